@@ -5,30 +5,35 @@
 // (fsi_asm_*).
 //
 // Per cell and quadrature point, with F = I + grad u, J = det F, A = grad(v) F^-1,
-// sigma_v = rho_f nu_f (A + A^T), dtt = dt theta, dto = dt (1 - theta):
-//   fluid cells   f0 = rho_f J [(v - v_old) - A (u - u_old) + dtt A v]      tested with phi
-//                 f1 = dtt J sigma_v F^-T - J p F^-T                         tested with grad phi
-//                 g0 = J tr(A)                                               tested with psi (Q1)
-//                 hm = grad(u) / J                                           tested with grad phi on mesh rows
-//                 (theta < 1: rho_f (1 - theta)(J_old - J)(v - v_old) + rho_f dto J_old A_old v_old in f0,
-//                  dto J_old sigma_v,old F_old^-T in f1: J^theta = theta J + (1 - theta) J_old)
+// X = J (mu (A + A^T) dtt - p I), mu = rho_f nu_f, dtt = dt theta, dto = dt (1 - theta),
+// J^theta = theta J + (1 - theta) J_old:
+//   fluid cells   f0 = rho_f [J^theta (v - v_old) - J A (u - u_old) + dtt J A v + dto J_old A_old v_old]
+//                 f1 = X F^-T + dto J_old sigma_v,old F_old^-T     f0 tested with phi, f1 with grad phi
+//                 g0 = J tr(A)                                     tested with psi (pressure)
+//                 hm = grad(u) / J                                 tested with grad phi on mesh rows
 //   solid cells   f0 = rho_s (v - v_old),  f1 = dtt F Sigma (+ dto F_old Sigma_old),
 //                 Sigma = 2 mu_s E + lambda_s tr(E) I,  E = (F^T F - I) / 2
-//                 k0 = (u - u_old) - dtt v (- dto v_old)                     tested with phi on u rows
-//   outflow face  c = -dtt rho_f nu_f J F^-T grad(v)^T F^-T n (n = e_0; theta < 1 adds the
-//   (fluid cells on x_0 = L_0)  previous level's term weighted dto)                  tested with phi on v rows
-// The Jacobian is the exact derivative of this discrete residual: every point
-// quantity is carried as a first-order dual number seeded along one local DOF,
-// so a CTA computes one chunk of columns of the element matrix.
+//                 k0 = (u - u_old) - dtt v (- dto v_old)           tested with phi on u rows
+//   outflow face  c = -dtt mu J A^T n', n' = F^-T e_0 (theta < 1 adds the previous level's
+//   (fluid cells on x_0 = L_0)  term weighted dto)                 tested with phi on v rows
+// The Jacobian is the exact derivative of this discrete residual, in closed form.  With
+// the deformed gradient G_b = F^-T grad phi_b of the trial function b, s_b = G_b . c,
+// c = dtt v - (u - u_old), the variations along component k of v or u at node b are
+//   dv:  dA_ij = delta_ik G_bj
+//        df0_i = delta_ik rho_f (J^theta phi_b + J s_b) + rho_f dtt J A_ik phi_b
+//        df1_ij = J dtt mu (delta_ik (F^-1 G_b)_j + G_bi F^-1_jk),          dg0 = J G_bk
+//   du:  dJ = J G_bk,  dA_ij = -A_ik G_bj,  dF^-1_jl = -F^-1_jk G_bl
+//        df0_i = G_bk rho_f J [theta (v - v_old) + A c]_i - A_ik rho_f J (s_b + phi_b)
+//        df1_ij = G_bk (X F^-T)_ij - (X G_b)_i F^-1_jk - J dtt mu (A_ik (F^-1 G_b)_j + G_bi (F^-1 A)_jk)
+//        dg0 = J (G_bk tr A - (A^T G_b)_k),  dhm_ij = (delta_ik d_j phi_b - (grad u)_ij G_bk) / J
+//   solid du: df1_ij = dtt [delta_ik (Sigma grad phi_b)_j + mu_s ((F F^T)_ik d_j phi_b + (F grad phi_b)_i F_kj)
+//                           + lambda_s (F grad phi_b)_k F_ij];  the mass terms are the same for every cell
 //
-// Work decomposition: one CTA per (cell, column chunk).  Phase 1: one thread per
-// (quadrature point, column) evaluates the point quantities above (value and one
-// derivative) into shared memory.  Phase 2: one thread per (element row, column)
-// sums its test-function weights over the points and adds the entry into the
-// global CSR values (binary search of the column in the row).  Cells are launched
-// colour by colour (the parities of their lattice coordinates): two cells of one
+// The GB300 retires 1.7 FP64 FMAs per clock and SM, so FP64 instructions are what an
+// assembly costs and the work is split to need few of them (see k_jacobian).  Cells are
+// launched colour by colour (the parities of their lattice coordinates): two cells of one
 // colour share no node, so the in-place additions never race, and the order in
-// which contributions reach an entry is fixed (deterministic, no atomics).
+// which contributions reach an entry is fixed (deterministic, no atomics on values).
 #include "../../include/fsi.h"
 #include "common.cuh"
 
@@ -39,35 +44,19 @@
 namespace fsi {
 namespace {
 
-// ------------------------------------------------------------------ first-order duals
-struct D1 {
-  double v, d;
-};
-__device__ __forceinline__ D1 dc(double a) { return {a, 0.0}; }
-__device__ __forceinline__ D1 operator+(D1 a, D1 b) { return {a.v + b.v, a.d + b.d}; }
-__device__ __forceinline__ D1 operator-(D1 a, D1 b) { return {a.v - b.v, a.d - b.d}; }
-__device__ __forceinline__ D1 operator*(D1 a, D1 b) { return {a.v * b.v, a.d * b.v + a.v * b.d}; }
-__device__ __forceinline__ D1 operator*(double s, D1 a) { return {s * a.v, s * a.d}; }
-__device__ __forceinline__ D1 operator+(D1 a, double s) { return {a.v + s, a.d}; }
-__device__ __forceinline__ D1 operator-(D1 a, double s) { return {a.v - s, a.d}; }
-__device__ __forceinline__ D1 inv(D1 b) {
-  const double r = 1.0 / b.v;
-  return {r, -b.d * r * r};
-}
-
 // Element shape: PD = 0 continuous Q1 pressure (2^D vertex functions), PD = 1 the
 // discontinuous P1 pressure of the paper's Q2-Q2-P1disc pair (D + 1 functions per cell).
 template <int D, int PD> struct Sh;
 template <int PD> struct Sh<2, PD> {
   static constexpr int NQ2 = 9, NQ1 = PD ? 3 : 4, NL = 36 + NQ1, NQP = 9, NFP = 3;
-  static constexpr int CHUNK = 40;   // columns per CTA (all)
+  static constexpr int JCELLS = 8;    // cells per CTA of the Jacobian: 36 units of a kind per cell, 9 full warps
+  static constexpr int RCELLS = 28;   // cells per CTA of the residual: 252 of 256 threads hold a point
 };
 template <int PD> struct Sh<3, PD> {
   static constexpr int NQ2 = 27, NQ1 = PD ? 4 : 8, NL = 162 + NQ1, NQP = 27, NFP = 9;
-  static constexpr int CHUNK = 17;   // 10 chunks of columns
+  static constexpr int JCELLS = 1;    // 243 units of a kind per cell: 7.6 of 8 warps
+  static constexpr int RCELLS = 4;
 };
-// shared slots per (point, column): f0 (D), f1 (D x D), then hm (D x D) and g0 (fluid) or k0 (solid)
-template <int D> constexpr int kSlots = D + D * D + D * D + 1;
 constexpr int kAsmThreads = 256;
 
 // Quadrature tables of one mesh (reference cell scaled by the cell size h).
@@ -79,6 +68,14 @@ struct Tables {
   const double* Nf;   // [NFP][NQ2]   outflow face x_0 = 1 of the reference cell
   const double* dNf;  // [NFP][NQ2][D]
   const double* wf;   // [NFP]
+  const double* M;    // [NQ2][NQ2]   sum_q w N_a N_b
+};
+// 1D factors of the Q2 basis at the three Gauss points: the basis function with lattice
+// index (a_0, a_1, a_2) is the product of N[q_d][a_d], its derivative along direction d
+// takes dN[d][q_d][a_d] there.  Kernel parameters, so FMAs read them as constants.
+struct Basis1 {
+  double N[3][3];
+  double dN[3][3][3];
 };
 
 struct Phys {
@@ -105,7 +102,7 @@ __device__ __forceinline__ int64_t colour_cell(const CellGeom& g, int64_t k, int
 }
 
 template <int D>
-__device__ __forceinline__ D1 det(const D1 (&F)[D][D]) {
+__device__ __forceinline__ double det(const double (&F)[D][D]) {
   if constexpr (D == 2) return F[0][0] * F[1][1] - F[0][1] * F[1][0];
   else
     return F[0][0] * (F[1][1] * F[2][2] - F[1][2] * F[2][1]) - F[0][1] * (F[1][0] * F[2][2] - F[1][2] * F[2][0]) +
@@ -113,378 +110,941 @@ __device__ __forceinline__ D1 det(const D1 (&F)[D][D]) {
 }
 // F^-1 = cof(F)^T / J
 template <int D>
-__device__ __forceinline__ void invert(const D1 (&F)[D][D], D1 iJ, D1 (&R)[D][D]) {
+__device__ __forceinline__ void invert(const double (&F)[D][D], double iJ, double (&R)[D][D]) {
   if constexpr (D == 2) {
-    R[0][0] = F[1][1] * iJ; R[0][1] = dc(0.0) - F[0][1] * iJ;
-    R[1][0] = dc(0.0) - F[1][0] * iJ; R[1][1] = F[0][0] * iJ;
+    R[0][0] = F[1][1] * iJ; R[0][1] = -F[0][1] * iJ;
+    R[1][0] = -F[1][0] * iJ; R[1][1] = F[0][0] * iJ;
   } else {
+#pragma unroll
     for (int i = 0; i < 3; ++i)
+#pragma unroll
       for (int j = 0; j < 3; ++j) {
         const int j1 = (j + 1) % 3, j2 = (j + 2) % 3, i1 = (i + 1) % 3, i2 = (i + 2) % 3;
-        // (F^-1)_ij = cofactor_ji / J
-        R[i][j] = (F[j1][i1] * F[j2][i2] - F[j1][i2] * F[j2][i1]) * iJ;
+        R[i][j] = (F[j1][i1] * F[j2][i2] - F[j1][i2] * F[j2][i1]) * iJ;   // cofactor_ji / J
       }
   }
 }
-
-// Previous-level point data (constants: no derivative).
+// C = A B
 template <int D>
-struct Old {
-  double vo[D], uo[D], Gvo[D][D], Fo[D][D], Jo, Fio[D][D];
+__device__ __forceinline__ void matmul(const double (&A)[D][D], const double (&B)[D][D], double (&C)[D][D]) {
+#pragma unroll
+  for (int i = 0; i < D; ++i)
+#pragma unroll
+    for (int j = 0; j < D; ++j) {
+      double s = A[i][0] * B[0][j];
+#pragma unroll
+      for (int k = 1; k < D; ++k) s += A[i][k] * B[k][j];
+      C[i][j] = s;
+    }
+}
+// C = A B^T
+template <int D>
+__device__ __forceinline__ void matmul_t(const double (&A)[D][D], const double (&B)[D][D], double (&C)[D][D]) {
+#pragma unroll
+  for (int i = 0; i < D; ++i)
+#pragma unroll
+    for (int j = 0; j < D; ++j) {
+      double s = A[i][0] * B[j][0];
+#pragma unroll
+      for (int k = 1; k < D; ++k) s += A[i][k] * B[j][k];
+      C[i][j] = s;
+    }
+}
+
+// Doubles that order as unsigned 64-bit integers (for atomicMin on min det F).
+__host__ __device__ inline unsigned long long order_key(double x) {
+#ifdef __CUDA_ARCH__
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+#else
+  unsigned long long b;
+  std::memcpy(&b, &x, 8);
+#endif
+  return (b >> 63) ? ~b : b | 0x8000000000000000ull;
+}
+inline double order_value(unsigned long long k) {
+  const unsigned long long b = (k >> 63) ? k & 0x7FFFFFFFFFFFFFFFull : ~k;
+  double x;
+  std::memcpy(&x, &b, 8);
+  return x;
+}
+
+// Scalars at a point, in the order they are interpolated: v (D), u (D), grad v (D x D),
+// grad u (D x D), then of the previous level v (D), u (D) and, for theta < 1, grad u, grad v.
+template <int D>
+struct Raw {
+  static constexpr int v = 0, u = D, Gv = 2 * D, Gu = 2 * D + D * D, vo = 2 * D + 2 * D * D, uo = vo + D,
+                       Guo = uo + D, Gvo = Guo + D * D, kNow = Guo, kAll = Gvo + D * D;
 };
 
-template <int D>
-__device__ __forceinline__ void old_point(const double* N, const double* dN, const double* Vo, const double* Uo,
-                                          bool need_grad, Old<D>& o) {
-  constexpr int NQ2 = Sh<D, 0>::NQ2;
-  for (int i = 0; i < D; ++i) {
-    double a = 0.0, b = 0.0;
-    for (int k = 0; k < NQ2; ++k) { a += N[k] * Vo[k * D + i]; b += N[k] * Uo[k * D + i]; }
-    o.vo[i] = a; o.uo[i] = b;
+// Quantity r of point pt (of the face when face) of an element with values U and Uold.
+template <int D, int PD>
+__device__ __forceinline__ double interpolate(const Tables& T, bool face, int pt, int r, const double* U,
+                                              const double* Uo) {
+  constexpr int NQ2 = Sh<D, PD>::NQ2;
+  const double* N = face ? T.Nf + pt * NQ2 : T.N + pt * NQ2;
+  const double* dN = face ? T.dNf + pt * NQ2 * D : T.dN + pt * NQ2 * D;
+  using R = Raw<D>;
+  const double* w;
+  const double* x;
+  int ws = 1;
+  if (r < R::Gv) {
+    w = N; x = U + (r < R::u ? r : NQ2 * D + r - R::u);
+  } else if (r < R::vo) {
+    const bool gu = r >= R::Gu;
+    const int e = r - (gu ? R::Gu : R::Gv);
+    w = dN + e % D; ws = D; x = U + (gu ? NQ2 * D : 0) + e / D;
+  } else if (r < R::Guo) {
+    w = N; x = Uo + (r < R::uo ? r - R::vo : NQ2 * D + r - R::uo);
+  } else {
+    const bool gv = r >= R::Gvo;
+    const int e = r - (gv ? R::Gvo : R::Guo);
+    w = dN + e % D; ws = D; x = Uo + (gv ? 0 : NQ2 * D) + e / D;
   }
-  o.Jo = 1.0;
-  if (!need_grad) return;
+  double s = 0.0;
+#pragma unroll 9
+  for (int k = 0; k < NQ2; ++k) s += w[k * ws] * x[k * D];
+  return s;
+}
+
+template <int D>
+__device__ __forceinline__ void read_mat(const double* p, double (&M)[D][D]) {
+#pragma unroll
   for (int i = 0; i < D; ++i)
-    for (int j = 0; j < D; ++j) {
-      double gv = 0.0, gu = 0.0;
-      for (int k = 0; k < NQ2; ++k) { gv += dN[k * D + j] * Vo[k * D + i]; gu += dN[k * D + j] * Uo[k * D + i]; }
-      o.Gvo[i][j] = gv;
-      o.Fo[i][j] = gu + (i == j ? 1.0 : 0.0);
-    }
-  D1 Fd[D][D], Rd[D][D];
-  for (int i = 0; i < D; ++i) for (int j = 0; j < D; ++j) Fd[i][j] = dc(o.Fo[i][j]);
-  const D1 J = det<D>(Fd);
-  o.Jo = J.v;
-  invert<D>(Fd, inv(J), Rd);
-  for (int i = 0; i < D; ++i) for (int j = 0; j < D; ++j) o.Fio[i][j] = Rd[i][j].v;
+#pragma unroll
+    for (int j = 0; j < D; ++j) M[i][j] = p[i * D + j];
 }
-
-// v, u, grad v, grad u at a point as duals seeded along local DOF `dir` (-1: none)
 template <int D>
-__device__ __forceinline__ void fields(const double* N, const double* dN, const double* U, int dir, D1 (&v)[D],
-                                       D1 (&u)[D], D1 (&Gv)[D][D], D1 (&Gu)[D][D]) {
-  constexpr int NQ2 = Sh<D, 0>::NQ2;
-  for (int i = 0; i < D; ++i) {
-    double a = 0.0, b = 0.0;
-    for (int k = 0; k < NQ2; ++k) { a += N[k] * U[k * D + i]; b += N[k] * U[NQ2 * D + k * D + i]; }
-    v[i] = dc(a); u[i] = dc(b);
-    for (int j = 0; j < D; ++j) {
-      double gv = 0.0, gu = 0.0;
-      for (int k = 0; k < NQ2; ++k) { gv += dN[k * D + j] * U[k * D + i]; gu += dN[k * D + j] * U[NQ2 * D + k * D + i]; }
-      Gv[i][j] = dc(gv); Gu[i][j] = dc(gu);
-    }
-  }
-  if (dir >= 0 && dir < 2 * NQ2 * D) {
-    const bool isv = dir < NQ2 * D;
-    const int l = isv ? dir : dir - NQ2 * D;
-    const int a = l / D, i = l % D;
-    if (isv) {
-      v[i].d = N[a];
-      for (int j = 0; j < D; ++j) Gv[i][j].d = dN[a * D + j];
-    } else {
-      u[i].d = N[a];
-      for (int j = 0; j < D; ++j) Gu[i][j].d = dN[a * D + j];
-    }
-  }
+__device__ __forceinline__ void write_mat(double* p, double s, const double (&M)[D][D]) {
+#pragma unroll
+  for (int i = 0; i < D; ++i)
+#pragma unroll
+    for (int j = 0; j < D; ++j) p[i * D + j] = s * M[i][j];
+}
+// F = I + grad u
+template <int D>
+__device__ __forceinline__ void read_F(const double* gu, double (&F)[D][D]) {
+  read_mat<D>(gu, F);
+#pragma unroll
+  for (int i = 0; i < D; ++i) F[i][i] += 1.0;
 }
 
-template <int D, int PD, bool JAC>
-__global__ void __launch_bounds__(kAsmThreads) k_assemble(CellGeom geom, int chunk0_stride, Tables T, Phys P,
+// ====================================================================== residual
+// One CTA takes RCELLS cells of a colour.  All threads interpolate (one scalar of one
+// point per step), then one thread per point forms the point fluxes, then one thread per
+// element row sums its test function over the points.  2D 256x128: about 3,000 FP64
+// instructions per cell.  256x128 P1disc: 0.37 ms.  An earlier form gave each cell a CTA of
+// its own, whose phase of point fluxes kept 12 of 256 threads busy: 3.35 ms.
+template <int D> constexpr int kFlux = 2 * D + 2 * D * D + 1;   // f0, f1, hm, k0 (D), g0
+template <int D, int PD>
+struct ResSmem {
+  using E = Sh<D, PD>;
+  double U[E::RCELLS][E::NL];
+  double Uo[E::RCELLS][2 * E::NQ2 * D];
+  double raw[E::RCELLS][E::NQP + E::NFP][Raw<D>::kAll];   // the point's fluxes replace its raw values
+  int gdof[E::RCELLS][E::NL];
+  unsigned flags[E::RCELLS];
+  unsigned long long minkey;
+};
+
+template <int D, int PD>
+__global__ void __launch_bounds__(kAsmThreads) k_residual(CellGeom geom, int64_t ncol, Tables T, Phys P,
                                                           const int* __restrict__ cell_dof,
                                                           const unsigned* __restrict__ cell_flags,
-                                                          const int64_t* __restrict__ rowptr,
-                                                          const int* __restrict__ colind,
                                                           const unsigned char* __restrict__ row_fixed,
                                                           const double* __restrict__ Ug,
-                                                          const double* __restrict__ Uold,
-                                                          double* __restrict__ out, double* __restrict__ cell_minJ,
-                                                          int* __restrict__ err) {
+                                                          const double* __restrict__ Uold, double* __restrict__ out,
+                                                          unsigned long long* __restrict__ minkey) {
   using E = Sh<D, PD>;
-  constexpr int NQ2 = E::NQ2, NQ1 = E::NQ1, NL = E::NL, NQP = E::NQP, NFP = E::NFP;
-  constexpr int S = kSlots<D>;
-  constexpr int NPT = NQP + NFP;
-  constexpr int C = JAC ? E::CHUNK : 1;
-  extern __shared__ double smem[];
-  double* U = smem;                        // NL
-  double* Vo = U + NL;                     // NQ2 * D
-  double* Uo = Vo + NQ2 * D;               // NQ2 * D
-  double* Q = Uo + NQ2 * D;                // [NPT][C][S]
-  __shared__ int gdof[NL];
-  __shared__ double jmin[kAsmThreads / 32];
-
-  const int64_t k = blockIdx.x / chunk0_stride;
-  const int chunk = blockIdx.x % chunk0_stride;
-  int c[3] = {0, 0, 0};
-  const int64_t cell = colour_cell<D>(geom, k, c);
-  const unsigned flags = cell_flags[cell];
-  const bool solid = flags & 1u;
-  const bool outflow = (flags & 2u) && !solid;
+  using R = Raw<D>;
+  constexpr int NQ2 = E::NQ2, NQ1 = E::NQ1, NL = E::NL, NQP = E::NQP, NFP = E::NFP, NV = NQ2 * D;
+  constexpr int F0 = 0, F1 = D, HM = D + D * D, K0 = HM + D * D, G0 = K0 + D;
+  static_assert(G0 + 1 == kFlux<D> && kFlux<D> <= R::kAll, "fluxes fit the raw slots");
+  extern __shared__ __align__(16) unsigned char asm_smem[];
+  ResSmem<D, PD>& S = *reinterpret_cast<ResSmem<D, PD>*>(asm_smem);
+  const int64_t k0 = (int64_t)blockIdx.x * E::RCELLS;
+  const int nc = (int)(ncol - k0 < E::RCELLS ? ncol - k0 : E::RCELLS);
   const bool prev = P.theta != 1.0;
-  const double dtt = P.dt * P.theta, dto = P.dt * (1.0 - P.theta);
-  const double mu = P.rho_f * P.nu_f;
-  for (int t = threadIdx.x; t < NL; t += blockDim.x) {
-    const int g = cell_dof[cell * NL + t];
-    gdof[t] = g;
-    U[t] = Ug[g];
+  const double dtt = P.dt * P.theta, dto = P.dt * (1.0 - P.theta), mu = P.rho_f * P.nu_f;
+  for (int t = threadIdx.x; t < nc * NL; t += blockDim.x) {
+    const int ce = t / NL, l = t % NL;
+    int cc[3];
+    const int64_t cell = colour_cell<D>(geom, k0 + ce, cc);
+    const int g = cell_dof[cell * NL + l];
+    S.gdof[ce][l] = g;
+    S.U[ce][l] = Ug[g];
+    if (l < 2 * NV) S.Uo[ce][l] = Uold ? Uold[g] : 0.0;
+    if (l == 0) S.flags[ce] = cell_flags[cell];
   }
-  for (int t = threadIdx.x; t < NQ2 * D; t += blockDim.x) {
-    Vo[t] = Uold ? Uold[cell_dof[cell * NL + t]] : 0.0;
-    Uo[t] = Uold ? Uold[cell_dof[cell * NL + NQ2 * D + t]] : 0.0;
+  if (threadIdx.x == 0) S.minkey = ~0ull;
+  __syncthreads();
+  const int nr = prev ? R::kAll : R::kNow;
+  for (int t = threadIdx.x; t < nc * NQP * nr; t += blockDim.x) {
+    const int ce = t / (NQP * nr), e = t % (NQP * nr);
+    S.raw[ce][e / nr][e % nr] = interpolate<D, PD>(T, false, e / nr, e % nr, S.U[ce], S.Uo[ce]);
   }
+  for (int ce = 0; ce < nc; ++ce)
+    if ((S.flags[ce] & 3u) == 2u)
+      for (int e = threadIdx.x; e < NFP * nr; e += blockDim.x)
+        S.raw[ce][NQP + e / nr][e % nr] = interpolate<D, PD>(T, true, e / nr, e % nr, S.U[ce], S.Uo[ce]);
   __syncthreads();
 
-  // ---- phase 1: point quantities
   double my_min = 1e300;
-  for (int idx = threadIdx.x; idx < NPT * C; idx += blockDim.x) {
-    const int pt = idx / C, cc = idx % C;
-    const int dir = JAC ? chunk * C + cc : -1;
-    double* q = Q + ((size_t)pt * C + cc) * S;
-    if (JAC && dir >= NL) {
-      for (int s = 0; s < S; ++s) q[s] = 0.0;
+  for (int t = threadIdx.x; t < nc * (NQP + NFP); t += blockDim.x) {
+    // volume points first, so that the cells' points fill whole warps
+    const bool face = t >= nc * NQP;
+    const int ce = face ? (t - nc * NQP) / NFP : t / NQP;
+    const int pt = face ? NQP + (t - nc * NQP) % NFP : t % NQP;
+    const bool solid = S.flags[ce] & 1u;
+    if (face && (S.flags[ce] & 3u) != 2u) continue;
+    double* q = S.raw[ce][pt];
+    double F[D][D], Gv[D][D], Fo[D][D], Gvo[D][D], v[D], dv[D], du[D], vo[D];
+    read_F<D>(q + R::Gu, F);
+    read_mat<D>(q + R::Gv, Gv);
+    if (prev) { read_F<D>(q + R::Guo, Fo); read_mat<D>(q + R::Gvo, Gvo); }
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      v[i] = q[R::v + i];
+      vo[i] = q[R::vo + i];
+      dv[i] = v[i] - vo[i];
+      du[i] = q[R::u + i] - q[R::uo + i];
+    }
+    const double J = det<D>(F);
+    if (!face && J < my_min) my_min = J;
+    if (solid) {
+      // E = (F^T F - I) / 2, f1 = w F Sigma
+      auto stress = [&](const double (&X)[D][D], double w, double (&O)[D][D]) {
+        double C[D][D], tr = 0.0;
+#pragma unroll
+        for (int i = 0; i < D; ++i)
+#pragma unroll
+          for (int j = 0; j < D; ++j) {
+            double s = X[0][i] * X[0][j];
+#pragma unroll
+            for (int m = 1; m < D; ++m) s += X[m][i] * X[m][j];
+            C[i][j] = 0.5 * (s - (i == j ? 1.0 : 0.0));
+          }
+#pragma unroll
+        for (int i = 0; i < D; ++i) tr += C[i][i];
+#pragma unroll
+        for (int i = 0; i < D; ++i)
+#pragma unroll
+          for (int j = 0; j < D; ++j) C[i][j] = w * (2.0 * P.mu_s * C[i][j] + (i == j ? P.lambda_s * tr : 0.0));
+        matmul<D>(X, C, O);
+      };
+      double f1[D][D], fo[D][D];
+      stress(F, dtt, f1);
+      if (prev) stress(Fo, dto, fo);
+#pragma unroll
+      for (int i = 0; i < D; ++i) {
+        q[F0 + i] = P.rho_s * dv[i];
+        q[K0 + i] = du[i] - dtt * v[i] - (prev ? dto * vo[i] : 0.0);
+#pragma unroll
+        for (int j = 0; j < D; ++j) q[F1 + i * D + j] = f1[i][j] + (prev ? fo[i][j] : 0.0);
+      }
       continue;
     }
-    const bool face = pt >= NQP;
-    if (face && !outflow) continue;
-    const double* N = face ? T.Nf + (pt - NQP) * NQ2 : T.N + pt * NQ2;
-    const double* dN = face ? T.dNf + (size_t)(pt - NQP) * NQ2 * D : T.dN + (size_t)pt * NQ2 * D;
-    D1 v[D], u[D], Gv[D][D], Gu[D][D];
-    fields<D>(N, dN, U, dir, v, u, Gv, Gu);
-    D1 F[D][D];
-    for (int i = 0; i < D; ++i) for (int j = 0; j < D; ++j) F[i][j] = Gu[i][j] + (i == j ? 1.0 : 0.0);
-    const D1 J = det<D>(F);
-    if (!face && J.v < my_min) my_min = J.v;
-    Old<D> o;
-    old_point<D>(N, dN, Vo, Uo, prev, o);
-    auto put = [&](int s, D1 x) { q[s] = JAC ? x.d : x.v; };
+    double Fi[D][D], A[D][D], Fio[D][D], Ao[D][D], Jo = 1.0;
+    const double iJ = 1.0 / J;
+    invert<D>(F, iJ, Fi);
+    matmul<D>(Gv, Fi, A);
+    if (prev) {
+      Jo = det<D>(Fo);
+      invert<D>(Fo, 1.0 / Jo, Fio);
+      matmul<D>(Gvo, Fio, Ao);
+    }
     if (face) {
-      // c_i = -dtt mu J sum_j Fi_ji t_j,  t_j = sum_k (grad v)_kj Fi_0k
-      D1 Fi[D][D];
-      invert<D>(F, inv(J), Fi);
-      D1 t[D];
-      for (int j = 0; j < D; ++j) {
-        D1 s = dc(0.0);
-        for (int kk = 0; kk < D; ++kk) s = s + Gv[kk][j] * Fi[0][kk];
-        t[j] = s;
-      }
-      double to[D] = {};
-      if (prev)
-        for (int j = 0; j < D; ++j) {
-          double s = 0.0;
-          for (int kk = 0; kk < D; ++kk) s += o.Gvo[kk][j] * o.Fio[0][kk];
-          to[j] = s;
-        }
+#pragma unroll
       for (int i = 0; i < D; ++i) {
-        D1 b = dc(0.0);
-        for (int j = 0; j < D; ++j) b = b + Fi[j][i] * t[j];
-        D1 cval = (-dtt * mu) * (J * b);
-        if (prev) {
-          double s = 0.0;
-          for (int j = 0; j < D; ++j) s += o.Fio[j][i] * to[j];
-          cval = cval + (-dto * mu * o.Jo * s);
-        }
-        put(i, cval);
+        double s = 0.0, so = 0.0;
+#pragma unroll
+        for (int m = 0; m < D; ++m) s += A[m][i] * Fi[0][m];
+        if (prev)
+#pragma unroll
+          for (int m = 0; m < D; ++m) so += Ao[m][i] * Fio[0][m];
+        q[F0 + i] = -dtt * mu * J * s - (prev ? dto * mu * Jo * so : 0.0);
       }
       continue;
     }
-    if (!solid) {
-      D1 Fi[D][D];
-      const D1 iJ = inv(J);
-      invert<D>(F, iJ, Fi);
-      const double* Np = T.Np + pt * NQ1;
-      D1 p = dc(0.0);
-      for (int a = 0; a < NQ1; ++a) p = p + Np[a] * dc(U[2 * NQ2 * D + a]);
-      if (dir >= 2 * NQ2 * D) p.d = Np[dir - 2 * NQ2 * D];
-      D1 A[D][D];
+    double p = 0.0;
+#pragma unroll
+    for (int a = 0; a < NQ1; ++a) p += T.Np[pt * NQ1 + a] * S.U[ce][2 * NV + a];
+    double X[D][D], f1[D][D], hm[D][D], trA = 0.0;
+    const double m = dtt * mu * J;
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      trA += A[i][i];
+#pragma unroll
+      for (int j = 0; j < D; ++j) {
+        X[i][j] = m * (A[i][j] + A[j][i]) - (i == j ? J * p : 0.0);
+        hm[i][j] = q[R::Gu + i * D + j] * iJ;
+      }
+    }
+    matmul_t<D>(X, Fi, f1);
+    if (prev) {
+      const double mo = dto * mu * Jo;
+      double Xo[D][D], fo[D][D];
+#pragma unroll
       for (int i = 0; i < D; ++i)
-        for (int j = 0; j < D; ++j) {
-          D1 s = dc(0.0);
-          for (int kk = 0; kk < D; ++kk) s = s + Gv[i][kk] * Fi[kk][j];
-          A[i][j] = s;
-        }
-      double Ao[D][D] = {};
+#pragma unroll
+        for (int j = 0; j < D; ++j) Xo[i][j] = mo * (Ao[i][j] + Ao[j][i]);
+      matmul_t<D>(Xo, Fio, fo);
+#pragma unroll
+      for (int i = 0; i < D; ++i)
+#pragma unroll
+        for (int j = 0; j < D; ++j) f1[i][j] += fo[i][j];
+    }
+    const double Jt = prev ? P.theta * J + (1.0 - P.theta) * Jo : J;
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      double ac = 0.0, co = 0.0;
+#pragma unroll
+      for (int j = 0; j < D; ++j) ac += A[i][j] * (dtt * v[j] - du[j]);
       if (prev)
-        for (int i = 0; i < D; ++i)
-          for (int j = 0; j < D; ++j) {
-            double s = 0.0;
-            for (int kk = 0; kk < D; ++kk) s += o.Gvo[i][kk] * o.Fio[kk][j];
-            Ao[i][j] = s;
-          }
-      for (int i = 0; i < D; ++i) {
-        const D1 dv = v[i] - o.vo[i];
-        D1 s = dv;
-        for (int j = 0; j < D; ++j) s = s - A[i][j] * (u[j] - o.uo[j]) + dtt * (A[i][j] * v[j]);
-        D1 f0 = (P.rho_f * J) * s;
-        if (prev) {
-          double co = 0.0;
-          for (int j = 0; j < D; ++j) co += Ao[i][j] * o.vo[j];
-          f0 = f0 + (P.rho_f * (1.0 - P.theta)) * (o.Jo * dv - J * dv) + P.rho_f * dto * o.Jo * co;
-        }
-        put(i, f0);
-      }
-      for (int i = 0; i < D; ++i)
-        for (int j = 0; j < D; ++j) {
-          D1 s = dc(0.0);
-          for (int kk = 0; kk < D; ++kk) s = s + (A[i][kk] + A[kk][i]) * Fi[j][kk];
-          D1 f1 = (dtt * mu) * (J * s) - (J * p) * Fi[j][i];
-          if (prev) {
-            double so = 0.0;
-            for (int kk = 0; kk < D; ++kk) so += (Ao[i][kk] + Ao[kk][i]) * o.Fio[j][kk];
-            f1 = f1 + dto * mu * o.Jo * so;
-          }
-          put(D + i * D + j, f1);
-          put(D + D * D + i * D + j, Gu[i][j] * iJ);     // mesh motion: grad(u) / J
-        }
-      D1 trA = dc(0.0);
-      for (int i = 0; i < D; ++i) trA = trA + A[i][i];
-      put(D + 2 * D * D, J * trA);
-    } else {
-      D1 E[D][D];
-      for (int i = 0; i < D; ++i)
-        for (int j = 0; j < D; ++j) {
-          D1 s = dc(0.0);
-          for (int kk = 0; kk < D; ++kk) s = s + F[kk][i] * F[kk][j];
-          E[i][j] = 0.5 * (s - (i == j ? 1.0 : 0.0));
-        }
-      D1 trE = dc(0.0);
-      for (int i = 0; i < D; ++i) trE = trE + E[i][i];
-      D1 Sg[D][D];
-      for (int i = 0; i < D; ++i)
-        for (int j = 0; j < D; ++j) {
-          Sg[i][j] = (2.0 * P.mu_s) * E[i][j];
-          if (i == j) Sg[i][j] = Sg[i][j] + P.lambda_s * trE;
-        }
-      double So[D][D] = {};
-      if (prev) {
-        double Eo[D][D], trEo = 0.0;
-        for (int i = 0; i < D; ++i)
-          for (int j = 0; j < D; ++j) {
-            double s = 0.0;
-            for (int kk = 0; kk < D; ++kk) s += o.Fo[kk][i] * o.Fo[kk][j];
-            Eo[i][j] = 0.5 * (s - (i == j ? 1.0 : 0.0));
-          }
-        for (int i = 0; i < D; ++i) trEo += Eo[i][i];
-        for (int i = 0; i < D; ++i)
-          for (int j = 0; j < D; ++j) So[i][j] = 2.0 * P.mu_s * Eo[i][j] + (i == j ? P.lambda_s * trEo : 0.0);
-      }
-      for (int i = 0; i < D; ++i) {
-        put(i, P.rho_s * (v[i] - o.vo[i]));
-        D1 k0 = (u[i] - o.uo[i]) - dtt * v[i];
-        if (prev) k0 = k0 - dto * o.vo[i];
-        put(D + D * D + i, k0);
-        for (int j = 0; j < D; ++j) {
-          D1 s = dc(0.0);
-          for (int kk = 0; kk < D; ++kk) s = s + F[i][kk] * Sg[kk][j];
-          D1 f1 = dtt * s;
-          if (prev) {
-            double so = 0.0;
-            for (int kk = 0; kk < D; ++kk) so += o.Fo[i][kk] * So[kk][j];
-            f1 = f1 + dto * so;
-          }
-          put(D + i * D + j, f1);
-        }
-      }
+#pragma unroll
+        for (int j = 0; j < D; ++j) co += Ao[i][j] * vo[j];
+      q[F0 + i] = P.rho_f * (Jt * dv[i] + J * ac + (prev ? dto * Jo * co : 0.0));
     }
+    write_mat<D>(q + F1, 1.0, f1);
+    write_mat<D>(q + HM, 1.0, hm);
+    q[G0] = J * trA;
   }
-  // smallest J of the cell's volume points (one value per cell, from the first chunk)
-  for (int off = 16; off > 0; off >>= 1) my_min = fmin(my_min, __shfl_down_sync(0xffffffffu, my_min, off));
-  if ((threadIdx.x & 31) == 0) jmin[threadIdx.x >> 5] = my_min;
+  if (my_min < 1e300) atomicMin(&S.minkey, order_key(my_min));
   __syncthreads();
-  if (threadIdx.x == 0 && chunk == 0) {
-    double m = jmin[0];
-    for (int wi = 1; wi < (int)(blockDim.x >> 5); ++wi) m = fmin(m, jmin[wi]);
-    cell_minJ[cell] = m;
-  }
+  if (threadIdx.x == 0 && S.minkey != ~0ull) atomicMin(minkey, S.minkey);
 
-  // ---- phase 2: element rows x columns, summed over the points
-  const int nentries = NL * C;
-  for (int e = threadIdx.x; e < nentries; e += blockDim.x) {
-    const int r = e / C, cc = e % C;
-    const int col = JAC ? chunk * C + cc : -1;
-    if (JAC && col >= NL) continue;
-    const int gr = gdof[r];
-    if (row_fixed[gr]) continue;
-    const bool prow = r >= 2 * NQ2 * D;
-    const bool urow = !prow && r >= NQ2 * D;
-    if (solid && prow) continue;                          // solid cells own no pressure rows
-    int a = 0, i = 0;
-    if (!prow) { const int l = urow ? r - NQ2 * D : r; a = l / D; i = l % D; }
-    if (!solid && urow && !((flags >> (2 + a)) & 1u)) continue;   // fluid cell: mesh rows only
-    if (JAC) {
-      const int gc = gdof[col];
-      if (row_fixed[gc] || (solid && col >= 2 * NQ2 * D)) continue;
-    }
+  for (int t = threadIdx.x; t < nc * NL; t += blockDim.x) {
+    const int ce = t / NL, r = t % NL;
+    const int gr = S.gdof[ce][r];
+    const unsigned flags = S.flags[ce];
+    const bool solid = flags & 1u, prow = r >= 2 * NV, urow = !prow && r >= NV;
+    if (row_fixed[gr] || (solid && prow)) continue;              // solid cells own no pressure rows
+    const int l = urow ? r - NV : r, a = l / D, i = l % D;
+    if (!solid && urow && !((flags >> (2 + a)) & 1u)) continue;  // fluid cell: mesh rows only
     double acc = 0.0;
     for (int pt = 0; pt < NQP; ++pt) {
-      const double* q = Q + ((size_t)pt * C + cc) * S;
-      const double w = T.w[pt];
+      const double* q = S.raw[ce][pt];
+      const double* dN = T.dN + (pt * NQ2 + a) * D;
+      double s;
       if (prow) {
-        acc += w * T.Np[pt * NQ1 + (r - 2 * NQ2 * D)] * q[D + 2 * D * D];
-      } else if (!urow) {
-        double s = T.N[pt * NQ2 + a] * q[i];
-        for (int j = 0; j < D; ++j) s += T.dN[((size_t)pt * NQ2 + a) * D + j] * q[D + i * D + j];
-        acc += w * s;
-      } else if (solid) {
-        acc += w * T.N[pt * NQ2 + a] * q[D + D * D + i];
+        s = T.Np[pt * NQ1 + (r - 2 * NV)] * q[G0];
+      } else if (!urow || solid) {
+        s = T.N[pt * NQ2 + a] * q[(urow ? K0 : F0) + i];
+        if (!urow)
+#pragma unroll
+          for (int j = 0; j < D; ++j) s += dN[j] * q[F1 + i * D + j];
       } else {
-        double s = 0.0;
-        for (int j = 0; j < D; ++j) s += T.dN[((size_t)pt * NQ2 + a) * D + j] * q[D + D * D + i * D + j];
-        acc += w * s;
+        s = dN[0] * q[HM + i * D];
+#pragma unroll
+        for (int j = 1; j < D; ++j) s += dN[j] * q[HM + i * D + j];
       }
+      acc += T.w[pt] * s;
     }
-    if (outflow && !urow && !prow)
-      for (int f = 0; f < NFP; ++f) acc += T.wf[f] * T.Nf[f * NQ2 + a] * Q[((size_t)(NQP + f) * C + cc) * S + i];
-    if (!JAC) {
-      out[gr] += acc;
+    if ((flags & 3u) == 2u && !urow && !prow)
+      for (int f = 0; f < NFP; ++f) acc += T.wf[f] * T.Nf[f * NQ2 + a] * S.raw[ce][NQP + f][F0 + i];
+    out[gr] += acc;
+  }
+}
+
+// ====================================================================== Jacobian
+// One CTA takes JCELLS cells of a colour.  What the variations above need is tabulated
+// in shared memory once per point (PT slots) and once per (point, trial node) (TR slots,
+// quadrature weight folded in).  A unit of work is one trial component (b, k) against
+// one test component i: a thread forms the unit's f0 and reference flux f1 at a line of
+// three points at a time and contracts them with the 3^D test functions by sum
+// factorisation (direction 0, then 1, then 2; the functions are products of 1D factors):
+// 729 FMAs per 3D unit instead of 2,916 for point x test function, 135 instead of 243
+// in 2D, and 4 to 14 more per point for the fields.  Neighbouring lanes take neighbouring
+// (b, k), so their additions into a CSR row are contiguous along a lattice line.
+// Positions in the CSR rows are searched once per (row, trial node), not per entry.
+// Measured, against one dual-number evaluation per point and column with a search per
+// entry: 256x128 16.17 -> 2.63 ms, 32x16x16 at theta = 1/2 197.0 -> 14.3 ms (0.77e6 FP64
+// FMAs per fluid cell; all cells take 9.9 ms at the FP64 pipe's measured 0.529e12 per second).
+template <int D>
+struct Pt {   // per point
+  static constexpr int Fi = 0, A = D * D, Fim = 2 * D * D, FA = 3 * D * D, PX = 4 * D * D, GuJ = 5 * D * D,
+                       e = 6 * D * D, wJ = e + D, trA = wJ + 1, wJi = trA + 1, kN = wJi + 1;
+  // solid cells: F, w dtt mu F, w dtt lambda F, w dtt mu F F^T, w dtt Sigma
+  static constexpr int sF = 0, smF = D * D, slF = 2 * D * D, sB = 3 * D * D, sS = 4 * D * D;
+  // face points: F^-1, A, A^T n', -w m J
+  static constexpr int fFi = 0, fA = D * D, fq = 2 * D * D, fm = fq + D;
+};
+template <int D>
+struct Tr {   // per (point, trial node)
+  static constexpr int G = 0, FG = D, XG = 2 * D, al = 3 * D, nb = al + 1, r = nb + 1, kN = r + 1;
+  // solid cells: F grad phi, w dtt Sigma grad phi, grad phi; mesh rows: w grad phi / J in FG
+  static constexpr int sf = 0, sS = D, sd = 2 * D;
+};
+constexpr unsigned short kNoPos = 0xFFFFu;
+
+template <int D, int PD>
+struct JacCell {
+  using E = Sh<D, PD>;
+  static constexpr int NC = 2 * E::NQ2 + E::NQ1;    // trial nodes: v, u, pressure functions
+  double U[E::NL];
+  double Uo[2 * E::NQ2 * D];
+  double pt[E::NQP][Pt<D>::kN];
+  double face[E::NFP][2 * D * D + D + 1];
+  double tr[E::NQP][E::NQ2][Tr<D>::kN];              // the raw point values first
+  long long row[E::NL];                              // first CSR entry of each local row, -1: not assembled
+  int gdof[E::NL];
+  unsigned flags;
+  unsigned short pos[E::NL][NC];                     // of the node's first component within the row
+  unsigned char cfix[E::NL];
+};
+template <int D, int PD>
+struct JacSmem {
+  JacCell<D, PD> c[Sh<D, PD>::JCELLS];
+  unsigned long long minkey;
+};
+
+// acc += the contraction of one unit's point fields with the test functions:
+// field(q, f0, f1) gives the fields of point q.  HAS0: f0 is not identically zero.
+template <int D, bool HAS0, class Field>
+__device__ __forceinline__ void contract(const Basis1& B, const Field& field, double (&acc)[D == 2 ? 9 : 27]) {
+#pragma unroll
+  for (int t = 0; t < (D == 2 ? 9 : 27); ++t) acc[t] = 0.0;
+#pragma unroll 1
+  for (int qz = 0; qz < (D == 2 ? 1 : 3); ++qz) {
+    double h[9], hz[9];   // sums over directions 0 and 1, for the value and the derivative in direction 2
+    if constexpr (D == 3)
+#pragma unroll
+      for (int t = 0; t < 9; ++t) h[t] = hz[t] = 0.0;
+#pragma unroll
+    for (int qy = 0; qy < 3; ++qy) {
+      double t0[3] = {0.0, 0.0, 0.0}, ty[3] = {0.0, 0.0, 0.0}, tz[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+      for (int qx = 0; qx < 3; ++qx) {
+        double f0 = 0.0, f1[D];
+        field(qx + 3 * qy + 9 * qz, f0, f1);
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+          if (HAS0) t0[ax] = fma(B.N[qx][ax], f0, t0[ax]);
+          t0[ax] = fma(B.dN[0][qx][ax], f1[0], t0[ax]);
+          ty[ax] = fma(B.N[qx][ax], f1[1], ty[ax]);
+          if constexpr (D == 3) tz[ax] = fma(B.N[qx][ax], f1[2], tz[ax]);
+        }
+      }
+#pragma unroll
+      for (int ay = 0; ay < 3; ++ay)
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+          double& o = D == 2 ? acc[3 * ay + ax] : h[3 * ay + ax];
+          o = fma(B.N[qy][ay], t0[ax], o);
+          o = fma(B.dN[1][qy][ay], ty[ax], o);
+          if constexpr (D == 3) hz[3 * ay + ax] = fma(B.N[qy][ay], tz[ax], hz[3 * ay + ax]);
+        }
+    }
+    if constexpr (D == 3) {
+#pragma unroll
+      for (int az = 0; az < 3; ++az)
+#pragma unroll
+        for (int t = 0; t < 9; ++t)
+          acc[9 * az + t] = fma(B.dN[2][qz][az], hz[t], fma(B.N[qz][az], h[t], acc[9 * az + t]));
+    }
+  }
+}
+
+// Position of column col in a CSR row of len sorted columns, or -1.
+__device__ __forceinline__ int find_col(const int* __restrict__ ci, int len, int col) {
+  int lo = 0, hi = len;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (__ldg(ci + mid) < col) lo = mid + 1; else hi = mid;
+  }
+  return lo < len && __ldg(ci + lo) == col ? lo : -1;
+}
+
+template <int D, int PD>
+__global__ void __launch_bounds__(kAsmThreads, 2) k_jacobian(CellGeom geom, int64_t ncol, Tables T,
+                                                             const __grid_constant__ Basis1 B, Phys P,
+                                                             const int* __restrict__ cell_dof,
+                                                             const unsigned* __restrict__ cell_flags,
+                                                             const int64_t* __restrict__ rowptr,
+                                                             const int* __restrict__ colind,
+                                                             const unsigned char* __restrict__ row_fixed,
+                                                             const double* __restrict__ Ug,
+                                                             const double* __restrict__ Uold,
+                                                             double* __restrict__ out,
+                                                             unsigned long long* __restrict__ minkey,
+                                                             int* __restrict__ err) {
+  using E = Sh<D, PD>;
+  using R = Raw<D>;
+  using C = JacCell<D, PD>;
+  constexpr int NQ2 = E::NQ2, NQ1 = E::NQ1, NL = E::NL, NQP = E::NQP, NFP = E::NFP, NV = NQ2 * D, NC = C::NC;
+  constexpr int UNITS = NQ2 * D * D;
+  static_assert(R::kAll <= NQ2 * Tr<D>::kN, "raw values fit a point's trial slots");
+  extern __shared__ __align__(16) unsigned char asm_smem[];
+  JacSmem<D, PD>& S = *reinterpret_cast<JacSmem<D, PD>*>(asm_smem);
+  const int64_t k0 = (int64_t)blockIdx.x * E::JCELLS;
+  const int nc = (int)(ncol - k0 < E::JCELLS ? ncol - k0 : E::JCELLS);
+  const bool prev = P.theta != 1.0;
+  const double dtt = P.dt * P.theta, mu = P.rho_f * P.nu_f;
+  for (int t = threadIdx.x; t < nc * NL; t += blockDim.x) {
+    C& c = S.c[t / NL];
+    const int l = t % NL;
+    int cc[3];
+    const int64_t cell = colour_cell<D>(geom, k0 + t / NL, cc);
+    const unsigned flags = cell_flags[cell];
+    const bool solid = flags & 1u, prow = l >= 2 * NV, urow = !prow && l >= NV;
+    const int g = cell_dof[cell * NL + l];
+    const bool fixed = row_fixed[g];
+    c.gdof[l] = g;
+    c.U[l] = Ug[g];
+    if (l < 2 * NV) c.Uo[l] = Uold ? Uold[g] : 0.0;
+    if (l == 0) c.flags = flags;
+    c.cfix[l] = fixed || (solid && prow);
+    const bool skip = fixed || (solid && prow) ||                            // solid cells own no pressure rows
+                      (!solid && urow && !((flags >> (2 + (l - NV) / D)) & 1u));   // fluid cells: mesh rows only
+    c.row[l] = skip ? -1 : rowptr[g];
+  }
+  if (threadIdx.x == 0) S.minkey = ~0ull;
+  __syncthreads();
+  // raw point values, in the trial slots of the point
+  const int nr = prev ? R::Gvo : R::kNow;
+  for (int t = threadIdx.x; t < nc * NQP * nr; t += blockDim.x) {
+    C& c = S.c[t / (NQP * nr)];
+    const int e = t % (NQP * nr);
+    c.tr[e / nr][0][e % nr] = interpolate<D, PD>(T, false, e / nr, e % nr, c.U, c.Uo);
+  }
+  // positions of the trial nodes in the rows (v and u rows of node a: the components' rows have equal
+  // patterns as a rule, so the first component's position is tried first)
+  for (int t = threadIdx.x; t < nc * NC * (2 * NQ2 + NQ1); t += blockDim.x) {
+    C& c = S.c[t / (NC * (2 * NQ2 + NQ1))];
+    const int e = t % (NC * (2 * NQ2 + NQ1)), rn = e / NC, cn = e % NC;
+    const int nrows = rn < 2 * NQ2 ? D : 1, r0 = rn < 2 * NQ2 ? rn * D : 2 * NV + rn - 2 * NQ2;
+    const int ncols = cn < 2 * NQ2 ? D : 1, col0 = c.gdof[cn < 2 * NQ2 ? cn * D : 2 * NV + cn - 2 * NQ2];
+    const bool solid = c.flags & 1u;
+    const bool urow = rn >= NQ2 && rn < 2 * NQ2;
+    if (!solid && urow && (cn < NQ2 || cn >= 2 * NQ2)) continue;             // mesh rows: u columns only
+    if (cn >= 2 * NQ2 && rn >= 2 * NQ2) continue;                            // no pressure-pressure coupling
+    int hint = -1;
+    for (int i = 0; i < nrows; ++i) {
+      const long long base = c.row[r0 + i];
+      unsigned short found = kNoPos;
+      if (base >= 0) {
+        const int len = (int)(rowptr[c.gdof[r0 + i] + 1] - base);
+        const int* ci = colind + base;
+        int p = hint >= 0 && hint < len && __ldg(ci + hint) == col0 ? hint : find_col(ci, len, col0);
+        if (p >= 0) {
+          hint = p;
+          bool all = p + ncols <= len && p < kNoPos;
+          for (int k = 1; k < ncols && all; ++k) all = __ldg(ci + p + k) == col0 + k;
+          if (all) found = (unsigned short)p;
+        }
+      }
+      c.pos[r0 + i][cn] = found;
+    }
+  }
+  __syncthreads();
+
+  // ---- point tables
+  double my_min = 1e300;
+  for (int t = threadIdx.x; t < nc * NQP; t += blockDim.x) {
+    C& c = S.c[t / NQP];
+    const int q = t % NQP;
+    const double* raw = c.tr[q][0];
+    double* o = c.pt[q];
+    const double w = T.w[q];
+    double F[D][D];
+    read_F<D>(raw + R::Gu, F);
+    const double J = det<D>(F);
+    if (J < my_min) my_min = J;
+    using K = Pt<D>;
+    if (c.flags & 1u) {
+      double Bm[D][D], Sg[D][D], tr = 0.0;
+      matmul_t<D>(F, F, Bm);
+#pragma unroll
+      for (int i = 0; i < D; ++i)
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+          double s = F[0][i] * F[0][j];
+#pragma unroll
+          for (int m = 1; m < D; ++m) s += F[m][i] * F[m][j];
+          Sg[i][j] = 0.5 * (s - (i == j ? 1.0 : 0.0));
+        }
+#pragma unroll
+      for (int i = 0; i < D; ++i) tr += Sg[i][i];
+#pragma unroll
+      for (int i = 0; i < D; ++i)
+#pragma unroll
+        for (int j = 0; j < D; ++j) Sg[i][j] = 2.0 * P.mu_s * Sg[i][j] + (i == j ? P.lambda_s * tr : 0.0);
+      write_mat<D>(o + K::sF, 1.0, F);
+      write_mat<D>(o + K::smF, w * dtt * P.mu_s, F);
+      write_mat<D>(o + K::slF, w * dtt * P.lambda_s, F);
+      write_mat<D>(o + K::sB, w * dtt * P.mu_s, Bm);
+      write_mat<D>(o + K::sS, w * dtt, Sg);
       continue;
     }
-    const int gc = gdof[col];
-    const int* ci = colind + rowptr[gr];
-    const int len = (int)(rowptr[gr + 1] - rowptr[gr]);
-    int lo = 0, hi = len;
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (ci[mid] < gc) lo = mid + 1; else hi = mid;
+    double Fi[D][D], A[D][D], Gv[D][D], X[D][D], Y[D][D], p = 0.0, trA = 0.0, Jo = 1.0;
+    read_mat<D>(raw + R::Gv, Gv);
+    const double iJ = 1.0 / J;
+    invert<D>(F, iJ, Fi);
+    matmul<D>(Gv, Fi, A);
+    if (prev) {
+      double Fo[D][D];
+      read_F<D>(raw + R::Guo, Fo);
+      Jo = det<D>(Fo);
     }
-    if (lo < len && ci[lo] == gc) out[rowptr[gr] + lo] += acc;
-    else if (acc != 0.0) atomicExch(err, 1);                // an entry outside the pattern
+#pragma unroll
+    for (int a = 0; a < NQ1; ++a) p += T.Np[q * NQ1 + a] * c.U[2 * NV + a];
+    const double m = dtt * mu, wJ = w * J;
+    write_mat<D>(o + K::Fi, 1.0, Fi);
+    write_mat<D>(o + K::A, 1.0, A);
+    write_mat<D>(o + K::Fim, wJ * m, Fi);
+    matmul<D>(Fi, A, Y);
+    write_mat<D>(o + K::FA, wJ * m, Y);
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      trA += A[i][i];
+#pragma unroll
+      for (int j = 0; j < D; ++j) X[i][j] = wJ * (m * (A[i][j] + A[j][i]) - (i == j ? p : 0.0));
+    }
+    matmul_t<D>(X, Fi, Y);
+    write_mat<D>(o + K::PX, 1.0, Y);
+    const double wi = w * iJ;
+#pragma unroll
+    for (int i = 0; i < D * D; ++i) o[K::GuJ + i] = wi * raw[R::Gu + i];
+    double cv[D];
+#pragma unroll
+    for (int j = 0; j < D; ++j) cv[j] = dtt * raw[R::v + j] - (raw[R::u + j] - raw[R::uo + j]);
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      double s = (prev ? P.theta : 1.0) * (raw[R::v + i] - raw[R::vo + i]);
+#pragma unroll
+      for (int j = 0; j < D; ++j) s += A[i][j] * cv[j];
+      o[K::e + i] = wJ * P.rho_f * s;
+    }
+    o[K::wJ] = wJ;
+    o[K::trA] = trA;
+    o[K::wJi] = wi;
+    // for the trial tables: c, and J^theta w rho_f; kept in raw slots that no other point reads
+    double* z = c.tr[q][0] + R::Gv;
+#pragma unroll
+    for (int j = 0; j < D; ++j) z[j] = cv[j];
+    z[D] = w * P.rho_f * (prev ? P.theta * J + (1.0 - P.theta) * Jo : J);
+    z[D + 1] = p;
+  }
+  if (my_min < 1e300) atomicMin(&S.minkey, order_key(my_min));
+  __syncthreads();
+  if (threadIdx.x == 0 && S.minkey != ~0ull) atomicMin(minkey, S.minkey);
+  // outflow faces of these cells
+  for (int ce = 0; ce < nc; ++ce) {
+    C& c = S.c[ce];
+    if ((c.flags & 3u) != 2u) continue;
+    for (int f = threadIdx.x; f < NFP; f += blockDim.x) {
+      double F[D][D], Gv[D][D], Fi[D][D], A[D][D];
+      for (int e = 0; e < D * D; ++e) {
+        Gv[e / D][e % D] = interpolate<D, PD>(T, true, f, R::Gv + e, c.U, c.Uo);
+        F[e / D][e % D] = interpolate<D, PD>(T, true, f, R::Gu + e, c.U, c.Uo) + (e / D == e % D ? 1.0 : 0.0);
+      }
+      const double J = det<D>(F);
+      invert<D>(F, 1.0 / J, Fi);
+      matmul<D>(Gv, Fi, A);
+      double* o = c.face[f];
+      write_mat<D>(o + Pt<D>::fFi, 1.0, Fi);
+      write_mat<D>(o + Pt<D>::fA, 1.0, A);
+#pragma unroll
+      for (int i = 0; i < D; ++i) {
+        double s = 0.0;
+#pragma unroll
+        for (int m = 0; m < D; ++m) s += A[m][i] * Fi[0][m];
+        o[Pt<D>::fq + i] = s;
+      }
+      o[Pt<D>::fm] = -T.wf[f] * dtt * mu * J;
+    }
+  }
+  // ---- trial tables: a warp takes whole points (3 in 2D, 1 in 3D), so that a point's c and J^theta
+  // (in the slots that the tables overwrite) are read by all of its lanes before any lane writes
+  {
+    constexpr int PW = 32 / NQ2;
+    static_assert(NQP % PW == 0, "whole points of one cell per warp");
+    const int lane = threadIdx.x & 31;
+    for (int u = threadIdx.x >> 5; u < nc * (NQP / PW); u += blockDim.x >> 5) {
+      C& c = S.c[u / (NQP / PW)];
+      const bool on = lane < PW * NQ2;
+      const int q = u % (NQP / PW) * PW + (on ? lane / NQ2 : 0), b = lane % NQ2;
+      const double* o = c.pt[q];
+      double cv[D], jt = 0.0, p = 0.0;
+      const bool solid = c.flags & 1u;
+      if (!solid) {
+        const double* z = c.tr[q][0] + R::Gv;
+#pragma unroll
+        for (int j = 0; j < D; ++j) cv[j] = z[j];
+        jt = z[D];
+        p = z[D + 1];
+      }
+      __syncwarp();
+      if (on) {
+        double* tr = c.tr[q][b];
+        const double* dN = T.dN + (q * NQ2 + b) * D;
+        const double N = T.N[q * NQ2 + b];
+        if (solid) {
+#pragma unroll
+          for (int i = 0; i < D; ++i) {
+            double f = 0.0, s = 0.0;
+#pragma unroll
+            for (int j = 0; j < D; ++j) {
+              f += o[Pt<D>::sF + i * D + j] * dN[j];
+              s += o[Pt<D>::sS + i * D + j] * dN[j];
+            }
+            tr[Tr<D>::sf + i] = f;
+            tr[Tr<D>::sS + i] = s;
+            tr[Tr<D>::sd + i] = dN[i];
+          }
+        } else {
+          double G[D], sb = 0.0;
+#pragma unroll
+          for (int k = 0; k < D; ++k) {
+            double g = 0.0;
+#pragma unroll
+            for (int l = 0; l < D; ++l) g += dN[l] * o[Pt<D>::Fi + l * D + k];
+            G[k] = g;
+            sb += g * cv[k];
+          }
+          const double wJ = o[Pt<D>::wJ], m = dtt * mu;
+#pragma unroll
+          for (int i = 0; i < D; ++i) {
+            double fg = 0.0, xg = 0.0;
+#pragma unroll
+            for (int j = 0; j < D; ++j) {
+              fg += o[Pt<D>::Fim + i * D + j] * G[j];
+              xg += (o[Pt<D>::A + i * D + j] + o[Pt<D>::A + j * D + i]) * G[j];
+            }
+            tr[Tr<D>::G + i] = G[i];
+            tr[Tr<D>::FG + i] = fg;
+            tr[Tr<D>::XG + i] = wJ * (m * xg - p * G[i]);
+          }
+          const double wr = wJ * P.rho_f;
+          tr[Tr<D>::al] = jt * N + wr * sb;
+          tr[Tr<D>::nb] = wr * dtt * N;
+          tr[Tr<D>::r] = wr * (sb + N);
+        }
+      }
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+
+  // ---- units
+  // adds acc (one value per test node) at column (node cn, component k of ncol) to the rows rbase + a * rstride
+  auto scatter = [&](C& c, int rbase, int cn, int col, int k, const double (&acc)[NQ2]) {
+    const int gc = c.gdof[col];
+#pragma unroll
+    for (int a0 = 0; a0 < NQ2; a0 += 9) {
+      double* at[9];
+      double old[9];
+#pragma unroll
+      for (int t = 0; t < 9; ++t) {
+        const int r = rbase + (a0 + t) * D;
+        const long long base = c.row[r];
+        at[t] = nullptr;
+        if (base < 0) continue;
+        int p = c.pos[r][cn];
+        if (p != kNoPos) p += k;
+        else p = find_col(colind + base, (int)(rowptr[c.gdof[r] + 1] - base), gc);
+        if (p >= 0) at[t] = out + base + p;
+        else if (acc[a0 + t] != 0.0) atomicExch(err, 1);      // an entry outside the pattern
+      }
+#pragma unroll
+      for (int t = 0; t < 9; ++t) old[t] = at[t] ? *at[t] : 0.0;
+#pragma unroll
+      for (int t = 0; t < 9; ++t)
+        if (at[t]) *at[t] = old[t] + acc[a0 + t];
+    }
+  };
+  // the outflow term of unit (i, b, k): added to the test nodes on the face (lattice index 2 in direction 0)
+  auto add_face = [&](const C& c, bool along_u, int i, int b, int k, double (&acc)[NQ2]) {
+    for (int f = 0; f < NFP; ++f) {
+      const double* o = c.face[f];
+      const double* dN = T.dNf + (f * NQ2 + b) * D;
+      double G[D];
+#pragma unroll
+      for (int j = 0; j < D; ++j) {
+        double g = 0.0;
+#pragma unroll
+        for (int l = 0; l < D; ++l) g += dN[l] * o[Pt<D>::fFi + l * D + j];
+        G[j] = g;
+      }
+      double gi = 0.0, gk = 0.0, ag = 0.0;
+#pragma unroll
+      for (int l = 0; l < D; ++l) {
+        gi = l == i ? G[l] : gi;
+        gk = l == k ? G[l] : gk;
+        ag += o[Pt<D>::fA + l * D + i] * G[l];
+      }
+      double d = gi * o[Pt<D>::fFi + k];                        // A^T n' along v
+      if (along_u) d = gk * o[Pt<D>::fq + i] - gi * o[Pt<D>::fq + k] - o[Pt<D>::fFi + k] * ag;
+      d *= o[Pt<D>::fm];
+#pragma unroll
+      for (int a = 2; a < NQ2; a += 3) acc[a] += T.Nf[f * NQ2 + a] * d;
+    }
+  };
+  // rows of v, columns of v (fluid); solid cells: the mass terms of all three pairs of v and u
+  for (int t = threadIdx.x; t < nc * UNITS; t += blockDim.x) {
+    C& c = S.c[t / UNITS];
+    const int u = t % UNITS, i = u / NV, b = (u % NV) / D, k = u % D;
+    if (c.flags & 1u) {
+      if (i != k) continue;
+      double m[NQ2], x[NQ2];
+#pragma unroll
+      for (int a = 0; a < NQ2; ++a) m[a] = T.M[a * NQ2 + b];
+      if (!c.cfix[b * D + k]) {
+#pragma unroll
+        for (int a = 0; a < NQ2; ++a) x[a] = P.rho_s * m[a];
+        scatter(c, i, b, b * D + k, k, x);
+#pragma unroll
+        for (int a = 0; a < NQ2; ++a) x[a] = -dtt * m[a];
+        scatter(c, NV + i, b, b * D + k, k, x);
+      }
+      if (!c.cfix[NV + b * D + k]) scatter(c, NV + i, NQ2 + b, NV + b * D + k, k, m);
+      continue;
+    }
+    if (c.cfix[b * D + k]) continue;
+    double acc[NQ2];
+    contract<D, true>(B, [&](int q, double& f0, double (&f1)[D]) {
+      const double* o = c.pt[q];
+      const double* tr = c.tr[q][b];
+      const double g = tr[Tr<D>::G + i];
+      f0 = fma(o[Pt<D>::A + i * D + k], tr[Tr<D>::nb], i == k ? tr[Tr<D>::al] : 0.0);
+#pragma unroll
+      for (int j = 0; j < D; ++j) f1[j] = fma(g, o[Pt<D>::Fim + j * D + k], i == k ? tr[Tr<D>::FG + j] : 0.0);
+    }, acc);
+    if (c.flags & 2u) add_face(c, false, i, b, k, acc);
+    scatter(c, i, b, b * D + k, k, acc);
+  }
+  // rows of v, columns of u
+  for (int t = threadIdx.x; t < nc * UNITS; t += blockDim.x) {
+    C& c = S.c[t / UNITS];
+    const int u = t % UNITS, i = u / NV, b = (u % NV) / D, k = u % D;
+    if (c.cfix[NV + b * D + k]) continue;
+    double acc[NQ2];
+    if (c.flags & 1u) {
+      contract<D, false>(B, [&](int q, double&, double (&f1)[D]) {
+        const double* o = c.pt[q];
+        const double* tr = c.tr[q][b];
+        const double bik = o[Pt<D>::sB + i * D + k], fi = tr[Tr<D>::sf + i], fk = tr[Tr<D>::sf + k];
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+          double s = fma(bik, tr[Tr<D>::sd + j], i == k ? tr[Tr<D>::sS + j] : 0.0);
+          s = fma(fi, o[Pt<D>::smF + k * D + j], s);
+          f1[j] = fma(fk, o[Pt<D>::slF + i * D + j], s);
+        }
+      }, acc);
+    } else {
+      contract<D, true>(B, [&](int q, double& f0, double (&f1)[D]) {
+        const double* o = c.pt[q];
+        const double* tr = c.tr[q][b];
+        const double gk = tr[Tr<D>::G + k], gi = tr[Tr<D>::G + i], xg = tr[Tr<D>::XG + i];
+        const double aik = o[Pt<D>::A + i * D + k];
+        f0 = fma(gk, o[Pt<D>::e + i], -aik * tr[Tr<D>::r]);
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+          double s = gk * o[Pt<D>::PX + i * D + j];
+          s = fma(-xg, o[Pt<D>::Fi + j * D + k], s);
+          s = fma(-aik, tr[Tr<D>::FG + j], s);
+          f1[j] = fma(-gi, o[Pt<D>::FA + j * D + k], s);
+        }
+      }, acc);
+      if (c.flags & 2u) add_face(c, true, i, b, k, acc);
+    }
+    scatter(c, i, NQ2 + b, NV + b * D + k, k, acc);
+  }
+  // rows of v, columns of the pressure: df1_ij = -J psi F^-1_ji
+  for (int t = threadIdx.x; t < nc * NQ1 * D; t += blockDim.x) {
+    C& c = S.c[t / (NQ1 * D)];
+    const int u = t % (NQ1 * D), i = u / NQ1, b = u % NQ1;
+    if (c.cfix[2 * NV + b]) continue;                     // solid cells: no pressure columns
+    double acc[NQ2];
+    contract<D, false>(B, [&](int q, double&, double (&f1)[D]) {
+      const double* o = c.pt[q];
+      const double s = -o[Pt<D>::wJ] * T.Np[q * NQ1 + b];
+#pragma unroll
+      for (int j = 0; j < D; ++j) f1[j] = s * o[Pt<D>::Fi + j * D + i];
+    }, acc);
+    scatter(c, i, 2 * NQ2 + b, 2 * NV + b, 0, acc);
+  }
+  // rows of the pressure, columns (b, k) of v and of u
+  for (int t = threadIdx.x; t < nc * NV; t += blockDim.x) {
+    C& c = S.c[t / NV];
+    const int b = (t % NV) / D, k = t % D;
+    if (c.flags & 1u) continue;
+    double av[NQ1], au[NQ1];
+#pragma unroll
+    for (int a = 0; a < NQ1; ++a) av[a] = au[a] = 0.0;
+#pragma unroll 3
+    for (int q = 0; q < NQP; ++q) {
+      const double* o = c.pt[q];
+      const double* tr = c.tr[q][b];
+      double ag = 0.0;
+#pragma unroll
+      for (int l = 0; l < D; ++l) ag += o[Pt<D>::A + l * D + k] * tr[Tr<D>::G + l];
+      const double gv = o[Pt<D>::wJ] * tr[Tr<D>::G + k];
+      const double gu = fma(gv, o[Pt<D>::trA], -o[Pt<D>::wJ] * ag);
+#pragma unroll
+      for (int a = 0; a < NQ1; ++a) {
+        av[a] = fma(T.Np[q * NQ1 + a], gv, av[a]);
+        au[a] = fma(T.Np[q * NQ1 + a], gu, au[a]);
+      }
+    }
+#pragma unroll
+    for (int a = 0; a < NQ1; ++a) {
+      const int r = 2 * NV + a;
+      const long long base = c.row[r];
+      if (base < 0) continue;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        if (c.cfix[h * NV + b * D + k]) continue;
+        const double x = h ? au[a] : av[a];
+        int p = c.pos[r][h * NQ2 + b];
+        if (p != kNoPos) p += k;
+        else p = find_col(colind + base, (int)(rowptr[c.gdof[r] + 1] - base), c.gdof[h * NV + b * D + k]);
+        if (p >= 0) out[base + p] += x;
+        else if (x != 0.0) atomicExch(err, 1);
+      }
+    }
+  }
+  __syncthreads();
+  // mesh rows, columns of u: w grad phi_b / J takes the place of FG
+  for (int t = threadIdx.x; t < nc * NQP * NQ2; t += blockDim.x) {
+    C& c = S.c[t / (NQP * NQ2)];
+    const int q = t % (NQP * NQ2) / NQ2, b = t % NQ2;
+    if (c.flags & 1u) continue;
+#pragma unroll
+    for (int j = 0; j < D; ++j)
+      c.tr[q][b][Tr<D>::FG + j] = c.pt[q][Pt<D>::wJi] * T.dN[(q * NQ2 + b) * D + j];
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < nc * UNITS; t += blockDim.x) {
+    C& c = S.c[t / UNITS];
+    const int u = t % UNITS, i = u / NV, b = (u % NV) / D, k = u % D;
+    if ((c.flags & 1u) || (c.flags >> 2) == 0u || c.cfix[NV + b * D + k]) continue;
+    double acc[NQ2];
+    contract<D, false>(B, [&](int q, double&, double (&f1)[D]) {
+      const double* o = c.pt[q];
+      const double* tr = c.tr[q][b];
+      const double gk = tr[Tr<D>::G + k];
+#pragma unroll
+      for (int j = 0; j < D; ++j) f1[j] = fma(-gk, o[Pt<D>::GuJ + i * D + j], i == k ? tr[Tr<D>::FG + j] : 0.0);
+    }, acc);
+    scatter(c, NV + i, NQ2 + b, NV + b * D + k, k, acc);
   }
 }
 
-// fixed rows: identity entry (Jacobian) or zero (residual)
+// fixed rows: the identity entry
 __global__ void k_fixed_rows(int64_t n, const int64_t* __restrict__ rowptr, const unsigned char* __restrict__ fixed,
-                             double* __restrict__ out, int jac) {
+                             double* __restrict__ vals) {
   const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= n || !fixed[r]) return;
-  if (jac) out[rowptr[r]] = 1.0; else out[r] = 0.0;
+  if (r < n && fixed[r]) vals[rowptr[r]] = 1.0;
 }
 
-__global__ void k_min_reduce(int64_t n, const double* __restrict__ x, double* __restrict__ out) {
-  __shared__ double sh[32];
-  double m = 1e300;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) m = fmin(m, x[i]);
-  for (int off = 16; off > 0; off >>= 1) m = fmin(m, __shfl_down_sync(0xffffffffu, m, off));
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmin(m, sh[w]);
-    out[0] = fmin(m, sh[0]);
-  }
-}
-
-// max |R_i| over the rows (deterministic: fixed blocks, fixed order)
-__global__ void k_absmax_partial(int64_t n, const double* __restrict__ x, double* __restrict__ part) {
-  __shared__ double sh[32];
-  const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
-  const int64_t lo = blockIdx.x * chunk, hi = lo + chunk < n ? lo + chunk : n;
+// max |R_i| over the rows into *key (the bits of a non-negative double order as integers; NaN
+// entries are passed over)
+__global__ void k_absmax(int64_t n, const double* __restrict__ x, unsigned long long* __restrict__ key) {
   double m = 0.0;
-  for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) m = fmax(m, fabs(x[i]));
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    m = fmax(m, fabs(x[i]));
   for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, off));
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmax(m, sh[w]);
-    part[blockIdx.x] = m;
-  }
+  if ((threadIdx.x & 31) == 0 && m > 0.0) atomicMax(key, (unsigned long long)__double_as_longlong(m));
 }
 
 __global__ void k_axpy_inplace(int64_t n, double alpha, const double* __restrict__ x, double* __restrict__ y) {
@@ -514,11 +1074,15 @@ struct Assembler {
   DBuf<int64_t> rowptr;
   DBuf<int> colind;
   DBuf<unsigned char> fixed;
-  DBuf<double> cell_minJ, scal, part;
-  DBuf<int> err;
+  Basis1 B1{};
+  // results of a call: [0] order key of min det F, [1] bits of max |R_i|, [2] entries outside the
+  // pattern (low 32 bits); the host reads them through `host`
+  DBuf<unsigned long long> res;
+  unsigned long long* host = nullptr;   // pinned
   int64_t nnz = 0;
   std::string msg;
   ~Assembler() {
+    if (host) cudaFreeHost(host);
     if (own_stream && s) cudaStreamDestroy(s);
   }
 };
@@ -576,10 +1140,19 @@ void build_tables(Assembler& A, const double* h) {
     wf[f] = ww;
     basis(xi, &Nf[f * NQ2], &dNf[(size_t)f * NQ2 * D], nullptr);
   }
+  std::vector<double> M((size_t)NQ2 * NQ2, 0.0);
+  for (int a = 0; a < NQ2; ++a)
+    for (int b = 0; b < NQ2; ++b)
+      for (int q = 0; q < NQP; ++q) M[a * NQ2 + b] += w[q] * N[q * NQ2 + a] * N[q * NQ2 + b];
+  for (int q = 0; q < 3; ++q)
+    for (int a = 0; a < 3; ++a) {
+      A.B1.N[q][a] = q2b(a, gx[q]);
+      for (int d = 0; d < D; ++d) A.B1.dN[d][q][a] = q2d(a, gx[q]) / h[d];
+    }
   std::vector<double> all;
-  size_t off[7];
-  const std::vector<double>* parts[7] = {&N, &dN, &Np, &w, &Nf, &dNf, &wf};
-  for (int t = 0; t < 7; ++t) {
+  size_t off[8];
+  const std::vector<double>* parts[8] = {&N, &dN, &Np, &w, &Nf, &dNf, &wf, &M};
+  for (int t = 0; t < 8; ++t) {
     off[t] = all.size();
     all.insert(all.end(), parts[t]->begin(), parts[t]->end());
   }
@@ -587,22 +1160,12 @@ void build_tables(Assembler& A, const double* h) {
   FSI_CUDA(cudaMemcpyAsync(A.tab.p, all.data(), sizeof(double) * all.size(), cudaMemcpyHostToDevice, A.s));
   FSI_CUDA(cudaStreamSynchronize(A.s));
   A.T = Tables{A.tab.p + off[0], A.tab.p + off[1], A.tab.p + off[2], A.tab.p + off[3],
-               A.tab.p + off[4], A.tab.p + off[5], A.tab.p + off[6]};
+               A.tab.p + off[4], A.tab.p + off[5], A.tab.p + off[6], A.tab.p + off[7]};
 }
 
-template <int D, int PD, bool JAC>
-size_t smem_bytes() {
-  using E = Sh<D, PD>;
-  constexpr int C = JAC ? E::CHUNK : 1;
-  return sizeof(double) * (E::NL + 2 * E::NQ2 * D + (size_t)(E::NQP + E::NFP) * C * kSlots<D>);
-}
-
-template <int D, int PD, bool JAC>
-void run_colours(Assembler& A, const double* U, const double* Uold, double* out) {
-  using E = Sh<D, PD>;
-  const size_t sm = smem_bytes<D, PD, JAC>();
-  FSI_CUDA(cudaFuncSetAttribute(k_assemble<D, PD, JAC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  const int chunks = JAC ? (E::NL + E::CHUNK - 1) / E::CHUNK : 1;
+// f(geometry, cells) for each colour that has cells
+template <int D, class F>
+void for_colours(const Assembler& A, F&& f) {
   for (int col = 0; col < (1 << D); ++col) {
     CellGeom g{};
     int64_t cnt = 1;
@@ -618,63 +1181,82 @@ void run_colours(Assembler& A, const double* U, const double* Uold, double* out)
     }
     g.color = col;
     if (cnt == 0) continue;
-    const int64_t blocks = cnt * chunks;
-    require(blocks < ((int64_t)1 << 31), "fsi_asm: too many cells for one launch");
-    k_assemble<D, PD, JAC><<<(unsigned)blocks, kAsmThreads, sm, A.s>>>(g, chunks, A.T, A.phys, A.cell_dof.p,
-                                                                    A.cell_flags.p, A.rowptr.p, A.colind.p, A.fixed.p,
-                                                                    U, Uold, out, A.cell_minJ.p, A.err.p);
+    require(cnt < ((int64_t)1 << 31), "fsi_asm: too many cells for one launch");
+    f(g, cnt);
     FSI_CHECK_LAUNCH();
   }
 }
 
-double finish(Assembler& A, double* out, bool jac, double* minJ) {
-  k_fixed_rows<<<div_up(A.n, 256), 256, 0, A.s>>>(A.n, A.rowptr.p, A.fixed.p, out, jac ? 1 : 0);
-  FSI_CHECK_LAUNCH();
-  k_min_reduce<<<1, 1024, 0, A.s>>>(A.ncell, A.cell_minJ.p, A.scal.p);
-  FSI_CHECK_LAUNCH();
-  double h[2] = {0, 0};
-  int e = 0;
-  FSI_CUDA(cudaMemcpyAsync(&h[0], A.scal.p, sizeof(double), cudaMemcpyDeviceToHost, A.s));
-  FSI_CUDA(cudaMemcpyAsync(&e, A.err.p, sizeof(int), cudaMemcpyDeviceToHost, A.s));
+template <int D, int PD>
+void run_residual(Assembler& A, const double* U, const double* Uold, double* out) {
+  constexpr size_t sm = sizeof(ResSmem<D, PD>);
+  static std::atomic<unsigned long long> attr{0};
+  once_per_device(attr, [](int) {
+    FSI_CUDA(cudaFuncSetAttribute(k_residual<D, PD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  });
+  for_colours<D>(A, [&](const CellGeom& g, int64_t cnt) {
+    k_residual<D, PD><<<div_up(cnt, Sh<D, PD>::RCELLS), kAsmThreads, sm, A.s>>>(
+        g, cnt, A.T, A.phys, A.cell_dof.p, A.cell_flags.p, A.fixed.p, U, Uold, out, A.res.p);
+  });
+}
+
+template <int D, int PD>
+void run_jacobian(Assembler& A, const double* U, const double* Uold, double* vals) {
+  constexpr size_t sm = sizeof(JacSmem<D, PD>);
+  static_assert(sm <= 227 * 1024, "Jacobian tables exceed the shared memory of a CTA");
+  static std::atomic<unsigned long long> attr{0};
+  once_per_device(attr, [](int) {
+    FSI_CUDA(cudaFuncSetAttribute(k_jacobian<D, PD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  });
+  for_colours<D>(A, [&](const CellGeom& g, int64_t cnt) {
+    k_jacobian<D, PD><<<div_up(cnt, Sh<D, PD>::JCELLS), kAsmThreads, sm, A.s>>>(
+        g, cnt, A.T, A.B1, A.phys, A.cell_dof.p, A.cell_flags.p, A.rowptr.p, A.colind.p, A.fixed.p, U, Uold, vals,
+        A.res.p, reinterpret_cast<int*>(A.res.p + 2));
+  });
+}
+
+void begin(Assembler& A) {
+  FSI_CUDA(cudaMemsetAsync(A.res.p, 0xFF, sizeof(unsigned long long), A.s));
+  FSI_CUDA(cudaMemsetAsync(A.res.p + 1, 0, 2 * sizeof(unsigned long long), A.s));
+}
+
+void finish(Assembler& A, double* minJ, double* rmax) {
+  FSI_CUDA(cudaMemcpyAsync(A.host, A.res.p, 3 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, A.s));
   FSI_CUDA(cudaStreamSynchronize(A.s));
-  if (minJ) *minJ = h[0];
-  require(e == 0, "fsi_asm: a Jacobian entry falls outside the CSR pattern");
-  return h[0];
+  if (minJ) *minJ = A.host[0] == ~0ull ? 1e300 : order_value(A.host[0]);   // 1e300: no point with a finite det F
+  if (rmax) std::memcpy(rmax, A.host + 1, sizeof(double));
+  require((int)(A.host[2] & 0xFFFFFFFFull) == 0, "fsi_asm: a Jacobian entry falls outside the CSR pattern");
 }
 
 }  // namespace
 
 void asm_residual(Assembler& A, const double* U, const double* Uold, double* R, double* minJ, double* rmax) {
-  FSI_CUDA(cudaMemsetAsync(R, 0, sizeof(double) * A.n, A.s));
-  FSI_CUDA(cudaMemsetAsync(A.err.p, 0, sizeof(int), A.s));
+  begin(A);
+  FSI_CUDA(cudaMemsetAsync(R, 0, sizeof(double) * A.n, A.s));   // fixed rows stay 0
   if (A.dim == 2) {
-    if (A.pdisc) run_colours<2, 1, false>(A, U, Uold, R); else run_colours<2, 0, false>(A, U, Uold, R);
+    if (A.pdisc) run_residual<2, 1>(A, U, Uold, R); else run_residual<2, 0>(A, U, Uold, R);
   } else {
-    if (A.pdisc) run_colours<3, 1, false>(A, U, Uold, R); else run_colours<3, 0, false>(A, U, Uold, R);
+    if (A.pdisc) run_residual<3, 1>(A, U, Uold, R); else run_residual<3, 0>(A, U, Uold, R);
   }
-  finish(A, R, false, minJ);
   if (rmax) {
-    const int nb = 256;
-    k_absmax_partial<<<nb, 256, 0, A.s>>>(A.n, R, A.part.p);
+    const int cap = device_sms() * 8, g = div_up(A.n, 256);
+    k_absmax<<<g < cap ? g : cap, 256, 0, A.s>>>(A.n, R, A.res.p + 1);
     FSI_CHECK_LAUNCH();
-    std::vector<double> hp(nb);
-    FSI_CUDA(cudaMemcpyAsync(hp.data(), A.part.p, sizeof(double) * nb, cudaMemcpyDeviceToHost, A.s));
-    FSI_CUDA(cudaStreamSynchronize(A.s));
-    double m = 0.0;
-    for (double v : hp) m = v > m ? v : m;
-    *rmax = m;
   }
+  finish(A, minJ, rmax);
 }
 
 void asm_jacobian(Assembler& A, const double* U, const double* Uold, double* vals, double* minJ) {
+  begin(A);
   FSI_CUDA(cudaMemsetAsync(vals, 0, sizeof(double) * A.nnz, A.s));
-  FSI_CUDA(cudaMemsetAsync(A.err.p, 0, sizeof(int), A.s));
   if (A.dim == 2) {
-    if (A.pdisc) run_colours<2, 1, true>(A, U, Uold, vals); else run_colours<2, 0, true>(A, U, Uold, vals);
+    if (A.pdisc) run_jacobian<2, 1>(A, U, Uold, vals); else run_jacobian<2, 0>(A, U, Uold, vals);
   } else {
-    if (A.pdisc) run_colours<3, 1, true>(A, U, Uold, vals); else run_colours<3, 0, true>(A, U, Uold, vals);
+    if (A.pdisc) run_jacobian<3, 1>(A, U, Uold, vals); else run_jacobian<3, 0>(A, U, Uold, vals);
   }
-  finish(A, vals, true, minJ);
+  k_fixed_rows<<<div_up(A.n, 256), 256, 0, A.s>>>(A.n, A.rowptr.p, A.fixed.p, vals);
+  FSI_CHECK_LAUNCH();
+  finish(A, minJ, nullptr);
 }
 
 void asm_axpy(Assembler& A, double alpha, const double* x, double* y) {
@@ -716,10 +1298,8 @@ void asm_create(Assembler& A, const fsi_asm_mesh& m, const fsi_asm_physics& p, v
   A.rowptr.alloc(A.n + 1);
   A.colind.alloc(A.nnz > 0 ? A.nnz : 1);
   A.fixed.alloc(A.n);
-  A.cell_minJ.alloc(A.ncell);
-  A.scal.alloc(2);
-  A.part.alloc(256);
-  A.err.alloc(1);
+  A.res.alloc(3);
+  FSI_CUDA(cudaMallocHost(&A.host, 3 * sizeof(unsigned long long)));
   FSI_CUDA(cudaMemcpyAsync(A.cell_dof.p, m.cell_dof, sizeof(int) * A.ncell * NL, cudaMemcpyHostToDevice, A.s));
   FSI_CUDA(cudaMemcpyAsync(A.cell_flags.p, m.cell_flags, sizeof(unsigned) * A.ncell, cudaMemcpyHostToDevice, A.s));
   FSI_CUDA(cudaMemcpyAsync(A.rowptr.p, m.rowptr, sizeof(int64_t) * (A.n + 1), cudaMemcpyHostToDevice, A.s));
