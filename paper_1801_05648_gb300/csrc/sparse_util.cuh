@@ -73,7 +73,7 @@ void bsr_make_pair_order(Bsr& A1, const Bsr& A2, cudaStream_t s);
 void bsr_to_dense(const Bsr& A, double* dense, cudaStream_t s);
 
 // Inverse of an n x n row-major dense matrix M into Minv (Gauss-Jordan with partial
-// pivoting, one launch per pivot over the whole GPU; M is destroyed); all-zero rows
+// pivoting in panels, dense.cu; M is destroyed); all-zero rows
 // are first replaced by identity rows.  Returns false when a pivot vanishes.
 bool dense_inverse(int n, double* M, double* Minv, cudaStream_t s);
 
