@@ -42,29 +42,55 @@ __device__ __forceinline__ double block_norm_at(const int* rp, const int* ci, co
   return (pos < rp[row + 1] && ci[pos] == col) ? fro[pos] : 0.0;
 }
 
-template <bool FILL>
-__global__ void k_strength(int nbr, const int* __restrict__ rp, const int* __restrict__ ci,
-                           const double* __restrict__ fro, double theta, int* __restrict__ cnt,
-                           const int* __restrict__ grp, int* __restrict__ gci) {
+// dnorm[i] = norm of row i's diagonal block (0 when absent)
+__global__ void k_diag_norm(int nbr, const int* __restrict__ rp, const int* __restrict__ ci,
+                            const double* __restrict__ fro, double* __restrict__ dnorm) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < nbr) dnorm[i] = block_norm_at(rp, ci, fro, i, i);
+}
+
+// One warp per row: strong[k] marks row i's strong neighbours, cnt[i] counts them.
+__global__ void __launch_bounds__(128) k_strength(int nbr, const int* __restrict__ rp, const int* __restrict__ ci,
+                                                  const double* __restrict__ fro, const double* __restrict__ dnorm,
+                                                  double theta, unsigned char* __restrict__ strong,
+                                                  int* __restrict__ cnt) {
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (i >= nbr) return;
-  const double dii = block_norm_at(rp, ci, fro, i, i);
+  const double dii = dnorm[i];
+  const int hi = rp[i + 1];
   int c = 0;
-  int pos = FILL ? grp[i] : 0;
-  for (int k = rp[i]; k < rp[i + 1]; ++k) {
+  for (int k = rp[i] + lane; k < hi; k += 32) {
     const int j = ci[k];
-    if (j == i) continue;
-    const double fij = fro[k];
-    const double fji = block_norm_at(rp, ci, fro, j, i);
-    const double djj = block_norm_at(rp, ci, fro, j, j);
-    const double m = fij > fji ? fij : fji;
-    const double thr = __dmul_rn(theta, __dsqrt_rn(__dmul_rn(dii, djj)));
-    if (m > 0.0 && m >= thr) {
-      if (FILL) gci[pos++] = j;
-      ++c;
+    bool on = false;
+    if (j != i) {
+      const double fij = fro[k];
+      const double fji = block_norm_at(rp, ci, fro, j, i);
+      const double m = fij > fji ? fij : fji;
+      const double thr = __dmul_rn(theta, __dsqrt_rn(__dmul_rn(dii, dnorm[j])));
+      on = m > 0.0 && m >= thr;
     }
+    strong[k] = on ? 1 : 0;
+    c += on;
   }
-  if (!FILL) cnt[i] = c;
+  c = __reduce_add_sync(0xffffffffu, c);
+  if (lane == 0) cnt[i] = c;
+}
+
+// The strong neighbours in order (one warp per row).
+__global__ void __launch_bounds__(128) k_strength_fill(int nbr, const int* __restrict__ rp,
+                                                       const int* __restrict__ ci,
+                                                       const unsigned char* __restrict__ strong,
+                                                       const int* __restrict__ grp, int* __restrict__ gci) {
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (i >= nbr) return;
+  const int lo = rp[i], hi = rp[i + 1];
+  int pos = grp[i];
+  for (int k0 = lo; k0 < hi; k0 += 32) {
+    const bool on = k0 + lane < hi && strong[k0 + lane];
+    const unsigned m = __ballot_sync(0xffffffffu, on);
+    if (on) gci[pos + __popc(m & ((1u << lane) - 1))] = ci[k0 + lane];
+    pos += __popc(m);
+  }
 }
 
 __global__ void k_mis_init(int n, const int* __restrict__ grp, int level, int* __restrict__ state,
@@ -165,71 +191,79 @@ __global__ void k_ptent_cols(int n, const int* __restrict__ agg, const int* __re
   if (i < n && agg[i] >= 0) pci[prp[i]] = agg[i];
 }
 
-// One thread per aggregate: modified Gram-Schmidt on the near-nullspace rows of
-// its members, Q written into P_tent's blocks, R into the coarse near-nullspace.
-__global__ void k_tentative(int nagg, int b, int k, const int* __restrict__ off, const int* __restrict__ mem,
-                            const int* __restrict__ prp, const double* __restrict__ B, double drop_tol,
-                            double* __restrict__ Q, double* __restrict__ Bc) {
-  const int J = blockIdx.x * blockDim.x + threadIdx.x;
+// One warp per aggregate: modified Gram-Schmidt on the near-nullspace rows of
+// its members, Q written into P_tent's blocks, R into the coarse near-nullspace.  The rows
+// (member-major, in order) are staged in shared memory when they fit `cap` doubles, else
+// worked on in a scratch slice.  Every sum runs over the rows in order, in one lane, as a
+// thread per aggregate did in global memory (1.0 ms per level of the 32x16x16
+// hierarchies); the columns' original norms are summed by one lane each, the updates by
+// all lanes.
+constexpr int kTentThreads = 64;
+__global__ void __launch_bounds__(kTentThreads) k_tentative(int nagg, int b, int k, int cap,
+                                                            const int* __restrict__ off, const int* __restrict__ mem,
+                                                            const int* __restrict__ prp, const double* __restrict__ B,
+                                                            double drop_tol, double* __restrict__ scratch,
+                                                            double* __restrict__ Q, double* __restrict__ Bc) {
+  extern __shared__ __align__(16) double tent_sm[];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int J = blockIdx.x * (kTentThreads / 32) + w;
   if (J >= nagg) return;
-  const int lo = off[J], hi = off[J + 1];
-  for (int e = lo; e < hi; ++e) {
-    const int m = mem[e];
-    for (int r = 0; r < b; ++r)
-      for (int c = 0; c < k; ++c) Q[((int64_t)prp[m] * b + r) * k + c] = B[((int64_t)m * b + r) * k + c];
-  }
+  const int lo = off[J], nm = off[J + 1] - lo, bk = b * k;
+  const int rows = nm * b, nv = nm * bk;
+  double* q = nv <= cap ? tent_sm + (size_t)w * cap : scratch + (int64_t)lo * bk;
+  for (int e = lane; e < nv; e += 32) q[e] = B[(int64_t)mem[lo + e / bk] * bk + e % bk];
   double* R = Bc + (int64_t)J * k * k;
-  for (int t = 0; t < k * k; ++t) R[t] = 0.0;
-  for (int c = 0; c < k; ++c) {
+  for (int t = lane; t < k * k; t += 32) R[t] = 0.0;
+  __syncwarp();
+  double orig = 0.0;   // lane c: the norm of column c (k <= 6)
+  if (lane < k) {
     double s = 0.0;
-    for (int e = lo; e < hi; ++e)
-      for (int r = 0; r < b; ++r) { const double q = Q[((int64_t)prp[mem[e]] * b + r) * k + c]; s += q * q; }
-    const double orig = sqrt(s);
+    for (int r = 0; r < rows; ++r) { const double v = q[r * k + lane]; s += v * v; }
+    orig = sqrt(s);
+  }
+  for (int c = 0; c < k; ++c) {
     for (int j = 0; j < c; ++j) {
       double rjc = 0.0;
-      for (int e = lo; e < hi; ++e)
-        for (int r = 0; r < b; ++r) {
-          const int64_t row = ((int64_t)prp[mem[e]] * b + r) * k;
-          rjc += Q[row + j] * Q[row + c];
-        }
-      R[j * k + c] = rjc;
-      for (int e = lo; e < hi; ++e)
-        for (int r = 0; r < b; ++r) {
-          const int64_t row = ((int64_t)prp[mem[e]] * b + r) * k;
-          Q[row + c] = Q[row + c] - rjc * Q[row + j];
-        }
-    }
-    s = 0.0;
-    for (int e = lo; e < hi; ++e)
-      for (int r = 0; r < b; ++r) { const double q = Q[((int64_t)prp[mem[e]] * b + r) * k + c]; s += q * q; }
-    const double nrm = sqrt(s);
-    const bool drop = (orig == 0.0) || (nrm <= drop_tol * orig);
-    for (int e = lo; e < hi; ++e)
-      for (int r = 0; r < b; ++r) {
-        const int64_t row = ((int64_t)prp[mem[e]] * b + r) * k;
-        Q[row + c] = drop ? 0.0 : Q[row + c] / nrm;
+      if (lane == 0) {
+        for (int r = 0; r < rows; ++r) rjc += q[r * k + j] * q[r * k + c];
+        R[j * k + c] = rjc;
       }
-    R[c * k + c] = drop ? 0.0 : nrm;
+      rjc = __shfl_sync(0xffffffffu, rjc, 0);
+      for (int r = lane; r < rows; r += 32) q[r * k + c] = q[r * k + c] - rjc * q[r * k + j];
+      __syncwarp();
+    }
+    double nrm = 0.0;
+    if (lane == 0) {
+      double s = 0.0;
+      for (int r = 0; r < rows; ++r) { const double v = q[r * k + c]; s += v * v; }
+      nrm = sqrt(s);
+    }
+    nrm = __shfl_sync(0xffffffffu, nrm, 0);
+    const double oc = __shfl_sync(0xffffffffu, orig, c);
+    const bool drop = (oc == 0.0) || (nrm <= drop_tol * oc);
+    for (int r = lane; r < rows; r += 32) q[r * k + c] = drop ? 0.0 : q[r * k + c] / nrm;
+    if (lane == 0) R[c * k + c] = drop ? 0.0 : nrm;
+    __syncwarp();
   }
+  for (int e = lane; e < nv; e += 32) Q[(int64_t)prp[mem[lo + e / bk]] * bk + e % bk] = q[e];
 }
 
 // P = P_tent - (omega * dinv) * AP on the pattern of AP (which contains P_tent's).
-__global__ void k_smooth_p(int nbr, int b, int k, const int* __restrict__ rp, const int* __restrict__ ci,
-                           const double* __restrict__ ap, const int* __restrict__ agg, const int* __restrict__ prp,
-                           const double* __restrict__ Q, const double* __restrict__ dinv, double omega,
-                           double* __restrict__ p) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// One warp per block row.
+__global__ void __launch_bounds__(128) k_smooth_p(int nbr, int b, int k, const int* __restrict__ rp,
+                                                  const int* __restrict__ ci, const double* __restrict__ ap,
+                                                  const int* __restrict__ agg, const int* __restrict__ prp,
+                                                  const double* __restrict__ Q, const double* __restrict__ dinv,
+                                                  double omega, double* __restrict__ p) {
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (i >= nbr) return;
-  for (int e = rp[i]; e < rp[i + 1]; ++e) {
-    const bool tent = agg[i] >= 0 && ci[e] == agg[i];
-    for (int r = 0; r < b; ++r) {
-      const double w = omega * dinv[(int64_t)i * b + r];
-      for (int c = 0; c < k; ++c) {
-        const int64_t o = ((int64_t)e * b + r) * k + c;
-        const double t = tent ? Q[((int64_t)prp[i] * b + r) * k + c] : 0.0;
-        p[o] = t - w * ap[o];
-      }
-    }
+  const int lo = rp[i], bk = b * k, ne = (rp[i + 1] - lo) * bk, ag = agg[i];
+  const int64_t q0 = ag >= 0 ? (int64_t)prp[i] * bk : 0;
+  for (int e = lane; e < ne; e += 32) {
+    const int t = e % bk, r = t / k;
+    const double w = omega * dinv[(int64_t)i * b + r];
+    const int64_t o = (int64_t)lo * bk + e;
+    p[o] = (ag >= 0 && ci[lo + e / bk] == ag ? Q[q0 + t] : 0.0) - w * ap[o];
   }
 }
 
@@ -238,6 +272,17 @@ __global__ void k_power_init(int64_t n, int stream_id, double* __restrict__ x) {
   if (i >= n) return;
   const unsigned long long z = splitmix64((unsigned long long)i + ((unsigned long long)stream_id << 32));
   x[i] = 1.0 + (double)(z >> 11) * 0x1.0p-53;
+}
+
+// x = y / ||y|| with ||y||^2 on the device; x stays when y = 0 (its next product is then 0 again)
+__global__ void k_power_scale(int64_t n, const double* __restrict__ yy, const double* __restrict__ y,
+                              double* __restrict__ x) {
+  dep_wait();
+  const double ny = __dsqrt_rn(*yy);
+  if (ny == 0.0) return;
+  const double a = __ddiv_rn(1.0, ny);
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    x[i] = a * y[i];
 }
 
 // d = dinv * b / theta; x = d   (first Chebyshev step from x = 0)
@@ -388,19 +433,21 @@ int sync_read_int(const int* dev, cudaStream_t s) {
 double power_lambda(const Bsr& A, const double* dinv, int iters, int stream_id, cudaStream_t s) {
   const int64_t n = A.rows();
   if (n == 0) return 0.0;
-  DBuf<double> x(n), y(n), part(kRedBlocks), out(1);
+  DBuf<double> x(n), y(n), part(kRedBlocks), out(2);
   k_power_init<<<div_up(n, 256), 256, 0, s>>>(n, stream_id, x.p);
   FSI_CHECK_LAUNCH();
-  double lam = 0.0;
+  // the norms stay on the device (one wait in all); x is needed as it enters the last product
+  const int cap = device_sms() * 16, g = div_up(n, 256) < cap ? div_up(n, 256) : cap;
   for (int it = 0; it < iters; ++it) {
+    if (it > 0) launch_k(k_power_scale, g, 256, 0, s, n, (const double*)out.p, (const double*)y.p, x.p);
     spmv_dinv<double>(A, x.p, dinv, y.p, s);
-    const double ny = std::sqrt(dot_host<double>(n, y.p, y.p, part.p, out.p, s));
-    const double nx = std::sqrt(dot_host<double>(n, x.p, x.p, part.p, out.p, s));
-    lam = ny / nx;
-    if (ny == 0.0) break;
-    axpby<double>(n, 1.0 / ny, y.p, 0.0, x.p, s);
+    dot_dev<double>(n, y.p, y.p, part.p, out.p, s);
   }
-  return lam;
+  dot_dev<double>(n, x.p, x.p, part.p, out.p + 1, s);
+  double h[2] = {0.0, 0.0};
+  FSI_CUDA(cudaMemcpyAsync(h, out.p, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
+  FSI_CUDA(cudaStreamSynchronize(s));
+  return std::sqrt(h[0]) / std::sqrt(h[1]);
 }
 
 double Hierarchy::operator_complexity() const {
@@ -465,13 +512,16 @@ void amg_setup(Hierarchy& H, Bsr&& A0, const double* B0, int k0, const AmgParams
       FSI_CHECK_LAUNCH();
     }
     DBuf<int> gcnt(nbr), grp(nbr + 1);
-    k_strength<false><<<div_up(nbr, 128), 128, 0, s>>>(nbr, L.A.rowptr.p, L.A.colind.p, fro.p, prm.theta, gcnt.p,
-                                                      nullptr, nullptr);
+    DBuf<double> dnorm(nbr);
+    DBuf<unsigned char> strong(L.A.nnzb > 0 ? L.A.nnzb : 1);
+    k_diag_norm<<<div_up(nbr, 128), 128, 0, s>>>(nbr, L.A.rowptr.p, L.A.colind.p, fro.p, dnorm.p);
+    FSI_CHECK_LAUNCH();
+    const int gw = div_up((int64_t)nbr * 32, 128);   // one warp per row
+    k_strength<<<gw, 128, 0, s>>>(nbr, L.A.rowptr.p, L.A.colind.p, fro.p, dnorm.p, prm.theta, strong.p, gcnt.p);
     FSI_CHECK_LAUNCH();
     const int64_t gnnz = exclusive_scan(gcnt.p, grp.p, nbr, s);
     DBuf<int> gci(gnnz > 0 ? gnnz : 1);
-    k_strength<true><<<div_up(nbr, 128), 128, 0, s>>>(nbr, L.A.rowptr.p, L.A.colind.p, fro.p, prm.theta, nullptr,
-                                                     grp.p, gci.p);
+    k_strength_fill<<<gw, 128, 0, s>>>(nbr, L.A.rowptr.p, L.A.colind.p, strong.p, grp.p, gci.p);
     FSI_CHECK_LAUNCH();
     // ---- distance-2 MIS
     DBuf<int> state(nbr), und(1);
@@ -479,6 +529,7 @@ void amg_setup(Hierarchy& H, Bsr&& A0, const double* B0, int k0, const AmgParams
     const int g = div_up(nbr, 256);
     k_mis_init<<<g, 256, 0, s>>>(nbr, grp.p, lvl, state.p, base.p);
     FSI_CHECK_LAUNCH();
+    // four rounds per look at the undecided count (a round after the last one changes nothing)
     for (int it = 0;; ++it) {
       require(it < 10000, "amg_setup: MIS iteration did not terminate");
       FSI_CUDA(cudaMemsetAsync(und.p, 0, sizeof(int), s));
@@ -487,7 +538,7 @@ void amg_setup(Hierarchy& H, Bsr&& A0, const double* B0, int k0, const AmgParams
       k_rowmax<<<g, 256, 0, s>>>(nbr, grp.p, gci.p, t1.p, t2.p);
       k_mis_update<<<g, 256, 0, s>>>(nbr, state.p, key.p, t2.p, und.p);
       FSI_CHECK_LAUNCH();
-      if (sync_read_int(und.p, s) == 0) break;
+      if (it % 4 == 3 && sync_read_int(und.p, s) == 0) break;
     }
     // ---- aggregates
     DBuf<int> flag(nbr), rid(nbr + 1), agg1(nbr), fail(1);
@@ -504,15 +555,15 @@ void amg_setup(Hierarchy& H, Bsr&& A0, const double* B0, int k0, const AmgParams
     L.nagg = nagg;
     if (nagg == 0 || (int64_t)nagg * k >= n) break;   // coarsening stalled: this level is the coarsest
     // ---- member lists (sorted by node index)
-    DBuf<int> acnt(nagg), aoff(nagg + 1), acur(nagg), mem(nbr);
+    DBuf<int> acnt(nagg), aoff(nagg + 1), acur(nagg), unsorted(nbr), mem(nbr);
     FSI_CUDA(cudaMemsetAsync(acnt.p, 0, sizeof(int) * nagg, s));
     FSI_CUDA(cudaMemsetAsync(acur.p, 0, sizeof(int) * nagg, s));
     k_count_agg<<<g, 256, 0, s>>>(nbr, L.agg.p, acnt.p);
     FSI_CHECK_LAUNCH();
-    exclusive_scan(acnt.p, aoff.p, nagg, s);
-    k_fill_members<<<g, 256, 0, s>>>(nbr, L.agg.p, aoff.p, acur.p, mem.p);
+    const int64_t nmem = exclusive_scan(acnt.p, aoff.p, nagg, s);
+    k_fill_members<<<g, 256, 0, s>>>(nbr, L.agg.p, aoff.p, acur.p, unsorted.p);
     FSI_CHECK_LAUNCH();
-    sort_segments(nagg, aoff.p, mem.p, nullptr, s);
+    sort_segments(nagg, nmem, aoff.p, unsorted.p, nullptr, mem.p, nullptr, s);
     // ---- tentative prolongator
     Bsr Pt;
     Pt.nbr = nbr; Pt.nbc = nagg; Pt.br = b; Pt.bc = k;
@@ -525,9 +576,14 @@ void amg_setup(Hierarchy& H, Bsr&& A0, const double* B0, int k0, const AmgParams
     k_ptent_cols<<<g, 256, 0, s>>>(nbr, L.agg.p, Pt.rowptr.p, Pt.colind.p);
     FSI_CHECK_LAUNCH();
     DBuf<double> Bc((int64_t)nagg * k * k);
-    k_tentative<<<div_up(nagg, 64), 64, 0, s>>>(nagg, b, k, aoff.p, mem.p, Pt.rowptr.p, B, prm.drop_tol, Pt.v64.p,
-                                                Bc.p);
-    FSI_CHECK_LAUNCH();
+    {
+      // 20 KB per warp: 850 rows of 3 modes, 420 of 6; larger aggregates work in the scratch
+      constexpr int kTentCap = 2560, kWarps = kTentThreads / 32;
+      DBuf<double> scratch(nmem > 0 ? nmem * b * k : 1);
+      k_tentative<<<div_up(nagg, kWarps), kTentThreads, kWarps * kTentCap * sizeof(double), s>>>(
+          nagg, b, k, kTentCap, aoff.p, mem.p, Pt.rowptr.p, B, prm.drop_tol, scratch.p, Pt.v64.p, Bc.p);
+      FSI_CHECK_LAUNCH();
+    }
     set_tpr(Pt);
     // ---- smoothed prolongator
     const double omega = 4.0 / (3.0 * L.lam);
@@ -537,7 +593,7 @@ void amg_setup(Hierarchy& H, Bsr&& A0, const double* B0, int k0, const AmgParams
     L.P.rowptr = std::move(AP.rowptr);
     L.P.colind = std::move(AP.colind);
     L.P.v64.alloc(AP.nnzb > 0 ? AP.nnzb * b * k : 1);
-    k_smooth_p<<<div_up(nbr, 128), 128, 0, s>>>(nbr, b, k, L.P.rowptr.p, L.P.colind.p, AP.v64.p, L.agg.p,
+    k_smooth_p<<<gw, 128, 0, s>>>(nbr, b, k, L.P.rowptr.p, L.P.colind.p, AP.v64.p, L.agg.p,
                                                 Pt.rowptr.p, Pt.v64.p, L.dinv64.p, omega, L.P.v64.p);
     FSI_CHECK_LAUNCH();
     set_tpr(L.P);
@@ -548,10 +604,12 @@ void amg_setup(Hierarchy& H, Bsr&& A0, const double* B0, int k0, const AmgParams
     // -(R A) where it pays: one pass over R and R A against b and x instead of the
     // residual (A, x, b read, r written) and its restriction (R, r read); kept when
     // that moves fewer bytes (in FP32) and the product's rows fit the SpGEMM table
-    if (bsr_spgemm_if_fits(L.R, L.A, L.RAn, s)) {
+    int longest = 0;
+    if (bsr_spgemm_pattern(L.R, L.A, L.RAn, longest, s)) {
       const double fused = L.R.spmv_bytes(4) + L.RAn.spmv_bytes(4) - 4.0 * L.R.rows();
       const double split = L.A.spmv_bytes(4) + 4.0 * L.A.rows() + L.R.spmv_bytes(4);
       if (fused < 0.95 * split) {
+        bsr_spgemm_values(L.R, L.A, L.RAn, longest, s);
         bsr_scale(L.RAn, -1.0, s);
         L.RAn.tpr = lanes_for(L.RAn.nnzb + L.R.nnzb, L.RAn.nbr, 2.0);   // one lane group reads both rows
         L.RAn.tpr64 = lanes_for(L.RAn.nnzb + L.R.nnzb, L.RAn.nbr, 8.0);

@@ -1,5 +1,6 @@
 #include "sparse_util.cuh"
 
+#include <algorithm>
 #include <climits>
 
 namespace fsi {
@@ -18,9 +19,8 @@ __device__ __forceinline__ long long warp_incl_scan(long long v, int lane) {
 }
 
 // Exclusive scan of a 1024-element tile; writes block totals.
-template <class Tin>
-__global__ void __launch_bounds__(kScanBlock) k_scan_tile(const Tin* __restrict__ in, long long* __restrict__ out,
-                                                          int64_t n, long long* __restrict__ bsum) {
+__global__ void __launch_bounds__(kScanBlock) k_scan_tile(const int* __restrict__ in, int* __restrict__ out, int64_t n,
+                                                          long long* __restrict__ bsum) {
   __shared__ long long wsum[32];
   const int64_t i = (int64_t)blockIdx.x * kScanBlock + threadIdx.x;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -35,39 +35,59 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_tile(const Tin* __restrict_
   }
   __syncthreads();
   long long base = w ? wsum[w - 1] : 0;
-  if (i < n) out[i] = base + inc - v;
+  if (i < n) out[i] = (int)(base + inc - v);   // total < 2^31, checked on the host
   if (threadIdx.x == kScanBlock - 1) bsum[blockIdx.x] = base + inc;
 }
 
-__global__ void k_scan_add(long long* __restrict__ out, int64_t n, const long long* __restrict__ boff) {
-  const int64_t i = (int64_t)blockIdx.x * kScanBlock + threadIdx.x;
-  if (i < n) out[i] += boff[blockIdx.x];
-}
-
-// exclusive scan of n long longs/ints into out (n entries); returns total on the host
-template <class Tin>
-long long scan_ll(const Tin* in, long long* out, int64_t n, cudaStream_t s) {
-  if (n == 0) return 0;
-  const int nb = div_up(n, kScanBlock);
-  DBuf<long long> bsum(nb), boff(nb);
-  k_scan_tile<Tin><<<nb, kScanBlock, 0, s>>>(in, out, n, bsum.p);
-  FSI_CHECK_LAUNCH();
-  long long total;
-  if (nb == 1) {
-    FSI_CUDA(cudaMemcpyAsync(&total, bsum.p, sizeof(long long), cudaMemcpyDeviceToHost, s));
-    FSI_CUDA(cudaStreamSynchronize(s));
-    return total;
+// Exclusive scan of the nb tile totals in place, by one block; bsum[nb] = the total.
+__global__ void __launch_bounds__(kScanBlock) k_scan_totals(long long* __restrict__ bsum, int nb) {
+  __shared__ long long wsum[32];
+  __shared__ long long carry;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (threadIdx.x == 0) carry = 0;
+  __syncthreads();
+  for (int b0 = 0; b0 < nb; b0 += kScanBlock) {
+    const int i = b0 + threadIdx.x;
+    const long long v = i < nb ? bsum[i] : 0;
+    const long long inc = warp_incl_scan(v, lane);
+    if (lane == 31) wsum[w] = inc;
+    __syncthreads();
+    if (w == 0) wsum[lane] = warp_incl_scan(wsum[lane], lane);
+    __syncthreads();
+    const long long ex = carry + (w ? wsum[w - 1] : 0) + inc - v;
+    if (i < nb) bsum[i] = ex;
+    __syncthreads();
+    if (threadIdx.x == kScanBlock - 1) carry = ex + v;
+    __syncthreads();
   }
-  total = scan_ll<long long>(bsum.p, boff.p, nb, s);
-  k_scan_add<<<nb, kScanBlock, 0, s>>>(out, n, boff.p);
-  FSI_CHECK_LAUNCH();
-  return total;
+  if (threadIdx.x == 0) bsum[nb] = carry;
 }
 
-__global__ void k_ll_to_int(const long long* __restrict__ in, int* __restrict__ out, int64_t n, long long total) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) out[i] = (int)in[i];
-  if (i == n) out[n] = (int)total;
+// Tile offsets added, out[n] = the total.
+__global__ void __launch_bounds__(kScanBlock) k_scan_add(int* __restrict__ out, int64_t n,
+                                                         const long long* __restrict__ bsum, int nb) {
+  const int64_t i = (int64_t)blockIdx.x * kScanBlock + threadIdx.x;
+  if (i < n) out[i] = (int)(out[i] + bsum[blockIdx.x]);
+  if (i == n) out[n] = (int)bsum[nb];
+}
+
+// exclusive scan of n ints into out (n + 1 entries); returns the total on the host (three launches,
+// one wait)
+long long scan_ints(const int* in, int* out, int64_t n, cudaStream_t s) {
+  const int nb = div_up(n, kScanBlock);
+  DBuf<long long> bsum(nb + 1);
+  if (n > 0) {
+    k_scan_tile<<<nb, kScanBlock, 0, s>>>(in, out, n, bsum.p);
+    FSI_CHECK_LAUNCH();
+  }
+  k_scan_totals<<<1, kScanBlock, 0, s>>>(bsum.p, nb);
+  FSI_CHECK_LAUNCH();
+  k_scan_add<<<div_up(n + 1, kScanBlock), kScanBlock, 0, s>>>(out, n, bsum.p, nb);
+  FSI_CHECK_LAUNCH();
+  long long total = 0;
+  FSI_CUDA(cudaMemcpyAsync(&total, bsum.p + nb, sizeof(long long), cudaMemcpyDeviceToHost, s));
+  FSI_CUDA(cudaStreamSynchronize(s));
+  return total;
 }
 
 __device__ __forceinline__ int lower_bound_i(const int* a, int lo, int hi, int key) {
@@ -86,20 +106,62 @@ __device__ __forceinline__ int64_t lower_bound_l(const int* a, int64_t lo, int64
 }
 
 // --------------------------------------------------------------- extraction
-// One thread per block row: merge the br sorted scalar rows restricted to the
-// column window into sorted block columns.
+// One warp per block row.  Rows of a node share their columns as a rule, and the columns
+// of a node come together: then the br scalar rows, restricted to the column window, are
+// the same list of whole blocks, and the lanes read and write them side by side.  Any
+// other block row (a Dirichlet node's identity rows, say) is merged entry by entry by one
+// lane.  (One thread per block row merging every row took 22 ms for the 18 class blocks of
+// the 32x16x16 operator.)
 template <bool FILL>
-__global__ void k_extract(const int64_t* __restrict__ rp, const int* __restrict__ ci, const double* __restrict__ va,
-                          int64_t r0, int nbr, int br, int64_t c0, int64_t c1, int bc, int* __restrict__ cnt,
-                          const int* __restrict__ orp, int* __restrict__ oci, double* __restrict__ ova) {
-  const int row = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(128) k_extract(const int64_t* __restrict__ rp, const int* __restrict__ ci,
+                                                 const double* __restrict__ va, int64_t r0, int nbr, int br,
+                                                 int64_t c0, int64_t c1, int bc, int* __restrict__ cnt,
+                                                 const int* __restrict__ orp, int* __restrict__ oci,
+                                                 double* __restrict__ ova) {
+  const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (row >= nbr) return;
-  int64_t ptr[6], end[6];
-  for (int q = 0; q < br; ++q) {
-    const int64_t r = r0 + (int64_t)row * br + q;
-    ptr[q] = lower_bound_l(ci, rp[r], rp[r + 1], (int)c0);
-    end[q] = lower_bound_l(ci, ptr[q], rp[r + 1], (int)c1);
+  // lanes 0 .. br - 1: the window [from, to) of their scalar row
+  int64_t from = 0;
+  int len = 0;
+  if (lane < br) {
+    const int64_t r = r0 + (int64_t)row * br + lane;
+    from = lower_bound_l(ci, rp[r], rp[r + 1], (int)c0);
+    len = (int)(lower_bound_l(ci, from, rp[r + 1], (int)c1) - from);
   }
+  const int64_t f0 = __shfl_sync(0xffffffffu, from, 0);
+  const int n0 = __shfl_sync(0xffffffffu, len, 0);
+  bool same = !__any_sync(0xffffffffu, lane < br && len != n0) && n0 % bc == 0;
+  for (int q = 0; q < br && same; ++q) {
+    const int64_t f = __shfl_sync(0xffffffffu, from, q);
+    bool ok = true;
+    for (int e = lane; e < n0; e += 32) {
+      const int c = ci[f + e];
+      // row 0: blocks of consecutive, aligned columns; other rows: row 0's columns
+      ok = ok && (q == 0 ? (c - (int)c0) % bc == e % bc && c == ci[f0 + e - e % bc] + e % bc : c == ci[f0 + e]);
+    }
+    same = __all_sync(0xffffffffu, ok);
+  }
+  if (same) {
+    const int nb = n0 / bc;
+    if (!FILL) {
+      if (lane == 0) cnt[row] = nb;
+      return;
+    }
+    const int64_t o = orp[row];
+    for (int e = lane; e < nb; e += 32) oci[o + e] = (int)((ci[f0 + (int64_t)e * bc] - c0) / bc);
+    for (int q = 0; q < br; ++q) {
+      const int64_t f = __shfl_sync(0xffffffffu, from, q);
+      for (int e = lane; e < n0; e += 32) ova[(o + e / bc) * (br * bc) + q * bc + e % bc] = va[f + e];
+    }
+    return;
+  }
+  int64_t ptr[6], end[6];
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    ptr[q] = __shfl_sync(0xffffffffu, from, q);
+    end[q] = ptr[q] + __shfl_sync(0xffffffffu, len, q);
+  }
+  if (lane != 0) return;
   int count = 0;
   int64_t outpos = FILL ? orp[row] : 0;
   while (true) {
@@ -130,14 +192,34 @@ __global__ void k_extract(const int64_t* __restrict__ rp, const int* __restrict_
 }
 
 // --------------------------------------------------------------- add
+// One warp per block row: equal patterns side by side, others merged by one lane.
 template <bool FILL>
-__global__ void k_add(int nbr, int bsz, const int* __restrict__ arp, const int* __restrict__ aci,
-                      const double* __restrict__ ava, const int* __restrict__ brp, const int* __restrict__ bci,
-                      const double* __restrict__ bva, double alpha, int* __restrict__ cnt, const int* __restrict__ crp,
-                      int* __restrict__ cci, double* __restrict__ cva) {
-  const int row = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(128) k_add(int nbr, int bsz, const int* __restrict__ arp,
+                                             const int* __restrict__ aci, const double* __restrict__ ava,
+                                             const int* __restrict__ brp, const int* __restrict__ bci,
+                                             const double* __restrict__ bva, double alpha, int* __restrict__ cnt,
+                                             const int* __restrict__ crp, int* __restrict__ cci,
+                                             double* __restrict__ cva) {
+  const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (row >= nbr) return;
   int ia = arp[row], ea = arp[row + 1], ib = brp[row], eb = brp[row + 1];
+  bool same = ea - ia == eb - ib;
+  if (same) {
+    for (int e = lane; e < ea - ia; e += 32) same = same && aci[ia + e] == bci[ib + e];
+    same = __all_sync(0xffffffffu, same);
+  }
+  if (same) {
+    if (!FILL) {
+      if (lane == 0) cnt[row] = ea - ia;
+      return;
+    }
+    const int64_t o = crp[row];
+    for (int e = lane; e < ea - ia; e += 32) cci[o + e] = aci[ia + e];
+    for (int64_t e = lane; e < (int64_t)(ea - ia) * bsz; e += 32)
+      cva[o * bsz + e] = ava[(int64_t)ia * bsz + e] + alpha * bva[(int64_t)ib * bsz + e];
+    return;
+  }
+  if (lane != 0) return;
   int count = 0;
   int pos = FILL ? crp[row] : 0;
   while (ia < ea || ib < eb) {
@@ -179,21 +261,36 @@ __global__ void k_scatter_t(int64_t nnzb, const int* __restrict__ ci, const int*
   trow[pos] = rowof[k];
   tsrc[pos] = (int)k;
 }
-// insertion sort of each segment by key (with a payload)
-__global__ void k_sort_segments(int nseg, const int* __restrict__ off, int* __restrict__ key, int* __restrict__ pay) {
-  const int sgm = blockIdx.x * blockDim.x + threadIdx.x;
-  if (sgm >= nseg) return;
-  const int lo = off[sgm], hi = off[sgm + 1];
-  for (int i = lo + 1; i < hi; ++i) {
-    int k = key[i], p = pay ? pay[i] : 0;
-    int j = i - 1;
-    while (j >= lo && key[j] > k) {
-      key[j + 1] = key[j];
-      if (pay) pay[j + 1] = pay[j];
-      --j;
-    }
-    key[j + 1] = k;
-    if (pay) pay[j + 1] = p;
+// Each segment of (distinct) keys sorted with its payload, from (key, pay) to (okey, opay):
+// an entry's place is the number of smaller keys.  `group` threads (a warp or the block)
+// per segment, the keys in shared memory where they fit.  (An insertion sort per thread
+// took 49 ms for the transposes of the 32x16x16 hierarchies.)
+constexpr int kSortThreads = 128, kSortKeys = 2048;
+__global__ void __launch_bounds__(kSortThreads) k_sort_segments(int nseg, int group, const int* __restrict__ off,
+                                                                const int* __restrict__ key,
+                                                                const int* __restrict__ pay, int* __restrict__ okey,
+                                                                int* __restrict__ opay) {
+  __shared__ __align__(16) int sk[kSortKeys];
+  const int per = kSortThreads / group, g = threadIdx.x / group, t = threadIdx.x % group;
+  const int cap = kSortKeys / per;
+  const int seg = blockIdx.x * per + g;
+  int lo = 0, n = 0;
+  if (seg < nseg) {
+    lo = off[seg];
+    n = off[seg + 1] - lo;
+  }
+  const bool fits = n <= cap;
+  int* k = sk + g * cap;
+  if (fits)
+    for (int e = t; e < n; e += group) k[e] = key[lo + e];
+  __syncthreads();
+  for (int e = t; e < n; e += group) {
+    const int v = fits ? k[e] : key[lo + e];
+    int rank = 0;
+    if (fits) for (int f = 0; f < n; ++f) rank += k[f] < v;
+    else for (int f = 0; f < n; ++f) rank += __ldg(key + lo + f) < v;
+    okey[lo + rank] = v;
+    if (pay) opay[lo + rank] = pay[lo + e];
   }
 }
 __global__ void k_gather_t(int64_t nnzb, int br, int bc, const int* __restrict__ tsrc, const double* __restrict__ va,
@@ -227,45 +324,62 @@ __device__ __forceinline__ int hash_insert(int* table, int key) {
 }
 
 // Symbolic pass, one warp per row of A.  FILL = false: count unique block
-// columns (flag overflow).  FILL = true: write them sorted.
+// columns (flag overflow; info[1] = the longest row).  FILL = true: write them sorted.
+// A batch of up to 32 entries of A's row has its B rows' bounds read together; `sub`
+// lanes then take one B row each time (about its mean length), so that several short
+// B rows are inserted at once.
 template <bool FILL>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32) k_spgemm_sym(int nbr, const int* __restrict__ arp,
+__global__ void __launch_bounds__(kWarpsPerBlock * 32) k_spgemm_sym(int nbr, int sub, const int* __restrict__ arp,
                                                                     const int* __restrict__ aci,
                                                                     const int* __restrict__ brp,
                                                                     const int* __restrict__ bci, int* __restrict__ cnt,
                                                                     const int* __restrict__ crp, int* __restrict__ cci,
-                                                                    int* __restrict__ overflow) {
+                                                                    int* __restrict__ info) {
   __shared__ int table[kWarpsPerBlock][kHashSize];
-  __shared__ int list[kWarpsPerBlock][kHashSize];
+  __shared__ __align__(16) int list[kWarpsPerBlock][FILL ? kHashSize : 4];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = blockIdx.x * kWarpsPerBlock + w;
   if (row >= nbr) return;   // whole warp exits together
   int* tb = table[w];
   for (int t = lane; t < kHashSize; t += 32) tb[t] = -1;
   __syncwarp();
-  int inserted = 0, full = 0;
-  for (int k = arp[row]; k < arp[row + 1]; ++k) {
-    const int kk = aci[k];
-    for (int q = brp[kk] + lane; q < brp[kk + 1]; q += 32) {
-      const int r = hash_insert(tb, bci[q]);
-      if (r < 0) full = 1; else inserted += r;
+  const int ka = arp[row], ke = arp[row + 1];
+  const int groups = 32 / sub, g = lane / sub, l = lane % sub;
+  int total = 0;
+  for (int k0 = ka; k0 < ke; k0 += 32) {
+    int lo = 0, hi = 0;
+    if (k0 + lane < ke) {
+      const int kk = aci[k0 + lane];
+      lo = brp[kk];
+      hi = brp[kk + 1];
     }
-    __syncwarp();
-    // bail out on overflow (table over 3/4 full or a failed insert)
-    int tot = inserted;
-    for (int off = 16; off > 0; off >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, off);
-    const int anyfull = __any_sync(0xffffffffu, full);
-    if (tot > kHashSize * 3 / 4 || anyfull) {
-      if (lane == 0) atomicExch(overflow, 1);
-      return;
+    const int nk = ke - k0 < 32 ? ke - k0 : 32;
+    for (int j = 0; j < nk; j += groups) {
+      int a = __shfl_sync(0xffffffffu, lo, (j + g) & 31), b = __shfl_sync(0xffffffffu, hi, (j + g) & 31);
+      if (j + g >= nk) b = a;
+      int fresh = 0, full = 0;
+      for (int q = a + l; q < b; q += sub) {
+        const int r = hash_insert(tb, bci[q]);
+        if (r < 0) { full = 1; break; }
+        fresh += r;
+      }
+      total += __reduce_add_sync(0xffffffffu, fresh);
+      // bail out on overflow (table over 3/4 full or a failed insert)
+      if (__any_sync(0xffffffffu, full) || total > kHashSize * 3 / 4) {
+        if (lane == 0) atomicExch(info, 1);
+        return;
+      }
     }
   }
-  for (int off = 16; off > 0; off >>= 1) inserted += __shfl_xor_sync(0xffffffffu, inserted, off);
   if (!FILL) {
-    if (lane == 0) cnt[row] = inserted;
+    if (lane == 0) {
+      cnt[row] = total;
+      if (total > __ldcg(info + 1)) atomicMax(info + 1, total);
+    }
     return;
   }
   // compact the table
+  __syncwarp();
   int* ls = list[w];
   int base = 0;
   for (int t0 = 0; t0 < kHashSize; t0 += 32) {
@@ -274,51 +388,119 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_spgemm_sym(int nbr, con
     if (v != -1) ls[base + __popc(m & ((1u << lane) - 1))] = v;
     base += __popc(m);
   }
+  if (lane < 4 && base + lane < kHashSize) ls[base + lane] = INT_MAX;   // pad the last group of four
   __syncwarp();
   const int out0 = crp[row];
   for (int e = lane; e < base; e += 32) {
     const int v = ls[e];
     int rank = 0;
-    for (int f = 0; f < base; ++f) rank += ls[f] < v;
+    for (int f = 0; f < base; f += 4) {
+      const int4 x = *reinterpret_cast<const int4*>(ls + f);
+      rank += (x.x < v) + (x.y < v) + (x.z < v) + (x.w < v);
+    }
     cci[out0 + rank] = v;
   }
 }
 
+// Numeric pass: C(row, J) = sum over k of A(row, k) B(k, J), every entry summed over k in
+// increasing order.  One warp takes a chunk (blockIdx.y) of a row's `cap` block columns,
+// with the sums in shared memory.  For a batch of up to 32 entries k it first finds where
+// each B entry goes (binary search in the chunk's sorted columns, all lanes on different
+// entries), then adds the B rows one after the other, lanes side by side on (entry,
+// component).  Bound by the FP64 pipe: BK FMAs per (match, component).  (One lane per C
+// entry searching every B row instead did five to ten times as many searches as there
+// are matches, in global memory: 125 ms of a 32x16x16 preconditioner build.)
+constexpr int kSlots = 256;          // matches placed at a time
+constexpr int kNumWarps = 4;
+struct NumScratch {
+  int pref[33], start[32];
+  short slot[kSlots];
+};
+template <int BR, int BC>
+__host__ __device__ constexpr size_t num_smem_per_warp(int cap) {
+  return ((size_t)cap * BR * BC * sizeof(double) + sizeof(int) * (size_t)cap + sizeof(NumScratch) + 15) / 16 * 16;
+}
+
 template <int BR, int BK, int BC>
-__global__ void __launch_bounds__(128) k_spgemm_num(int nbr, const int* __restrict__ arp, const int* __restrict__ aci,
-                                                    const double* __restrict__ ava, const int* __restrict__ brp,
-                                                    const int* __restrict__ bci, const double* __restrict__ bva,
-                                                    const int* __restrict__ crp, const int* __restrict__ cci,
-                                                    double* __restrict__ cva) {
+__global__ void __launch_bounds__(kNumWarps * 32) k_spgemm_num(int nbr, int cap, const int* __restrict__ arp,
+                                                               const int* __restrict__ aci,
+                                                               const double* __restrict__ ava,
+                                                               const int* __restrict__ brp,
+                                                               const int* __restrict__ bci,
+                                                               const double* __restrict__ bva,
+                                                               const int* __restrict__ crp,
+                                                               const int* __restrict__ cci,
+                                                               double* __restrict__ cva) {
+  constexpr int BS = BR * BC;
+  extern __shared__ __align__(16) unsigned char num_sm[];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int row = blockIdx.x * 4 + w;
+  const int row = blockIdx.x * kNumWarps + w;
   if (row >= nbr) return;
-  for (int e = crp[row] + lane; e < crp[row + 1]; e += 32) {
-    const int J = cci[e];
-    double acc[BR * BC];
+  const int c0 = crp[row] + blockIdx.y * cap;
+  const int nc = min(crp[row + 1] - c0, cap);
+  if (nc <= 0) return;
+  unsigned char* base = num_sm + (size_t)w * num_smem_per_warp<BR, BC>(cap);
+  double* acc = reinterpret_cast<double*>(base);
+  int* cols = reinterpret_cast<int*>(acc + (size_t)cap * BS);
+  NumScratch& sc = *reinterpret_cast<NumScratch*>(cols + cap);
+  for (int e = lane; e < nc; e += 32) cols[e] = cci[c0 + e];
+  for (int e = lane; e < nc * BS; e += 32) acc[e] = 0.0;
+  __syncwarp();
+  const int ka = arp[row], ke = arp[row + 1];
+  for (int k0 = ka; k0 < ke; k0 += 32) {
+    const int nk = ke - k0 < 32 ? ke - k0 : 32;
+    int len = 0;
+    if (lane < nk) {
+      const int kk = aci[k0 + lane];
+      const int lo = brp[kk];
+      len = brp[kk + 1] - lo;
+      sc.start[lane] = lo;
+    }
+    int inc = len;
 #pragma unroll
-    for (int t = 0; t < BR * BC; ++t) acc[t] = 0.0;
-    for (int k = arp[row]; k < arp[row + 1]; ++k) {
-      const int kk = aci[k];
-      const int pos = lower_bound_i(bci, brp[kk], brp[kk + 1], J);
-      if (pos < brp[kk + 1] && bci[pos] == J) {
-        const double* a = ava + (int64_t)k * BR * BK;
-        const double* b = bva + (int64_t)pos * BK * BC;
+    for (int off = 1; off < 32; off <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, inc, off);
+      if (lane >= off) inc += t;
+    }
+    sc.pref[lane + 1] = inc;
+    if (lane == 0) sc.pref[0] = 0;
+    __syncwarp();
+    const int tot = sc.pref[32];
+    int k = 0;                                     // the B row that the first match of the part belongs to
+    for (int m0 = 0; m0 < tot; m0 += kSlots) {
+      const int m1 = min(m0 + kSlots, tot);
+      for (int m = m0 + lane; m < m1; m += 32) {
+        int lo = 0, hi = nk;                       // last k with pref[k] <= m
+        while (hi - lo > 1) {
+          const int mid = (lo + hi) >> 1;
+          if (sc.pref[mid] <= m) lo = mid; else hi = mid;
+        }
+        const int J = __ldg(bci + sc.start[lo] + (m - sc.pref[lo]));
+        const int pos = lower_bound_i(cols, 0, nc, J);
+        sc.slot[m - m0] = pos < nc && cols[pos] == J ? (short)pos : (short)-1;
+      }
+      __syncwarp();
+      for (; k < nk; ++k) {
+        const int f = max(sc.pref[k], m0), l = min(sc.pref[k + 1], m1);
+        const double* a = ava + (int64_t)(k0 + k) * BR * BK;
+        const double* b = bva + ((int64_t)sc.start[k] + (f - sc.pref[k])) * BK * BC;
+        for (int e = lane; e < (l - f) * BS; e += 32) {
+          const int m = e / BS, t = e % BS, i = t / BC, j = t % BC;
+          const int p = sc.slot[f - m0 + m];
+          if (p >= 0) {
+            double sum = acc[p * BS + t];
 #pragma unroll
-        for (int i = 0; i < BR; ++i)
-#pragma unroll
-          for (int j = 0; j < BC; ++j) {
-            double s = acc[i * BC + j];
-#pragma unroll
-            for (int q = 0; q < BK; ++q) s += a[i * BK + q] * b[q * BC + j];
-            acc[i * BC + j] = s;
+            for (int q = 0; q < BK; ++q) sum += __ldg(a + i * BK + q) * __ldg(b + (m * BK + q) * BC + j);
+            acc[p * BS + t] = sum;
           }
+        }
+        __syncwarp();
+        if (sc.pref[k + 1] > m1) break;            // the row goes on in the next part
       }
     }
-    double* c = cva + (int64_t)e * BR * BC;
-#pragma unroll
-    for (int t = 0; t < BR * BC; ++t) c[t] = acc[t];
+    __syncwarp();
   }
+  for (int e = lane; e < nc * BS; e += 32) cva[(int64_t)c0 * BS + e] = acc[e];
 }
 
 // --------------------------------------------------------------- misc
@@ -422,26 +604,21 @@ void spgemm_dispatch(int br, int bk, int bc, F&& f) {
                            std::to_string(bc));
 }
 
+// row pointers from the row lengths, and the index array
 void finalize_rowptr(const int* cnt, Bsr& C, cudaStream_t s) {
-  DBuf<long long> tmp(C.nbr + 1);
-  long long total = scan_ll<int>(cnt, tmp.p, C.nbr, s);
-  require(total < INT_MAX, "sparse matrix too large for 32-bit block indices");
   C.rowptr.alloc(C.nbr + 1);
-  k_ll_to_int<<<div_up(C.nbr + 1, 256), 256, 0, s>>>(tmp.p, C.rowptr.p, C.nbr, total);
-  FSI_CHECK_LAUNCH();
+  const long long total = scan_ints(cnt, C.rowptr.p, C.nbr, s);
+  require(total < INT_MAX, "sparse matrix too large for 32-bit block indices");
   C.nnzb = total;
   C.colind.alloc(total > 0 ? total : 1);
-  C.v64.alloc(total > 0 ? total * C.br * C.bc : 1);
 }
+void alloc_values(Bsr& C) { C.v64.alloc(C.nnzb > 0 ? C.nnzb * C.br * C.bc : 1); }
 
 }  // namespace
 
 int64_t exclusive_scan(const int* in, int* out, int64_t n, cudaStream_t s) {
-  DBuf<long long> tmp(n + 1);
-  long long total = scan_ll<int>(in, tmp.p, n, s);
+  const long long total = scan_ints(in, out, n, s);
   require(total < INT_MAX, "scan overflow");
-  k_ll_to_int<<<div_up(n + 1, 256), 256, 0, s>>>(tmp.p, out, n, total);
-  FSI_CHECK_LAUNCH();
   return total;
 }
 
@@ -453,13 +630,14 @@ void extract_bsr(const CsrView& A, int64_t r0, int nbr, int br, int64_t c0, int 
   DBuf<int> cnt(nbr > 0 ? nbr : 1);
   const int64_t c1 = c0 + (int64_t)nbc * bc;
   if (nbr > 0) {
-    k_extract<false><<<div_up(nbr, 128), 128, 0, s>>>(A.rowptr, A.colind, A.vals, r0, nbr, br, c0, c1, bc, cnt.p,
+    k_extract<false><<<div_up((int64_t)nbr * 32, 128), 128, 0, s>>>(A.rowptr, A.colind, A.vals, r0, nbr, br, c0, c1, bc, cnt.p,
                                                     nullptr, nullptr, nullptr);
     FSI_CHECK_LAUNCH();
   }
   finalize_rowptr(cnt.p, out, s);
+  alloc_values(out);
   if (nbr > 0) {
-    k_extract<true><<<div_up(nbr, 128), 128, 0, s>>>(A.rowptr, A.colind, A.vals, r0, nbr, br, c0, c1, bc, nullptr,
+    k_extract<true><<<div_up((int64_t)nbr * 32, 128), 128, 0, s>>>(A.rowptr, A.colind, A.vals, r0, nbr, br, c0, c1, bc, nullptr,
                                                    out.rowptr.p, out.colind.p, out.v64.p);
     FSI_CHECK_LAUNCH();
   }
@@ -473,13 +651,14 @@ void bsr_add(const Bsr& A, const Bsr& B, double alpha, Bsr& C, cudaStream_t s) {
   DBuf<int> cnt(A.nbr > 0 ? A.nbr : 1);
   const int bsz = A.br * A.bc;
   if (A.nbr > 0) {
-    k_add<false><<<div_up(A.nbr, 128), 128, 0, s>>>(A.nbr, bsz, A.rowptr.p, A.colind.p, A.v64.p, B.rowptr.p,
+    k_add<false><<<div_up((int64_t)A.nbr * 32, 128), 128, 0, s>>>(A.nbr, bsz, A.rowptr.p, A.colind.p, A.v64.p, B.rowptr.p,
                                                    B.colind.p, B.v64.p, alpha, cnt.p, nullptr, nullptr, nullptr);
     FSI_CHECK_LAUNCH();
   }
   finalize_rowptr(cnt.p, C, s);
+  alloc_values(C);
   if (A.nbr > 0) {
-    k_add<true><<<div_up(A.nbr, 128), 128, 0, s>>>(A.nbr, bsz, A.rowptr.p, A.colind.p, A.v64.p, B.rowptr.p,
+    k_add<true><<<div_up((int64_t)A.nbr * 32, 128), 128, 0, s>>>(A.nbr, bsz, A.rowptr.p, A.colind.p, A.v64.p, B.rowptr.p,
                                                   B.colind.p, B.v64.p, alpha, nullptr, C.rowptr.p, C.colind.p,
                                                   C.v64.p);
     FSI_CHECK_LAUNCH();
@@ -498,61 +677,84 @@ void bsr_transpose(const Bsr& A, Bsr& C, cudaStream_t s) {
     FSI_CHECK_LAUNCH();
   }
   finalize_rowptr(cnt.p, C, s);
+  alloc_values(C);
   if (A.nnzb == 0) { set_tpr(C); return; }
-  DBuf<int> rowof(A.nnzb), tsrc(A.nnzb);
+  DBuf<int> rowof(A.nnzb), trow(A.nnzb), tsrc(A.nnzb), src(A.nnzb);
   k_row_of_block<<<div_up(A.nbr, 128), 128, 0, s>>>(A.nbr, A.rowptr.p, rowof.p);
   FSI_CHECK_LAUNCH();
-  k_scatter_t<<<div_up(A.nnzb, 256), 256, 0, s>>>(A.nnzb, A.colind.p, rowof.p, C.rowptr.p, cursor.p, C.colind.p,
-                                                 tsrc.p);
+  k_scatter_t<<<div_up(A.nnzb, 256), 256, 0, s>>>(A.nnzb, A.colind.p, rowof.p, C.rowptr.p, cursor.p, trow.p, tsrc.p);
   FSI_CHECK_LAUNCH();
-  k_sort_segments<<<div_up(C.nbr, 128), 128, 0, s>>>(C.nbr, C.rowptr.p, C.colind.p, tsrc.p);
-  FSI_CHECK_LAUNCH();
-  k_gather_t<<<div_up(A.nnzb, 256), 256, 0, s>>>(A.nnzb, A.br, A.bc, tsrc.p, A.v64.p, C.v64.p);
+  sort_segments(C.nbr, A.nnzb, C.rowptr.p, trow.p, tsrc.p, C.colind.p, src.p, s);
+  k_gather_t<<<div_up(A.nnzb, 256), 256, 0, s>>>(A.nnzb, A.br, A.bc, src.p, A.v64.p, C.v64.p);
   FSI_CHECK_LAUNCH();
   set_tpr(C);
 }
 
 void bsr_spgemm(const Bsr& A, const Bsr& B, Bsr& C, cudaStream_t s) {
-  require(bsr_spgemm_if_fits(A, B, C, s), "bsr_spgemm: a product row has more than 768 block columns");
+  int longest = 0;
+  require(bsr_spgemm_pattern(A, B, C, longest, s), "bsr_spgemm: a product row has more than 768 block columns");
+  bsr_spgemm_values(A, B, C, longest, s);
 }
 
-bool bsr_spgemm_if_fits(const Bsr& A, const Bsr& B, Bsr& C, cudaStream_t s) {
+bool bsr_spgemm_pattern(const Bsr& A, const Bsr& B, Bsr& C, int& longest, cudaStream_t s) {
   require(A.bc == B.br && A.nbc == B.nbr, "bsr_spgemm: inner dimensions differ");
   C = Bsr();
   C.nbr = A.nbr; C.nbc = B.nbc; C.br = A.br; C.bc = B.bc;
-  DBuf<int> cnt(A.nbr > 0 ? A.nbr : 1), overflow(1);
-  FSI_CUDA(cudaMemsetAsync(overflow.p, 0, sizeof(int), s));
+  DBuf<int> cnt(A.nbr > 0 ? A.nbr : 1), info(2);
+  FSI_CUDA(cudaMemsetAsync(info.p, 0, 2 * sizeof(int), s));
   const int grid = div_up(A.nbr, kWarpsPerBlock);
+  int sub = 4;
+  while (sub < 32 && B.nbr > 0 && (double)B.nnzb / B.nbr > sub) sub *= 2;
   if (A.nbr > 0) {
-    k_spgemm_sym<false><<<grid, kWarpsPerBlock * 32, 0, s>>>(A.nbr, A.rowptr.p, A.colind.p, B.rowptr.p, B.colind.p,
-                                                            cnt.p, nullptr, nullptr, overflow.p);
+    k_spgemm_sym<false><<<grid, kWarpsPerBlock * 32, 0, s>>>(A.nbr, sub, A.rowptr.p, A.colind.p, B.rowptr.p,
+                                                            B.colind.p, cnt.p, nullptr, nullptr, info.p);
     FSI_CHECK_LAUNCH();
   }
-  int of = 0;
-  FSI_CUDA(cudaMemcpyAsync(&of, overflow.p, sizeof(int), cudaMemcpyDeviceToHost, s));
+  int h[2] = {0, 0};
+  FSI_CUDA(cudaMemcpyAsync(h, info.p, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
   FSI_CUDA(cudaStreamSynchronize(s));
-  if (of) {
+  if (h[0]) {
     C = Bsr();
     return false;
   }
+  longest = h[1];
   finalize_rowptr(cnt.p, C, s);
   if (A.nbr > 0) {
-    k_spgemm_sym<true><<<grid, kWarpsPerBlock * 32, 0, s>>>(A.nbr, A.rowptr.p, A.colind.p, B.rowptr.p, B.colind.p,
-                                                           nullptr, C.rowptr.p, C.colind.p, overflow.p);
+    k_spgemm_sym<true><<<grid, kWarpsPerBlock * 32, 0, s>>>(A.nbr, sub, A.rowptr.p, A.colind.p, B.rowptr.p,
+                                                           B.colind.p, nullptr, C.rowptr.p, C.colind.p, info.p);
     FSI_CHECK_LAUNCH();
-    spgemm_dispatch(A.br, A.bc, B.bc, [&]<int BR, int BK, int BC>() {
-      k_spgemm_num<BR, BK, BC><<<grid, 128, 0, s>>>(A.nbr, A.rowptr.p, A.colind.p, A.v64.p, B.rowptr.p, B.colind.p,
-                                                    B.v64.p, C.rowptr.p, C.colind.p, C.v64.p);
-      FSI_CHECK_LAUNCH();
-    });
   }
   set_tpr(C);
   return true;
 }
 
-void sort_segments(int nseg, const int* off, int* key, int* pay, cudaStream_t s) {
+void bsr_spgemm_values(const Bsr& A, const Bsr& B, Bsr& C, int longest, cudaStream_t s) {
+  alloc_values(C);
+  if (A.nbr == 0 || longest == 0) return;
+  spgemm_dispatch(A.br, A.bc, B.bc, [&]<int BR, int BK, int BC>() {
+    // columns per warp: all of a row's, at most 24 KB of sums, and fewer (up to 4 chunks per
+    // row) when there are too few rows to give every SM about 12 warps
+    const int fits = (int)((24 * 1024) / (BR * BC * sizeof(double)));
+    int chunks = std::min(4, div_up((int64_t)12 * device_sms(), A.nbr));
+    const int cap = std::min(fits, std::max(16, div_up(longest, chunks)));
+    chunks = div_up(longest, cap);
+    const size_t sm = kNumWarps * num_smem_per_warp<BR, BC>(cap);
+    static std::atomic<unsigned long long> attr{0};
+    once_per_device(attr, [](int) {
+      FSI_CUDA(cudaFuncSetAttribute(k_spgemm_num<BR, BK, BC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    128 * 1024));
+    });
+    k_spgemm_num<BR, BK, BC><<<dim3(div_up(A.nbr, kNumWarps), chunks), kNumWarps * 32, sm, s>>>(
+        A.nbr, cap, A.rowptr.p, A.colind.p, A.v64.p, B.rowptr.p, B.colind.p, B.v64.p, C.rowptr.p, C.colind.p, C.v64.p);
+    FSI_CHECK_LAUNCH();
+  });
+}
+
+void sort_segments(int nseg, int64_t n, const int* off, const int* key, const int* pay, int* okey, int* opay,
+                   cudaStream_t s) {
   if (nseg <= 0) return;
-  k_sort_segments<<<div_up(nseg, 128), 128, 0, s>>>(nseg, off, key, pay);
+  const int group = n / nseg > 96 ? kSortThreads : 32;   // long segments: the block's threads share one
+  k_sort_segments<<<div_up(nseg, kSortThreads / group), kSortThreads, 0, s>>>(nseg, group, off, key, pay, okey, opay);
   FSI_CHECK_LAUNCH();
 }
 

@@ -41,8 +41,10 @@ void bsr_transpose(const Bsr& A, Bsr& C, cudaStream_t s);
 // C = A * B  (A: br x bk blocks, B: bk x bc blocks), FP64 values.  A product row
 // may have at most 768 block columns (FSI_EINVAL otherwise).
 void bsr_spgemm(const Bsr& A, const Bsr& B, Bsr& C, cudaStream_t s);
-// The same, returning false (C left empty) instead when a row has more columns.
-bool bsr_spgemm_if_fits(const Bsr& A, const Bsr& B, Bsr& C, cudaStream_t s);
+// The two passes on their own: C's pattern (false and C left empty when a row has more
+// columns; longest: the longest row), then its values.
+bool bsr_spgemm_pattern(const Bsr& A, const Bsr& B, Bsr& C, int& longest, cudaStream_t s);
+void bsr_spgemm_values(const Bsr& A, const Bsr& B, Bsr& C, int longest, cudaStream_t s);
 
 // Scale the scalar rows of A: A[r, :] *= w[r].
 void bsr_scale_rows(Bsr& A, const double* w, cudaStream_t s);
@@ -56,9 +58,10 @@ void bsr_point_diagonal(const Bsr& A, double* diag, cudaStream_t s);
 // dinv = 1/diag where diag != 0, else 0.
 void invert_nonzero(int64_t n, const double* diag, double* dinv, cudaStream_t s);
 
-// Sort each segment [off[i], off[i+1]) of key ascending, carrying pay along
-// (pay may be null).  Segments are short (set-up use).
-void sort_segments(int nseg, const int* off, int* key, int* pay, cudaStream_t s);
+// Sort each segment [off[i], off[i+1]) of the n distinct keys ascending, carrying pay along
+// (pay and opay may be null), into other arrays.
+void sort_segments(int nseg, int64_t n, const int* off, const int* key, const int* pay, int* okey, int* opay,
+                   cudaStream_t s);
 
 // FP32 copy of the values.
 void bsr_make_fp32(Bsr& A, cudaStream_t s);
