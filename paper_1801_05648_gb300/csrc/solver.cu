@@ -152,14 +152,7 @@ inline int grid_n(int64_t n) {
   return (int)(b < 1 ? 1 : b);
 }
 
-// near-nullspaces (host-built, node-major rows, row-major columns)
-std::vector<double> translations(int64_t nodes, int d) {
-  std::vector<double> B((size_t)nodes * d * d, 0.0);
-  for (int64_t i = 0; i < nodes; ++i)
-    for (int r = 0; r < d; ++r) B[((size_t)i * d + r) * d + r] = 1.0;
-  return B;
-}
-
+// rigid-body modes of the solid nodes (host-built once, node-major rows, row-major columns)
 std::vector<double> rigid_modes(const double* X, int64_t nodes, int d) {
   const int k = d == 2 ? 3 : 6;
   std::vector<double> B((size_t)nodes * d * k, 0.0);
@@ -184,6 +177,19 @@ void upload(DBuf<double>& dst, const std::vector<double>& src, cudaStream_t s) {
   if (!src.empty())
     FSI_CUDA(cudaMemcpyAsync(dst.p, src.data(), sizeof(double) * src.size(), cudaMemcpyHostToDevice, s));
   FSI_CUDA(cudaStreamSynchronize(s));
+}
+
+// translations: the d x d identity for each node
+__global__ void k_translations(int64_t n, int d, double* __restrict__ B) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) B[i] = i % d == i / d % d ? 1.0 : 0.0;
+}
+void translations(DBuf<double>& B, int64_t nodes, int d, cudaStream_t s) {
+  const int64_t n = nodes * d * d;
+  B.alloc(n > 0 ? n : 1);
+  if (n == 0) return;
+  k_translations<<<div_up(n, 256), 256, 0, s>>>(n, d, B.p);
+  FSI_CHECK_LAUNCH();
 }
 
 // ------------------------------------------------------------------ sub-solves
@@ -464,7 +470,7 @@ static void extract_blocks(Context& C, const CsrView& A) {
 
 void context_setup(Context& C, const int64_t* rowptr, const int32_t* colind, const double* vals,
                    const double* solid_coords) {
-  SetupPhase setup_phase;
+  SetupPhase setup_phase(C.pool);
   auto t0 = clk::now();
   FSI_CUDA(cudaGetDevice(&C.device));
   FSI_CUDA(cudaStreamCreateWithFlags(&C.s2, cudaStreamNonBlocking));
@@ -498,7 +504,7 @@ void context_setup(Context& C, const int64_t* rowptr, const int32_t* colind, con
 }
 
 void context_update_values(Context& C, const double* vals_dev) {
-  SetupPhase setup_phase;
+  SetupPhase setup_phase(C.pool);
   CsrView v = C.pattern.view();
   v.vals = vals_dev;
   extract_blocks(C, v);
@@ -511,7 +517,7 @@ void context_update_values(Context& C, const double* vals_dev) {
 }
 
 void precond_build(Context& C, int precision) {
-  SetupPhase setup_phase;
+  SetupPhase setup_phase(C.pool);
   auto t0 = clk::now();
   auto& s = C.s;
   const int d = C.dim;
@@ -531,12 +537,12 @@ void precond_build(Context& C, int precision) {
     bsr_add(C.Cpp, BDB, -1.0, Sp, s);
     // hierarchies
     DBuf<double> Bm, Bf, Bp;
-    upload(Bm, translations(C.Mblk.nbr, d), s);
-    upload(Bf, translations(C.Aff.nbr, d), s);
-    upload(Bp, std::vector<double>((size_t)Sp.nbr, 1.0), s);
+    translations(Bm, C.Mblk.nbr, d, s);
+    translations(Bf, C.Aff.nbr, d, s);
+    translations(Bp, Sp.nbr, 1, s);
     const bool rigid = C.solid_B.p != nullptr;
     DBuf<double> Bst;
-    if (!rigid) upload(Bst, translations(Shat.nbr, d), s);
+    if (!rigid) translations(Bst, Shat.nbr, d, s);
     const int ks = rigid ? (d == 2 ? 3 : 6) : d;
     for (auto& H : C.H)
       H.coarse_mode = (C.prm.flags & CLUSTER_COARSE) ? COARSE_CLUSTER

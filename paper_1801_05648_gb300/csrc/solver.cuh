@@ -56,6 +56,7 @@ struct PrecWork {
 };
 
 struct Context {
+  std::shared_ptr<MemPool> pool = std::make_shared<MemPool>();   // buffers of the set-up calls (all on stream s)
   cudaStream_t s = nullptr;
   bool own_stream = false;
   int device = -1;                        // CUDA device current at fsi_setup; every entry point runs on it
