@@ -49,12 +49,13 @@ namespace {
 template <int D, int PD> struct Sh;
 template <int PD> struct Sh<2, PD> {
   static constexpr int NQ2 = 9, NQ1 = PD ? 3 : 4, NL = 36 + NQ1, NQP = 9, NFP = 3;
-  static constexpr int JCELLS = 8;    // cells per CTA of the Jacobian: 36 units of a kind per cell, 9 full warps
+  static constexpr int JCELLS = 8;    // cells per CTA of the Jacobian: 36 units of a kind per cell,
+  static constexpr int JTHREADS = 288;   // 288 in all, one per thread
   static constexpr int RCELLS = 28;   // cells per CTA of the residual: 252 of 256 threads hold a point
 };
 template <int PD> struct Sh<3, PD> {
   static constexpr int NQ2 = 27, NQ1 = PD ? 4 : 8, NL = 162 + NQ1, NQP = 27, NFP = 9;
-  static constexpr int JCELLS = 1;    // 243 units of a kind per cell: 7.6 of 8 warps
+  static constexpr int JCELLS = 1, JTHREADS = 256;   // 243 units of a kind per cell
   static constexpr int RCELLS = 4;
 };
 constexpr int kAsmThreads = 256;
@@ -457,7 +458,7 @@ __global__ void __launch_bounds__(kAsmThreads) k_residual(CellGeom geom, int64_t
 // (b, k), so their additions into a CSR row are contiguous along a lattice line.
 // Positions in the CSR rows are searched once per (row, trial node), not per entry.
 // Measured, against one dual-number evaluation per point and column with a search per
-// entry: 256x128 16.17 -> 2.63 ms, 32x16x16 at theta = 1/2 197.0 -> 14.3 ms (0.77e6 FP64
+// entry: 256x128 16.17 -> 2.52 ms, 32x16x16 at theta = 1/2 197.0 -> 14.0 ms (0.77e6 FP64
 // FMAs per fluid cell; all cells take 9.9 ms at the FP64 pipe's measured 0.529e12 per second).
 template <int D>
 struct Pt {   // per point
@@ -555,7 +556,7 @@ __device__ __forceinline__ int find_col(const int* __restrict__ ci, int len, int
 }
 
 template <int D, int PD>
-__global__ void __launch_bounds__(kAsmThreads, 2) k_jacobian(CellGeom geom, int64_t ncol, Tables T,
+__global__ void __launch_bounds__(Sh<D, PD>::JTHREADS, 2) k_jacobian(CellGeom geom, int64_t ncol, Tables T,
                                                              const __grid_constant__ Basis1 B, Phys P,
                                                              const int* __restrict__ cell_dof,
                                                              const unsigned* __restrict__ cell_flags,
@@ -575,7 +576,9 @@ __global__ void __launch_bounds__(kAsmThreads, 2) k_jacobian(CellGeom geom, int6
   static_assert(R::kAll <= NQ2 * Tr<D>::kN, "raw values fit a point's trial slots");
   extern __shared__ __align__(16) unsigned char asm_smem[];
   JacSmem<D, PD>& S = *reinterpret_cast<JacSmem<D, PD>*>(asm_smem);
-  const int64_t k0 = (int64_t)blockIdx.x * E::JCELLS;
+  // the last cells first: the solid ones, a third of a fluid cell's work, lie at the low end of
+  // the last direction in the meshes of Sec. 6 and fill the SMs' last slots better
+  const int64_t k0 = (int64_t)(gridDim.x - 1 - blockIdx.x) * E::JCELLS;
   const int nc = (int)(ncol - k0 < E::JCELLS ? ncol - k0 : E::JCELLS);
   const bool prev = P.theta != 1.0;
   const double dtt = P.dt * P.theta, mu = P.rho_f * P.nu_f;
@@ -606,9 +609,104 @@ __global__ void __launch_bounds__(kAsmThreads, 2) k_jacobian(CellGeom geom, int6
     const int e = t % (NQP * nr);
     c.tr[e / nr][0][e % nr] = interpolate<D, PD>(T, false, e / nr, e % nr, c.U, c.Uo);
   }
-  // positions of the trial nodes in the rows (v and u rows of node a: the components' rows have equal
-  // patterns as a rule, so the first component's position is tried first)
-  for (int t = threadIdx.x; t < nc * NC * (2 * NQ2 + NQ1); t += blockDim.x) {
+  __syncthreads();
+
+  // ---- point tables, in the first warps
+  constexpr int kPointThreads = (E::JCELLS * NQP + 31) / 32 * 32;
+  static_assert(kPointThreads < E::JTHREADS, "warps left for the positions");
+  double my_min = 1e300;
+  if ((int)threadIdx.x < nc * NQP) {
+    const int t = threadIdx.x;
+    C& c = S.c[t / NQP];
+    const int q = t % NQP;
+    const double* raw = c.tr[q][0];
+    double* o = c.pt[q];
+    const double w = T.w[q];
+    double F[D][D];
+    read_F<D>(raw + R::Gu, F);
+    const double J = det<D>(F);
+    if (J < my_min) my_min = J;
+    using K = Pt<D>;
+    const bool solid = c.flags & 1u;
+    if (solid) {
+      double Bm[D][D], Sg[D][D], tr = 0.0;
+      matmul_t<D>(F, F, Bm);
+#pragma unroll
+      for (int i = 0; i < D; ++i)
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+          double s = F[0][i] * F[0][j];
+#pragma unroll
+          for (int m = 1; m < D; ++m) s += F[m][i] * F[m][j];
+          Sg[i][j] = 0.5 * (s - (i == j ? 1.0 : 0.0));
+        }
+#pragma unroll
+      for (int i = 0; i < D; ++i) tr += Sg[i][i];
+#pragma unroll
+      for (int i = 0; i < D; ++i)
+#pragma unroll
+        for (int j = 0; j < D; ++j) Sg[i][j] = 2.0 * P.mu_s * Sg[i][j] + (i == j ? P.lambda_s * tr : 0.0);
+      write_mat<D>(o + K::sF, 1.0, F);
+      write_mat<D>(o + K::smF, w * dtt * P.mu_s, F);
+      write_mat<D>(o + K::slF, w * dtt * P.lambda_s, F);
+      write_mat<D>(o + K::sB, w * dtt * P.mu_s, Bm);
+      write_mat<D>(o + K::sS, w * dtt, Sg);
+    }
+    if (!solid) {
+      double Fi[D][D], A[D][D], Gv[D][D], X[D][D], Y[D][D], p = 0.0, trA = 0.0, Jo = 1.0;
+      read_mat<D>(raw + R::Gv, Gv);
+      const double iJ = 1.0 / J;
+      invert<D>(F, iJ, Fi);
+      matmul<D>(Gv, Fi, A);
+      if (prev) {
+        double Fo[D][D];
+        read_F<D>(raw + R::Guo, Fo);
+        Jo = det<D>(Fo);
+      }
+#pragma unroll
+      for (int a = 0; a < NQ1; ++a) p += T.Np[q * NQ1 + a] * c.U[2 * NV + a];
+      const double m = dtt * mu, wJ = w * J;
+      write_mat<D>(o + K::Fi, 1.0, Fi);
+      write_mat<D>(o + K::A, 1.0, A);
+      write_mat<D>(o + K::Fim, wJ * m, Fi);
+      matmul<D>(Fi, A, Y);
+      write_mat<D>(o + K::FA, wJ * m, Y);
+#pragma unroll
+      for (int i = 0; i < D; ++i) {
+        trA += A[i][i];
+#pragma unroll
+        for (int j = 0; j < D; ++j) X[i][j] = wJ * (m * (A[i][j] + A[j][i]) - (i == j ? p : 0.0));
+      }
+      matmul_t<D>(X, Fi, Y);
+      write_mat<D>(o + K::PX, 1.0, Y);
+      const double wi = w * iJ;
+#pragma unroll
+      for (int i = 0; i < D * D; ++i) o[K::GuJ + i] = wi * raw[R::Gu + i];
+      double cv[D];
+#pragma unroll
+      for (int j = 0; j < D; ++j) cv[j] = dtt * raw[R::v + j] - (raw[R::u + j] - raw[R::uo + j]);
+#pragma unroll
+      for (int i = 0; i < D; ++i) {
+        double s = (prev ? P.theta : 1.0) * (raw[R::v + i] - raw[R::vo + i]);
+#pragma unroll
+        for (int j = 0; j < D; ++j) s += A[i][j] * cv[j];
+        o[K::e + i] = wJ * P.rho_f * s;
+      }
+      o[K::wJ] = wJ;
+      o[K::trA] = trA;
+      o[K::wJi] = wi;
+      // for the trial tables: c, and J^theta w rho_f; kept in raw slots that no other point reads
+      double* z = c.tr[q][0] + R::Gv;
+#pragma unroll
+      for (int j = 0; j < D; ++j) z[j] = cv[j];
+      z[D] = w * P.rho_f * (prev ? P.theta * J + (1.0 - P.theta) * Jo : J);
+      z[D + 1] = p;
+    }
+  }
+  // meanwhile, in the other warps: positions of the trial nodes in the rows (the components' rows of a
+  // node have equal patterns as a rule, so the first component's position is tried first)
+  for (int t = (int)threadIdx.x - kPointThreads; t >= 0 && t < nc * NC * (2 * NQ2 + NQ1);
+       t += (int)blockDim.x - kPointThreads) {
     C& c = S.c[t / (NC * (2 * NQ2 + NQ1))];
     const int e = t % (NC * (2 * NQ2 + NQ1)), rn = e / NC, cn = e % NC;
     const int nrows = rn < 2 * NQ2 ? D : 1, r0 = rn < 2 * NQ2 ? rn * D : 2 * NV + rn - 2 * NQ2;
@@ -634,95 +732,6 @@ __global__ void __launch_bounds__(kAsmThreads, 2) k_jacobian(CellGeom geom, int6
       }
       c.pos[r0 + i][cn] = found;
     }
-  }
-  __syncthreads();
-
-  // ---- point tables
-  double my_min = 1e300;
-  for (int t = threadIdx.x; t < nc * NQP; t += blockDim.x) {
-    C& c = S.c[t / NQP];
-    const int q = t % NQP;
-    const double* raw = c.tr[q][0];
-    double* o = c.pt[q];
-    const double w = T.w[q];
-    double F[D][D];
-    read_F<D>(raw + R::Gu, F);
-    const double J = det<D>(F);
-    if (J < my_min) my_min = J;
-    using K = Pt<D>;
-    if (c.flags & 1u) {
-      double Bm[D][D], Sg[D][D], tr = 0.0;
-      matmul_t<D>(F, F, Bm);
-#pragma unroll
-      for (int i = 0; i < D; ++i)
-#pragma unroll
-        for (int j = 0; j < D; ++j) {
-          double s = F[0][i] * F[0][j];
-#pragma unroll
-          for (int m = 1; m < D; ++m) s += F[m][i] * F[m][j];
-          Sg[i][j] = 0.5 * (s - (i == j ? 1.0 : 0.0));
-        }
-#pragma unroll
-      for (int i = 0; i < D; ++i) tr += Sg[i][i];
-#pragma unroll
-      for (int i = 0; i < D; ++i)
-#pragma unroll
-        for (int j = 0; j < D; ++j) Sg[i][j] = 2.0 * P.mu_s * Sg[i][j] + (i == j ? P.lambda_s * tr : 0.0);
-      write_mat<D>(o + K::sF, 1.0, F);
-      write_mat<D>(o + K::smF, w * dtt * P.mu_s, F);
-      write_mat<D>(o + K::slF, w * dtt * P.lambda_s, F);
-      write_mat<D>(o + K::sB, w * dtt * P.mu_s, Bm);
-      write_mat<D>(o + K::sS, w * dtt, Sg);
-      continue;
-    }
-    double Fi[D][D], A[D][D], Gv[D][D], X[D][D], Y[D][D], p = 0.0, trA = 0.0, Jo = 1.0;
-    read_mat<D>(raw + R::Gv, Gv);
-    const double iJ = 1.0 / J;
-    invert<D>(F, iJ, Fi);
-    matmul<D>(Gv, Fi, A);
-    if (prev) {
-      double Fo[D][D];
-      read_F<D>(raw + R::Guo, Fo);
-      Jo = det<D>(Fo);
-    }
-#pragma unroll
-    for (int a = 0; a < NQ1; ++a) p += T.Np[q * NQ1 + a] * c.U[2 * NV + a];
-    const double m = dtt * mu, wJ = w * J;
-    write_mat<D>(o + K::Fi, 1.0, Fi);
-    write_mat<D>(o + K::A, 1.0, A);
-    write_mat<D>(o + K::Fim, wJ * m, Fi);
-    matmul<D>(Fi, A, Y);
-    write_mat<D>(o + K::FA, wJ * m, Y);
-#pragma unroll
-    for (int i = 0; i < D; ++i) {
-      trA += A[i][i];
-#pragma unroll
-      for (int j = 0; j < D; ++j) X[i][j] = wJ * (m * (A[i][j] + A[j][i]) - (i == j ? p : 0.0));
-    }
-    matmul_t<D>(X, Fi, Y);
-    write_mat<D>(o + K::PX, 1.0, Y);
-    const double wi = w * iJ;
-#pragma unroll
-    for (int i = 0; i < D * D; ++i) o[K::GuJ + i] = wi * raw[R::Gu + i];
-    double cv[D];
-#pragma unroll
-    for (int j = 0; j < D; ++j) cv[j] = dtt * raw[R::v + j] - (raw[R::u + j] - raw[R::uo + j]);
-#pragma unroll
-    for (int i = 0; i < D; ++i) {
-      double s = (prev ? P.theta : 1.0) * (raw[R::v + i] - raw[R::vo + i]);
-#pragma unroll
-      for (int j = 0; j < D; ++j) s += A[i][j] * cv[j];
-      o[K::e + i] = wJ * P.rho_f * s;
-    }
-    o[K::wJ] = wJ;
-    o[K::trA] = trA;
-    o[K::wJi] = wi;
-    // for the trial tables: c, and J^theta w rho_f; kept in raw slots that no other point reads
-    double* z = c.tr[q][0] + R::Gv;
-#pragma unroll
-    for (int j = 0; j < D; ++j) z[j] = cv[j];
-    z[D] = w * P.rho_f * (prev ? P.theta * J + (1.0 - P.theta) * Jo : J);
-    z[D + 1] = p;
   }
   if (my_min < 1e300) atomicMin(&S.minkey, order_key(my_min));
   __syncthreads();
@@ -1209,7 +1218,7 @@ void run_jacobian(Assembler& A, const double* U, const double* Uold, double* val
     FSI_CUDA(cudaFuncSetAttribute(k_jacobian<D, PD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   });
   for_colours<D>(A, [&](const CellGeom& g, int64_t cnt) {
-    k_jacobian<D, PD><<<div_up(cnt, Sh<D, PD>::JCELLS), kAsmThreads, sm, A.s>>>(
+    k_jacobian<D, PD><<<div_up(cnt, Sh<D, PD>::JCELLS), Sh<D, PD>::JTHREADS, sm, A.s>>>(
         g, cnt, A.T, A.B1, A.phys, A.cell_dof.p, A.cell_flags.p, A.rowptr.p, A.colind.p, A.fixed.p, U, Uold, vals,
         A.res.p, reinterpret_cast<int*>(A.res.p + 2));
   });

@@ -9,13 +9,12 @@
 // leaves the kNb multipliers of every row, and one launch over the whole GPU
 // (k_gj_update), which applies the panel's swaps and its kNb rank-1 updates to the other
 // columns.  Every entry sees the operations of the column-by-column elimination in the
-// same order with the same rounding (one fused multiply-add per step with a nonzero
-// multiplier), so the inverse has the same bits as one launch per pivot gave.
+// same order with the same rounding (one fused multiply-add per step), so the inverse has the same bits as one launch per pivot gave.
 //
 // Why panels: one launch per pivot took 11 us (n = 300) to 40 us (n = 1100) because each
 // read and wrote 2 n^2 entries and ended with one CTA's search for the next pivot.  The
-// four inverses of a 32x16x16 preconditioner (3,315 pivots) went from 133 to 33 ms, those
-// of a 256x128 one (1,139 pivots) from 20 to 6.5 ms.
+// four inverses of a 32x16x16 preconditioner (3,315 pivots) went from 133 to 21 ms, those
+// of a 256x128 one (1,139 pivots) from 20 to 5 ms.
 #include "sparse_util.cuh"
 
 #include <cooperative_groups.h>
@@ -31,10 +30,10 @@ constexpr int kPanelThreads = 256;
 constexpr int kMaxCluster = 16;
 constexpr int kLd = kNb + 1;          // row stride of the panel in shared memory
 
-// Zero tests and magnitude comparisons on the bits: an FP64 comparison would take the
-// FP64 pipe as long as a multiply-add does.
-__device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
-// orders like |x|, 0 for NaN (never a pivot), at least 1 otherwise
+// Magnitudes compared on the bits: an FP64 comparison would take the FP64 pipe as long as
+// a multiply-add does.  (For the same reason a zero multiplier is not tested for: fma(-0, u, w)
+// is w for every finite pivot row u, up to the sign of a zero.)
+// Orders like |x|, 0 for NaN (never a pivot), at least 1 otherwise
 __device__ __forceinline__ unsigned long long pivot_key(double x) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
   return b > 0x7FF0000000000000ull ? 0ull : b + 1;
@@ -143,7 +142,7 @@ __global__ void __launch_bounds__(kPanelThreads) k_gj_panel(int n, int P0, int n
         l[c] = c == s ? 0.0 : (none ? box.l[c] : o.l[c]);
       } else {
         const double y = c == s ? 0.0 : x;
-        w[c] = nonzero(f) ? __fma_rn(-f, u, y) : y;
+        w[c] = __fma_rn(-f, u, y);
         if (c == s) l[c] = f;
         else if (swapped) l[c] = box.l[c];
       }
@@ -213,8 +212,7 @@ __global__ void __launch_bounds__(kUpThreads) k_gj_update(int n, int P0, int nb,
       U[p][lane] = u[p];
 #pragma unroll
       for (int q = p + 1; q < kNb; ++q) {
-        const double f = Lp[q][p], y = __fma_rn(-f, u[p], u[q]);
-        u[q] = nonzero(f) ? y : u[q];
+        u[q] = __fma_rn(-Lp[q][p], u[p], u[q]);
       }
     }
   }
@@ -228,8 +226,7 @@ __global__ void __launch_bounds__(kUpThreads) k_gj_update(int n, int P0, int nb,
     double w = in_panel >= 0 && in_panel < nb ? U[in_panel][lane] : (on ? Win[(int64_t)src[i] * n + c] : 0.0);
 #pragma unroll
     for (int p = 0; p < kNb; ++p) {
-      const double f = Ls[i][p], y = __fma_rn(-f, u[p], w);
-      w = nonzero(f) ? y : w;
+      w = __fma_rn(-Ls[i][p], u[p], w);
     }
     if (on) Wout[(int64_t)(r0 + i) * n + c] = w;
   }

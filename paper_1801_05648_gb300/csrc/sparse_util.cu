@@ -2,6 +2,7 @@
 
 #include <algorithm>
 #include <climits>
+#include <type_traits>
 
 namespace fsi {
 
@@ -323,30 +324,34 @@ __device__ __forceinline__ int hash_insert(int* table, int key) {
   return -1;
 }
 
-// Symbolic pass, one warp per row of A.  FILL = false: count unique block
-// columns (flag overflow; info[1] = the longest row).  FILL = true: write them sorted.
-// A batch of up to 32 entries of A's row has its B rows' bounds read together; `sub`
-// lanes then take one B row each time (about its mean length), so that several short
-// B rows are inserted at once.
-template <bool FILL>
+// Symbolic pass, WPR warps per row of A (the whole block, for products of few long
+// rows, or one).  FILL = false: count unique block columns (flag overflow; info[1] = the
+// longest row).  FILL = true: write them sorted.  Each warp takes batches of 32 entries of
+// A's row and reads their B rows' bounds together; `sub` lanes then take one B row each
+// time (about its mean length), so that several short B rows are inserted at once.
+template <bool FILL, int WPR>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_spgemm_sym(int nbr, int sub, const int* __restrict__ arp,
                                                                     const int* __restrict__ aci,
                                                                     const int* __restrict__ brp,
                                                                     const int* __restrict__ bci, int* __restrict__ cnt,
                                                                     const int* __restrict__ crp, int* __restrict__ cci,
                                                                     int* __restrict__ info) {
-  __shared__ int table[kWarpsPerBlock][kHashSize];
-  __shared__ __align__(16) int list[kWarpsPerBlock][FILL ? kHashSize : 4];
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int row = blockIdx.x * kWarpsPerBlock + w;
-  if (row >= nbr) return;   // whole warp exits together
-  int* tb = table[w];
-  for (int t = lane; t < kHashSize; t += 32) tb[t] = -1;
-  __syncwarp();
+  static_assert(WPR == 1 || WPR == kWarpsPerBlock, "a warp or the block per row");
+  constexpr int ROWS = kWarpsPerBlock / WPR, T = WPR * 32;
+  __shared__ int table[ROWS][kHashSize];
+  __shared__ __align__(16) int list[ROWS][FILL ? kHashSize : 4];
+  __shared__ int found[ROWS], wide[ROWS], place[ROWS];
+  const int g = threadIdx.x / T, t = threadIdx.x % T, lane = threadIdx.x & 31, wr = t / 32;
+  const int row = blockIdx.x * ROWS + g;
+  if (row >= nbr) return;   // a row's threads leave together
+  auto sync = [] { if constexpr (WPR == 1) __syncwarp(); else __syncthreads(); };
+  int* tb = table[g];
+  for (int e = t; e < kHashSize; e += T) tb[e] = -1;
+  if (t == 0) found[g] = wide[g] = place[g] = 0;
+  sync();
   const int ka = arp[row], ke = arp[row + 1];
-  const int groups = 32 / sub, g = lane / sub, l = lane % sub;
-  int total = 0;
-  for (int k0 = ka; k0 < ke; k0 += 32) {
+  const int groups = 32 / sub, q0 = lane / sub, l = lane % sub;
+  for (int k0 = ka + 32 * wr; k0 < ke; k0 += T) {
     int lo = 0, hi = 0;
     if (k0 + lane < ke) {
       const int kk = aci[k0 + lane];
@@ -354,47 +359,60 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_spgemm_sym(int nbr, int
       hi = brp[kk + 1];
     }
     const int nk = ke - k0 < 32 ? ke - k0 : 32;
-    for (int j = 0; j < nk; j += groups) {
-      int a = __shfl_sync(0xffffffffu, lo, (j + g) & 31), b = __shfl_sync(0xffffffffu, hi, (j + g) & 31);
-      if (j + g >= nk) b = a;
+    bool stop = false;
+    for (int j = 0; j < nk && !stop; j += groups) {
+      int a = __shfl_sync(0xffffffffu, lo, (j + q0) & 31), b = __shfl_sync(0xffffffffu, hi, (j + q0) & 31);
+      if (j + q0 >= nk) b = a;
       int fresh = 0, full = 0;
       for (int q = a + l; q < b; q += sub) {
         const int r = hash_insert(tb, bci[q]);
         if (r < 0) { full = 1; break; }
         fresh += r;
       }
-      total += __reduce_add_sync(0xffffffffu, fresh);
-      // bail out on overflow (table over 3/4 full or a failed insert)
-      if (__any_sync(0xffffffffu, full) || total > kHashSize * 3 / 4) {
-        if (lane == 0) atomicExch(info, 1);
-        return;
+      fresh = __reduce_add_sync(0xffffffffu, fresh);
+      full = __any_sync(0xffffffffu, full);
+      // over 3/4 of the table in use, or a failed insert: the row does not fit
+      int total = 0;
+      if (lane == 0) {
+        total = (fresh ? atomicAdd(&found[g], fresh) : *(volatile int*)&found[g]) + fresh;
+        if (full || total > kHashSize * 3 / 4) *(volatile int*)&wide[g] = 1;
       }
+      stop = __shfl_sync(0xffffffffu, lane == 0 && (full || total > kHashSize * 3 / 4), 0);
     }
+    if (stop || *(volatile int*)&wide[g]) break;
+  }
+  sync();
+  if (wide[g]) {
+    if (t == 0) atomicExch(info, 1);
+    return;
   }
   if (!FILL) {
-    if (lane == 0) {
+    if (t == 0) {
+      const int total = found[g];
       cnt[row] = total;
       if (total > __ldcg(info + 1)) atomicMax(info + 1, total);
     }
     return;
   }
-  // compact the table
-  __syncwarp();
-  int* ls = list[w];
-  int base = 0;
-  for (int t0 = 0; t0 < kHashSize; t0 += 32) {
-    int v = tb[t0 + lane];
-    unsigned m = __ballot_sync(0xffffffffu, v != -1);
+  // compact the table (in any order: the ranks put it in order)
+  int* ls = list[g];
+  for (int t0 = 32 * wr; t0 < kHashSize; t0 += T) {
+    const int v = tb[t0 + lane];
+    const unsigned m = __ballot_sync(0xffffffffu, v != -1);
+    int base = 0;
+    if (lane == 0) base = atomicAdd(&place[g], __popc(m));
+    base = __shfl_sync(0xffffffffu, base, 0);
     if (v != -1) ls[base + __popc(m & ((1u << lane) - 1))] = v;
-    base += __popc(m);
   }
-  if (lane < 4 && base + lane < kHashSize) ls[base + lane] = INT_MAX;   // pad the last group of four
-  __syncwarp();
+  sync();
+  const int n = found[g];
+  if (t < 4 && n + t < kHashSize) ls[n + t] = INT_MAX;   // pad the last group of four
+  sync();
   const int out0 = crp[row];
-  for (int e = lane; e < base; e += 32) {
+  for (int e = t; e < n; e += T) {
     const int v = ls[e];
     int rank = 0;
-    for (int f = 0; f < base; f += 4) {
+    for (int f = 0; f < n; f += 4) {
       const int4 x = *reinterpret_cast<const int4*>(ls + f);
       rank += (x.x < v) + (x.y < v) + (x.z < v) + (x.w < v);
     }
@@ -403,13 +421,16 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_spgemm_sym(int nbr, int
 }
 
 // Numeric pass: C(row, J) = sum over k of A(row, k) B(k, J), every entry summed over k in
-// increasing order.  One warp takes a chunk (blockIdx.y) of a row's `cap` block columns,
-// with the sums in shared memory.  For a batch of up to 32 entries k it first finds where
-// each B entry goes (binary search in the chunk's sorted columns, all lanes on different
-// entries), then adds the B rows one after the other, lanes side by side on (entry,
-// component).  Bound by the FP64 pipe: BK FMAs per (match, component).  (One lane per C
-// entry searching every B row instead did five to ten times as many searches as there
-// are matches, in global memory: 125 ms of a 32x16x16 preconditioner build.)
+// increasing order.  One warp takes a chunk (blockIdx.y) of `cap` consecutive block
+// columns of a row, with the sums in shared memory.  For a batch of up to 32 entries k the
+// lanes first cut each B row to the chunk's columns, then find where each of the batch's
+// remaining entries goes (binary search in the chunk's columns, all lanes on different
+// entries), and then add the B rows one after the other, lanes side by side on (entry,
+// component), several loads ahead of the sums.  Bound by the FP64 pipe (BK FMAs per match
+// and component) as long as an SM holds about eight warps: the chunks are kept small for
+// that, and smaller when there are few rows.  All products of a 32x16x16 preconditioner build:
+// 24 ms; one lane per C entry searching every B row took 125 ms, whole rows per warp (two
+// CTAs' worth of sums per SM) 66 ms.
 constexpr int kSlots = 256;          // matches placed at a time
 constexpr int kNumWarps = 4;
 struct NumScratch {
@@ -431,7 +452,7 @@ __global__ void __launch_bounds__(kNumWarps * 32) k_spgemm_num(int nbr, int cap,
                                                                const int* __restrict__ crp,
                                                                const int* __restrict__ cci,
                                                                double* __restrict__ cva) {
-  constexpr int BS = BR * BC;
+  constexpr int BS = BR * BC, U = BK <= 3 ? 4 : 2;   // U items per lane loaded before their sums
   extern __shared__ __align__(16) unsigned char num_sm[];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = blockIdx.x * kNumWarps + w;
@@ -446,14 +467,20 @@ __global__ void __launch_bounds__(kNumWarps * 32) k_spgemm_num(int nbr, int cap,
   for (int e = lane; e < nc; e += 32) cols[e] = cci[c0 + e];
   for (int e = lane; e < nc * BS; e += 32) acc[e] = 0.0;
   __syncwarp();
+  const int first = cols[0], last = cols[nc - 1];
+  const bool part = nc < crp[row + 1] - crp[row];
   const int ka = arp[row], ke = arp[row + 1];
   for (int k0 = ka; k0 < ke; k0 += 32) {
     const int nk = ke - k0 < 32 ? ke - k0 : 32;
     int len = 0;
     if (lane < nk) {
       const int kk = aci[k0 + lane];
-      const int lo = brp[kk];
-      len = brp[kk + 1] - lo;
+      int lo = brp[kk], hi = brp[kk + 1];
+      if (part) {
+        lo = lower_bound_i(bci, lo, hi, first);
+        hi = lower_bound_i(bci, lo, hi, last + 1);
+      }
+      len = hi - lo;
       sc.start[lane] = lo;
     }
     int inc = len;
@@ -476,22 +503,38 @@ __global__ void __launch_bounds__(kNumWarps * 32) k_spgemm_num(int nbr, int cap,
           if (sc.pref[mid] <= m) lo = mid; else hi = mid;
         }
         const int J = __ldg(bci + sc.start[lo] + (m - sc.pref[lo]));
-        const int pos = lower_bound_i(cols, 0, nc, J);
-        sc.slot[m - m0] = pos < nc && cols[pos] == J ? (short)pos : (short)-1;
+        sc.slot[m - m0] = (short)lower_bound_i(cols, 0, nc, J);   // present: C's pattern covers every match
       }
       __syncwarp();
       for (; k < nk; ++k) {
         const int f = max(sc.pref[k], m0), l = min(sc.pref[k + 1], m1);
         const double* a = ava + (int64_t)(k0 + k) * BR * BK;
         const double* b = bva + ((int64_t)sc.start[k] + (f - sc.pref[k])) * BK * BC;
-        for (int e = lane; e < (l - f) * BS; e += 32) {
-          const int m = e / BS, t = e % BS, i = t / BC, j = t % BC;
-          const int p = sc.slot[f - m0 + m];
-          if (p >= 0) {
-            double sum = acc[p * BS + t];
+        const int ne = (l - f) * BS;
+        for (int e0 = lane; e0 < ne; e0 += 32 * U) {
+          double av[U][BK], bv[U][BK];
 #pragma unroll
-            for (int q = 0; q < BK; ++q) sum += __ldg(a + i * BK + q) * __ldg(b + (m * BK + q) * BC + j);
-            acc[p * BS + t] = sum;
+          for (int u = 0; u < U; ++u) {
+            const int e = e0 + 32 * u;
+            if (e < ne) {
+              const int m = e / BS, t = e % BS, i = t / BC, j = t % BC;
+#pragma unroll
+              for (int q = 0; q < BK; ++q) {
+                av[u][q] = __ldg(a + i * BK + q);
+                bv[u][q] = __ldg(b + (m * BK + q) * BC + j);
+              }
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int e = e0 + 32 * u;
+            if (e < ne) {
+              double* s = acc + sc.slot[f - m0 + e / BS] * BS + e % BS;
+              double sum = *s;
+#pragma unroll
+              for (int q = 0; q < BK; ++q) sum += av[u][q] * bv[u][q];
+              *s = sum;
+            }
           }
         }
         __syncwarp();
@@ -702,14 +745,19 @@ bool bsr_spgemm_pattern(const Bsr& A, const Bsr& B, Bsr& C, int& longest, cudaSt
   C.nbr = A.nbr; C.nbc = B.nbc; C.br = A.br; C.bc = B.bc;
   DBuf<int> cnt(A.nbr > 0 ? A.nbr : 1), info(2);
   FSI_CUDA(cudaMemsetAsync(info.p, 0, 2 * sizeof(int), s));
-  const int grid = div_up(A.nbr, kWarpsPerBlock);
   int sub = 4;
   while (sub < 32 && B.nbr > 0 && (double)B.nnzb / B.nbr > sub) sub *= 2;
-  if (A.nbr > 0) {
-    k_spgemm_sym<false><<<grid, kWarpsPerBlock * 32, 0, s>>>(A.nbr, sub, A.rowptr.p, A.colind.p, B.rowptr.p,
-                                                            B.colind.p, cnt.p, nullptr, nullptr, info.p);
+  // a block per row when a warp per row would leave an SM fewer than 16 warps
+  const bool wide = A.nbr < 16 * device_sms();
+  const int grid = wide ? A.nbr : div_up(A.nbr, kWarpsPerBlock);
+  auto pass = [&](auto fill) {
+    constexpr bool FILL = decltype(fill)::value;
+    if (A.nbr == 0) return;
+    (wide ? k_spgemm_sym<FILL, kWarpsPerBlock> : k_spgemm_sym<FILL, 1>)<<<grid, kWarpsPerBlock * 32, 0, s>>>(
+        A.nbr, sub, A.rowptr.p, A.colind.p, B.rowptr.p, B.colind.p, cnt.p, C.rowptr.p, C.colind.p, info.p);
     FSI_CHECK_LAUNCH();
-  }
+  };
+  pass(std::false_type());
   int h[2] = {0, 0};
   FSI_CUDA(cudaMemcpyAsync(h, info.p, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
   FSI_CUDA(cudaStreamSynchronize(s));
@@ -719,11 +767,7 @@ bool bsr_spgemm_pattern(const Bsr& A, const Bsr& B, Bsr& C, int& longest, cudaSt
   }
   longest = h[1];
   finalize_rowptr(cnt.p, C, s);
-  if (A.nbr > 0) {
-    k_spgemm_sym<true><<<grid, kWarpsPerBlock * 32, 0, s>>>(A.nbr, sub, A.rowptr.p, A.colind.p, B.rowptr.p,
-                                                           B.colind.p, nullptr, C.rowptr.p, C.colind.p, info.p);
-    FSI_CHECK_LAUNCH();
-  }
+  pass(std::true_type());
   set_tpr(C);
   return true;
 }
@@ -732,18 +776,15 @@ void bsr_spgemm_values(const Bsr& A, const Bsr& B, Bsr& C, int longest, cudaStre
   alloc_values(C);
   if (A.nbr == 0 || longest == 0) return;
   spgemm_dispatch(A.br, A.bc, B.bc, [&]<int BR, int BK, int BC>() {
-    // columns per warp: all of a row's, at most 24 KB of sums, and fewer (up to 4 chunks per
-    // row) when there are too few rows to give every SM about 12 warps
-    const int fits = (int)((24 * 1024) / (BR * BC * sizeof(double)));
-    int chunks = std::min(4, div_up((int64_t)12 * device_sms(), A.nbr));
-    const int cap = std::min(fits, std::max(16, div_up(longest, chunks)));
-    chunks = div_up(longest, cap);
+    // columns per warp: about 5 KB of sums (a row a little longer is not split), fewer when
+    // rows x chunks would leave an SM fewer than 16 warps, at least 12
+    const int most = (int)(5 * 1024 / (BR * BC * sizeof(double)));
+    int cap = longest <= most + most / 2 ? longest : most;
+    const int64_t tasks = (int64_t)16 * device_sms();
+    if ((int64_t)A.nbr * div_up(longest, cap) < tasks)
+      cap = std::min(cap, std::max(12, (int)((int64_t)A.nbr * longest / tasks)));
+    const int chunks = div_up(longest, cap);
     const size_t sm = kNumWarps * num_smem_per_warp<BR, BC>(cap);
-    static std::atomic<unsigned long long> attr{0};
-    once_per_device(attr, [](int) {
-      FSI_CUDA(cudaFuncSetAttribute(k_spgemm_num<BR, BK, BC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    128 * 1024));
-    });
     k_spgemm_num<BR, BK, BC><<<dim3(div_up(A.nbr, kNumWarps), chunks), kNumWarps * 32, sm, s>>>(
         A.nbr, cap, A.rowptr.p, A.colind.p, A.v64.p, B.rowptr.p, B.colind.p, B.v64.p, C.rowptr.p, C.colind.p, C.v64.p);
     FSI_CHECK_LAUNCH();
