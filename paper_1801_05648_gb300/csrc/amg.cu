@@ -620,8 +620,7 @@ void amg_setup(Hierarchy& H, Bsr&& A0, const double* B0, int k0, const AmgParams
     A = std::move(Ac);
     Bcur = std::move(Bc);
     B = Bcur.p;
-    k = k;   // coarse block size equals the near-nullspace dimension
-    FSI_CUDA(cudaStreamSynchronize(s));
+    // (the coarse block size equals the near-nullspace dimension k)
   }
   // ---- coarsest level: dense inverse
   AmgLevel& C = H.levels.back();

@@ -34,9 +34,9 @@ enum Status { OK = 0, EINVAL_ = -1, ENOMEM_ = -2, ECUDA_ = -3, ENOTCONV_ = -4, E
     }                                                                                           \
   } while (0)
 
-// Kernel launches issued by the library (captured launches are re-counted per
+// Kernel launches issued by this thread (captured launches are re-counted per
 // graph replay by the solver).
-inline int64_t g_kernel_launches = 0;
+inline thread_local int64_t g_kernel_launches = 0;
 
 #define FSI_CHECK_LAUNCH()        \
   do {                            \
@@ -143,14 +143,35 @@ void once_per_device(std::atomic<unsigned long long>& done, F&& setup) {
 // makes about a thousand allocations, most of them temporaries of the sizes that the
 // build before had; cudaMalloc and cudaFree (which waits for the device) took a third of a
 // 256x128 rebuild.  A buffer allocated inside a SetupPhase comes from the context's pool
-// and goes back to it when it is released, without waiting: every set-up call works on
-// the context's own stream, so a block's next user is ordered behind its last one.  The pool
+// and goes back to it when it is released, without waiting: a pool's buffers are only taken for
+// work on one stream (the context's, or that of a hierarchy's branch, see precond_build), so a
+// block's next user is ordered behind its last one.  The pool
 // holds at most kKeep bytes of released blocks (the rest is freed at once), returns them
 // when the context is freed, and gives them up when any allocation of the library fails.
+// Blocks of up to kSmall bytes are cut from slabs that the context's pools share, so that a small
+// system's arrays lie in a few large pages and cost no driver call each.  Slabs live as long as
+// the context.
+class Slabs {
+ public:
+  static constexpr size_t kSmall = (size_t)1 << 20, kSlab = (size_t)32 << 20;
+  Slabs() = default;
+  Slabs(const Slabs&) = delete;
+  Slabs& operator=(const Slabs&) = delete;
+  ~Slabs() {
+    for (void* p : slabs_) cudaFree(p);
+  }
+  void* take(size_t bytes);
+
+ private:
+  std::mutex lock_;
+  std::vector<void*> slabs_;
+  size_t left_ = 0;
+};
+
 class MemPool {
  public:
-  static constexpr size_t kKeep = (size_t)2 << 30;
-  MemPool() {
+  static constexpr size_t kKeep = (size_t)1 << 30;
+  explicit MemPool(std::shared_ptr<Slabs> slabs) : slabs_(std::move(slabs)) {
     std::lock_guard<std::mutex> g(registry_lock());
     registry().insert(this);
   }
@@ -167,37 +188,40 @@ class MemPool {
   // at least `bytes` bytes; got: the block's size, to be handed back with it
   void* take(size_t bytes, size_t& got) {
     size_t step = 256;
-    while (step * 16 <= bytes) step *= 2;              // sizes rounded up by at most an eighth
+    while (step * 16 <= bytes && bytes > Slabs::kSmall) step *= 2;   // sizes rounded up by at most an eighth
     bytes = (bytes + step - 1) / step * step;
     {
       std::lock_guard<std::mutex> g(lock_);
       auto it = free_.lower_bound(bytes);
-      if (it != free_.end() && it->first <= bytes + bytes / 4 + 4096) {
+      if (it != free_.end() && it->first <= bytes + bytes / 4 + 4096 &&
+          (it->first <= Slabs::kSmall) == (bytes <= Slabs::kSmall)) {
         void* p = it->second;
         got = it->first;
-        held_ -= got;
+        if (got > Slabs::kSmall) held_ -= got;
         free_.erase(it);
         return p;
       }
     }
     got = bytes;
-    return device_malloc(bytes);
+    return bytes <= Slabs::kSmall ? slabs_->take(bytes) : device_malloc(bytes);
   }
   void give(void* p, size_t bytes) {
     {
       std::lock_guard<std::mutex> g(lock_);
-      if (held_ + bytes <= kKeep) {
+      if (bytes <= Slabs::kSmall || held_ + bytes <= kKeep) {
         free_.emplace(bytes, p);
-        held_ += bytes;
+        if (bytes > Slabs::kSmall) held_ += bytes;
         return;
       }
     }
     cudaFree(p);
   }
+  // frees the blocks held (those of the slabs stay)
   void trim() {
     std::lock_guard<std::mutex> g(lock_);
-    for (auto& b : free_) cudaFree(b.second);
-    free_.clear();
+    auto it = free_.upper_bound(Slabs::kSmall);
+    for (auto i = it; i != free_.end(); ++i) cudaFree(i->second);
+    free_.erase(it, free_.end());
     held_ = 0;
   }
   // cudaMalloc; when it fails, once more after every pool has freed what it holds
@@ -225,10 +249,23 @@ class MemPool {
     static auto* r = new std::set<MemPool*>;   // never destroyed: a context may outlive static objects
     return *r;
   }
+  std::shared_ptr<Slabs> slabs_;
   std::mutex lock_;
   std::multimap<size_t, void*> free_;
   size_t held_ = 0;
 };
+
+inline void* Slabs::take(size_t bytes) {
+  std::lock_guard<std::mutex> g(lock_);
+  if (slabs_.empty() || left_ < bytes) {
+    slabs_.reserve(slabs_.size() + 1);
+    slabs_.push_back(MemPool::device_malloc(kSlab));
+    left_ = kSlab;
+  }
+  void* p = static_cast<char*>(slabs_.back()) + (kSlab - left_);
+  left_ -= bytes;
+  return p;
+}
 
 // The pool that this thread's set-up call allocates from (null outside one).
 inline std::shared_ptr<MemPool>& current_pool() {

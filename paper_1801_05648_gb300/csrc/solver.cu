@@ -21,6 +21,8 @@
 #include <chrono>
 #include <cmath>
 #include <cstring>
+#include <exception>
+#include <thread>
 
 namespace fsi {
 
@@ -414,6 +416,8 @@ Context::~Context() {
   if (ev_fork) cudaEventDestroy(ev_fork);
   if (ev_join) cudaEventDestroy(ev_join);
   if (s2) cudaStreamDestroy(s2);
+  for (SetupBranch& b : branch)
+    if (b.done) cudaEventDestroy(b.done);
   if (pinned) cudaFreeHost(pinned);
   if (pinned_j) cudaFreeHost(pinned_j);
   if (own_stream && s) cudaStreamDestroy(s);
@@ -422,6 +426,7 @@ Context::~Context() {
 // Class blocks of the operator (Eq. mat:small): the four pieces of the outer
 // operator and the preconditioner's blocks, all extracted on the device.
 static void extract_blocks(Context& C, const CsrView& A) {
+  C.blocks_used = false;
   const int d = C.dim;
   const int64_t* o = C.off;
   const int nV = (int)(o[4] / d);
@@ -516,70 +521,153 @@ void context_update_values(Context& C, const double* vals_dev) {
   FSI_CUDA(cudaStreamSynchronize(C.s));
 }
 
+// The four streams of the hierarchies' set-ups on the current device, shared by its contexts
+// (work of several contexts on one of them only waits its turn).  Four more streams per
+// context slowed the launches of small captured solves by 6%: the device multiplexes
+// streams onto few connections.
+cudaStream_t branch_stream(int h) {
+  static std::atomic<unsigned long long> done{0};
+  static std::atomic<cudaStream_t> streams[64][4];
+  static std::mutex making;
+  std::lock_guard<std::mutex> g(making);
+  once_per_device(done, [](int dev) {
+    for (auto& st : streams[dev]) {
+      cudaStream_t x = nullptr;
+      FSI_CUDA(cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking));
+      st.store(x);
+    }
+  });
+  int dev = 0;
+  FSI_CUDA(cudaGetDevice(&dev));
+  return streams[dev][h].load();
+}
+
+// Runs build(h, stream) for the four hierarchies side by side, each in a thread of its own
+// on its branch's stream and pool, behind the work queued on C.s, and `own` on this
+// thread and C.s meanwhile; C.s then waits for the branches.  A hierarchy's set-up is
+// a chain of short launches and waits for counts on its coarse levels: one after the other, the
+// four left the GPU idle or a few SMs busy most of the time.  Every launch knob of this thread
+// applies to the branches.  An error in any of them is raised after all have ended.
+template <class Build, class Own>
+void run_branches(Context& C, Build&& build, Own&& own) {
+  for (int h = 0; h < 4; ++h) {
+    SetupBranch& b = C.branch[h];
+    b.s = branch_stream(h);
+    if (!b.done) FSI_CUDA(cudaEventCreateWithFlags(&b.done, cudaEventDisableTiming));
+    if (!b.pool) b.pool = std::make_shared<MemPool>(C.slabs);
+  }
+  FSI_CUDA(cudaEventRecord(C.ev_fork, C.s));
+  const SpmvTuning tuning = spmv_tuning();
+  const bool pdl = pdl_enabled();
+  const double coarse_bytes = coarse_max_bytes();
+  int64_t launches[4] = {0, 0, 0, 0};
+  std::exception_ptr failed[5];
+  auto work = [&](int h) {
+    try {
+      FSI_CUDA(cudaSetDevice(C.device));
+      spmv_tuning() = tuning;
+      pdl_enabled() = pdl;
+      coarse_max_bytes() = coarse_bytes;
+      SetupPhase phase(C.branch[h].pool);
+      FSI_CUDA(cudaStreamWaitEvent(C.branch[h].s, C.ev_fork, 0));
+      build(h, C.branch[h].s);
+      FSI_CUDA(cudaEventRecord(C.branch[h].done, C.branch[h].s));
+    } catch (...) {
+      failed[h] = std::current_exception();
+    }
+    launches[h] = g_kernel_launches;
+  };
+  std::thread threads[4];
+  int started = 0;
+  try {
+    for (; started < 4; ++started) threads[started] = std::thread(work, started);
+    own();
+  } catch (...) {
+    failed[4] = std::current_exception();
+    cudaStreamSynchronize(C.s);
+  }
+  for (int h = 0; h < started; ++h) {
+    threads[h].join();
+    g_kernel_launches += launches[h];
+  }
+  for (const std::exception_ptr& e : failed)
+    if (e) {
+      for (SetupBranch& b : C.branch) cudaStreamSynchronize(b.s);   // they read the caller's buffers
+      std::rethrow_exception(e);
+    }
+  for (SetupBranch& b : C.branch) FSI_CUDA(cudaStreamWaitEvent(C.s, b.done, 0));
+}
+
 void precond_build(Context& C, int precision) {
   SetupPhase setup_phase(C.pool);
   auto t0 = clk::now();
   auto& s = C.s;
   const int d = C.dim;
-  if (!C.built) {
-    // S_hat = A_vv + c A_vu  (Alg. 3)
-    Bsr Shat;
-    bsr_add(C.Avv, C.A_vu, C.prm.dt_theta, Shat, s);
-    // S_p = C_pp - B_pv diag(A_ff)^-1 B_vp
-    const int64_t nfv = C.Aff.rows();
-    DBuf<double> diag(nfv > 0 ? nfv : 1), dinv(nfv > 0 ? nfv : 1);
-    bsr_point_diagonal(C.Aff, diag.p, s);
-    invert_nonzero(nfv, diag.p, dinv.p, s);
-    Bsr Bs, BDB, Sp;
-    bsr_clone(C.B_vp, Bs, s);
-    bsr_scale_rows(Bs, dinv.p, s);
-    bsr_spgemm(C.B_pv, Bs, BDB, s);
-    bsr_add(C.Cpp, BDB, -1.0, Sp, s);
-    // hierarchies
-    DBuf<double> Bm, Bf, Bp;
-    translations(Bm, C.Mblk.nbr, d, s);
-    translations(Bf, C.Aff.nbr, d, s);
-    translations(Bp, Sp.nbr, 1, s);
+  const bool first = !C.built, demote = precision == 1 && !C.fp32_ready;
+  if (first || demote) {
+    Bsr Shat, Sp;
+    DBuf<double> B[4];   // near-nullspaces; the solid's rigid-body modes are kept by the context
     const bool rigid = C.solid_B.p != nullptr;
-    DBuf<double> Bst;
-    if (!rigid) translations(Bst, Shat.nbr, d, s);
-    const int ks = rigid ? (d == 2 ? 3 : 6) : d;
-    for (auto& H : C.H)
-      H.coarse_mode = (C.prm.flags & CLUSTER_COARSE) ? COARSE_CLUSTER
-                      : (C.prm.flags & GRID_COARSE)  ? COARSE_GRID
-                                                     : COARSE_PER_LEVEL;
-    amg_setup(C.H[0], std::move(C.Mblk), Bm.p, d, C.prm.amg, s);
-    amg_setup(C.H[1], std::move(Shat), rigid ? C.solid_B.p : Bst.p, ks, C.prm.amg, s);
-    amg_setup(C.H[2], std::move(C.Aff), Bf.p, d, C.prm.amg, s);
-    amg_setup(C.H[3], std::move(Sp), Bp.p, 1, C.prm.amg, s);
-    cheb_setup(C.mass, std::move(C.Auu), C.prm.mass_degree, C.prm.mass_ratio, C.prm.amg.cheb_upper,
-               C.prm.amg.power_iters, s);
-    {
-      const int64_t nsu = C.off[3] - C.off[2];
-      C.uv_w64.alloc(nsu > 0 ? nsu : 1);
-      if (nsu > 0) {
-        k_row_weight<<<div_up(nsu, 256), 256, 0, s>>>(C.A_uv.nbr, C.A_uv.br, C.A_uv.rowptr.p, C.prm.dt_theta,
-                                                       C.uv_w64.p);
-        FSI_CHECK_LAUNCH();
-      }
+    if (first) {
+      require(!C.blocks_used, "fsi_precond_build: an earlier build of these values failed; give new ones (fsi_update_values)");
+      C.blocks_used = true;   // the diagonal blocks move into the hierarchies
+      // S_hat = A_vv + c A_vu  (Alg. 3)
+      bsr_add(C.Avv, C.A_vu, C.prm.dt_theta, Shat, s);
+      // S_p = C_pp - B_pv diag(A_ff)^-1 B_vp
+      const int64_t nfv = C.Aff.rows();
+      DBuf<double> diag(nfv > 0 ? nfv : 1), dinv(nfv > 0 ? nfv : 1);
+      bsr_point_diagonal(C.Aff, diag.p, s);
+      invert_nonzero(nfv, diag.p, dinv.p, s);
+      Bsr Bs, BDB;
+      bsr_clone(C.B_vp, Bs, s);
+      bsr_scale_rows(Bs, dinv.p, s);
+      bsr_spgemm(C.B_pv, Bs, BDB, s);
+      bsr_add(C.Cpp, BDB, -1.0, Sp, s);
+      translations(B[0], C.Mblk.nbr, d, s);
+      if (!rigid) translations(B[1], Shat.nbr, d, s);
+      translations(B[2], C.Aff.nbr, d, s);
+      translations(B[3], Sp.nbr, 1, s);
+      for (auto& H : C.H)
+        H.coarse_mode = (C.prm.flags & CLUSTER_COARSE) ? COARSE_CLUSTER
+                        : (C.prm.flags & GRID_COARSE)  ? COARSE_GRID
+                                                       : COARSE_PER_LEVEL;
     }
-    C.Avv = Bsr();
-    C.Cpp = Bsr();
-    alloc_pw(C.pw64, C.n);
+    // hierarchies M, S_hat, A_ff, S_p
+    Bsr* A0[4] = {&C.Mblk, &Shat, &C.Aff, &Sp};
+    const int modes[4] = {d, rigid ? (d == 2 ? 3 : 6) : d, d, 1};
+    run_branches(
+        C,
+        [&](int h, cudaStream_t st) {
+          if (first) amg_setup(C.H[h], std::move(*A0[h]), h == 1 && rigid ? C.solid_B.p : B[h].p, modes[h], C.prm.amg, st);
+          if (demote) amg_make_fp32(C.H[h], st);
+        },
+        [&] {
+          const int64_t nsu = C.off[3] - C.off[2];
+          if (first) {
+            cheb_setup(C.mass, std::move(C.Auu), C.prm.mass_degree, C.prm.mass_ratio, C.prm.amg.cheb_upper,
+                       C.prm.amg.power_iters, s);
+            C.uv_w64.alloc(nsu > 0 ? nsu : 1);
+            if (nsu > 0) {
+              k_row_weight<<<div_up(nsu, 256), 256, 0, s>>>(C.A_uv.nbr, C.A_uv.br, C.A_uv.rowptr.p, C.prm.dt_theta,
+                                                             C.uv_w64.p);
+              FSI_CHECK_LAUNCH();
+            }
+            C.Avv = Bsr();
+            C.Cpp = Bsr();
+            alloc_pw(C.pw64, C.n);
+          }
+          if (demote) {
+            cheb_make_fp32(C.mass, s);
+            C.uv_w32.alloc(nsu > 0 ? nsu : 1);
+            if (nsu > 0) cast<double, float>(nsu, C.uv_w64.p, C.uv_w32.p, s);
+            for (Bsr* Q : {&C.C_ms, &C.A_vu, &C.A_uv, &C.C_sv_f, &C.C_sv_p, &C.C_fv_ms, &C.C_p_ms, &C.B_vp, &C.B_pv})
+              bsr_make_fp32(*Q, s);
+            alloc_pw(C.pw32, C.n);
+          }
+        });
+    FSI_CUDA(cudaStreamSynchronize(s));   // before the near-nullspaces go
     C.built = true;
-  }
-  if (precision == 1 && !C.fp32_ready) {
-    for (auto& H : C.H) amg_make_fp32(H, s);
-    cheb_make_fp32(C.mass, s);
-    {
-      const int64_t nsu = C.off[3] - C.off[2];
-      C.uv_w32.alloc(nsu > 0 ? nsu : 1);
-      if (nsu > 0) cast<double, float>(nsu, C.uv_w64.p, C.uv_w32.p, s);
-    }
-    for (Bsr* B : {&C.C_ms, &C.A_vu, &C.A_uv, &C.C_sv_f, &C.C_sv_p, &C.C_fv_ms, &C.C_p_ms, &C.B_vp, &C.B_pv})
-      bsr_make_fp32(*B, s);
-    alloc_pw(C.pw32, C.n);
-    C.fp32_ready = true;
+    if (demote) C.fp32_ready = true;
   }
   C.precision = precision;
   if (C.iter_graph) { cudaGraphExecDestroy(C.iter_graph); C.iter_graph = nullptr; }

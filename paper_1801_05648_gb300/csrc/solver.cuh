@@ -55,8 +55,18 @@ struct PrecWork {
   bool ready = false;
 };
 
+// Stream (the device's, not owned) and pool of one hierarchy's set-up (precond_build runs the
+// four side by side).
+struct SetupBranch {
+  cudaStream_t s = nullptr;
+  cudaEvent_t done = nullptr;
+  std::shared_ptr<MemPool> pool;
+};
+
 struct Context {
-  std::shared_ptr<MemPool> pool = std::make_shared<MemPool>();   // buffers of the set-up calls (all on stream s)
+  std::shared_ptr<Slabs> slabs = std::make_shared<Slabs>();
+  std::shared_ptr<MemPool> pool = std::make_shared<MemPool>(slabs);   // buffers of the set-up calls on stream s
+  SetupBranch branch[4];                  // made at the first preconditioner build
   cudaStream_t s = nullptr;
   bool own_stream = false;
   int device = -1;                        // CUDA device current at fsi_setup; every entry point runs on it
@@ -82,6 +92,7 @@ struct Context {
   Bsr Mblk, Avv, Auu, Aff, Cpp;   // diagonal blocks, consumed by precond_build
   Hierarchy H[4];             // M, S_hat, A_ff, S_p
   ChebSolver mass;            // A_uu (solid mass)
+  bool blocks_used = false;   // a build (perhaps a failed one) has taken the diagonal blocks
   bool built = false;
   bool fp32_ready = false;    // FP32 copies of the current hierarchies and couplings exist
   Csr pattern;                // device CSR pattern of the operator (values not kept), for fsi_update_values
