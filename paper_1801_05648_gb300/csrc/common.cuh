@@ -375,6 +375,7 @@ struct SpmvTuning {
   int keep_x64 = 1;    // FP64 launches gather x with the L2 evict-last policy (see OuterOperatorScope)
   int stage = 0;       // 2 x 2 FP32 Chebyshev steps with the column offsets staged in shared memory
   int order = 1;       // two-matrix launches take their rows in the order of Bsr::ord2 when it is built
+  int wide64 = 0;      // FP64 launches take more lanes per row on small matrices (see WideRows64)
   int setup_depth = 0; // > 0 while matrices are being built: no reads before the dependency wait
 };
 inline SpmvTuning& spmv_tuning() {
@@ -409,6 +410,18 @@ struct OuterOperatorScope {
   ~OuterOperatorScope() { spmv_tuning().keep_x64 = saved; }
   OuterOperatorScope(const OuterOperatorScope&) = delete;
   OuterOperatorScope& operator=(const OuterOperatorScope&) = delete;
+};
+
+// The FP64 preconditioner's launches spread a row over more lanes where its matrix would
+// otherwise leave the GPU a few warps per SM (widened() in spmv.cu).  That changes the order of a
+// row's sum, so only the FP64 preconditioner takes it: the outer operator and the set-up,
+// which the FP32 form shares, keep theirs.
+struct WideRows64 {
+  int saved;
+  explicit WideRows64(bool on) : saved(spmv_tuning().wide64) { spmv_tuning().wide64 = on ? 1 : 0; }
+  ~WideRows64() { spmv_tuning().wide64 = saved; }
+  WideRows64(const WideRows64&) = delete;
+  WideRows64& operator=(const WideRows64&) = delete;
 };
 
 inline void set_tpr(Bsr& A) {

@@ -58,6 +58,7 @@ extern "C" int fsi_mass_solve_noalloc(fsi_ctx* ctx, const double* in_dev, double
     if (rc != FSI_OK) { C.err = err; return rc; }
     // xb = scratch[0, n), d = scratch[max, max + n); the first Chebyshev step
     // overwrites both, so nothing needs clearing between calls.
+    fsi::WideRows64 wide(true);   // as fsi_apply_block in FP64
     fsi::cheb_apply_scratch(C.mass, in_dev, out_dev, scratch, scratch + kNoAllocMaxRows, C.s);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { C.err = cudaGetErrorString(e); return FSI_ECUDA; }

@@ -677,6 +677,7 @@ void precond_build(Context& C, int precision) {
 
 template <class T>
 void precond_apply(Context& C, const T* r, T* z) {
+  WideRows64 wide(sizeof(T) == 8);
   PrecWork<T>& W = pwork<T>(C);
   const int64_t* o = C.off;
   const T* r_m = r + o[0];
@@ -723,6 +724,7 @@ void precond_apply(Context& C, const T* r, T* z) {
 
 template <class T>
 void apply_block(Context& C, int which, const T* in, T* out) {
+  WideRows64 wide(sizeof(T) == 8);
   ensure_fluid_gmres(C);
   switch (which) {
     case 0: amg_solve<T>(C, 0, C.prm.vc_mesh, in, out, C.s); break;

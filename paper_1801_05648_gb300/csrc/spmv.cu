@@ -54,6 +54,21 @@ void launch_staged(const Bsr& A1, const G1& g1, const Epi& epi, int tpr, int row
            A1.stage_max, stage_err_ptr());
 }
 
+// FP64 launches of the preconditioner (WideRows64): lanes doubled until the launch holds
+// about 16 warps per SM or a lane has a single block of an average row.  The 8 blocks per lane of
+// the FP64 rule save shuffle additions, but leave the levels of small and mid-size systems a
+// few warps per SM walking rows of 64 blocks in dependent trips: the 21x11x10 FP64 solve went
+// from 25.3 to 16.0 ms with this and the epilogues per component.
+inline int widened(const Bsr& A, int tpr) {
+  const double mean = (double)A.nnzb / A.nbr;
+  while (tpr < 32 && (int64_t)A.nbr * tpr < (int64_t)device_sms() * 16 * 32 && mean >= 2 * tpr) tpr *= 2;
+  return tpr;
+}
+
+// Whether an epilogue comes per component (load1 / store1).
+template <class Epi>
+concept PerComponent = requires { typename Epi::Pre1; };
+
 // ALLOW16: the first matrix's 16-bit column offsets are read when present (FP32
 // Chebyshev steps on the square level matrices).
 template <class T, int BR, int BC1, int BC2, class Epi, class G1, bool ALLOW16 = false>
@@ -61,6 +76,7 @@ void launch_g(const Bsr& A1, const G1& g1, const Bsr* A2, const T* x2, const Epi
   if (A1.nbr == 0) return;
   const SpmvTuning& tu = spmv_tuning();
   int tpr = sizeof(T) == 8 ? A1.tpr64 : A1.tpr;
+  if (sizeof(T) == 8 && tu.wide64) tpr = widened(A1, tpr);
   if (sizeof(T) == 4) tpr = (tpr >> tu.lane_shift) > 0 ? (tpr >> tu.lane_shift) : 1;
   const int threads = 256;
   const int per_pass = threads / tpr;
@@ -91,23 +107,33 @@ void launch_g(const Bsr& A1, const G1& g1, const Bsr* A2, const T* x2, const Epi
       }
     }
     if (A1.cd16.p) {
+      auto go = [&](auto kernel) {
+        launch_k(kernel, blocks, threads, 0, s, A1.nbr, tpr, rows_per_cta, pf, pre_wait, ord2, A1.rowptr.p,
+                 (const int16_t*)A1.cd16.p, A1.vals<T>(), A1.nnzb, g1, rp2, ci2, v2, nnzb2, x2, epi);
+      };
       if (tu.unroll >= 8 && unroll_for<T, BR, BC1, 8>() == 8)
-        launch_k(k_bsr_spmv<T, BR, BC1, BC2, Epi, G1, 8, int16_t>, blocks, threads, 0, s, A1.nbr, tpr, rows_per_cta,
-                 pf, pre_wait, ord2, A1.rowptr.p, (const int16_t*)A1.cd16.p, A1.vals<T>(), A1.nnzb, g1, rp2, ci2, v2, nnzb2,
-                 x2, epi);
+        go(k_bsr_spmv<T, BR, BC1, BC2, Epi, G1, 8, int16_t>);
       else
-        launch_k(k_bsr_spmv<T, BR, BC1, BC2, Epi, G1, 4, int16_t>, blocks, threads, 0, s, A1.nbr, tpr, rows_per_cta,
-                 pf, pre_wait, ord2, A1.rowptr.p, (const int16_t*)A1.cd16.p, A1.vals<T>(), A1.nnzb, g1, rp2, ci2, v2, nnzb2,
-                 x2, epi);
+        go(k_bsr_spmv<T, BR, BC1, BC2, Epi, G1, 4, int16_t>);
+      return;
+    }
+  }
+  auto go = [&](auto kernel) {
+    launch_k(kernel, blocks, threads, 0, s, A1.nbr, tpr, rows_per_cta, pf, pre_wait, ord2, A1.rowptr.p, A1.colind.p,
+             A1.vals<T>(), A1.nnzb, g1, rp2, ci2, v2, nnzb2, x2, epi);
+  };
+  // a lane per component in FP64, where the epilogue's instructions count (each takes the FP64
+  // pipe for a whole warp); in FP32 it was slower (1024x512 solve 257 -> 275 ms)
+  if constexpr (sizeof(T) == 8 && BC2 == 0 && BR == BC1 && BR > 1 && PerComponent<Epi>) {
+    if (tpr >= BR) {
+      go(k_bsr_spmv<T, BR, BC1, BC2, Epi, G1, 4, int, true>);
       return;
     }
   }
   if (tu.unroll >= 8 && unroll_for<T, BR, BC1, 8>() == 8)
-    launch_k(k_bsr_spmv<T, BR, BC1, BC2, Epi, G1, 8>, blocks, threads, 0, s, A1.nbr, tpr, rows_per_cta, pf, pre_wait,
-             ord2, A1.rowptr.p, A1.colind.p, A1.vals<T>(), A1.nnzb, g1, rp2, ci2, v2, nnzb2, x2, epi);
+    go(k_bsr_spmv<T, BR, BC1, BC2, Epi, G1, 8>);
   else
-    launch_k(k_bsr_spmv<T, BR, BC1, BC2, Epi, G1, 4>, blocks, threads, 0, s, A1.nbr, tpr, rows_per_cta, pf, pre_wait,
-             ord2, A1.rowptr.p, A1.colind.p, A1.vals<T>(), A1.nnzb, g1, rp2, ci2, v2, nnzb2, x2, epi);
+    go(k_bsr_spmv<T, BR, BC1, BC2, Epi, G1, 4>);
 }
 
 template <class T, int BR, int BC1, int BC2, class Epi, bool ALLOW16 = false>

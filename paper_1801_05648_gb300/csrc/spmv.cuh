@@ -157,7 +157,8 @@ struct GatherScaled {
 
 // ------------------------------------------------------------------ epilogues
 // Each epilogue loads its row's own operands (load) before the row product is
-// accumulated, so those loads overlap the gathers, and combines them (store).
+// accumulated, so those loads overlap the gathers, and combines them (store).  load1 and
+// store1 do the same for one component of the row (launches with a lane per component).
 
 // y = alpha * (A x) + beta * y   (y not read when beta == 0)
 template <class T, int BR>
@@ -195,6 +196,9 @@ struct EpiResid {
 #pragma unroll
     for (int i = 0; i < BR; ++i) r[(size_t)row * BR + i] = p.b[i] - acc[i];
   }
+  struct Pre1 { T b; };
+  __device__ __forceinline__ Pre1 load1(size_t k) const { return {b[k]}; }
+  __device__ __forceinline__ void store1(size_t k, T acc, const Pre1& p) const { r[k] = p.b - acc; }
 };
 
 // One Chebyshev step (Saad Alg. 12.1, residual recomputed):
@@ -228,6 +232,15 @@ struct EpiCheb {
       xo[k] = p.x[i] + dn;
     }
   }
+  struct Pre1 { T b, dinv, x, d; };
+  __device__ __forceinline__ Pre1 load1(size_t k) const { return {b[k], dinv[k], x[k], c1 != T(0) ? d[k] : T(0)}; }
+  __device__ __forceinline__ void store1(size_t k, T acc, const Pre1& p) const {
+    const T r = mul_rn(p.dinv, p.b - acc);
+    T dn = mul_rn(c2, r);
+    if (c1 != T(0)) dn = fma_rn(c1, p.d, dn);
+    d[k] = dn;
+    xo[k] = p.x + dn;
+  }
 };
 
 // Second Chebyshev step from x = 0 with the first step folded in: the gathered
@@ -257,6 +270,15 @@ struct EpiChebFromZero {
       d[k] = dn;
       xo[k] = d1 + dn;
     }
+  }
+  struct Pre1 { T b, dinv; };
+  __device__ __forceinline__ Pre1 load1(size_t k) const { return {b[k], dinv[k]}; }
+  __device__ __forceinline__ void store1(size_t k, T acc, const Pre1& p) const {
+    const T d1 = mul_rn(mul_rn(p.dinv, p.b), inv_theta);
+    const T r = mul_rn(p.dinv, p.b - acc);
+    const T dn = fma_rn(c1, d1, mul_rn(c2, r));
+    d[k] = dn;
+    xo[k] = d1 + dn;
   }
 };
 
@@ -374,7 +396,12 @@ __device__ __forceinline__ void prefetch_blocks(const T* v, int64_t nnzb, int a,
 // rows when r0 is a multiple of 32, i.e. tpr <= 8), so the rows of a warp have equal
 // length and no lane idles while a longer row in its warp finishes.  A slot's record
 // replaces the four row-pointer loads; each row is summed exactly as without it.
-template <class T, int BR, int BC1, int BC2, class Epi, class G1 = GatherX<T, BC1>, int UREQ = 4, class CI1 = int>
+// COMP: the row group's first BR lanes take one component of the epilogue each (tpr >= BR)
+// instead of lane 0 all of them: a BR-th of the epilogue's instructions, and its loads and
+// stores side by side.  The butterfly leaves every lane the sums that the reduction to lane 0
+// gives (each addition has the same operands), so the results are the same bits.
+template <class T, int BR, int BC1, int BC2, class Epi, class G1 = GatherX<T, BC1>, int UREQ = 4, class CI1 = int,
+          bool COMP = false>
 __global__ void __launch_bounds__(256) k_bsr_spmv(int nbr, int tpr, int rows_per_cta, int prefetch, int pre_wait,
     const int4* __restrict__ ord2,
     const int* __restrict__ rp1, const CI1* __restrict__ ci1, const T* __restrict__ v1, int64_t nnzb1, G1 g1,
@@ -425,6 +452,23 @@ __global__ void __launch_bounds__(256) k_bsr_spmv(int nbr, int tpr, int rows_per
     T acc[BR];
 #pragma unroll
     for (int i = 0; i < BR; ++i) acc[i] = T(0);
+    if constexpr (COMP) {
+      const bool mine = valid && lane < BR;
+      const size_t k = (size_t)row * BR + lane;
+      typename Epi::Pre1 pre1;
+      if (mine) pre1 = epi.load1(k);
+      if (valid)
+        row_accumulate<T, BR, BC1, UREQ, G1, CI1>(ci1, sizeof(CI1) == 4 ? 0 : row, v1, nnzb1, g1, kb1, ke1, lane, tpr,
+                                                  acc);
+      for (int off = tpr >> 1; off > 0; off >>= 1)
+#pragma unroll
+        for (int i = 0; i < BR; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], off);
+      T sum = acc[0];
+#pragma unroll
+      for (int i = 1; i < BR; ++i) sum = lane == i ? acc[i] : sum;
+      if (mine) epi.store1(k, sum, pre1);
+      continue;
+    }
     typename Epi::Pre pre;
     if (valid && lane == 0) pre = epi.load(row);
     if (valid) {
