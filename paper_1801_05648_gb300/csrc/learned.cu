@@ -45,8 +45,11 @@ __host__ __device__ inline uint16_t f32_to_bf16(float f) {   // round to nearest
 }
 
 __device__ __forceinline__ float gelu(float x) { return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_grad(float x) {
-  return 0.5f * (1.0f + erff(x * 0.70710678118654752f)) + x * expf(-0.5f * x * x) * 0.39894228040143268f;
+// gelu(x), and its derivative in d
+__device__ __forceinline__ float gelu_both(float x, float& d) {
+  const float e = 1.0f + erff(x * 0.70710678118654752f);
+  d = 0.5f * e + x * expf(-0.5f * x * x) * 0.39894228040143268f;
+  return 0.5f * x * e;
 }
 
 __device__ __forceinline__ int cls_of(const MlpGeom& g, int64_t d) {
@@ -74,8 +77,9 @@ __device__ __forceinline__ int parity_of(int fl) {
 }
 
 // One thread per node: gather the patch, normalise, run the MLP (MODE_APPLY,
-// MODE_TRAIN) and scatter the correction; MODE_TRAIN also stores the features
-// and pre-activations column-major (row k of node a at [k * ld + a]).
+// MODE_TRAIN) and scatter the correction; MODE_TRAIN also stores the features F and, for
+// both hidden layers, the activations G = gelu(h) and derivatives D = gelu'(h),
+// column-major (row k of node a at [k * ld + a]).
 //
 // Dynamic shared memory: the weights as FP32 (params_padded<D>() floats), then
 // one column per thread (act[k * kNodeThreads + t]) holding the hidden
@@ -128,7 +132,8 @@ template <int D, int MODE>
 __global__ void __launch_bounds__(kNodeThreads) k_mlp(MlpGeom g, const uint16_t* __restrict__ w16,
                                                       const double* __restrict__ rp, double* __restrict__ c,
                                                       float* __restrict__ F, float* __restrict__ rho_out,
-                                                      float* __restrict__ H1, float* __restrict__ H2, int64_t ld) {
+                                                      float* __restrict__ G1, float* __restrict__ D1,
+                                                      float* __restrict__ G2, float* __restrict__ D2, int64_t ld) {
   using N = Net<D>;
   constexpr int kC = N::kComp, kH = N::kHidden;
   extern __shared__ __align__(16) float smem[];
@@ -277,12 +282,20 @@ __global__ void __launch_bounds__(kNodeThreads) k_mlp(MlpGeom g, const uint16_t*
       }
     }
 #pragma unroll
-    for (int j = 0; j < kH; ++j) {
-      act[j * kNodeThreads + t] = h[j];
-      if (MODE == MODE_TRAIN) H1[j * ld + a] = h[j];
-    }
+    for (int j = 0; j < kH; ++j) act[j * kNodeThreads + t] = h[j];
 #pragma unroll 1
-    for (int j = 0; j < kH; ++j) act[j * kNodeThreads + t] = gelu(act[j * kNodeThreads + t]);
+    for (int j = 0; j < kH; ++j) {
+      const float x = act[j * kNodeThreads + t];
+      if constexpr (MODE == MODE_TRAIN) {
+        float d;
+        const float v = gelu_both(x, d);
+        act[j * kNodeThreads + t] = v;
+        G1[j * ld + a] = v;
+        D1[j * ld + a] = d;
+      } else {
+        act[j * kNodeThreads + t] = gelu(x);
+      }
+    }
     // layer 2: h = W2^T gelu(h1) + b2
 #pragma unroll
     for (int j = 0; j < kH; ++j) h[j] = W[N::kB2 + j];
@@ -297,17 +310,23 @@ __global__ void __launch_bounds__(kNodeThreads) k_mlp(MlpGeom g, const uint16_t*
       }
     }
 #pragma unroll
-    for (int j = 0; j < kH; ++j) {
-      act[j * kNodeThreads + t] = h[j];
-      if (MODE == MODE_TRAIN) H2[j * ld + a] = h[j];
-    }
+    for (int j = 0; j < kH; ++j) act[j * kNodeThreads + t] = h[j];
     // layer 3: y = W3^T gelu(h2) + b3
     float y[N::kOut];
 #pragma unroll
     for (int o = 0; o < N::kOut; ++o) y[o] = W[N::kB3 + o];
 #pragma unroll 1
     for (int j = 0; j < kH; ++j) {
-      const float a2 = gelu(act[j * kNodeThreads + t]);
+      const float x2 = act[j * kNodeThreads + t];
+      float a2;
+      if constexpr (MODE == MODE_TRAIN) {
+        float d;
+        a2 = gelu_both(x2, d);
+        G2[j * ld + a] = a2;
+        D2[j * ld + a] = d;
+      } else {
+        a2 = gelu(x2);
+      }
       const float* w3 = W + N::kW3 + j * N::kOut;
 #pragma unroll
       for (int o = 0; o < N::kOut; ++o) y[o] += a2 * w3[o];
@@ -332,7 +351,7 @@ __global__ void __launch_bounds__(kNodeThreads) k_mlp(MlpGeom g, const uint16_t*
 
 template <int D, int MODE>
 void launch_mlp(const MlpGeom& g, const uint16_t* w16, const double* rp, double* c, float* F, float* rho,
-                float* H1, float* H2, int64_t ld, cudaStream_t s) {
+                float* G1, float* D1, float* G2, float* D2, int64_t ld, cudaStream_t s) {
   constexpr size_t smem = mlp_smem<D, MODE>();
   static std::atomic<unsigned long long> attr{0};   // the opt-in above 48 KB, per instantiation and device
   once_per_device(attr, [](int) {
@@ -343,19 +362,22 @@ void launch_mlp(const MlpGeom& g, const uint16_t* w16, const double* rp, double*
   constexpr int per_sm = (int)((228u * 1024u) / (smem + 1024u)) < 1 ? 1 : (int)((228u * 1024u) / (smem + 1024u));
   int64_t b = (g.n_nodes + kNodeThreads - 1) / kNodeThreads;
   if (b > (int64_t)device_sms() * per_sm) b = (int64_t)device_sms() * per_sm;
-  launch_k(k_mlp<D, MODE>, (int)(b < 1 ? 1 : b), kNodeThreads, smem, s, g, w16, rp, c, F, rho, H1, H2, ld);
+  launch_k(k_mlp<D, MODE>, (int)(b < 1 ? 1 : b), kNodeThreads, smem, s, g, w16, rp, c, F, rho, G1, D1, G2, D2, ld);
 }
 
-// Backward through the MLP for one node: dY from dL/dc, then dH2 and dH1.  Shared
-// memory holds the parameters from W2 on (W2, b2, W3, b3), the only ones read.
+// Backward through the MLP for one node: dY from dL/dc, then dH2 and dH1 (the derivatives
+// D1, D2 come from the forward pass).  Shared memory holds the parameters from W2 on (W2,
+// b2, W3, b3), the only ones read.  Four rows of W2 at a time: four independent sums per
+// thread and four derivatives in flight.  131,841 nodes: 94 us; 180 us with one row at a
+// time and erf and exp evaluated again.
 template <int D>
-__global__ void __launch_bounds__(kNodeThreads) k_mlp_bwd(MlpGeom g, const uint16_t* __restrict__ w16,
+__global__ void __launch_bounds__(kNodeThreads, 4) k_mlp_bwd(MlpGeom g, const uint16_t* __restrict__ w16,
                                                           const double* __restrict__ gc, const float* __restrict__ rho_s,
-                                                          const float* __restrict__ H1, const float* __restrict__ H2,
+                                                          const float* __restrict__ D1, const float* __restrict__ D2,
                                                           float* __restrict__ dY, float* __restrict__ dH1,
                                                           float* __restrict__ dH2, int64_t ld) {
   using N = Net<D>;
-  constexpr int kH = N::kHidden, kO = N::kOut, kTail = N::kParams - N::kW2;
+  constexpr int kH = N::kHidden, kO = N::kOut, kTail = N::kParams - N::kW2, kR = 4;
   __shared__ __align__(16) float W[(kTail + 3) / 4 * 4];
   for (int i = threadIdx.x; i < kTail; i += blockDim.x) W[i] = bf16_to_f32(w16[N::kW2 + i]);
   __syncthreads();
@@ -388,96 +410,147 @@ __global__ void __launch_bounds__(kNodeThreads) k_mlp_bwd(MlpGeom g, const uint1
     for (int o = 0; o < kO; ++o) dY[o * ld + a] = dy[o];
     float d2[kH];
 #pragma unroll
+    for (int j = 0; j < kH; ++j) d2[j] = D2[j * ld + a];
+#pragma unroll
     for (int j = 0; j < kH; ++j) {
       float s = 0.f;
 #pragma unroll
       for (int o = 0; o < kO; ++o) s += W3[j * kO + o] * dy[o];
-      d2[j] = s * gelu_grad(H2[j * ld + a]);
+      d2[j] *= s;
       dH2[j * ld + a] = d2[j];
     }
 #pragma unroll 1
-    for (int i = 0; i < kH; ++i) {
-      const float4* w4 = reinterpret_cast<const float4*>(W2 + i * kH);
-      float s = 0.f;
+    for (int i = 0; i < kH; i += kR) {
+      float d[kR], s[kR];
 #pragma unroll
-      for (int q = 0; q < kH / 4; ++q) {
-        const float4 w = w4[q];
-        s += w.x * d2[4 * q] + w.y * d2[4 * q + 1] + w.z * d2[4 * q + 2] + w.w * d2[4 * q + 3];
+      for (int r = 0; r < kR; ++r) {
+        d[r] = D1[(i + r) * ld + a];
+        s[r] = 0.f;
       }
-      dH1[i * ld + a] = s * gelu_grad(H1[i * ld + a]);
+#pragma unroll
+      for (int q = 0; q < kH / 4; ++q)
+#pragma unroll
+        for (int r = 0; r < kR; ++r) {
+          const float4 w = *reinterpret_cast<const float4*>(W2 + (i + r) * kH + 4 * q);
+          s[r] += w.x * d2[4 * q] + w.y * d2[4 * q + 1] + w.z * d2[4 * q + 2] + w.w * d2[4 * q + 3];
+        }
+#pragma unroll
+      for (int r = 0; r < kR; ++r) dH1[(i + r) * ld + a] = s[r] * d[r];
     }
   }
 }
 
 // partial[b][(P+bias) x Q] = sum over block b's nodes of [X; 1] Y^T, the ones row
-// only when bias is set (X: P <= 64 rows, optionally through gelu; Y: Q <= 64
-// rows; column-major with leading dimension ld).  A layer with more than 64
+// only when bias is set (X: P <= 64 rows; Y: Q <= 64 rows; column-major with leading
+// dimension ld, a multiple of 4).  A layer with more than 64
 // inputs is taken in chunks of 64 rows, the last one with the bias row.
-constexpr int kOuterThreads = 256, kOuterRows = 64;
-template <bool GX>
+// Tiles of 32 nodes are transposed into shared memory (the groups of four rows of node k are
+// permuted by k / 4, so that neither the stores of a tile nor the 16-byte reads of a node
+// conflict) while the next tile's loads are in flight; a thread sums an 8 x 4 piece, 32 FMAs
+// per three 16-byte reads.  131,841 nodes: 39 us on average over the layers; one 4-byte read
+// per two FMAs and gelu evaluated on loading took 132 us.
+constexpr int kOuterThreads = 128, kOuterRows = 64, kOuterTile = 32;
+__device__ __forceinline__ int outer_at(int k, int r) { return k * 64 + ((((r >> 2) ^ (k >> 2)) & 15) << 2) + (r & 3); }
 __global__ void __launch_bounds__(kOuterThreads) k_outer(int P, int bias, int Q, const float* __restrict__ X,
                                                          const float* __restrict__ Y, int64_t ld, int64_t n,
                                                          int64_t chunk, float* __restrict__ partial) {
-  __shared__ float xs[kOuterRows][33];
-  __shared__ float ys[kOuterRows][33];
+  __shared__ __align__(16) float xs[kOuterTile * 64];
+  __shared__ __align__(16) float ys[kOuterTile * 64];
   const int t = threadIdx.x, tq = t & 15, tp = t >> 4;
-  const int R = P + bias;   // rows of the partial; p = tp + 16 kk covers up to 80
-  float acc[5][4];
-#pragma unroll
-  for (int k = 0; k < 5; ++k)
-#pragma unroll
-    for (int u = 0; u < 4; ++u) acc[k][u] = 0.f;
+  const int R = P + bias;
   const int64_t lo = blockIdx.x * chunk;
   const int64_t hi = lo + chunk < n ? lo + chunk : n;
-  for (int64_t base = lo; base < hi; base += 32) {
-    const int cnt = (int)(hi - base < 32 ? hi - base : 32);
-    __syncthreads();
-    for (int e = t; e < P * 32; e += kOuterThreads) {
-      const int r = e >> 5, k = e & 31;
-      float v = k < cnt ? X[r * ld + base + k] : 0.f;
-      if (GX) v = gelu(v);
-      xs[r][k] = v;
-    }
-    for (int e = t; e < Q * 32; e += kOuterThreads) {
-      const int r = e >> 5, k = e & 31;
-      ys[r][k] = k < cnt ? Y[r * ld + base + k] : 0.f;
-    }
-    __syncthreads();
-    for (int k = 0; k < cnt; ++k) {
-      float yv[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int q = tq * 4 + u;
-        yv[u] = q < Q ? ys[q][k] : 0.f;
+  // loads: thread t takes nodes 4 (t & 7) .. + 3 of rows t / 8 + 16 i
+  const int lk = 4 * (t & 7), lr = t >> 3;
+  float4 xv[4], yv[4];
+  auto fetch = [&](int64_t base) {
+    const int cnt = (int)(hi - base < kOuterTile ? hi - base : kOuterTile);
+    auto row = [&](const float* __restrict__ M, int r, int rows) {
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (r < rows && lk < cnt) {
+        v = __ldg(reinterpret_cast<const float4*>(M + r * ld + base + lk));   // the row's tail past n is allocated
+        if (lk + 1 >= cnt) v.y = 0.f;
+        if (lk + 2 >= cnt) v.z = 0.f;
+        if (lk + 3 >= cnt) v.w = 0.f;
       }
+      return v;
+    };
 #pragma unroll
-      for (int kk = 0; kk < 5; ++kk) {
-        const int p = tp + 16 * kk;
-        const float xv = p < P ? xs[p][k] : (p < R ? 1.f : 0.f);
+    for (int i = 0; i < 4; ++i) {
+      xv[i] = row(X, lr + 16 * i, P);
+      yv[i] = row(Y, lr + 16 * i, Q);
+    }
+  };
+  float acc[8][4], ones[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int u = 0; u < 4; ++u) acc[kk][u] += xv * yv[u];
+  for (int k = 0; k < 8; ++k)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc[k][u] = 0.f;
+  if (lo < hi) fetch(lo);
+  for (int64_t base = lo; base < hi; base += kOuterTile) {
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = lr + 16 * i;
+      const float x4[4] = {xv[i].x, xv[i].y, xv[i].z, xv[i].w}, y4[4] = {yv[i].x, yv[i].y, yv[i].z, yv[i].w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        xs[outer_at(lk + e, r)] = x4[e];
+        ys[outer_at(lk + e, r)] = y4[e];
+      }
+    }
+    __syncthreads();
+    if (base + kOuterTile < hi) fetch(base + kOuterTile);
+    if (4 * tq < Q) {
+#pragma unroll 4
+      for (int k = 0; k < kOuterTile; ++k) {
+        const float4 x0 = *reinterpret_cast<const float4*>(xs + outer_at(k, 8 * tp));
+        const float4 x1 = *reinterpret_cast<const float4*>(xs + outer_at(k, 8 * tp + 4));
+        const float4 y = *reinterpret_cast<const float4*>(ys + outer_at(k, 4 * tq));
+        const float xa[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w}, ya[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) acc[i][u] += xa[i] * ya[u];
+        if (tp == 0)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) ones[u] += ya[u];
       }
     }
   }
   float* out = partial + (size_t)blockIdx.x * R * Q;
 #pragma unroll
-  for (int kk = 0; kk < 5; ++kk)
+  for (int i = 0; i < 8; ++i)
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const int p = tp + 16 * kk, q = tq * 4 + u;
-      if (p < R && q < Q) out[p * Q + q] = acc[kk][u];
+      const int p = 8 * tp + i, q = 4 * tq + u;
+      if (p < P && q < Q) out[p * Q + q] = acc[i][u];
     }
+  if (bias && tp == 0)
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (4 * tq + u < Q) out[P * Q + 4 * tq + u] = ones[u];
 }
 
-// grad[param(p, q)] += sum_b partial[b][p][q] in block order (FP64 sum); rows
-// p < P are the weights at wofs + p Q + q, row P (when bias) the biases at bofs + q
-__global__ void k_reduce_grad(const float* __restrict__ partial, int G, int P, int bias, int Q, int wofs, int bofs,
-                              float* __restrict__ grad) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+// grad[param(p, q)] += sum_b partial[b][p][q] in a fixed order (FP64 sums of every eighth
+// block, then of these); rows p < P are the weights at wofs + p Q + q, row P (when bias)
+// the biases at bofs + q.  32 entries per block, eight threads each (one thread per entry left
+// 17 blocks walking all partials: 49 us, now 14).
+constexpr int kReduceParts = 8;
+__global__ void __launch_bounds__(32 * kReduceParts) k_reduce_grad(const float* __restrict__ partial, int G, int P,
+                                                                   int bias, int Q, int wofs, int bofs,
+                                                                   float* __restrict__ grad) {
+  __shared__ double sh[kReduceParts][33];
+  const int l = threadIdx.x & 31, part = threadIdx.x >> 5;
+  const int e = blockIdx.x * 32 + l;
   const int total = (P + bias) * Q;
-  if (e >= total) return;
   double s = 0.0;
-  for (int b = 0; b < G; ++b) s += (double)partial[(size_t)b * total + e];
+  if (e < total)
+    for (int b = part; b < G; b += kReduceParts) s += (double)partial[(size_t)b * total + e];
+  sh[part][l] = s;
+  __syncthreads();
+  if (part != 0 || e >= total) return;
+  for (int k = 1; k < kReduceParts; ++k) s += sh[k][l];
   const int p = e / Q, q = e % Q;
   const int idx = p < P ? wofs + p * Q + q : bofs + q;
   grad[idx] += (float)s;
@@ -766,19 +839,19 @@ MlpGeom learned_geom(const Learned& L, const int64_t off[6]) {
 
 void mlp_apply(const MlpGeom& g, const uint16_t* w16, const double* rp, double* c, cudaStream_t s) {
   if (g.dim == 3) {
-    launch_mlp<3, MODE_APPLY>(g, w16, rp, c, nullptr, nullptr, nullptr, nullptr, 0, s);
+    launch_mlp<3, MODE_APPLY>(g, w16, rp, c, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0, s);
     return;
   }
   if (mlp_tensor_cores() && g.err) {
     mlp_apply_tc(g, w16, rp, c, g.err, s);
     return;
   }
-  launch_mlp<2, MODE_APPLY>(g, w16, rp, c, nullptr, nullptr, nullptr, nullptr, 0, s);
+  launch_mlp<2, MODE_APPLY>(g, w16, rp, c, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0, s);
 }
 
 void mlp_features(const MlpGeom& g, const double* rp, float* F, float* rho, cudaStream_t s) {
-  if (g.dim == 3) launch_mlp<3, MODE_FEATURES>(g, nullptr, rp, nullptr, F, rho, nullptr, nullptr, 0, s);
-  else launch_mlp<2, MODE_FEATURES>(g, nullptr, rp, nullptr, F, rho, nullptr, nullptr, 0, s);
+  if (g.dim == 3) launch_mlp<3, MODE_FEATURES>(g, nullptr, rp, nullptr, F, rho, nullptr, nullptr, nullptr, nullptr, 0, s);
+  else launch_mlp<2, MODE_FEATURES>(g, nullptr, rp, nullptr, F, rho, nullptr, nullptr, nullptr, nullptr, 0, s);
 }
 
 void learned_residual(int64_t n, const double* V, int64_t ldv, const int* jdev, const double* w, double* rp,
@@ -888,14 +961,12 @@ double trainer_step_d(Trainer& T, Context& C, const double* rp, bool grad) {
   const int64_t n = C.n, nn = L.n_nodes;
   cudaStream_t s = C.s;
   if (T.cap_nodes < nn) {
-    T.cap_nodes = nn;
-    T.F.alloc((size_t)N::kIn * nn);
-    T.rho.alloc((size_t)nn);
-    T.H1.alloc((size_t)N::kHidden * nn);
-    T.H2.alloc((size_t)N::kHidden * nn);
-    T.dY.alloc((size_t)N::kOut * nn);
-    T.dH1.alloc((size_t)N::kHidden * nn);
-    T.dH2.alloc((size_t)N::kHidden * nn);
+    const size_t rows = ((size_t)nn + 31) / 32 * 32;   // row length: 16-byte aligned rows
+    T.cap_nodes = (int64_t)rows;
+    T.F.alloc(N::kIn * rows);
+    T.rho.alloc(rows);
+    for (DBuf<float>* h : {&T.G1, &T.D1, &T.G2, &T.D2, &T.dH1, &T.dH2}) h->alloc(N::kHidden * rows);
+    T.dY.alloc(N::kOut * rows);
   }
   if (T.cap_n < n) {
     T.cap_n = n;
@@ -911,7 +982,7 @@ double trainer_step_d(Trainer& T, Context& C, const double* rp, bool grad) {
     g.sig_out[k] = T.prm.sig_out[k];
   }
   const int64_t ld = T.cap_nodes;
-  launch_mlp<D, MODE_TRAIN>(g, T.w16.p, rp, T.c.p, T.F.p, T.rho.p, T.H1.p, T.H2.p, ld, s);
+  launch_mlp<D, MODE_TRAIN>(g, T.w16.p, rp, T.c.p, T.F.p, T.rho.p, T.G1.p, T.D1.p, T.G2.p, T.D2.p, ld, s);
   apply_operator(C, T.c.p, T.t.p);
   k_square_partial<<<kRedBlocks, kRT, 0, s>>>(n, rp, T.part.p);
   FSI_CHECK_LAUNCH();
@@ -927,28 +998,27 @@ double trainer_step_d(Trainer& T, Context& C, const double* rp, bool grad) {
   k_scale_dev<<<grid_elem(n), 256, 0, s>>>(n, T.scal.p + 2, T.res.p);   // res = -2 (r' - A c) / ||r'||^2
   FSI_CHECK_LAUNCH();
   apply_operator_t(C, T.res.p, T.g.p);                                     // dL/dc
-  k_mlp_bwd<D><<<grid_nodes(nn), kNodeThreads, 0, s>>>(g, T.w16.p, T.g.p, T.rho.p, T.H1.p, T.H2.p, T.dY.p, T.dH1.p,
+  k_mlp_bwd<D><<<grid_nodes(nn), kNodeThreads, 0, s>>>(g, T.w16.p, T.g.p, T.rho.p, T.D1.p, T.D2.p, T.dY.p, T.dH1.p,
                                                     T.dH2.p, ld);
   FSI_CHECK_LAUNCH();
   // weight gradients: dW1 = [F;1] dH1^T, dW2 = [gelu(H1);1] dH2^T, dW3 = [gelu(H2);1] dY^T
-  const int G = (int)std::min<int64_t>(2 * device_sms(), std::max<int64_t>(1, (nn + 255) / 256));
+  const int G = (int)std::min<int64_t>(4 * device_sms(), std::max<int64_t>(1, (nn + 127) / 128));
   const int64_t chunk = ((nn + G - 1) / G + 31) / 32 * 32;
   const size_t need = (size_t)G * (kOuterRows + 1) * N::kHidden;
   if (T.partial.n < need) T.partial.alloc(need);
   // layer 1 in chunks of kOuterRows inputs, the bias row with the last chunk
-  struct Lyr { int P, Q; const float* X; const float* Y; bool gx; int wofs, bofs; };
-  const Lyr lyr[3] = {{N::kIn, N::kHidden, T.F.p, T.dH1.p, false, N::kW1, N::kB1},
-                      {N::kHidden, N::kHidden, T.H1.p, T.dH2.p, true, N::kW2, N::kB2},
-                      {N::kHidden, N::kOut, T.H2.p, T.dY.p, true, N::kW3, N::kB3}};
+  struct Lyr { int P, Q; const float* X; const float* Y; int wofs, bofs; };
+  const Lyr lyr[3] = {{N::kIn, N::kHidden, T.F.p, T.dH1.p, N::kW1, N::kB1},
+                      {N::kHidden, N::kHidden, T.G1.p, T.dH2.p, N::kW2, N::kB2},
+                      {N::kHidden, N::kOut, T.G2.p, T.dY.p, N::kW3, N::kB3}};
   for (const Lyr& l : lyr) {
     for (int p0 = 0; p0 < l.P; p0 += kOuterRows) {
       const int P = std::min(kOuterRows, l.P - p0), bias = p0 + P == l.P ? 1 : 0;
       const float* X = l.X + (int64_t)p0 * ld;
-      if (l.gx) k_outer<true><<<G, kOuterThreads, 0, s>>>(P, bias, l.Q, X, l.Y, ld, nn, chunk, T.partial.p);
-      else k_outer<false><<<G, kOuterThreads, 0, s>>>(P, bias, l.Q, X, l.Y, ld, nn, chunk, T.partial.p);
+      k_outer<<<G, kOuterThreads, 0, s>>>(P, bias, l.Q, X, l.Y, ld, nn, chunk, T.partial.p);
       FSI_CHECK_LAUNCH();
       const int total = (P + bias) * l.Q;
-      k_reduce_grad<<<div_up(total, 256), 256, 0, s>>>(T.partial.p, G, P, bias, l.Q, l.wofs + p0 * l.Q, l.bofs,
+      k_reduce_grad<<<div_up(total, 32), 32 * kReduceParts, 0, s>>>(T.partial.p, G, P, bias, l.Q, l.wofs + p0 * l.Q, l.bofs,
                                                        T.grad.p);
       FSI_CHECK_LAUNCH();
     }

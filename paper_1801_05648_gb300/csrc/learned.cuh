@@ -131,7 +131,8 @@ struct Trainer {
   int64_t cap_nodes = 0, cap_n = 0;
   DBuf<float> master, m, v, grad;  // Net<prm.dim>::kParams each
   DBuf<uint16_t> w16;
-  DBuf<float> F, rho, H1, H2, dY, dH1, dH2;   // column-major: row k of node a at [k * cap_nodes + a]
+  // column-major: row k of node a at [k * cap_nodes + a]; G, D: gelu and its derivative of the hidden layers
+  DBuf<float> F, rho, G1, D1, G2, D2, dY, dH1, dH2;
   DBuf<float> partial;
   DBuf<double> c, t, res, g, part, scal;
   int grads = 0;        // gradient contributions since the last update
