@@ -8,6 +8,9 @@ namespace fsi {
 
 namespace {
 
+// FP64 gathers take the evict-last policy from this many entries of x on (16 MB).
+constexpr int64_t kKeepCols = (int64_t)2 << 20;
+
 // L2 prefetch per CTA and matrix: at most this many bytes from the head of its slice.
 constexpr int kPrefetchCap = 32768;
 
@@ -139,7 +142,9 @@ void launch_g(const Bsr& A1, const G1& g1, const Bsr* A2, const T* x2, const Epi
 template <class T, int BR, int BC1, int BC2, class Epi, bool ALLOW16 = false>
 void launch(const Bsr& A1, const T* x1, const Bsr* A2, const T* x2, const Epi& epi, cudaStream_t s) {
   if constexpr (sizeof(T) == 8) {
-    if (spmv_tuning().keep_x64) {
+    // (a vector that L2 holds beside the matrix stream anyway needs no policy, which costs the
+    // kernel 20 to 30 registers)
+    if (spmv_tuning().keep_x64 && A1.cols() >= kKeepCols) {
       launch_g<T, BR, BC1, BC2, Epi, GatherX<T, BC1, true>, ALLOW16>(A1, GatherX<T, BC1, true>{x1}, A2, x2, epi, s);
       return;
     }
