@@ -424,8 +424,9 @@ Context::~Context() {
 }
 
 // Class blocks of the operator (Eq. mat:small): the four pieces of the outer
-// operator and the preconditioner's blocks, all extracted on the device.
-static void extract_blocks(Context& C, const CsrView& A) {
+// operator and the preconditioner's blocks, all extracted on the device.  keep: the blocks
+// hold an earlier extraction from the same pattern.
+static void extract_blocks(Context& C, const CsrView& A, bool keep) {
   C.blocks_used = false;
   const int d = C.dim;
   const int64_t* o = C.off;
@@ -435,22 +436,24 @@ static void extract_blocks(Context& C, const CsrView& A) {
   const int ns = nsv + nsu, nfv = (int)((o[4] - o[3]) / d), nms = (int)(o[3] / d);
   cudaStream_t s = C.s;
   // outer operator
-  extract_bsr(A, 0, nV, d, 0, nV, d, C.AVV, s);
-  extract_bsr(A, 0, nV, d, o[4], nP, 1, C.AVP, s);
-  extract_bsr(A, o[4], nP, 1, 0, nV, d, C.APV, s);
-  extract_bsr(A, o[4], nP, 1, o[4], nP, 1, C.APP, s);
-  bsr_make_pair_order(C.AVV, C.AVP, s);
-  bsr_make_pair_order(C.APV, C.APP, s);
+  extract_bsr(A, 0, nV, d, 0, nV, d, C.AVV, keep, s);
+  extract_bsr(A, 0, nV, d, o[4], nP, 1, C.AVP, keep, s);
+  extract_bsr(A, o[4], nP, 1, 0, nV, d, C.APV, keep, s);
+  extract_bsr(A, o[4], nP, 1, o[4], nP, 1, C.APP, keep, s);
+  if (!keep) {
+    bsr_make_pair_order(C.AVV, C.AVP, s);
+    bsr_make_pair_order(C.APV, C.APP, s);
+  }
   // preconditioner blocks
-  extract_bsr(A, o[0], nm, d, o[0], nm, d, C.Mblk, s);
-  extract_bsr(A, o[0], nm, d, o[1], ns, d, C.C_ms, s);
-  extract_bsr(A, o[1], nsv, d, o[1], nsv, d, C.Avv, s);
-  extract_bsr(A, o[1], nsv, d, o[2], nsu, d, C.A_vu, s);
-  extract_bsr(A, o[2], nsu, d, o[1], nsv, d, C.A_uv, s);
-  extract_bsr(A, o[2], nsu, d, o[2], nsu, d, C.Auu, s);
-  extract_bsr(A, o[1], ns, d, o[3], nfv, d, C.C_sv_f, s);
-  extract_bsr(A, o[1], ns, d, o[4], nP, 1, C.C_sv_p, s);
-  {
+  extract_bsr(A, o[0], nm, d, o[0], nm, d, C.Mblk, keep, s);
+  extract_bsr(A, o[0], nm, d, o[1], ns, d, C.C_ms, keep, s);
+  extract_bsr(A, o[1], nsv, d, o[1], nsv, d, C.Avv, keep, s);
+  extract_bsr(A, o[1], nsv, d, o[2], nsu, d, C.A_vu, keep, s);
+  extract_bsr(A, o[2], nsu, d, o[1], nsv, d, C.A_uv, keep, s);
+  extract_bsr(A, o[2], nsu, d, o[2], nsu, d, C.Auu, keep, s);
+  extract_bsr(A, o[1], ns, d, o[3], nfv, d, C.C_sv_f, keep, s);
+  extract_bsr(A, o[1], ns, d, o[4], nP, 1, C.C_sv_p, keep, s);
+  if (!keep) {
     // do the s_u rows of C_sf hold entries?  (The displacement equation couples
     // no fluid unknown, so normally not: then the S^-1 of step 4 of Alg. 2 sees
     // r_u = 0 and skips its mass solve, see solid_solve.)
@@ -465,12 +468,12 @@ static void extract_blocks(Context& C, const CsrView& A) {
     };
     C.csf_u_zero = tail_empty(C.C_sv_f) && tail_empty(C.C_sv_p);
   }
-  extract_bsr(A, o[3], nfv, d, o[0], nms, d, C.C_fv_ms, s);
-  extract_bsr(A, o[4], nP, 1, o[0], nms, d, C.C_p_ms, s);
-  extract_bsr(A, o[3], nfv, d, o[3], nfv, d, C.Aff, s);
-  extract_bsr(A, o[3], nfv, d, o[4], nP, 1, C.B_vp, s);
-  extract_bsr(A, o[4], nP, 1, o[3], nfv, d, C.B_pv, s);
-  extract_bsr(A, o[4], nP, 1, o[4], nP, 1, C.Cpp, s);
+  extract_bsr(A, o[3], nfv, d, o[0], nms, d, C.C_fv_ms, keep, s);
+  extract_bsr(A, o[4], nP, 1, o[0], nms, d, C.C_p_ms, keep, s);
+  extract_bsr(A, o[3], nfv, d, o[3], nfv, d, C.Aff, keep, s);
+  extract_bsr(A, o[3], nfv, d, o[4], nP, 1, C.B_vp, keep, s);
+  extract_bsr(A, o[4], nP, 1, o[3], nfv, d, C.B_pv, keep, s);
+  extract_bsr(A, o[4], nP, 1, o[4], nP, 1, C.Cpp, keep, s);
 }
 
 void context_setup(Context& C, const int64_t* rowptr, const int32_t* colind, const double* vals,
@@ -497,7 +500,7 @@ void context_setup(Context& C, const int64_t* rowptr, const int32_t* colind, con
     else   // pattern only: the values come later from the device (fsi_update_values)
       FSI_CUDA(cudaMemsetAsync(A.vals.p, 0, sizeof(double) * A.nnz, C.s));
   }
-  extract_blocks(C, A.view());
+  extract_blocks(C, A.view(), false);
   // keep the pattern (not the values) for fsi_update_values
   FSI_CUDA(cudaStreamSynchronize(C.s));
   A.vals.release();
@@ -512,7 +515,13 @@ void context_update_values(Context& C, const double* vals_dev) {
   SetupPhase setup_phase(C.pool);
   CsrView v = C.pattern.view();
   v.vals = vals_dev;
-  extract_blocks(C, v);
+  if (C.built) {   // the diagonal blocks that the hierarchies took come back with their patterns
+    C.Mblk = std::move(C.H[0].levels[0].A);
+    C.Aff = std::move(C.H[2].levels[0].A);
+    C.Auu = std::move(C.mass.A);
+    C.built = false;
+  }
+  extract_blocks(C, v, true);
   // every hierarchy, Schur operator, FP32 copy and captured graph refers to the old values
   C.built = false;
   C.fp32_ready = false;
@@ -652,8 +661,6 @@ void precond_build(Context& C, int precision) {
                                                              C.uv_w64.p);
               FSI_CHECK_LAUNCH();
             }
-            C.Avv = Bsr();
-            C.Cpp = Bsr();
             alloc_pw(C.pw64, C.n);
           }
           if (demote) {

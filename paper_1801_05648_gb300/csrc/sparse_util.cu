@@ -665,23 +665,28 @@ int64_t exclusive_scan(const int* in, int* out, int64_t n, cudaStream_t s) {
   return total;
 }
 
-void extract_bsr(const CsrView& A, int64_t r0, int nbr, int br, int64_t c0, int nbc, int bc, Bsr& out,
+void extract_bsr(const CsrView& A, int64_t r0, int nbr, int br, int64_t c0, int nbc, int bc, Bsr& out, bool keep,
                  cudaStream_t s) {
   require(br <= 6, "extract_bsr: block rows > 6");
-  out = Bsr();
-  out.nbr = nbr; out.nbc = nbc; out.br = br; out.bc = bc;
-  DBuf<int> cnt(nbr > 0 ? nbr : 1);
   const int64_t c1 = c0 + (int64_t)nbc * bc;
-  if (nbr > 0) {
-    k_extract<false><<<div_up((int64_t)nbr * 32, 128), 128, 0, s>>>(A.rowptr, A.colind, A.vals, r0, nbr, br, c0, c1, bc, cnt.p,
-                                                    nullptr, nullptr, nullptr);
-    FSI_CHECK_LAUNCH();
+  const int grid = div_up((int64_t)nbr * 32, 128);
+  keep = keep && out.rowptr.p && out.colind.p && out.v64.p && out.nbr == nbr && out.nbc == nbc && out.br == br &&
+         out.bc == bc;
+  if (!keep) {
+    out = Bsr();
+    out.nbr = nbr; out.nbc = nbc; out.br = br; out.bc = bc;
+    DBuf<int> cnt(nbr > 0 ? nbr : 1);
+    if (nbr > 0) {
+      k_extract<false><<<grid, 128, 0, s>>>(A.rowptr, A.colind, A.vals, r0, nbr, br, c0, c1, bc, cnt.p, nullptr,
+                                            nullptr, nullptr);
+      FSI_CHECK_LAUNCH();
+    }
+    finalize_rowptr(cnt.p, out, s);
+    alloc_values(out);
   }
-  finalize_rowptr(cnt.p, out, s);
-  alloc_values(out);
   if (nbr > 0) {
-    k_extract<true><<<div_up((int64_t)nbr * 32, 128), 128, 0, s>>>(A.rowptr, A.colind, A.vals, r0, nbr, br, c0, c1, bc, nullptr,
-                                                   out.rowptr.p, out.colind.p, out.v64.p);
+    k_extract<true><<<grid, 128, 0, s>>>(A.rowptr, A.colind, A.vals, r0, nbr, br, c0, c1, bc, nullptr, out.rowptr.p,
+                                         out.colind.p, out.v64.p);
     FSI_CHECK_LAUNCH();
   }
   set_tpr(out);
