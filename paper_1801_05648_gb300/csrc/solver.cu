@@ -78,10 +78,12 @@ __global__ void k_col_out(int64_t n, const T* __restrict__ in, double* __restric
     dst[i] = v;
   }
 }
-// V_{j+1} = sign * w / h  (left zero when h == 0)
+// V_{j+1} = sign * w / h  (left zero when h == 0); nothing while a second pass is due (*ready == 0)
 __global__ void k_scale_col(int64_t n, const double* __restrict__ w, const double* __restrict__ h,
-                            double* __restrict__ V, int64_t ldv, const int* __restrict__ jdev, double sign) {
+                            double* __restrict__ V, int64_t ldv, const int* __restrict__ jdev, double sign,
+                            const int* __restrict__ ready) {
   dep_wait();
+  if (*ready == 0) return;
   const double hv = *h;
   double* dst = V + (size_t)(*jdev + 1) * ldv;
   const double inv = hv > 0.0 ? sign / hv : 0.0;
@@ -89,25 +91,49 @@ __global__ void k_scale_col(int64_t n, const double* __restrict__ w, const doubl
     dst[i] = w[i] * inv;
 }
 
-// Hessenberg column j = h1 + h2 (two Gram-Schmidt passes on w), or, with defect != 0,
-// e_j - (h1 + h2) (the passes ran on the defect v_j - w), h_{j+1,j} = ||w||; apply the
-// previous rotations, form the new one, update g.  Writes |g_{j+1}|/||b|| and a
-// breakdown flag to host-mapped memory.  One thread.
-__global__ void k_givens(int ldh, const int* __restrict__ jdev, const double* __restrict__ h1,
-                         const double* __restrict__ h2, const double* __restrict__ hnorm, double* __restrict__ H,
-                         double* __restrict__ cs, double* __restrict__ sn, double* __restrict__ g,
-                         const double* __restrict__ inv_bnorm_p, double* __restrict__ out, int defect) {
+// The end of an Arnoldi step, one block.  pa: partial sums of squares of the vector d that the
+// Gram-Schmidt pass left, pb: of the vector before it.
+// First pass (second == 0): when it kept less than eta of the norm, a second pass is due:
+// flag[0] = 0, flag[1] += 1, out[5] = 1, and the rest is left to the end of that pass, which
+// the host launches.  Otherwise flag[0] = 1, out[5] = 0, hnorm = ||d||, and one thread updates the
+// least-squares problem: Hessenberg column j = e_j - h1 (- h2 after a second pass),
+// h_{j+1,j} = ||d||; the previous rotations applied, the new one formed, g updated;
+// |g_{j+1}|/||b|| and a breakdown flag to host-mapped memory.
+// (The second pass, its sums, the test and the norm as launches of their own in every step, most
+// of which had nothing to do, were 5 of a small system's 83 launches per iteration.)
+__global__ void __launch_bounds__(kRedThreads) k_arnoldi_finish(
+    const double* __restrict__ pa, const double* __restrict__ pb, int np, double eta2, int second,
+    int* __restrict__ flag, double* __restrict__ hnorm, int ldh, const int* __restrict__ jdev,
+    const double* __restrict__ h1, const double* __restrict__ h2, double* __restrict__ H, double* __restrict__ cs,
+    double* __restrict__ sn, double* __restrict__ g, const double* __restrict__ inv_bnorm_p,
+    double* __restrict__ out) {
   dep_wait();
+  __shared__ double sh[32];
+  double a = 0.0, b = 0.0;
+  for (int k = threadIdx.x; k < np; k += blockDim.x) { a += pa[k]; b += pb[k]; }
+  a = block_sum(a, sh);
+  b = block_sum(b, sh);
+  if (threadIdx.x != 0) return;
+  if (!second) {
+    const int need = (a < eta2 * b) ? 1 : 0;
+    flag[0] = 1 - need;
+    flag[1] += need;
+    out[5] = (double)need;
+    if (need) return;
+  } else {
+    flag[0] = 1;
+  }
   const double inv_bnorm = *inv_bnorm_p;
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
   const int j = *jdev;
   double* col = H + (size_t)j * ldh;
   double w0 = 0.0;
   for (int i = 0; i <= j; ++i) {
-    col[i] = defect ? (i == j ? 1.0 : 0.0) - (h1[i] + h2[i]) : h1[i] + h2[i];
+    const double h = second ? h1[i] + h2[i] : h1[i];
+    col[i] = (i == j ? 1.0 : 0.0) - h;
     w0 += col[i] * col[i];
   }
-  const double hn = *hnorm;
+  const double hn = sqrt(a);
+  *hnorm = hn;
   col[j + 1] = hn;
   w0 = sqrt(w0 + hn * hn);
   for (int i = 0; i < j; ++i) {
@@ -854,12 +880,31 @@ void ensure_krylov(Context& C) {
   if (C.iter_graph) { cudaGraphExecDestroy(C.iter_graph); C.iter_graph = nullptr; }
 }
 
-// One FGMRES iteration for the index held in C.jdev: Z_j = P^-1 V_j,
-// w = A Z_j, Gram-Schmidt against V_0..V_j, Givens update, V_{j+1} = w / ||w||.
 // Second-pass threshold of the Arnoldi Gram-Schmidt: one pass leaves the new
 // vector orthogonal to about u ||d|| / ||d'|| (u the unit roundoff), so a pass that
 // keeps at least 1% of the norm leaves it within ~1e-14.
 constexpr double kReorthEta = 1e-2;
+
+// The end of the Arnoldi step on the vector that the last Gram-Schmidt pass left in C.wfix.
+void arnoldi_end(Context& C, int second) {
+  const int m = C.prm.restart;
+  launch_k(k_arnoldi_finish, 1, kRedThreads, 0, C.s, (const double*)C.npart.p, (const double*)C.dpart.p, kRedBlocks,
+           kReorthEta * kReorthEta, second, C.reorth.p, C.scal.p, m + 1, (const int*)C.jdev.p, (const double*)C.h1.p,
+           (const double*)C.h2.p, C.Hh.p, C.cs.p, C.sn.p, C.g.p, (const double*)(C.scal.p + 5), C.pinned_dev);
+  launch_k(k_scale_col, grid_n(C.n), 256, 0, C.s, C.n, (const double*)C.wfix.p, (const double*)C.scal.p, C.V.p, C.ldv,
+           (const int*)C.jdev.p, -1.0, (const int*)C.reorth.p);
+}
+
+// The second Gram-Schmidt pass of a step that asked for it (rare).
+void second_pass(Context& C) {
+  const int m = C.prm.restart;
+  mdot(C.n, C.V.p, C.ldv, C.jdev.p, 1, C.wfix.p, C.partials.p, C.h2.p, m + 1, C.s);
+  maxpy(C.n, C.V.p, C.ldv, C.jdev.p, 1, C.h2.p, 1.0, C.wfix.p, C.npart.p, m + 1, C.s);
+  arnoldi_end(C, 1);
+}
+
+// One FGMRES iteration for the index held in C.jdev: Z_j = P^-1 V_j,
+// w = A Z_j, Gram-Schmidt against V_0..V_j, Givens update, V_{j+1} = w / ||w||.
 template <class T>
 void iteration_body(Context& C) {
   const int64_t n = C.n;
@@ -882,18 +927,12 @@ void iteration_body(Context& C) {
     learned_commit(n, L.counters.p, L.c.p, L.t.p, C.Z.p, C.ldv, C.jdev.p, C.wfix.p, C.s);
   }
   // Arnoldi step on the defect d = v_j - w (classical Gram-Schmidt, a second pass
-  // only when the first kept less than kReorthEta of ||d||): h = e_j - V^T d,
+  // only when the first kept less than kReorthEta of ||d||, see fgmres_solve): h = e_j - V^T d,
   // w - V h = -(d - V V^T d), so v_{j+1} = -d' / ||d'||.
   arnoldi_defect(n, C.V.p, C.ldv, C.jdev.p, C.wfix.p, C.dpart.p, C.s);
   mdot(n, C.V.p, C.ldv, C.jdev.p, 1, C.wfix.p, C.partials.p, C.h1.p, m + 1, C.s);
   maxpy(n, C.V.p, C.ldv, C.jdev.p, 1, C.h1.p, 1.0, C.wfix.p, C.npart.p, m + 1, C.s);
-  reorth_flag(C.npart.p, C.dpart.p, kReorthEta, C.reorth.p, C.s);
-  mdot(n, C.V.p, C.ldv, C.jdev.p, 1, C.wfix.p, C.partials.p, C.h2.p, m + 1, C.s, C.reorth.p);
-  maxpy(n, C.V.p, C.ldv, C.jdev.p, 1, C.h2.p, 1.0, C.wfix.p, C.npart.p, m + 1, C.s, C.reorth.p);
-  finish_norm(C.npart.p, C.scal.p, C.s);
-  launch_k(k_givens, 1, 32, 0, C.s, m + 1, C.jdev.p, C.h1.p, C.h2.p, C.scal.p, C.Hh.p, C.cs.p, C.sn.p, C.g.p,
-           C.scal.p + 5, C.pinned_dev, 1);
-  launch_k(k_scale_col, grid_n(n), 256, 0, C.s, n, C.wfix.p, C.scal.p, C.V.p, C.ldv, C.jdev.p, -1.0);
+  arnoldi_end(C, 0);
 }
 
 void run_iteration(Context& C) {
@@ -985,6 +1024,10 @@ int fgmres_solve(Context& C, const double* b, double* x, double tol) {
       run_iteration(C);
       FSI_CUDA(cudaStreamSynchronize(C.s));
       volatile double* pv = C.pinned;
+      if (pv[5] != 0.0) {
+        second_pass(C);
+        FSI_CUDA(cudaStreamSynchronize(C.s));
+      }
       const double est = pv[0];
       const bool bd = pv[1] != 0.0;
       nonfinite = pv[3] != 0.0;

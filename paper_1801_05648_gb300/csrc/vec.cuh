@@ -12,6 +12,20 @@ namespace fsi {
 constexpr int kRedBlocks = 608;
 constexpr int kRedThreads = 256;
 
+// Block-wide sum of one double per thread; result valid in thread 0.
+__device__ __forceinline__ double block_sum(double v, double* sh) {
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  __syncthreads();
+  if (l == 0) sh[w] = v;
+  __syncthreads();
+  v = 0.0;
+  if (threadIdx.x < (blockDim.x >> 5)) v = sh[threadIdx.x];
+  if (w == 0)
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+  return v;
+}
+
 // y = a x + b y  (y not read when b == 0)
 template <class T> void axpby(int64_t n, T a, const T* x, T b, T* y, cudaStream_t s);
 // z = a x + b y
@@ -30,25 +44,18 @@ template <class T> double dot_host(int64_t n, const T* x, const T* y, double* pa
 // Gram-Schmidt pieces.  V holds basis vectors of length n with leading dimension
 // ldv (vector i at V + i*ldv); the number of active vectors is read on the
 // device from *jcount (+ joff), so a captured graph can be replayed for every j.
-// h[i] = <V_i, w>, i < *jcount + joff.  With skip != nullptr and *skip != 0 (read on
-// the device) the products are not formed and h[i] = 0.
+// h[i] = <V_i, w>, i < *jcount + joff.
 void mdot(int64_t n, const double* V, int64_t ldv, const int* jcount, int joff, const double* w, double* partials,
-          double* h, int maxcols, cudaStream_t s, const int* skip = nullptr);
+          double* h, int maxcols, cudaStream_t s);
 // w -= sign * sum_i h[i] V_i; if nrm_partials != nullptr also writes per-block sums of w^2.
 // maxcols bounds the number of vectors (*jcount + joff) for the shared-memory copy
 // of h (0: unknown, the unvectorised kernel runs).  Both multi-products use 16-byte
-// loads when V's columns and w are 16-byte aligned (ldv even).  With *skip != 0
-// nothing is written (w and the partial sums keep their values).
+// loads when V's columns and w are 16-byte aligned (ldv even).
 void maxpy(int64_t n, const double* V, int64_t ldv, const int* jcount, int joff, const double* h, double sign,
-           double* w, double* nrm_partials, int maxcols, cudaStream_t s, const int* skip = nullptr);
+           double* w, double* nrm_partials, int maxcols, cudaStream_t s);
 // out = sqrt(sum partials)
 void finish_norm(const double* partials, double* out, cudaStream_t s);
 // Arnoldi defect: w = V_j - w (j = *jcount), partials = per-block sums of w^2.
 void arnoldi_defect(int64_t n, const double* V, int64_t ldv, const int* jcount, double* w, double* partials,
                     cudaStream_t s);
-// Second-pass test of Gram-Schmidt (kRedBlocks partial sums of squares of the vector
-// after and before one pass): flag[0] = 0 when sum(after) < eta^2 sum(before) (a second
-// pass is needed), else 1 (the skip flag of that pass); flag[1] += 1 - flag[0].
-void reorth_flag(const double* after, const double* before, double eta, int* flag, cudaStream_t s);
-
 }  // namespace fsi

@@ -176,3 +176,27 @@ def test_assembly_on_patterns_without_the_zero_couplings(cells, torch_cuda):
     rowptr = np.concatenate([[0], np.cumsum(np.bincount(rows[keep], minlength=pb.n))])
     with pytest.raises(P.FSIError):
         _assembled(torch_cuda, P, pb, U, U, rowptr, pb.colind[keep])
+
+
+@pytest.mark.parametrize("graphs", [False, True])
+def test_second_gram_schmidt_pass(graphs, torch_cuda):
+    """A system whose preconditioned operator is 2/3 I on the right-hand side's space: the Arnoldi defect
+    v - A z = v / 3 is parallel to v, the first pass cancels it to rounding, and the step asks
+    for its second pass; the first iterate is the solution (10 u for a handful of roundings)."""
+    torch = torch_cuda
+    import paper_1801_05648_gb300 as P
+    off = np.array([0, 2, 6, 10, 12, 13], np.int64)
+    rows = [[i] if not 2 <= i < 6 else [i, i + 4] for i in range(13)]      # A_vv = A_vu = I
+    rowptr = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int64)
+    colind = np.concatenate(rows).astype(np.int32)
+    S = P.FSISolver(2, rowptr, colind, np.ones(len(colind)), off, None,
+                    P.default_params(2, dt_theta=0.5, flags=P.FSI_USE_GRAPHS if graphs else 0))
+    S.precond_build("fp64")
+    b = np.zeros(13)
+    b[2:6] = np.random.default_rng(0).standard_normal(4)
+    x = torch.zeros(13, dtype=torch.float64, device="cuda")
+    for _ in range(2):
+        st = S.solve(torch.tensor(b, device="cuda"), x, 1e-10)
+        assert (st.iters, st.reorth_passes) == (1, 1)
+        assert np.abs(x.cpu().numpy() - b).max() <= 10 * np.finfo(float).eps * np.abs(b).max()
+    S.close()
