@@ -94,8 +94,8 @@ __global__ void k_scale_col(int64_t n, const double* __restrict__ w, const doubl
 // The end of an Arnoldi step, one block.  pa: partial sums of squares of the vector d that the
 // Gram-Schmidt pass left, pb: of the vector before it.
 // First pass (second == 0): when it kept less than eta of the norm, a second pass is due:
-// flag[0] = 0, flag[1] += 1, out[5] = 1, and the rest is left to the end of that pass, which
-// the host launches.  Otherwise flag[0] = 1, out[5] = 0, hnorm = ||d||, and one thread updates the
+// *ready = 0, out[5] = 1, and the rest is left to the end of that pass, which
+// the host launches.  Otherwise *ready = 1, out[5] = 0, hnorm = ||d||, and one thread updates the
 // least-squares problem: Hessenberg column j = e_j - h1 (- h2 after a second pass),
 // h_{j+1,j} = ||d||; the previous rotations applied, the new one formed, g updated;
 // |g_{j+1}|/||b|| and a breakdown flag to host-mapped memory.
@@ -103,7 +103,7 @@ __global__ void k_scale_col(int64_t n, const double* __restrict__ w, const doubl
 // of which had nothing to do, were 5 of a small system's 83 launches per iteration.)
 __global__ void __launch_bounds__(kRedThreads) k_arnoldi_finish(
     const double* __restrict__ pa, const double* __restrict__ pb, int np, double eta2, int second,
-    int* __restrict__ flag, double* __restrict__ hnorm, int ldh, const int* __restrict__ jdev,
+    int* __restrict__ ready, double* __restrict__ hnorm, int ldh, const int* __restrict__ jdev,
     const double* __restrict__ h1, const double* __restrict__ h2, double* __restrict__ H, double* __restrict__ cs,
     double* __restrict__ sn, double* __restrict__ g, const double* __restrict__ inv_bnorm_p,
     double* __restrict__ out) {
@@ -116,12 +116,11 @@ __global__ void __launch_bounds__(kRedThreads) k_arnoldi_finish(
   if (threadIdx.x != 0) return;
   if (!second) {
     const int need = (a < eta2 * b) ? 1 : 0;
-    flag[0] = 1 - need;
-    flag[1] += need;
+    *ready = 1 - need;
     out[5] = (double)need;
     if (need) return;
   } else {
-    flag[0] = 1;
+    *ready = 1;
   }
   const double inv_bnorm = *inv_bnorm_p;
   const int j = *jdev;
@@ -870,7 +869,7 @@ void ensure_krylov(Context& C) {
   C.npart.alloc(kRedBlocks);
   C.zfix.alloc(n); C.wfix.alloc(n); C.rvec.alloc(n);
   C.jdev.alloc(1); C.kdev.alloc(1);
-  C.dpart.alloc(kRedBlocks); C.reorth.alloc(2);
+  C.dpart.alloc(kRedBlocks); C.ready.alloc(1);
   if (!C.pinned) {
     FSI_CUDA(cudaHostAlloc(&C.pinned, 8 * sizeof(double), cudaHostAllocMapped));
     FSI_CUDA(cudaHostGetDevicePointer(&C.pinned_dev, C.pinned, 0));
@@ -889,10 +888,10 @@ constexpr double kReorthEta = 1e-2;
 void arnoldi_end(Context& C, int second) {
   const int m = C.prm.restart;
   launch_k(k_arnoldi_finish, 1, kRedThreads, 0, C.s, (const double*)C.npart.p, (const double*)C.dpart.p, kRedBlocks,
-           kReorthEta * kReorthEta, second, C.reorth.p, C.scal.p, m + 1, (const int*)C.jdev.p, (const double*)C.h1.p,
+           kReorthEta * kReorthEta, second, C.ready.p, C.scal.p, m + 1, (const int*)C.jdev.p, (const double*)C.h1.p,
            (const double*)C.h2.p, C.Hh.p, C.cs.p, C.sn.p, C.g.p, (const double*)(C.scal.p + 5), C.pinned_dev);
   launch_k(k_scale_col, grid_n(C.n), 256, 0, C.s, C.n, (const double*)C.wfix.p, (const double*)C.scal.p, C.V.p, C.ldv,
-           (const int*)C.jdev.p, -1.0, (const int*)C.reorth.p);
+           (const int*)C.jdev.p, -1.0, (const int*)C.ready.p);
 }
 
 // The second Gram-Schmidt pass of a step that asked for it (rare).
@@ -972,6 +971,13 @@ void run_iteration(Context& C) {
 
 }  // namespace
 
+// ||v||, through host-mapped memory (no copy)
+static double norm_host(Context& C, const double* v) {
+  dot_dev<double>(C.n, v, v, C.partials.p, C.pinned_dev + 6, C.s);
+  FSI_CUDA(cudaStreamSynchronize(C.s));
+  return std::sqrt(*(volatile double*)(C.pinned + 6));
+}
+
 int fgmres_solve(Context& C, const double* b, double* x, double tol) {
   auto t0 = clk::now();
   const int64_t launches0 = g_kernel_launches;
@@ -984,11 +990,10 @@ int fgmres_solve(Context& C, const double* b, double* x, double tol) {
   C.last_accepted = 0;
   C.last_reorth = 0;
   if (C.prm.flags & LEARNED) FSI_CUDA(cudaMemsetAsync(C.learned.counters.p, 0, 2 * sizeof(int), C.s));
-  FSI_CUDA(cudaMemsetAsync(C.reorth.p, 0, 2 * sizeof(int), C.s));
   const int64_t n = C.n;
   const int m = C.prm.restart;
   C.hist.clear();
-  const double bnorm = std::sqrt(dot_host<double>(n, b, b, C.partials.p, C.scal.p + 4, C.s));
+  const double bnorm = norm_host(C, b);
   C.last_iters = 0; C.last_cycles = 0;
   if (!std::isfinite(bnorm)) {
     C.last_status = ENONFINITE_;
@@ -1010,7 +1015,7 @@ int fgmres_solve(Context& C, const double* b, double* x, double tol) {
   bool breakdown = false, nonfinite = false;
   while (true) {
     operator_resid(C, x, b, C.rvec.p);
-    const double beta = std::sqrt(dot_host<double>(n, C.rvec.p, C.rvec.p, C.partials.p, C.scal.p + 4, C.s));
+    const double beta = norm_host(C, C.rvec.p);
     relres = beta / bnorm;
     if (!std::isfinite(relres)) { nonfinite = true; break; }
     if (relres <= tol) { status = OK; break; }
@@ -1027,6 +1032,7 @@ int fgmres_solve(Context& C, const double* b, double* x, double tol) {
       if (pv[5] != 0.0) {
         second_pass(C);
         FSI_CUDA(cudaStreamSynchronize(C.s));
+        ++C.last_reorth;
       }
       const double est = pv[0];
       const bool bd = pv[1] != 0.0;
@@ -1046,7 +1052,6 @@ int fgmres_solve(Context& C, const double* b, double* x, double tol) {
     ++C.last_cycles;
   }
   FSI_CUDA(cudaStreamSynchronize(C.s));
-  FSI_CUDA(cudaMemcpy(&C.last_reorth, C.reorth.p + 1, sizeof(int), cudaMemcpyDeviceToHost));
   if (C.learned.counters.p) {
     int cnt[3] = {0, 0, 0};
     FSI_CUDA(cudaMemcpy(cnt, C.learned.counters.p, sizeof(cnt), cudaMemcpyDeviceToHost));
@@ -1058,7 +1063,7 @@ int fgmres_solve(Context& C, const double* b, double* x, double tol) {
       throw Error(ECUDA_, "a wait of the tensor-core MLP timed out; its corrections are not valid");
     }
   }
-  if (spmv_stage_failed(C.s)) {
+  if (C.prm.spmv_stage && spmv_stage_failed(C.s)) {
     C.last_status = ECUDA_;
     C.solve_s = secs(t0, clk::now());
     throw Error(ECUDA_, "a staged Chebyshev step timed out waiting for its copies; the result is not valid");

@@ -115,9 +115,9 @@ struct Context {
   DBuf<double> V, Z, Hh, cs, sn, g, y, h1, h2, scal, partials, npart, zfix, wfix, rvec;
   DBuf<int> jdev, kdev;
   DBuf<double> dpart;         // per-block sums of squares of the Arnoldi defect
-  DBuf<int> reorth;           // [0] 0 while a second pass is due, [1] second passes in this solve
+  DBuf<int> ready;            // 0 while a second Gram-Schmidt pass of the current step is due
   double* pinned = nullptr;   // host-mapped: [0] |g_{j+1}|/|b|, [1] breakdown flag, [2] h_{j+1,j},
-                              // [3] non-finite, [4] 1/|b| on its way to the device, [5] second pass due
+                              // [3] non-finite, [4] 1/|b| on its way to the device, [5] second pass due, [6] norms
   double* pinned_dev = nullptr;
   int* pinned_j = nullptr;    // pinned host staging for the iteration index
   cudaGraphExec_t iter_graph = nullptr;

@@ -301,14 +301,6 @@ void dot_dev(int64_t n, const T* x, const T* y, double* partials, double* out, c
   launch_k(k_dot_partial<T>, kRedBlocks, kRedThreads, 0, s, n, x, y, partials);
   launch_k(k_reduce_cols, 1, kRedThreads, 0, s, partials, kRedBlocks, (const int*)nullptr, 1, out, 0);
 }
-template <class T>
-double dot_host(int64_t n, const T* x, const T* y, double* partials, double* out, cudaStream_t s) {
-  dot_dev<T>(n, x, y, partials, out, s);
-  double h = 0.0;
-  FSI_CUDA(cudaMemcpyAsync(&h, out, sizeof(double), cudaMemcpyDeviceToHost, s));
-  FSI_CUDA(cudaStreamSynchronize(s));
-  return h;
-}
 
 void mdot(int64_t n, const double* V, int64_t ldv, const int* jcount, int joff, const double* w, double* partials,
           double* h, int maxcols, cudaStream_t s) {
@@ -349,7 +341,5 @@ template void cast<double, float>(int64_t, const double*, float*, cudaStream_t);
 template void cast<float, double>(int64_t, const float*, double*, cudaStream_t);
 template void dot_dev<double>(int64_t, const double*, const double*, double*, double*, cudaStream_t);
 template void dot_dev<float>(int64_t, const float*, const float*, double*, double*, cudaStream_t);
-template double dot_host<double>(int64_t, const double*, const double*, double*, double*, cudaStream_t);
-template double dot_host<float>(int64_t, const float*, const float*, double*, double*, cudaStream_t);
 
 }  // namespace fsi

@@ -39,7 +39,6 @@ template <class Ti, class To> void cast(int64_t n, const Ti* x, To* y, cudaStrea
 // out[0] = sum_i x_i y_i (FP64 accumulation), device result; partials has kRedBlocks doubles
 template <class T> void dot_dev(int64_t n, const T* x, const T* y, double* partials, double* out, cudaStream_t s);
 // host convenience: synchronous dot
-template <class T> double dot_host(int64_t n, const T* x, const T* y, double* partials, double* out, cudaStream_t s);
 
 // Gram-Schmidt pieces.  V holds basis vectors of length n with leading dimension
 // ldv (vector i at V + i*ldv); the number of active vectors is read on the
