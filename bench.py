@@ -289,7 +289,7 @@ def kernel_traffic(profile_name: str, source_files):
         return None
 
 
-SPMV_SRCS = ["paper_1801_05648_gb300/csrc/spmv.cuh", "paper_1801_05648_gb300/csrc/spmv.cu"]
+SPMV_SRCS = ["paper_1801_05648_gb300/csrc/spmv.cuh", "paper_1801_05648_gb300/csrc/spmv_inst.cuh"]
 
 
 def dist_setup(args=None):

@@ -297,15 +297,29 @@ __global__ void k_cheb_first(int64_t n, const T* __restrict__ b, const T* __rest
   x[i] = v;
 }
 
-// x = M b, M dense row-major n x n; one warp per row
+// x = M b, M dense row-major n x n; one warp per row.  The first 8 entries of a lane are loaded
+// before the wait for the previous kernel (built: M is not being written), which leaves b's round
+// trip behind it.
 template <class T>
-__global__ void k_dense_gemv(int n, const T* __restrict__ M, const T* __restrict__ b, T* __restrict__ x) {
-  dep_wait();
+__global__ void k_dense_gemv(int n, const T* __restrict__ M, const T* __restrict__ b, T* __restrict__ x, int built) {
+  constexpr int U = 8;
+  dep_trigger();
+  if (!built) dep_wait_only();
   const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
+  T m[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int c = lane + 32 * u;
+    m[u] = row < n && c < n ? M[(int64_t)row * n + c] : T(0);
+  }
+  if (built) dep_wait_only();
   if (row >= n) return;
   T acc = 0;
-  for (int c = lane; c < n; c += 32) acc += M[(int64_t)row * n + c] * b[c];
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+    if (lane + 32 * u < n) acc += m[u] * b[lane + 32 * u];
+  for (int c = lane + 32 * U; c < n; c += 32) acc += M[(int64_t)row * n + c] * b[c];
   for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
   if (lane == 0) x[row] = acc;
 }
@@ -394,7 +408,8 @@ void vcycle_level(Hierarchy& H, int l, const T* b, T* x, cudaStream_t s) {
   if (l == last) {
     const int n = H.ncoarse;
     if (n == 0) return;
-    launch_k(k_dense_gemv<T>, div_up((int64_t)n * 32, 256), 256, 0, s, n, cinv_of<T>(H), b, x);
+    launch_k(k_dense_gemv<T>, div_up((int64_t)n * 32, 256), 256, 0, s, n, cinv_of<T>(H), b, x,
+             spmv_tuning().setup_depth == 0 ? 1 : 0);
     return;
   }
   {

@@ -45,16 +45,32 @@ inline thread_local int64_t g_kernel_launches = 0;
   } while (0)
 
 // Programmatic dependent launch (sm_90 and later).  A kernel started with
-// launch_k() may be scheduled while the previous kernel of its stream drains
-// (its blocks become resident during that kernel's tail); it executes
-// dep_wait() before its first global-memory access, which returns once the
-// previous kernel has completed and its writes are visible.  Every kernel
-// launched through launch_k() therefore starts with dep_wait().  Off for the
-// whole process when a context was set up with FSI_NO_PDL.
-__device__ __forceinline__ void dep_wait() {
+// launch_k() may be scheduled before the previous kernel of its stream has finished:
+// once every block of that kernel has called dep_trigger() or ended, its blocks become
+// resident where there is room, and dep_wait_only() returns when that kernel (and with
+// it all before it) has completed and its writes are visible.  Before that wait a
+// kernel touches only what no queued kernel writes: the launch's arguments, and, outside
+// set-up, matrices and weights, which every call that writes them leaves with a
+// stream synchronisation.  Every kernel launched through launch_k() waits, as its first
+// act (dep_wait: trigger and wait) or after such loads.  Triggering first takes the
+// launch itself out of the chain of short dependent kernels: 256x128 solve 9.5 -> 9.2 ms.
+// A kernel that precedes or is a product bound by the FP64 pipe does not trigger: blocks that
+// arrive early settle where there happens to be room, and the fullest SM's FP64 pipe then sets
+// the pace (64x32 solve 1.99 ms with such triggers, 1.92 without; training step 800 / 762 us).
+// Off for the whole process when a context was set up with FSI_NO_PDL.
+__device__ __forceinline__ void dep_trigger() {
+#if defined(__CUDA_ARCH__) && (__CUDA_ARCH__ >= 900)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+#endif
+}
+__device__ __forceinline__ void dep_wait_only() {
 #if defined(__CUDA_ARCH__) && (__CUDA_ARCH__ >= 900)
   asm volatile("griddepcontrol.wait;" ::: "memory");
 #endif
+}
+__device__ __forceinline__ void dep_wait() {
+  dep_trigger();
+  dep_wait_only();
 }
 
 // Launch knobs (programmatic dependent launch here; the SpMV shape and the coarse
@@ -372,7 +388,6 @@ struct SpmvTuning {
   int prefetch = 1;    // 0 none, 1 L2 bulk prefetch of each CTA's matrix slice, 2 also persistent CTAs
   int ctas_per_sm = 5; // persistent grid size per SM (prefetch 2)
   int lane_shift = 0;  // FP32 launches: lanes per block row divided by 2^lane_shift (at least 1)
-  int keep_x64 = 1;    // FP64 launches gather x with the L2 evict-last policy (see OuterOperatorScope)
   int stage = 0;       // 2 x 2 FP32 Chebyshev steps with the column offsets staged in shared memory
   int order = 1;       // two-matrix launches take their rows in the order of Bsr::ord2 when it is built
   int wide64 = 0;      // FP64 launches take more lanes per row on small matrices (see WideRows64)
@@ -400,20 +415,8 @@ struct SetupPhase {
   SetupPhase& operator=(const SetupPhase&) = delete;
 };
 
-// The outer FP64 operator gathers x with the default L2 policy: measured on the
-// 1024x512 system, evict-last gathers cut its DRAM traffic from 7.5 to 6.4 GB but
-// made it 5% slower (it is bound by the FP64 pipe), while the FP64 V-cycles, bound
-// by memory, ran 8% faster with them.
-struct OuterOperatorScope {
-  int saved;
-  OuterOperatorScope() : saved(spmv_tuning().keep_x64) { spmv_tuning().keep_x64 = 0; }
-  ~OuterOperatorScope() { spmv_tuning().keep_x64 = saved; }
-  OuterOperatorScope(const OuterOperatorScope&) = delete;
-  OuterOperatorScope& operator=(const OuterOperatorScope&) = delete;
-};
-
 // The FP64 preconditioner's launches spread a row over more lanes where its matrix would
-// otherwise leave the GPU a few warps per SM (widened() in spmv.cu).  That changes the order of a
+// otherwise leave the GPU a few warps per SM (widened() in spmv_inst.cuh).  That changes the order of a
 // row's sum, so only the FP64 preconditioner takes it: the outer operator and the set-up,
 // which the FP32 form shares, keep theirs.
 struct WideRows64 {

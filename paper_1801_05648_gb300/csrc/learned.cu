@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kNodeThreads) k_mlp(MlpGeom g, const uint16_t*
   const int t = threadIdx.x;
   // the weights do not depend on earlier kernels: load them before waiting for the previous one
   if (MODE != MODE_FEATURES) load_weights<D>(W, w16);
-  dep_wait();
+  dep_wait_only();   // the FP64 operator follows
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   // the block loops in lockstep so that the weights stay loaded; idle threads skip the work
   const int64_t nb = (g.n_nodes + blockDim.x - 1) / blockDim.x * blockDim.x;

@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_mlp_tc(MlpGeom g, const uint1
   const uint32_t hcol = 32u * (uint32_t)half;                         // this half's hidden columns
   const float* b2 = reinterpret_cast<const float*>(sm + kOffB2v);
   const float* b3 = reinterpret_cast<const float*>(sm + kOffB3v);
-  dep_wait();
+  dep_wait_only();   // the FP64 operator follows
   uint32_t phase = 0;
   bool failed = false;
   const int64_t ntiles = (g.n_nodes + kTcRows - 1) / kTcRows;

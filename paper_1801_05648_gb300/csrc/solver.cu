@@ -70,7 +70,7 @@ __global__ void k_col_in(int64_t n, const Ti* __restrict__ V, int64_t ldv, const
 template <class T>
 __global__ void k_col_out(int64_t n, const T* __restrict__ in, double* __restrict__ zfix, double* __restrict__ Z,
                           int64_t ldz, const int* __restrict__ jdev) {
-  dep_wait();
+  dep_wait_only();   // the FP64 operator follows
   double* dst = Z + (size_t)(*jdev) * ldz;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const double v = (double)in[i];
@@ -771,45 +771,12 @@ void apply_block(Context& C, int which, const T* in, T* out) {
   }
 }
 
-// Work on the second stream, behind C.s's queued work and next to what follows on C.s; join()
-// makes C.s wait for it.  Small systems stay on C.s: the two full dependencies (no
-// programmatic overlap across them) cost more than the overlap gives.  So do large ones, whose
-// main launch fills the GPU (1024x512 solve 255.5 ms on one stream, 256.6 on two).
-struct SideBranch {
-  static constexpr int64_t kFrom = 100000, kTo = 2000000;   // unknowns
-  Context& C;
-  const bool on;
-  explicit SideBranch(Context& c) : C(c), on(c.n >= kFrom && c.n < kTo) {
-    if (!on) return;
-    FSI_CUDA(cudaEventRecord(C.ev_fork, C.s));
-    FSI_CUDA(cudaStreamWaitEvent(C.s2, C.ev_fork, 0));
-  }
-  cudaStream_t stream() const { return on ? C.s2 : C.s; }
-  void join() {
-    if (!on) return;
-    FSI_CUDA(cudaEventRecord(C.ev_join, C.s2));
-    FSI_CUDA(cudaStreamWaitEvent(C.s, C.ev_join, 0));
-  }
-};
-
-// The pressure rows (latency bound: 14.6 us of the 256x128 operator's 96) run next to the vector
-// rows: 256x128 solve 10.37 -> 10.23 ms.
 void apply_operator(Context& C, const double* x, double* y) {
-  OuterOperatorScope outer;
-  const int64_t nv = C.off[4];
-  SideBranch side(C);
-  spmv2_axpby<double>(C.APV, x, &C.APP, x + nv, 1.0, 0.0, y + nv, side.stream());
-  spmv2_axpby<double>(C.AVV, x, &C.AVP, x + nv, 1.0, 0.0, y, C.s);
-  side.join();
+  spmv_operator(C.AVV, C.AVP, C.APV, C.APP, x, nullptr, y, C.s);
 }
 
 static void operator_resid(Context& C, const double* x, const double* b, double* r) {
-  OuterOperatorScope outer;
-  const int64_t nv = C.off[4];
-  SideBranch side(C);
-  spmv2_resid<double>(C.APV, x, &C.APP, x + nv, b + nv, r + nv, side.stream());
-  spmv2_resid<double>(C.AVV, x, &C.AVP, x + nv, b, r, C.s);
-  side.join();
+  spmv_operator(C.AVV, C.AVP, C.APV, C.APP, x, b, r, C.s);
 }
 
 double operator_bytes(const Context& C) {

@@ -76,7 +76,8 @@ __device__ __forceinline__ void load_gather(const T* __restrict__ p, T* out) {
 
 // FP64 gathers with the L2 evict-last policy: the gathered vector (71 MB in FP64 on
 // the 1024x512 system) then outlives the evict-first matrix stream in L2.  FP64
-// launches use them unless the caller turns them off (OuterOperatorScope).
+// launches of the preconditioner and the set-up use them on large vectors (kKeepCols): the
+// 1024x512 V-cycles ran 8% faster with them.
 __device__ __forceinline__ uint64_t l2_evict_last_policy() {
   uint64_t pol;
   asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
@@ -311,19 +312,20 @@ __host__ __device__ constexpr int unroll_for() {
          : (int)(sizeof(T) * (BR * BC + BC)) <= 24 ? UREQ : ((int)(sizeof(T) * (BR * BC + BC)) <= 64 ? 4 : 2);
 }
 
-// acc += sum over the lane's share of row entries [kb, ke) of block * x[col].
+// One trip of a lane over its share of a row, and acc += sum over that share of row entries [kb, ke) of block * x[col].
 // The U column indices and the U blocks are requested together (which entries
 // exist follows from the position alone), then the x segments, which need the
 // indices: one dependent memory round trip for the matrix data, one for x.
 // Column indices are int32 block columns (base 0), or int16 offsets from the
 // block row (base = the row) for square matrices whose offsets fit.
-template <class T, int BR, int BC, int UREQ, class G, class CI = int>
-__device__ __forceinline__ void row_accumulate(const CI* __restrict__ ci, int base, const T* __restrict__ v,
-                                               int64_t nnzb, const G& gx, int kb, int ke, int lane, int tpr, T* acc) {
-  constexpr int U = unroll_for<T, BR, BC, UREQ>();
-  for (int k0 = kb + lane; k0 < ke; k0 += tpr * U) {
-    int col[U];
-    T blk[U][BR * BC], xv[U][BC];
+template <class T, int BR, int BC, int UREQ, class CI = int>
+struct Trip {
+  static constexpr int U = unroll_for<T, BR, BC, UREQ>();
+  int col[U];
+  T blk[U][BR * BC];
+
+  __device__ __forceinline__ void load(const CI* __restrict__ ci, int base, const T* __restrict__ v, int64_t nnzb,
+                                       int k0, int ke, int tpr) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int k = k0 + u * tpr;
@@ -336,6 +338,10 @@ __device__ __forceinline__ void row_accumulate(const CI* __restrict__ ci, int ba
         for (int t = 0; t < BR * BC; ++t) blk[u][t] = T(0);
       }
     }
+  }
+  template <class G>
+  __device__ __forceinline__ void apply(const G& gx, int k0, int ke, int tpr, T* acc) const {
+    T xv[U][BC];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       if (k0 + u * tpr < ke) {
@@ -351,6 +357,28 @@ __device__ __forceinline__ void row_accumulate(const CI* __restrict__ ci, int ba
       for (int i = 0; i < BR; ++i)
 #pragma unroll
         for (int j = 0; j < BC; ++j) acc[i] = fma_rn(blk[u][i * BC + j], xv[u][j], acc[i]);
+  }
+};
+
+template <class T, int BR, int BC, int UREQ, class G, class CI = int>
+__device__ __forceinline__ void row_accumulate(const CI* __restrict__ ci, int base, const T* __restrict__ v,
+                                               int64_t nnzb, const G& gx, int kb, int ke, int lane, int tpr, T* acc) {
+  Trip<T, BR, BC, UREQ, CI> trip;
+  for (int k0 = kb + lane; k0 < ke; k0 += tpr * trip.U) {
+    trip.load(ci, base, v, nnzb, k0, ke, tpr);
+    trip.apply(gx, k0, ke, tpr, acc);
+  }
+}
+
+// The same with the trip at kb + lane already loaded.
+template <class T, int BR, int BC, int UREQ, class G, class CI>
+__device__ __forceinline__ void row_accumulate_loaded(Trip<T, BR, BC, UREQ, CI>& trip, const CI* __restrict__ ci,
+                                                      int base, const T* __restrict__ v, int64_t nnzb, const G& gx,
+                                                      int kb, int ke, int lane, int tpr, T* acc) {
+  for (int k0 = kb + lane; k0 < ke;) {
+    trip.apply(gx, k0, ke, tpr, acc);
+    k0 += tpr * trip.U;
+    if (k0 < ke) trip.load(ci, base, v, nnzb, k0, ke, tpr);
   }
 }
 
@@ -381,7 +409,11 @@ __device__ __forceinline__ void prefetch_blocks(const T* v, int64_t nnzb, int a,
   }
 }
 
-// One CTA handles the contiguous block rows [blockIdx.x * rows_per_cta, + rows_per_cta),
+// Bits of a launch's dep argument: the matrices are built (they may be read before the wait for
+// the previous kernel); the next kernel may be scheduled from this one's start.
+enum { kDepBuilt = 1, kDepTrigger = 2 };
+
+// CTA cta handles the contiguous block rows [cta * rows_per_cta, + rows_per_cta),
 // blockDim.x / tpr rows per pass, tpr lanes per row.  With prefetch (> 0, a byte cap),
 // thread 0 first asks L2 for the head of the CTA's slice of the (constant) matrix
 // arrays, at most `prefetch` bytes of each matrix, before waiting for the previous
@@ -390,42 +422,52 @@ __device__ __forceinline__ void prefetch_blocks(const T* v, int64_t nnzb, int a,
 // flight for all resident CTAs well inside L2: a whole 80 KB FP64 slice per CTA
 // (about 60 MB for the resident CTAs) was evicted before use and read twice.  Reading the
 // row pointers before the wait is only allowed once the matrices are built
-// (pre_wait != 0); during set-up the previous kernel may still be writing them.
+// (kDepBuilt); during set-up the previous kernel may still be writing them.
 // Two-matrix launches may take a slot table (ord2, Bsr::ord2): the CTA's slots
 // [r0, r1) are then its block rows sorted by length within 32-row windows (the same
 // rows when r0 is a multiple of 32, i.e. tpr <= 8), so the rows of a warp have equal
 // length and no lane idles while a longer row in its warp finishes.  A slot's record
 // replaces the four row-pointer loads; each row is summed exactly as without it.
+// EARLY (built matrices only): the row pointers and every lane's first trip of columns and
+// blocks are loaded before the wait for the previous kernel, which leaves the gathers, the
+// epilogue's operands and the sums behind it: two of the three dependent memory round trips of a
+// small launch.  It costs up to 12 registers (2 x 2 FP32) that large launches need for
+// occupancy, see launch_g.
 // COMP: the row group's first BR lanes take one component of the epilogue each (tpr >= BR)
 // instead of lane 0 all of them: a BR-th of the epilogue's instructions, and its loads and
 // stores side by side.  The butterfly leaves every lane the sums that the reduction to lane 0
 // gives (each addition has the same operands), so the results are the same bits.
-template <class T, int BR, int BC1, int BC2, class Epi, class G1 = GatherX<T, BC1>, int UREQ = 4, class CI1 = int,
-          bool COMP = false>
-__global__ void __launch_bounds__(256) k_bsr_spmv(int nbr, int tpr, int rows_per_cta, int prefetch, int pre_wait,
+template <class T, int BR, int BC1, int BC2, class Epi, class G1, int UREQ, class CI1, bool COMP, bool EARLY>
+__device__ __forceinline__ void bsr_rows(int cta, int nbr, int tpr, int rows_per_cta, int prefetch, int dep,
     const int4* __restrict__ ord2,
-    const int* __restrict__ rp1, const CI1* __restrict__ ci1, const T* __restrict__ v1, int64_t nnzb1, G1 g1,
+    const int* __restrict__ rp1, const CI1* __restrict__ ci1, const T* __restrict__ v1, int64_t nnzb1, const G1& g1,
     const int* __restrict__ rp2, const int* __restrict__ ci2, const T* __restrict__ v2, int64_t nnzb2,
     const T* __restrict__ x2,
-    Epi epi) {
-  const int r0 = blockIdx.x * rows_per_cta;
+    const Epi& epi) {
+  const int r0 = cta * rows_per_cta;
   const int r1 = r0 + rows_per_cta < nbr ? r0 + rows_per_cta : nbr;
-  if (!pre_wait) dep_wait();
-  if (prefetch && threadIdx.x == 0 && r0 < r1) {
-    const int a = rp1[r0];
-    const int cap1 = prefetch / (int)(BR * BC1 * sizeof(T) + sizeof(CI1));
-    const int b = rp1[r1] - a < cap1 ? rp1[r1] : a + cap1;
-    prefetch_blocks<T, BR, BC1>(v1, nnzb1, a, b);
-    prefetch_l2(ci1 + a, sizeof(CI1) * (size_t)(b - a));
-    if constexpr (BC2 > 0) {
-      const int a2 = rp2[r0];
-      const int cap2 = prefetch / (int)(BR * BC2 * sizeof(T) + sizeof(int));
-      const int b2 = rp2[r1] - a2 < cap2 ? rp2[r1] : a2 + cap2;
-      prefetch_blocks<T, BR, BC2>(v2, nnzb2, a2, b2);
-      prefetch_l2(ci2 + a2, sizeof(int) * (size_t)(b2 - a2));
+  if (dep & kDepTrigger) dep_trigger();
+  if (!(dep & kDepBuilt)) dep_wait_only();
+  auto prefetch_slice = [&] {
+    if (prefetch && threadIdx.x == 0 && r0 < r1) {
+      const int a = rp1[r0];
+      const int cap1 = prefetch / (int)(BR * BC1 * sizeof(T) + sizeof(CI1));
+      const int b = rp1[r1] - a < cap1 ? rp1[r1] : a + cap1;
+      prefetch_blocks<T, BR, BC1>(v1, nnzb1, a, b);
+      prefetch_l2(ci1 + a, sizeof(CI1) * (size_t)(b - a));
+      if constexpr (BC2 > 0) {
+        const int a2 = rp2[r0];
+        const int cap2 = prefetch / (int)(BR * BC2 * sizeof(T) + sizeof(int));
+        const int b2 = rp2[r1] - a2 < cap2 ? rp2[r1] : a2 + cap2;
+        prefetch_blocks<T, BR, BC2>(v2, nnzb2, a2, b2);
+        prefetch_l2(ci2 + a2, sizeof(int) * (size_t)(b2 - a2));
+      }
     }
+  };
+  if constexpr (!EARLY) {
+    prefetch_slice();
+    if (dep & kDepBuilt) dep_wait_only();
   }
-  if (pre_wait) dep_wait();
   const int per_pass = blockDim.x / tpr;
   const int lane = threadIdx.x & (tpr - 1);
   for (int base = r0; base < r1; base += per_pass) {
@@ -449,17 +491,30 @@ __global__ void __launch_bounds__(256) k_bsr_spmv(int nbr, int tpr, int rows_per
         }
       }
     }
+    const int base1 = sizeof(CI1) == 4 ? 0 : row;
+    Trip<T, BR, BC1, UREQ, CI1> trip;
+    if constexpr (EARLY) {
+      trip.load(ci1, base1, v1, nnzb1, kb1 + lane, ke1, tpr);
+      if (base == r0 && (dep & kDepBuilt)) {
+        prefetch_slice();
+        dep_wait_only();
+      }
+    }
     T acc[BR];
 #pragma unroll
     for (int i = 0; i < BR; ++i) acc[i] = T(0);
+    auto product = [&] {
+      if constexpr (EARLY)
+        row_accumulate_loaded(trip, ci1, base1, v1, nnzb1, g1, kb1, ke1, lane, tpr, acc);
+      else
+        row_accumulate<T, BR, BC1, UREQ, G1, CI1>(ci1, base1, v1, nnzb1, g1, kb1, ke1, lane, tpr, acc);
+    };
     if constexpr (COMP) {
       const bool mine = valid && lane < BR;
       const size_t k = (size_t)row * BR + lane;
       typename Epi::Pre1 pre1;
       if (mine) pre1 = epi.load1(k);
-      if (valid)
-        row_accumulate<T, BR, BC1, UREQ, G1, CI1>(ci1, sizeof(CI1) == 4 ? 0 : row, v1, nnzb1, g1, kb1, ke1, lane, tpr,
-                                                  acc);
+      if (valid) product();
       for (int off = tpr >> 1; off > 0; off >>= 1)
 #pragma unroll
         for (int i = 0; i < BR; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], off);
@@ -472,8 +527,7 @@ __global__ void __launch_bounds__(256) k_bsr_spmv(int nbr, int tpr, int rows_per
     typename Epi::Pre pre;
     if (valid && lane == 0) pre = epi.load(row);
     if (valid) {
-      row_accumulate<T, BR, BC1, UREQ, G1, CI1>(ci1, sizeof(CI1) == 4 ? 0 : row, v1, nnzb1, g1, kb1, ke1, lane, tpr,
-                                                acc);
+      product();
       if constexpr (BC2 > 0)
         row_accumulate<T, BR, BC2, UREQ>(ci2, 0, v2, nnzb2, GatherX<T, BC2, G1::kKeep>{x2}, kb2, ke2, lane, tpr,
                                          acc);
@@ -483,6 +537,48 @@ __global__ void __launch_bounds__(256) k_bsr_spmv(int nbr, int tpr, int rows_per
       for (int i = 0; i < BR; ++i) acc[i] += __shfl_down_sync(0xffffffffu, acc[i], off, tpr);
     if (valid && lane == 0) epi.store(row, acc, pre);
   }
+}
+
+template <class T, int BR, int BC1, int BC2, class Epi, class G1 = GatherX<T, BC1>, int UREQ = 4, class CI1 = int,
+          bool COMP = false, bool EARLY = false>
+__global__ void __launch_bounds__(256) k_bsr_spmv(int nbr, int tpr, int rows_per_cta, int prefetch, int dep,
+    const int4* __restrict__ ord2,
+    const int* __restrict__ rp1, const CI1* __restrict__ ci1, const T* __restrict__ v1, int64_t nnzb1, G1 g1,
+    const int* __restrict__ rp2, const int* __restrict__ ci2, const T* __restrict__ v2, int64_t nnzb2,
+    const T* __restrict__ x2,
+    Epi epi) {
+  bsr_rows<T, BR, BC1, BC2, Epi, G1, UREQ, CI1, COMP, EARLY>(blockIdx.x, nbr, tpr, rows_per_cta, prefetch, dep, ord2,
+                                                            rp1, ci1, v1, nnzb1, g1, rp2, ci2, v2, nnzb2, x2, epi);
+}
+
+// The outer operator's rows: D velocity components of a node (D x D blocks, and D x 1 to the
+// pressures) and pressures (1 x D and 1 x 1), in one launch.  The first ctas_p CTAs take the
+// pressure rows: few, long ones, which as a launch of their own wait on latency (10 us of the
+// 16x16 operator's 22, 14.6 of the 256x128 operator's 96) and here run beside the rest.  x is gathered with the default L2 policy: on the 1024x512 system
+// evict-last gathers cut the DRAM traffic from 7.5 to 6.4 GB but made the product 5% slower (it is
+// bound by the FP64 pipe).
+struct RowClass {
+  int nbr, tpr, rows_per_cta;
+  const int4* ord2;
+  const int *rp1, *ci1; const double* v1; int64_t nnzb1;
+  const int *rp2, *ci2; const double* v2; int64_t nnzb2;
+};
+
+template <int D, template <class, int> class Epi, bool EARLY>
+__global__ void __launch_bounds__(256) k_operator_rows(const __grid_constant__ RowClass V,
+                                                       const __grid_constant__ RowClass P, int ctas_p, int prefetch,
+                                                       int dep, const double* __restrict__ xv,
+                                                       const double* __restrict__ xp, Epi<double, D> epi_v,
+                                                       Epi<double, 1> epi_p) {
+  const GatherX<double, D> g{xv};
+  if ((int)blockIdx.x < ctas_p)
+    bsr_rows<double, 1, D, 1, Epi<double, 1>, GatherX<double, D>, 4, int, false, EARLY>(
+        blockIdx.x, P.nbr, P.tpr, P.rows_per_cta, prefetch, dep, P.ord2, P.rp1, P.ci1, P.v1, P.nnzb1, g, P.rp2, P.ci2,
+        P.v2, P.nnzb2, xp, epi_p);
+  else
+    bsr_rows<double, D, D, 1, Epi<double, D>, GatherX<double, D>, 4, int, false, EARLY>(
+        blockIdx.x - ctas_p, V.nbr, V.tpr, V.rows_per_cta, prefetch, dep, V.ord2, V.rp1, V.ci1, V.v1, V.nnzb1, g, V.rp2,
+        V.ci2, V.v2, V.nnzb2, xp, epi_v);
 }
 
 // ------------------------------------------------------------------ staged 2 x 2 FP32 steps
@@ -547,7 +643,7 @@ __device__ __forceinline__ void stage_issue(int c, int nchunks, int R, int nbr, 
 }
 
 template <class Epi, class G1, int UREQ>
-__global__ void __launch_bounds__(256) k_bsr_cheb_staged(int nbr, int tpr, int R, int nchunks, int pre_wait,
+__global__ void __launch_bounds__(256) k_bsr_cheb_staged(int nbr, int tpr, int R, int nchunks, int dep,
                                                          const int* __restrict__ rp, const int16_t* __restrict__ ci,
                                                          const float* __restrict__ v, G1 g1, Epi epi, int smax,
                                                          int* __restrict__ err) {
@@ -564,12 +660,13 @@ __global__ void __launch_bounds__(256) k_bsr_cheb_staged(int nbr, int tpr, int R
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   __syncthreads();
-  if (!pre_wait) dep_wait();
+  if (dep & kDepTrigger) dep_trigger();
+  if (!(dep & kDepBuilt)) dep_wait_only();
   if (threadIdx.x == 0)
     for (int st = 0; st < kStageDepth; ++st)
       stage_issue(blockIdx.x + st * gridDim.x, nchunks, R, nbr, st, sbase, smax, rp, ci, v, s_a8);
   __syncthreads();
-  if (pre_wait) dep_wait();
+  if (dep & kDepBuilt) dep_wait_only();
   const int lane = threadIdx.x & (tpr - 1);
   for (int i = 0;; ++i) {
     const int c = blockIdx.x + i * gridDim.x;
@@ -635,6 +732,10 @@ __global__ void __launch_bounds__(256) k_bsr_cheb_staged(int nbr, int tpr, int R
 template <class T> void spmv_axpby(const Bsr& A, const T* x, T alpha, T beta, T* y, cudaStream_t s);
 // y = alpha * (A1 x1 + A2 x2) + beta * y   (A2 may have 0 block rows == none)
 template <class T> void spmv2_axpby(const Bsr& A1, const T* x1, const Bsr* A2, const T* x2, T alpha, T beta, T* y, cudaStream_t s);
+// The outer operator: y = A x (b == nullptr) or b - A x with A = [AVV AVP; APV APP] and x = [velocity
+// rows; pressures], in one launch.
+void spmv_operator(const Bsr& AVV, const Bsr& AVP, const Bsr& APV, const Bsr& APP, const double* x, const double* b,
+                   double* y, cudaStream_t s);
 // r = b - A1 x1 - A2 x2
 template <class T> void spmv2_resid(const Bsr& A1, const T* x1, const Bsr* A2, const T* x2, const T* b, T* r, cudaStream_t s);
 // Coarse right-hand side of a V-cycle level in one pass: y = RAn x + R b with

@@ -1,7 +1,8 @@
 """Set-up kernels at the sizes where they can go wrong: the panelled dense inverse of the
 coarsest level around its panel, tile and cluster sizes (with pivoting), preconditioner
 rebuilds that reuse a context's memory, builds in several threads, and the device
-assembly on meshes smaller than its cell groups and on patterns that lack entries."""
+assembly on meshes smaller than its cell groups and on patterns that lack entries; and the
+solver's launches that overlap or are left out (queued products, the second Gram-Schmidt pass)."""
 import threading
 
 import numpy as np
@@ -200,3 +201,40 @@ def test_second_gram_schmidt_pass(graphs, torch_cuda):
         assert (st.iters, st.reorth_passes) == (1, 1)
         assert np.abs(x.cpu().numpy() - b).max() <= 10 * np.finfo(float).eps * np.abs(b).max()
     S.close()
+
+
+@pytest.mark.parametrize("cells,precision", [((3, 3), "fp32"), ((16, 16), "fp64"), ((16, 16), "fp32"), ((37, 19), "fp32"),
+                                             ((64, 48), "fp32"), ((4, 4, 4), "fp32"), ((7, 5, 6), "fp64")])
+def test_queued_products_read_finished_inputs(cells, precision, torch_cuda):
+    """Products queued one behind the other, each reading the last one's result, with launches that load
+    their matrix before the previous kernel has finished (small levels, and operators on both sides of the
+    size where that ends): the bits of the same products with a wait after each, and of a context without overlapped
+    launches; and the operator within its rounding, (row length + 2) u |A| |x|, of the host's product."""
+    torch = torch_cuda
+    import paper_1801_05648_gb300 as P
+    from scipy.sparse import csr_matrix
+    base = fsigen.CONFIGS["2d_tiny" if len(cells) == 2 else "3d"]
+    pb = fsigen.get_problem(base.with_(name="q", n=cells))
+    U = pb.seeded_state(0, 5e-3)
+    vals = pb.jacobian(U, U)
+    x0 = torch.tensor(np.random.default_rng(3).standard_normal(pb.n), device="cuda")
+
+    def chain(flags, sync):
+        S = P.FSISolver(pb.dim, pb.rowptr, pb.colind, vals, pb.offsets, pb.solid_node_coords(),
+                        P.default_params(pb.dim, flags=flags))
+        S.precond_build(precision)
+        v = [x0] + [torch.empty_like(x0) for _ in range(12)]
+        torch.cuda.synchronize()
+        for k in range(0, 12, 2):
+            S.apply_operator(v[k], v[k + 1], sync=sync)
+            S.apply_block("precond", v[k + 1], v[k + 2], sync=sync)
+        torch.cuda.synchronize()
+        S.close()
+        return v[1:]
+    want = chain(P.FSI_NO_PDL, True)
+    for sync in (True, False, False):
+        assert all(torch.equal(a, b) for a, b in zip(chain(0, sync), want))
+    A = csr_matrix((vals, pb.colind, pb.rowptr))
+    x = x0.cpu().numpy()
+    bound = (np.diff(pb.rowptr) + 2) * np.finfo(float).eps * (abs(A) @ np.abs(x))
+    assert (np.abs(want[0].cpu().numpy() - A @ x) <= bound).all()
