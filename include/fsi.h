@@ -332,7 +332,7 @@ int fsi_update_values(fsi_ctx* ctx, const double* vals_dev);
  * outflow and solid stress terms and of the kinematic velocity, and the fluid
  * time derivative carries theta J + (1 - theta) J_old.  3^dim Gauss points per
  * cell, 3^(dim-1) on the outflow face.  The Jacobian is the exact derivative of
- * this discrete residual (dual numbers).  Fixed rows: residual 0, Jacobian row =
+ * this discrete residual (closed form).  Fixed rows: residual 0, Jacobian row =
  * the identity entry.
  */
 typedef struct fsi_asm fsi_asm;

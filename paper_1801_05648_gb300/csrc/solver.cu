@@ -12,8 +12,8 @@
 //   y = A_ff^-1 r_v;  x_p = S_p^-1 (r_p - B_pv y);  x_v = A_ff^-1 (r_v - B_vp x_p).
 // Inverses: smoothed-aggregation V-cycles (M, S_hat, A_ff, S_p) and a Chebyshev
 // polynomial for the solid mass matrix A_uu.  The outer iteration is
-// right-preconditioned FGMRES (Saad Alg. 9.6) with classical Gram-Schmidt applied
-// twice and Givens rotations kept on the device.
+// right-preconditioned FGMRES (Saad Alg. 9.6) with classical Gram-Schmidt on the Arnoldi
+// defect (a second pass when needed) and Givens rotations kept on the device.
 #include "solver.cuh"
 #include "spmv.cuh"
 #include "vec.cuh"
