@@ -379,7 +379,9 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_spgemm_sym(int nbr, int
       }
       stop = __shfl_sync(0xffffffffu, lane == 0 && (full || total > kHashSize * 3 / 4), 0);
     }
-    if (stop || *(volatile int*)&wide[g]) break;
+    // another warp of the row may be setting the flag: the lanes' looks at it are pooled, so that all 32 leave
+    // here or none does
+    if (__any_sync(0xffffffffu, stop || *(volatile int*)&wide[g])) break;
   }
   sync();
   if (wide[g]) {

@@ -1,0 +1,50 @@
+"""Rules of the device code that a run cannot show to be broken (a race or a hang that a build happens not to
+have), checked on the sources."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1801_05648_gb300", "csrc")
+
+
+def _source(name):
+    """The file without comments and line continuations."""
+    with open(os.path.join(CSRC, name)) as f:
+        text = f.read()
+    return re.sub(r"//[^\n]*|/\*.*?\*/", "", text, flags=re.S)
+
+
+def _kernels():
+    """{kernel name: (file, parameter list, body)} of every __global__ function defined in the sources."""
+    found = {}
+    for name in sorted(os.listdir(CSRC)):
+        if not name.endswith((".cu", ".cuh")):
+            continue
+        text = _source(name)
+        for m in re.finditer(r"__global__\s+void\s+(?:__launch_bounds__\((?:[^()]|\([^()]*\))*\)\s*)?(\w+)\s*\(", text):
+            depth, i = 1, m.end()
+            while depth:
+                depth += {"(": 1, ")": -1}.get(text[i], 0)
+                i += 1
+            params = text[m.end():i - 1]
+            body = text.index("{", i)
+            depth, j = 1, body + 1
+            while depth:
+                depth += {"{": 1, "}": -1}.get(text[j], 0)
+                j += 1
+            found[m.group(1)] = (name, params, text[body:j])
+    return found
+
+
+def test_kernels_are_found():
+    k = _kernels()
+    assert {"k_bsr_spmv", "k_operator_rows", "k_spgemm_sym", "k_gj_panel", "k_mlp_tc", "k_jacobian"} <= set(k)
+
+
+def test_spgemm_rows_leave_their_loop_together():
+    """A flag in shared memory that another warp may be setting can look different to the 32 lanes of a
+    warp; lanes that leave a loop on it would miss the warp-wide operations that the others wait in."""
+    body = _kernels()["k_spgemm_sym"][2]
+    exits = re.findall(r"if \(([^;{}]*)\) break;", body)
+    assert exits
+    for cond in exits:
+        assert "volatile" not in cond or cond.startswith("__any_sync(0xffffffffu,"), cond

@@ -1,0 +1,94 @@
+"""Calls at the edges of what the solver takes: product rows around the length of the SpGEMM
+table and aggregates larger than shared memory."""
+import numpy as np
+import pytest
+import scipy.sparse as sp
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch_cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1801_05648_gb300 import build
+    build.build()
+    return torch
+
+
+def _system(**blocks):
+    """CSR and class offsets of a 2D system: `blocks` names class pairs such as m_m, v_p (classes m, sv, su, v, p);
+    a class without a diagonal block is one node of identity rows (one entry for p)."""
+    names = ("m", "sv", "su", "v", "p")
+    size = {k: (blocks[f"{k}_{k}"].shape[0] if f"{k}_{k}" in blocks else 1 if k == "p" else 2) for k in names}
+    grid = [[blocks.get(f"{r}_{c}", sp.identity(size[r]) if r == c else sp.csr_matrix((size[r], size[c])))
+             for c in names] for r in names]
+    A = sp.block_array(grid, format="csr") if hasattr(sp, "block_array") else sp.bmat(grid, format="csr")
+    A.sort_indices()
+    return A, np.cumsum([0] + [size[k] for k in names]).astype(np.int64)
+
+
+def _context(A, off, **params):
+    import paper_1801_05648_gb300 as P
+    return P.FSISolver(2, A.indptr.astype(np.int64), A.indices.astype(np.int32), A.data.astype(np.float64), off, None,
+                       P.default_params(2, **params))
+
+
+# pressures below and above 16 rows per SM: a block or a warp per product row
+@pytest.mark.parametrize("n_p", [900, 2600])
+@pytest.mark.parametrize("cols", [767, 768, 769, 900])
+def test_product_rows_around_the_table(n_p, cols, torch_cuda):
+    """S_p = I - e_0 w^T with w on `cols` pressures: a row of up to 768 columns is taken, and S_p^-1 b is
+    b + e_0 (w.b) / (1 - w_0) to the rounding of a well-conditioned inverse; a longer one is refused, and
+    the context is good again with the next values."""
+    torch = torch_cuda
+    import paper_1801_05648_gb300 as P
+    w = np.zeros(n_p)
+    w[:cols] = 0.5 / cols
+    first = np.arange(n_p) * 2
+    v_p = sp.csr_matrix((np.ones(n_p), (first, np.arange(n_p))), (2 * n_p, n_p))
+    p_v = sp.csr_matrix((w[:cols], (np.zeros(cols, int), first[:cols])), (n_p, 2 * n_p))
+    A, off = _system(v_v=sp.identity(2 * n_p), v_p=v_p, p_v=p_v, p_p=sp.identity(n_p))
+    S = _context(A, off, coarse_max=8000)
+    b = np.random.default_rng(cols).standard_normal(n_p)
+    x = torch.empty(n_p, dtype=torch.float64, device="cuda")
+    for _ in range(2):
+        if cols <= 768:
+            S.precond_build("fp64")
+            S.apply_block("pressure_schur", torch.tensor(b, device="cuda"), x)
+            want = b.copy()
+            want[0] += (w @ b) / (1 - w[0])
+            assert np.abs(x.cpu().numpy() - want).max() <= 1e-12 * np.abs(b).max()
+        else:
+            with pytest.raises(P.FSIError) as e:
+                S.precond_build("fp64")
+            assert e.value.code == P.FSI_EINVAL and "768" in str(e.value)
+        S.update_values(torch.tensor(A.data, device="cuda"))
+    S.close()
+
+
+def test_an_aggregate_larger_than_shared_memory(torch_cuda):
+    """A star of 1,001 nodes is one aggregate: 4,004 values to orthogonalise, more than the 2,560 that a
+    warp keeps in shared memory; and R A has one row of 1,001 columns, which the optional product
+    -(R A) does not take.  A V-cycle as the oracle's (sums of 2,002 terms, some ten passes: 1e-10)."""
+    torch = torch_cuda
+    from oracle import amg
+    n = 1001
+    S1 = sp.diags(np.concatenate([[1000.0], np.full(n - 1, 1.5)])).tolil()
+    S1[0, 1:] = -1.0
+    S1[1:, 0] = -1.0
+    M = sp.kron(S1.tocsr(), sp.identity(2)).tocsr()
+    A, off = _system(m_m=M)
+    S = _context(A, off, coarse_max=8, strength_theta=0.01)
+    S.precond_build("fp64")
+    H = amg.sa_setup(A[: 2 * n, : 2 * n].tocsr(), 2, amg.translations(n, 2),
+                     amg.AMGParams(coarse_max=8, theta=0.01))
+    assert S.amg_info("mesh")["levels"] == len(H.levels) == 2
+    assert H.levels[0].nagg == 1
+    b = np.random.default_rng(0).standard_normal(2 * n)
+    x = torch.empty(2 * n, dtype=torch.float64, device="cuda")
+    S.apply_block("mesh", torch.tensor(b, device="cuda"), x)
+    want = amg.vcycle(H, b)
+    assert np.linalg.norm(x.cpu().numpy() - want) <= 1e-10 * np.linalg.norm(want)
+    S.close()
