@@ -275,7 +275,7 @@ __global__ void k_power_init(int64_t n, int stream_id, double* __restrict__ x) {
 }
 
 // x = y / ||y|| with ||y||^2 on the device; x stays when y = 0 (its next product is then 0 again)
-__global__ void k_power_scale(int64_t n, const double* __restrict__ yy, const double* __restrict__ y,
+__global__ void k_power_scale(int64_t n, const double* yy, const double* y,
                               double* __restrict__ x) {
   dep_wait();
   const double ny = __dsqrt_rn(*yy);
@@ -287,7 +287,7 @@ __global__ void k_power_scale(int64_t n, const double* __restrict__ yy, const do
 
 // d = dinv * b / theta; x = d   (first Chebyshev step from x = 0)
 template <class T>
-__global__ void k_cheb_first(int64_t n, const T* __restrict__ b, const T* __restrict__ dinv, T inv_theta,
+__global__ void k_cheb_first(int64_t n, const T* b, const T* __restrict__ dinv, T inv_theta,
                              T* __restrict__ d, T* __restrict__ x) {
   dep_wait();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -301,7 +301,7 @@ __global__ void k_cheb_first(int64_t n, const T* __restrict__ b, const T* __rest
 // before the wait for the previous kernel (built: M is not being written), which leaves b's round
 // trip behind it.
 template <class T>
-__global__ void k_dense_gemv(int n, const T* __restrict__ M, const T* __restrict__ b, T* __restrict__ x, int built) {
+__global__ void k_dense_gemv(int n, const T* __restrict__ M, const T* b, T* __restrict__ x, int built) {
   constexpr int U = 8;
   dep_trigger();
   if (!built) dep_wait_only();

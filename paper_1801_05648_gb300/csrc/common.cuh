@@ -58,6 +58,10 @@ inline thread_local int64_t g_kernel_launches = 0;
 // arrive early settle where there happens to be room, and the fullest SM's FP64 pipe then sets
 // the pace (64x32 solve 1.99 ms with such triggers, 1.92 without; training step 800 / 762 us).
 // Off for the whole process when a context was set up with FSI_NO_PDL.
+// Such a kernel's lifetime overlaps writes of the kernels before it, so nothing that a queued kernel
+// may write counts as read-only in it: those arguments carry no __restrict__ and are read by ordinary loads
+// behind the wait, not by __ldg or ld.global.nc, which the compiler may move ahead of it and which
+// need not see the write.  Matrices, patterns, weights and the arguments themselves may be.
 __device__ __forceinline__ void dep_trigger() {
 #if defined(__CUDA_ARCH__) && (__CUDA_ARCH__ >= 900)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

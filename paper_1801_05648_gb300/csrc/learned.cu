@@ -105,7 +105,7 @@ __device__ __forceinline__ int4 node_rec(const MlpGeom& g, int q) {
 
 // Issue the loads of one patch node's r' values (raw FP64) and class scales.
 template <int D>
-__device__ __forceinline__ void load_node_vals(const MlpGeom& g, const double* __restrict__ rp, int4 r,
+__device__ __forceinline__ void load_node_vals(const MlpGeom& g, const double* rp, int4 r,
                                                double (&ev)[2 * D + 1], float (&sc)[3]) {
 #pragma unroll
   for (int k = 0; k < 2 * D + 1; ++k) ev[k] = 0.0;
@@ -130,7 +130,7 @@ __device__ __forceinline__ void load_node_vals(const MlpGeom& g, const double* _
 #pragma nv_diag_suppress 128
 template <int D, int MODE>
 __global__ void __launch_bounds__(kNodeThreads) k_mlp(MlpGeom g, const uint16_t* __restrict__ w16,
-                                                      const double* __restrict__ rp, double* __restrict__ c,
+                                                      const double* rp, double* __restrict__ c,
                                                       float* __restrict__ F, float* __restrict__ rho_out,
                                                       float* __restrict__ G1, float* __restrict__ D1,
                                                       float* __restrict__ G2, float* __restrict__ D2, int64_t ld) {
@@ -590,8 +590,8 @@ __device__ __forceinline__ double block_sum_d(double v, double* sh) {
 }
 
 // rp = V_j - w; part[blk] = sum of rp^2 over the block's contiguous chunk
-__global__ void __launch_bounds__(kRT) k_learned_residual(int64_t n, const double* __restrict__ V, int64_t ldv,
-                                                          const int* __restrict__ jdev, const double* __restrict__ w,
+__global__ void __launch_bounds__(kRT) k_learned_residual(int64_t n, const double* V, int64_t ldv,
+                                                          const int* jdev, const double* w,
                                                           double* __restrict__ rp, double* __restrict__ part) {
   dep_wait();
   __shared__ double sh[32];
@@ -610,8 +610,8 @@ __global__ void __launch_bounds__(kRT) k_learned_residual(int64_t n, const doubl
 }
 
 // part[blk] = sum of (rp - t)^2; optionally res = rp - t
-__global__ void __launch_bounds__(kRT) k_diff_sq(int64_t n, const double* __restrict__ rp,
-                                                 const double* __restrict__ t, double* __restrict__ res,
+__global__ void __launch_bounds__(kRT) k_diff_sq(int64_t n, const double* rp,
+                                                 const double* t, double* __restrict__ res,
                                                  double* __restrict__ part) {
   dep_wait();
   __shared__ double sh[32];
@@ -629,7 +629,7 @@ __global__ void __launch_bounds__(kRT) k_diff_sq(int64_t n, const double* __rest
 }
 
 // sums of both partial arrays (fixed order); accept iff ||rp - t||^2 < tau^2 ||rp||^2
-__global__ void __launch_bounds__(kRT) k_learned_decide(const double* __restrict__ part, int np, double tau2,
+__global__ void __launch_bounds__(kRT) k_learned_decide(const double* part, int np, double tau2,
                                                         int* counters) {
   dep_wait();
   __shared__ double sh[32];
@@ -647,9 +647,9 @@ __global__ void __launch_bounds__(kRT) k_learned_decide(const double* __restrict
   }
 }
 
-__global__ void k_learned_commit(int64_t n, const int* __restrict__ counters, const double* __restrict__ c,
-                                 const double* __restrict__ t, double* __restrict__ Z, int64_t ldz,
-                                 const int* __restrict__ jdev, double* __restrict__ w) {
+__global__ void k_learned_commit(int64_t n, const int* counters, const double* c,
+                                 const double* t, double* __restrict__ Z, int64_t ldz,
+                                 const int* jdev, double* __restrict__ w) {
   dep_wait();
   if (counters[0] == 0) return;
   double* z = Z + (int64_t)(*jdev) * ldz;
@@ -659,8 +659,8 @@ __global__ void k_learned_commit(int64_t n, const int* __restrict__ counters, co
   }
 }
 
-__global__ void k_harvest(int64_t n, const double* __restrict__ V, int64_t ldv, const int* __restrict__ jdev,
-                          const double* __restrict__ w, double* __restrict__ buf, int nvec) {
+__global__ void k_harvest(int64_t n, const double* V, int64_t ldv, const int* jdev,
+                          const double* w, double* __restrict__ buf, int nvec) {
   dep_wait();
   const int j = *jdev;
   if (j >= nvec) return;

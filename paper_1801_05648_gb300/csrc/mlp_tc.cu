@@ -153,7 +153,7 @@ __device__ __forceinline__ void issue_layer(uint32_t sbase, uint32_t boff, uint3
 //   layers 1-2 half 0: hidden columns 0-31; half 1: 32-63
 //   layer 3    half 0: the outputs and the scatter
 __global__ void __launch_bounds__(kTcThreads, 2) k_mlp_tc(MlpGeom g, const uint16_t* __restrict__ w16,
-                                                          const double* __restrict__ rp, double* __restrict__ c,
+                                                          const double* rp, double* __restrict__ c,
                                                           int* __restrict__ err, int no_commit) {
   extern __shared__ __align__(1024) unsigned char sm[];
   const int t = threadIdx.x, warp = t >> 5;

@@ -58,7 +58,7 @@ void bsr_clone(const Bsr& A, Bsr& B, cudaStream_t s) {
 
 // ------------------------------------------------------------------ kernels
 template <class Ti, class To>
-__global__ void k_col_in(int64_t n, const Ti* __restrict__ V, int64_t ldv, const int* __restrict__ jdev, int joff,
+__global__ void k_col_in(int64_t n, const Ti* V, int64_t ldv, const int* jdev, int joff,
                          To* __restrict__ out) {
   dep_wait();
   const int j = *jdev + joff;
@@ -68,8 +68,8 @@ __global__ void k_col_in(int64_t n, const Ti* __restrict__ V, int64_t ldv, const
 }
 // zfix = (double) in; Z_j = zfix
 template <class T>
-__global__ void k_col_out(int64_t n, const T* __restrict__ in, double* __restrict__ zfix, double* __restrict__ Z,
-                          int64_t ldz, const int* __restrict__ jdev) {
+__global__ void k_col_out(int64_t n, const T* in, double* __restrict__ zfix, double* __restrict__ Z,
+                          int64_t ldz, const int* jdev) {
   dep_wait_only();   // the FP64 operator follows
   double* dst = Z + (size_t)(*jdev) * ldz;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -79,9 +79,9 @@ __global__ void k_col_out(int64_t n, const T* __restrict__ in, double* __restric
   }
 }
 // V_{j+1} = sign * w / h  (left zero when h == 0); nothing while a second pass is due (*ready == 0)
-__global__ void k_scale_col(int64_t n, const double* __restrict__ w, const double* __restrict__ h,
-                            double* __restrict__ V, int64_t ldv, const int* __restrict__ jdev, double sign,
-                            const int* __restrict__ ready) {
+__global__ void k_scale_col(int64_t n, const double* w, const double* h,
+                            double* __restrict__ V, int64_t ldv, const int* jdev, double sign,
+                            const int* ready) {
   dep_wait();
   if (*ready == 0) return;
   const double hv = *h;
@@ -102,10 +102,10 @@ __global__ void k_scale_col(int64_t n, const double* __restrict__ w, const doubl
 // (The second pass, its sums, the test and the norm as launches of their own in every step, most
 // of which had nothing to do, were 5 of a small system's 83 launches per iteration.)
 __global__ void __launch_bounds__(kRedThreads) k_arnoldi_finish(
-    const double* __restrict__ pa, const double* __restrict__ pb, int np, double eta2, int second,
-    int* __restrict__ ready, double* __restrict__ hnorm, int ldh, const int* __restrict__ jdev,
-    const double* __restrict__ h1, const double* __restrict__ h2, double* __restrict__ H, double* __restrict__ cs,
-    double* __restrict__ sn, double* __restrict__ g, const double* __restrict__ inv_bnorm_p,
+    const double* pa, const double* pb, int np, double eta2, int second,
+    int* __restrict__ ready, double* __restrict__ hnorm, int ldh, const int* jdev,
+    const double* h1, const double* h2, double* __restrict__ H, double* __restrict__ cs,
+    double* __restrict__ sn, double* __restrict__ g, const double* inv_bnorm_p,
     double* __restrict__ out) {
   dep_wait();
   __shared__ double sh[32];
@@ -155,8 +155,8 @@ __global__ void __launch_bounds__(kRedThreads) k_arnoldi_finish(
 }
 
 // H y = g, k x k upper triangular (column-major, leading dimension ldh); one thread
-__global__ void k_backsolve(int ldh, const int* __restrict__ kdev, const double* __restrict__ H,
-                            const double* __restrict__ g, double* __restrict__ y) {
+__global__ void k_backsolve(int ldh, const int* kdev, const double* H,
+                            const double* g, double* __restrict__ y) {
   dep_wait();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   const int k = *kdev;
@@ -286,7 +286,7 @@ void solid_solve(Context& C, const T* r, T* x, cudaStream_t st, bool r_u_zero = 
 // whole sequence is enqueued once and can be captured into the iteration graph.
 
 // out = w / a with a = nrm[0] (sqrt(nrm[0]) when squared); out = 0 when a == 0
-__global__ void k_unit_scale(int64_t n, const double* __restrict__ w, const double* __restrict__ nrm, int squared,
+__global__ void k_unit_scale(int64_t n, const double* w, const double* nrm, int squared,
                              double* __restrict__ out) {
   dep_wait();
   const double a = squared ? sqrt(nrm[0]) : nrm[0];
@@ -298,8 +298,8 @@ __global__ void k_unit_scale(int64_t n, const double* __restrict__ w, const doub
 // step: H(i, j) = h1[j ld + i] + h2[j ld + i] for i <= j (the two Gram-Schmidt
 // passes), H(j+1, j) = nrm[j]; beta = sqrt(beta2[0]).  A zero pivot (exact
 // breakdown) gives y_i = 0 for that column.
-__global__ void k_inner_ls(int k, const double* __restrict__ h1, const double* __restrict__ h2, int ld,
-                           const double* __restrict__ nrm, const double* __restrict__ beta2, double* __restrict__ y) {
+__global__ void k_inner_ls(int k, const double* h1, const double* h2, int ld,
+                           const double* nrm, const double* beta2, double* __restrict__ y) {
   __shared__ double R[kFluidGmresMax + 1][kFluidGmresMax];   // shared, not local: no stack frame
   __shared__ double g[kFluidGmresMax + 1], cs[kFluidGmresMax], sn[kFluidGmresMax];
   dep_wait();

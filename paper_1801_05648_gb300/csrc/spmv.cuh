@@ -4,7 +4,7 @@
 // row: lane l reads blocks l, l+tpr, ... of the row, so the lanes of a group
 // stream consecutive blocks (row-major br x bc values, 16-byte vector loads
 // whenever the block size allows) and the block-column indices coalesced; the
-// x entries are gathered through the read-only path.  Each lane issues several
+// x entries are gathered with ordinary loads (see dep_wait in common.cuh).  Each lane issues several
 // blocks' loads before multiplying (bytes in flight hide the DRAM latency).
 // Lane 0 loads its row's own epilogue operands first, then the group reduces its
 // br partial sums with shuffles and lane 0 applies the epilogue.  The lane count
@@ -55,47 +55,48 @@ __device__ __forceinline__ void load_stream(const T* __restrict__ p, T* out) {
 }
 
 template <class T, int N>
-__device__ __forceinline__ void load_gather(const T* __restrict__ p, T* out) {
+__device__ __forceinline__ void load_gather(const T* p, T* out) {
   if constexpr (sizeof(T) == 8 && N % 2 == 0) {
 #pragma unroll
     for (int i = 0; i < N / 2; ++i) {
-      double2 v = __ldg(reinterpret_cast<const double2*>(p) + i);
+      const double2 v = reinterpret_cast<const double2*>(p)[i];
       out[2 * i] = v.x; out[2 * i + 1] = v.y;
     }
   } else if constexpr (sizeof(T) == 4 && N % 2 == 0) {
 #pragma unroll
     for (int i = 0; i < N / 2; ++i) {
-      float2 v = __ldg(reinterpret_cast<const float2*>(p) + i);
+      const float2 v = reinterpret_cast<const float2*>(p)[i];
       out[2 * i] = v.x; out[2 * i + 1] = v.y;
     }
   } else {
 #pragma unroll
-    for (int i = 0; i < N; ++i) out[i] = __ldg(p + i);
+    for (int i = 0; i < N; ++i) out[i] = p[i];
   }
 }
 
 // FP64 gathers with the L2 evict-last policy: the gathered vector (71 MB in FP64 on
 // the 1024x512 system) then outlives the evict-first matrix stream in L2.  FP64
 // launches of the preconditioner and the set-up use them on large vectors (kKeepCols): the
-// 1024x512 V-cycles ran 8% faster with them.
+// 1024x512 V-cycles ran 8% faster with them.  (volatile: they stay behind the wait for the previous kernel.)
 __device__ __forceinline__ uint64_t l2_evict_last_policy() {
   uint64_t pol;
   asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
   return pol;
 }
 template <int N>
-__device__ __forceinline__ void load_gather_keep(const double* __restrict__ p, double* out) {
+__device__ __forceinline__ void load_gather_keep(const double* p, double* out) {
 #if defined(__CUDA_ARCH__) && (__CUDA_ARCH__ >= 900)
   const uint64_t pol = l2_evict_last_policy();
   if constexpr (N % 2 == 0) {
 #pragma unroll
     for (int i = 0; i < N / 2; ++i)
-      asm("ld.global.nc.L2::cache_hint.v2.f64 {%0, %1}, [%2], %3;"
-          : "=d"(out[2 * i]), "=d"(out[2 * i + 1])
-          : "l"(p + 2 * i), "l"(pol));
+      asm volatile("ld.global.L2::cache_hint.v2.f64 {%0, %1}, [%2], %3;"
+                   : "=d"(out[2 * i]), "=d"(out[2 * i + 1])
+                   : "l"(p + 2 * i), "l"(pol));
   } else {
 #pragma unroll
-    for (int i = 0; i < N; ++i) asm("ld.global.nc.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(out[i]) : "l"(p + i), "l"(pol));
+    for (int i = 0; i < N; ++i)
+      asm volatile("ld.global.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(out[i]) : "l"(p + i), "l"(pol));
   }
 #else
   for (int i = 0; i < N; ++i) out[i] = p[i];
@@ -442,7 +443,7 @@ __device__ __forceinline__ void bsr_rows(int cta, int nbr, int tpr, int rows_per
     const int4* __restrict__ ord2,
     const int* __restrict__ rp1, const CI1* __restrict__ ci1, const T* __restrict__ v1, int64_t nnzb1, const G1& g1,
     const int* __restrict__ rp2, const int* __restrict__ ci2, const T* __restrict__ v2, int64_t nnzb2,
-    const T* __restrict__ x2,
+    const T* x2,
     const Epi& epi) {
   const int r0 = cta * rows_per_cta;
   const int r1 = r0 + rows_per_cta < nbr ? r0 + rows_per_cta : nbr;
@@ -545,7 +546,7 @@ __global__ void __launch_bounds__(256) k_bsr_spmv(int nbr, int tpr, int rows_per
     const int4* __restrict__ ord2,
     const int* __restrict__ rp1, const CI1* __restrict__ ci1, const T* __restrict__ v1, int64_t nnzb1, G1 g1,
     const int* __restrict__ rp2, const int* __restrict__ ci2, const T* __restrict__ v2, int64_t nnzb2,
-    const T* __restrict__ x2,
+    const T* x2,
     Epi epi) {
   bsr_rows<T, BR, BC1, BC2, Epi, G1, UREQ, CI1, COMP, EARLY>(blockIdx.x, nbr, tpr, rows_per_cta, prefetch, dep, ord2,
                                                             rp1, ci1, v1, nnzb1, g1, rp2, ci2, v2, nnzb2, x2, epi);
@@ -567,8 +568,8 @@ struct RowClass {
 template <int D, template <class, int> class Epi, bool EARLY>
 __global__ void __launch_bounds__(256) k_operator_rows(const __grid_constant__ RowClass V,
                                                        const __grid_constant__ RowClass P, int ctas_p, int prefetch,
-                                                       int dep, const double* __restrict__ xv,
-                                                       const double* __restrict__ xp, Epi<double, D> epi_v,
+                                                       int dep, const double* xv,
+                                                       const double* xp, Epi<double, D> epi_v,
                                                        Epi<double, 1> epi_p) {
   const GatherX<double, D> g{xv};
   if ((int)blockIdx.x < ctas_p)

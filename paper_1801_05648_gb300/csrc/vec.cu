@@ -13,7 +13,7 @@ inline int grid_for(int64_t n) {
 }
 
 template <class T>
-__global__ void k_axpby(int64_t n, T a, const T* __restrict__ x, T b, T* __restrict__ y) {
+__global__ void k_axpby(int64_t n, T a, const T* x, T b, T* __restrict__ y) {
   dep_wait();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     T v = a * x[i];
@@ -23,28 +23,28 @@ __global__ void k_axpby(int64_t n, T a, const T* __restrict__ x, T b, T* __restr
 }
 
 template <class T>
-__global__ void k_axpbyz(int64_t n, T a, const T* __restrict__ x, T b, const T* __restrict__ y, T* __restrict__ z) {
+__global__ void k_axpbyz(int64_t n, T a, const T* x, T b, const T* y, T* __restrict__ z) {
   dep_wait();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     z[i] = a * x[i] + b * y[i];
 }
 
 template <class T>
-__global__ void k_vmul(int64_t n, const T* __restrict__ x, const T* __restrict__ w, T* __restrict__ y) {
+__global__ void k_vmul(int64_t n, const T* x, const T* w, T* __restrict__ y) {
   dep_wait();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = x[i] * w[i];
 }
 
 template <class T>
-__global__ void k_vfma(int64_t n, const T* __restrict__ w, const T* __restrict__ x, T* __restrict__ y) {
+__global__ void k_vfma(int64_t n, const T* w, const T* x, T* __restrict__ y) {
   dep_wait();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] += w[i] * x[i];
 }
 
 template <class Ti, class To>
-__global__ void k_cast(int64_t n, const Ti* __restrict__ x, To* __restrict__ y) {
+__global__ void k_cast(int64_t n, const Ti* x, To* __restrict__ y) {
   dep_wait();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = (To)x[i];
@@ -52,8 +52,8 @@ __global__ void k_cast(int64_t n, const Ti* __restrict__ x, To* __restrict__ y) 
 
 // partials[blockIdx] = sum over this block's contiguous chunk of x*y
 template <class T>
-__global__ void __launch_bounds__(kRedThreads) k_dot_partial(int64_t n, const T* __restrict__ x,
-                                                              const T* __restrict__ y, double* __restrict__ partials) {
+__global__ void __launch_bounds__(kRedThreads) k_dot_partial(int64_t n, const T* x,
+                                                              const T* y, double* __restrict__ partials) {
   dep_wait();
   __shared__ double sh[32];
   const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_partial(int64_t n, const T*
 }
 
 // out[c] = (sqrt?) sum_k partials[c * np + k], one block per column c
-__global__ void __launch_bounds__(kRedThreads) k_reduce_cols(const double* __restrict__ partials, int np,
+__global__ void __launch_bounds__(kRedThreads) k_reduce_cols(const double* partials, int np,
                                                              const int* jcount, int joff, double* out,
                                                              int take_sqrt) {
   dep_wait();
@@ -82,9 +82,9 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce_cols(const double* __res
 
 // Multi-dot: partials[i * gridDim + block] = <V_i, w> over the block's chunk, i < J.
 // Four basis vectors per pass over the chunk of w.
-__global__ void __launch_bounds__(kRedThreads) k_mdot_partial(int64_t n, const double* __restrict__ V, int64_t ldv,
-                                                              const int* __restrict__ jcount, int joff,
-                                                              const double* __restrict__ w,
+__global__ void __launch_bounds__(kRedThreads) k_mdot_partial(int64_t n, const double* V, int64_t ldv,
+                                                              const int* jcount, int joff,
+                                                              const double* w,
                                                               double* __restrict__ partials) {
   dep_wait();
   __shared__ double sh[32];
@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(kRedThreads) k_mdot_partial(int64_t n, const d
     const int ni = J - i0 < 4 ? J - i0 : 4;
     const double* v0 = V + (size_t)i0 * ldv;
     for (int64_t r = lo + threadIdx.x; r < hi; r += blockDim.x) {
-      const double wr = __ldg(w + r);
+      const double wr = w[r];
       a0 += __ldcs(v0 + r) * wr;
       if (ni > 1) a1 += __ldcs(v0 + ldv + r) * wr;
       if (ni > 2) a2 += __ldcs(v0 + 2 * ldv + r) * wr;
@@ -112,9 +112,9 @@ __global__ void __launch_bounds__(kRedThreads) k_mdot_partial(int64_t n, const d
 }
 
 // w -= sign * sum_i h[i] V_i  over the block's chunk; optional per-block sum of w^2
-__global__ void __launch_bounds__(kRedThreads) k_maxpy(int64_t n, const double* __restrict__ V, int64_t ldv,
-                                                       const int* __restrict__ jcount, int joff,
-                                                       const double* __restrict__ h, double sign,
+__global__ void __launch_bounds__(kRedThreads) k_maxpy(int64_t n, const double* V, int64_t ldv,
+                                                       const int* jcount, int joff,
+                                                       const double* h, double sign,
                                                        double* __restrict__ w, double* __restrict__ nrm_partials) {
   dep_wait();
   __shared__ double hs[256];
@@ -159,9 +159,9 @@ __device__ __forceinline__ void chunk_of(int64_t n, int64_t& lo, int64_t& hi) {
   hi = lo + chunk < n ? lo + chunk : n;
 }
 
-__global__ void __launch_bounds__(kRedThreads, 4) k_mdot_partial_v2(int64_t n, const double* __restrict__ V,
-                                                                 int64_t ldv, const int* __restrict__ jcount,
-                                                                 int joff, const double* __restrict__ w,
+__global__ void __launch_bounds__(kRedThreads, 4) k_mdot_partial_v2(int64_t n, const double* V,
+                                                                 int64_t ldv, const int* jcount,
+                                                                 int joff, const double* w,
                                                                  double* __restrict__ partials) {
   dep_wait();
   __shared__ double sh[kDotCols][kRedThreads / 32];
@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(kRedThreads, 4) k_mdot_partial_v2(int64_t n, c
     for (int u = 0; u < kDotCols; ++u) acc[u] = 0.0;
     for (int64_t r = lo + 2 * threadIdx.x; r < hi; r += 2 * blockDim.x) {
       if (r + 1 < hi) {
-        const double2 wr = __ldg(reinterpret_cast<const double2*>(w + r));
+        const double2 wr = *reinterpret_cast<const double2*>(w + r);
 #pragma unroll
         for (int u = 0; u < kDotCols; ++u)
           if (u < ni) {
@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(kRedThreads, 4) k_mdot_partial_v2(int64_t n, c
             acc[u] = fma(v.y, wr.y, fma(v.x, wr.x, acc[u]));
           }
       } else {
-        const double wr = __ldg(w + r);
+        const double wr = w[r];
 #pragma unroll
         for (int u = 0; u < kDotCols; ++u)
           if (u < ni) acc[u] = fma(__ldcs(v0 + (size_t)u * ldv + r), wr, acc[u]);
@@ -209,9 +209,9 @@ __global__ void __launch_bounds__(kRedThreads, 4) k_mdot_partial_v2(int64_t n, c
 
 // w -= sign * sum_i h[i] V_i over the block's chunk, two elements per thread and
 // load; each element sums the basis vectors in increasing order (as k_maxpy).
-__global__ void __launch_bounds__(kRedThreads) k_maxpy_v2(int64_t n, const double* __restrict__ V, int64_t ldv,
-                                                          const int* __restrict__ jcount, int joff,
-                                                          const double* __restrict__ h, double sign,
+__global__ void __launch_bounds__(kRedThreads) k_maxpy_v2(int64_t n, const double* V, int64_t ldv,
+                                                          const int* jcount, int joff,
+                                                          const double* h, double sign,
                                                           double* __restrict__ w, double* __restrict__ nrm_partials) {
   dep_wait();
   extern __shared__ double hs[];
@@ -248,8 +248,8 @@ __global__ void __launch_bounds__(kRedThreads) k_maxpy_v2(int64_t n, const doubl
 }
 
 // Arnoldi defect: w = V_j - w over the block's chunk (j = *jcount), per-block sums of w^2.
-__global__ void __launch_bounds__(kRedThreads) k_defect(int64_t n, const double* __restrict__ V, int64_t ldv,
-                                                        const int* __restrict__ jcount, double* __restrict__ w,
+__global__ void __launch_bounds__(kRedThreads) k_defect(int64_t n, const double* V, int64_t ldv,
+                                                        const int* jcount, double* __restrict__ w,
                                                         double* __restrict__ partials) {
   dep_wait();
   __shared__ double sh[32];

@@ -48,3 +48,29 @@ def test_spgemm_rows_leave_their_loop_together():
     assert exits
     for cond in exits:
         assert "volatile" not in cond or cond.startswith("__any_sync(0xffffffffu,"), cond
+
+
+# What no queued kernel writes while another may be resident: matrices with their patterns, the inverse
+# diagonals and the coarse inverse of a built preconditioner, the weights.
+_CONSTANT = {"ord2", "rp1", "ci1", "v1", "rp2", "ci2", "v2", "rp", "ci", "v", "M", "dinv", "w16"}
+
+
+def test_overlapping_kernels_read_vectors_with_ordinary_loads():
+    """A kernel that may be resident before the kernel ahead of it has finished must not declare what
+    that kernel writes read-only: an invariant load may be moved ahead of the wait."""
+    overlapping = {k: v for k, v in _kernels().items() if re.search(r"\bdep_wait|\bbsr_rows<", v[2])}
+    assert len(overlapping) >= 28, sorted(overlapping)
+    for kernel, (name, params, _) in overlapping.items():
+        declared = set(re.findall(r"const\s+\w+\s*\*\s*__restrict__\s+(\w+)", params))
+        assert declared <= _CONSTANT, (name, kernel, declared - _CONSTANT)
+    text = _source("spmv.cuh")
+    assert set(re.findall(r"__ldg\((\w+)", text)) == {"ord2"}
+    for loader in ("load_gather", "load_gather_keep"):
+        assert re.search(r"void %s\(const \w+\* p," % loader, text), loader
+    rows = text[text.index("void bsr_rows("):]
+    assert set(re.findall(r"const\s+\w+\*\s*__restrict__\s+(\w+)", rows[:rows.index("{")])) <= _CONSTANT
+    for name in os.listdir(CSRC):
+        if name.endswith((".cu", ".cuh")):
+            assert "ld.global.nc" not in _source(name), name
+    for name in ("vec.cu", "solver.cu", "mlp_tc.cu", "amg.cu"):
+        assert "__ldg" not in _source(name), name
