@@ -29,9 +29,10 @@ void launch_operator(const Bsr& AVV, const Bsr& AVP, const Bsr& APV, const Bsr& 
 void spmv_operator(const Bsr& AVV, const Bsr& AVP, const Bsr& APV, const Bsr& APP, const double* x, const double* b,
                    double* y, cudaStream_t s) {
   const int64_t nv = AVV.rows();
-  if (AVP.nbr == 0 || APP.nbr == 0) {   // no pressures
-    if (b) spmv2_resid<double>(AVV, x, nullptr, nullptr, b, y, s);
-    else spmv2_axpby<double>(AVV, x, nullptr, nullptr, 1.0, 0.0, y, s);
+  if (AVV.nbr == 0 || APP.nbr == 0) {   // (AVP has the velocity rows, APV the pressure rows)
+    const Bsr& A = AVV.nbr ? AVV : APP;   // no pressures, or no velocities: then nv = 0
+    if (b) spmv2_resid<double>(A, x, nullptr, nullptr, b, y, s);
+    else spmv2_axpby<double>(A, x, nullptr, nullptr, 1.0, 0.0, y, s);
     return;
   }
   auto run = [&]<int D>() {

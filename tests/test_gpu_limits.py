@@ -1,5 +1,5 @@
 """Calls at the edges of what the solver takes: product rows around the length of the SpGEMM
-table and aggregates larger than shared memory."""
+table, aggregates larger than shared memory, empty classes of unknowns."""
 import numpy as np
 import pytest
 import scipy.sparse as sp
@@ -91,4 +91,34 @@ def test_an_aggregate_larger_than_shared_memory(torch_cuda):
     S.apply_block("mesh", torch.tensor(b, device="cuda"), x)
     want = amg.vcycle(H, b)
     assert np.linalg.norm(x.cpu().numpy() - want) <= 1e-10 * np.linalg.norm(want)
+    S.close()
+
+
+# the classes of unknowns that are left out, out of m, sv, su, v, p
+@pytest.mark.parametrize("empty", [("m",), ("sv", "su"), ("v",), ("p",), ("v", "p"), ("m", "sv", "su", "v"),
+                                   ("m", "sv", "su", "p"), ("sv", "su", "v", "p")])
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_empty_classes(empty, precision, torch_cuda):
+    """A system without one or several classes: the operator is the host's product within its rounding,
+    (row length + 2) u |A| |x|, into a vector that held something else, and the solution has a
+    residual of 1e-10."""
+    torch = torch_cuda
+    rng = np.random.default_rng(7)
+    size = {k: 0 if k in empty else 30 if k == "p" else 60 for k in ("m", "sv", "su", "v", "p")}
+    n = sum(size.values())
+    A = sp.random(n, n, 0.1, random_state=rng, data_rvs=rng.standard_normal).tocsr()
+    A = (A + sp.identity(n) * 20.0).tocsr()
+    A.sort_indices()
+    off = np.cumsum([0] + list(size.values())).astype(np.int64)
+    S = _context(A, off, maxit=300)
+    x = rng.standard_normal(n)
+    y = torch.full((n,), 7.0, dtype=torch.float64, device="cuda")
+    S.apply_operator(torch.tensor(x, device="cuda"), y)
+    bound = (np.diff(A.indptr) + 2) * np.finfo(float).eps * (abs(A) @ np.abs(x))
+    assert (np.abs(y.cpu().numpy() - A @ x) <= bound).all()
+    S.precond_build(precision)
+    b = A @ x
+    z = torch.full((n,), 7.0, dtype=torch.float64, device="cuda")
+    st = S.solve(torch.tensor(b, device="cuda"), z, 1e-10)
+    assert st.status == 0 and np.linalg.norm(b - A @ z.cpu().numpy()) <= 1.001e-10 * np.linalg.norm(b)
     S.close()
