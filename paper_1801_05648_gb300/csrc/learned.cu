@@ -751,7 +751,7 @@ void learned_set_geometry(Learned& L, int64_t n, int64_t n_nodes, const int32_t*
     }
   }
   for (int64_t d = 0; d < n; ++d) require(seen[(size_t)d], "learned stage: a DOF belongs to no node");
-  L.n_nodes = n_nodes;
+  L.n_nodes = 0;   // until every array is there
   L.node_dof.alloc((size_t)n_nodes);
   L.patch.alloc((size_t)n_nodes * slots);
   FSI_CUDA(cudaMemcpyAsync(L.node_dof.p, node_dof, sizeof(int4) * n_nodes, cudaMemcpyHostToDevice, s));
@@ -763,6 +763,7 @@ void learned_set_geometry(Learned& L, int64_t n, int64_t n_nodes, const int32_t*
   L.counters.alloc(3);
   FSI_CUDA(cudaMemsetAsync(L.counters.p, 0, 3 * sizeof(int), s));
   FSI_CUDA(cudaStreamSynchronize(s));
+  L.n_nodes = n_nodes;
 }
 
 void learned_set_weights(Learned& L, const float* sig_in, const float* sig_out, const uint16_t* params,
@@ -962,18 +963,20 @@ double trainer_step_d(Trainer& T, Context& C, const double* rp, bool grad) {
   cudaStream_t s = C.s;
   if (T.cap_nodes < nn) {
     const size_t rows = ((size_t)nn + 31) / 32 * 32;   // row length: 16-byte aligned rows
-    T.cap_nodes = (int64_t)rows;
+    T.cap_nodes = 0;                                    // until every array is there
     T.F.alloc(N::kIn * rows);
     T.rho.alloc(rows);
     for (DBuf<float>* h : {&T.G1, &T.D1, &T.G2, &T.D2, &T.dH1, &T.dH2}) h->alloc(N::kHidden * rows);
     T.dY.alloc(N::kOut * rows);
+    T.cap_nodes = (int64_t)rows;
   }
   if (T.cap_n < n) {
-    T.cap_n = n;
+    T.cap_n = 0;
     T.c.alloc((size_t)n);
     T.t.alloc((size_t)n);
     T.res.alloc((size_t)n);
     T.g.alloc((size_t)n);
+    T.cap_n = n;
   }
   MlpGeom g = learned_geom(L, C.off);
   for (int k = 0; k < 5; ++k) {

@@ -387,9 +387,13 @@ void ensure_fluid_gmres(Context& C) {
   const int k = C.prm.fluid_gmres_iters;
   const int64_t n = C.off[4] - C.off[3];
   if (F.k == k && F.n == n) return;
-  F.k = k;
+  F.k = 0;   // until every array is there
   F.n = n;
-  if (n == 0) return;
+  if (C.iter_graph) { cudaGraphExecDestroy(C.iter_graph); C.iter_graph = nullptr; }
+  if (n == 0) {
+    F.k = k;
+    return;
+  }
   F.V.alloc((size_t)(k + 1) * n);
   F.Z.alloc((size_t)k * n);
   F.w.alloc(n);
@@ -404,7 +408,7 @@ void ensure_fluid_gmres(Context& C) {
   F.npart.alloc(kRedBlocks);
   F.zero.alloc(1);
   FSI_CUDA(cudaMemsetAsync(F.zero.p, 0, sizeof(int), C.s));
-  if (C.iter_graph) { cudaGraphExecDestroy(C.iter_graph); C.iter_graph = nullptr; }
+  F.k = k;
 }
 
 // A_ff^-1 of the fluid solve: V-cycle(s), or the inner GMRES with FLUID_GMRES

@@ -1,8 +1,12 @@
 """Calls at the edges of what the solver takes: product rows around the length of the SpGEMM
-table, aggregates larger than shared memory, empty classes of unknowns."""
+table, aggregates larger than shared memory, empty classes of unknowns, too little device memory."""
+import contextlib
+
 import numpy as np
 import pytest
 import scipy.sparse as sp
+
+import fsigen
 
 pytestmark = pytest.mark.gpu
 
@@ -121,4 +125,55 @@ def test_empty_classes(empty, precision, torch_cuda):
     z = torch.full((n,), 7.0, dtype=torch.float64, device="cuda")
     st = S.solve(torch.tensor(b, device="cuda"), z, 1e-10)
     assert st.status == 0 and np.linalg.norm(b - A @ z.cpu().numpy()) <= 1.001e-10 * np.linalg.norm(b)
+    S.close()
+
+
+@contextlib.contextmanager
+def _memory_left(torch, nbytes):
+    """The device with about nbytes free while the block runs."""
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    ballast = []
+    for size in (32 << 30, 4 << 30, 512 << 20, 64 << 20, 8 << 20, 2 << 20):
+        while torch.cuda.mem_get_info()[0] >= nbytes + size:
+            try:
+                ballast.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+            except torch.OutOfMemoryError:
+                break
+    try:
+        yield
+    finally:
+        torch.cuda.synchronize()
+        del ballast
+        torch.cuda.empty_cache()
+
+
+def test_training_step_after_a_failed_allocation(torch_cuda):
+    """A training step that does not get its memory says so, and the next one, with memory, has the loss and the
+    gradient of a trainer that never failed."""
+    torch = torch_cuda
+    import paper_1801_05648_gb300 as P
+    pb = fsigen.get_problem(fsigen.CONFIGS["2d_tiny"].with_(name="t", n=(96, 64)))
+    U = pb.seeded_state(0, 5e-3)
+    S = P.FSISolver(pb.dim, pb.rowptr, pb.colind, pb.jacobian(U, U), pb.offsets, pb.solid_node_coords(),
+                    P.default_params(2))
+    S.learned_setup(*pb.node_map())
+    r = torch.tensor(np.random.default_rng(1).standard_normal(pb.n), device="cuda")
+    ref = P.Trainer(seed=3)
+    loss = ref.step(S, r)
+    grad = ref.get()[2]
+    failed = 0
+    for mb in (1, 6, 12, 24, 40):
+        T = P.Trainer(seed=3)
+        with _memory_left(torch, mb << 20):
+            try:
+                T.step(S, r)
+            except P.FSIError as e:
+                assert e.code == P.FSI_ENOMEM
+                failed += 1
+            else:
+                continue
+        assert T.step(S, r) == loss and np.array_equal(T.get()[2], grad)
+        T.close()
+    assert failed >= 2
     S.close()
