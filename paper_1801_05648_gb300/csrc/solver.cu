@@ -456,7 +456,6 @@ Context::~Context() {
 // operator and the preconditioner's blocks, all extracted on the device.  keep: the blocks
 // hold an earlier extraction from the same pattern.
 static void extract_blocks(Context& C, const CsrView& A, bool keep) {
-  C.blocks_used = false;
   const int d = C.dim;
   const int64_t* o = C.off;
   const int nV = (int)(o[4] / d);
@@ -540,19 +539,25 @@ void context_setup(Context& C, const int64_t* rowptr, const int32_t* colind, con
   C.setup_s = secs(t0, clk::now());
 }
 
+// The diagonal blocks that the hierarchies and the mass solve took, back in their places (with their patterns
+// and, until new ones come, values).
+static void take_blocks_back(Context& C) {
+  auto back = [](Bsr& to, Bsr& from) {
+    if (from.rowptr.p) to = std::move(from);
+  };
+  if (!C.H[0].levels.empty()) back(C.Mblk, C.H[0].levels[0].A);
+  if (!C.H[2].levels.empty()) back(C.Aff, C.H[2].levels[0].A);
+  back(C.Auu, C.mass.A);
+  C.built = false;
+}
+
 void context_update_values(Context& C, const double* vals_dev) {
   SetupPhase setup_phase(C.pool);
   CsrView v = C.pattern.view();
   v.vals = vals_dev;
-  if (C.built) {   // the diagonal blocks that the hierarchies took come back with their patterns
-    C.Mblk = std::move(C.H[0].levels[0].A);
-    C.Aff = std::move(C.H[2].levels[0].A);
-    C.Auu = std::move(C.mass.A);
-    C.built = false;
-  }
+  take_blocks_back(C);
   extract_blocks(C, v, true);
   // every hierarchy, Schur operator, FP32 copy and captured graph refers to the old values
-  C.built = false;
   C.fp32_ready = false;
   C.At_built = false;
   if (C.iter_graph) { cudaGraphExecDestroy(C.iter_graph); C.iter_graph = nullptr; }
@@ -636,72 +641,96 @@ void run_branches(Context& C, Build&& build, Own&& own) {
   for (SetupBranch& b : C.branch) FSI_CUDA(cudaStreamWaitEvent(C.s, b.done, 0));
 }
 
+// The hierarchies and the mass solve of the context's values (first) and their FP32 copies (demote).
+// done[h]: what FP64 needs of hierarchy h (done[4]: of the rest) is there.
+static void build_parts(Context& C, bool first, bool demote, bool (&done)[5]) {
+  auto& s = C.s;
+  const int d = C.dim;
+  Bsr Shat, Sp;
+  DBuf<double> B[4];   // near-nullspaces; the solid's rigid-body modes are kept by the context
+  const bool rigid = C.solid_B.p != nullptr;
+  if (first) {
+    require(C.Mblk.rowptr.p && C.Aff.rowptr.p && C.Auu.rowptr.p, "fsi_precond_build: no values (fsi_update_values)");
+    // S_hat = A_vv + c A_vu  (Alg. 3)
+    bsr_add(C.Avv, C.A_vu, C.prm.dt_theta, Shat, s);
+    // S_p = C_pp - B_pv diag(A_ff)^-1 B_vp
+    const int64_t nfv = C.Aff.rows();
+    DBuf<double> diag(nfv > 0 ? nfv : 1), dinv(nfv > 0 ? nfv : 1);
+    bsr_point_diagonal(C.Aff, diag.p, s);
+    invert_nonzero(nfv, diag.p, dinv.p, s);
+    Bsr Bs, BDB;
+    bsr_clone(C.B_vp, Bs, s);
+    bsr_scale_rows(Bs, dinv.p, s);
+    bsr_spgemm(C.B_pv, Bs, BDB, s);
+    bsr_add(C.Cpp, BDB, -1.0, Sp, s);
+    translations(B[0], C.Mblk.nbr, d, s);
+    if (!rigid) translations(B[1], Shat.nbr, d, s);
+    translations(B[2], C.Aff.nbr, d, s);
+    translations(B[3], Sp.nbr, 1, s);
+    for (auto& H : C.H)
+      H.coarse_mode = (C.prm.flags & CLUSTER_COARSE) ? COARSE_CLUSTER
+                      : (C.prm.flags & GRID_COARSE)  ? COARSE_GRID
+                                                     : COARSE_PER_LEVEL;
+  }
+  // hierarchies M, S_hat, A_ff, S_p
+  Bsr* A0[4] = {&C.Mblk, &Shat, &C.Aff, &Sp};
+  const int modes[4] = {d, rigid ? (d == 2 ? 3 : 6) : d, d, 1};
+  run_branches(
+      C,
+      [&](int h, cudaStream_t st) {
+        if (first) amg_setup(C.H[h], std::move(*A0[h]), h == 1 && rigid ? C.solid_B.p : B[h].p, modes[h], C.prm.amg, st);
+        done[h] = true;
+        if (demote) amg_make_fp32(C.H[h], st);
+      },
+      [&] {
+        const int64_t nsu = C.off[3] - C.off[2];
+        if (first) {
+          cheb_setup(C.mass, std::move(C.Auu), C.prm.mass_degree, C.prm.mass_ratio, C.prm.amg.cheb_upper,
+                     C.prm.amg.power_iters, s);
+          C.uv_w64.alloc(nsu > 0 ? nsu : 1);
+          if (nsu > 0) {
+            k_row_weight<<<div_up(nsu, 256), 256, 0, s>>>(C.A_uv.nbr, C.A_uv.br, C.A_uv.rowptr.p, C.prm.dt_theta,
+                                                           C.uv_w64.p);
+            FSI_CHECK_LAUNCH();
+          }
+          alloc_pw(C.pw64, C.n);
+        }
+        done[4] = true;
+        if (demote) {
+          cheb_make_fp32(C.mass, s);
+          C.uv_w32.alloc(nsu > 0 ? nsu : 1);
+          if (nsu > 0) cast<double, float>(nsu, C.uv_w64.p, C.uv_w32.p, s);
+          for (Bsr* Q : {&C.C_ms, &C.A_vu, &C.A_uv, &C.C_sv_f, &C.C_sv_p, &C.C_fv_ms, &C.C_p_ms, &C.B_vp, &C.B_pv})
+            bsr_make_fp32(*Q, s);
+          alloc_pw(C.pw32, C.n);
+        }
+      });
+  FSI_CUDA(cudaStreamSynchronize(s));   // before the near-nullspaces go
+}
+
 void precond_build(Context& C, int precision) {
   SetupPhase setup_phase(C.pool);
   auto t0 = clk::now();
   auto& s = C.s;
-  const int d = C.dim;
   const bool first = !C.built, demote = precision == 1 && !C.fp32_ready;
   if (first || demote) {
-    Bsr Shat, Sp;
-    DBuf<double> B[4];   // near-nullspaces; the solid's rigid-body modes are kept by the context
-    const bool rigid = C.solid_B.p != nullptr;
-    if (first) {
-      require(!C.blocks_used, "fsi_precond_build: an earlier build of these values failed; give new ones (fsi_update_values)");
-      C.blocks_used = true;   // the diagonal blocks move into the hierarchies
-      // S_hat = A_vv + c A_vu  (Alg. 3)
-      bsr_add(C.Avv, C.A_vu, C.prm.dt_theta, Shat, s);
-      // S_p = C_pp - B_pv diag(A_ff)^-1 B_vp
-      const int64_t nfv = C.Aff.rows();
-      DBuf<double> diag(nfv > 0 ? nfv : 1), dinv(nfv > 0 ? nfv : 1);
-      bsr_point_diagonal(C.Aff, diag.p, s);
-      invert_nonzero(nfv, diag.p, dinv.p, s);
-      Bsr Bs, BDB;
-      bsr_clone(C.B_vp, Bs, s);
-      bsr_scale_rows(Bs, dinv.p, s);
-      bsr_spgemm(C.B_pv, Bs, BDB, s);
-      bsr_add(C.Cpp, BDB, -1.0, Sp, s);
-      translations(B[0], C.Mblk.nbr, d, s);
-      if (!rigid) translations(B[1], Shat.nbr, d, s);
-      translations(B[2], C.Aff.nbr, d, s);
-      translations(B[3], Sp.nbr, 1, s);
-      for (auto& H : C.H)
-        H.coarse_mode = (C.prm.flags & CLUSTER_COARSE) ? COARSE_CLUSTER
-                        : (C.prm.flags & GRID_COARSE)  ? COARSE_GRID
-                                                       : COARSE_PER_LEVEL;
+    // A build that fails (out of memory, say) leaves the context as it can be used: with its FP64 form when
+    // only the FP32 copies are missing, else unbuilt with its blocks, so that the call may be repeated.
+    bool done[5] = {};
+    try {
+      build_parts(C, first, demote, done);
+    } catch (...) {
+      cudaStreamSynchronize(s);
+      if (!first || (done[0] && done[1] && done[2] && done[3] && done[4])) {
+        C.built = true;
+        C.precision = 0;
+      } else {
+        take_blocks_back(C);
+        for (Hierarchy& H : C.H) H = Hierarchy();
+        C.mass = ChebSolver();
+      }
+      throw;
     }
-    // hierarchies M, S_hat, A_ff, S_p
-    Bsr* A0[4] = {&C.Mblk, &Shat, &C.Aff, &Sp};
-    const int modes[4] = {d, rigid ? (d == 2 ? 3 : 6) : d, d, 1};
-    run_branches(
-        C,
-        [&](int h, cudaStream_t st) {
-          if (first) amg_setup(C.H[h], std::move(*A0[h]), h == 1 && rigid ? C.solid_B.p : B[h].p, modes[h], C.prm.amg, st);
-          if (demote) amg_make_fp32(C.H[h], st);
-        },
-        [&] {
-          const int64_t nsu = C.off[3] - C.off[2];
-          if (first) {
-            cheb_setup(C.mass, std::move(C.Auu), C.prm.mass_degree, C.prm.mass_ratio, C.prm.amg.cheb_upper,
-                       C.prm.amg.power_iters, s);
-            C.uv_w64.alloc(nsu > 0 ? nsu : 1);
-            if (nsu > 0) {
-              k_row_weight<<<div_up(nsu, 256), 256, 0, s>>>(C.A_uv.nbr, C.A_uv.br, C.A_uv.rowptr.p, C.prm.dt_theta,
-                                                             C.uv_w64.p);
-              FSI_CHECK_LAUNCH();
-            }
-            alloc_pw(C.pw64, C.n);
-          }
-          if (demote) {
-            cheb_make_fp32(C.mass, s);
-            C.uv_w32.alloc(nsu > 0 ? nsu : 1);
-            if (nsu > 0) cast<double, float>(nsu, C.uv_w64.p, C.uv_w32.p, s);
-            for (Bsr* Q : {&C.C_ms, &C.A_vu, &C.A_uv, &C.C_sv_f, &C.C_sv_p, &C.C_fv_ms, &C.C_p_ms, &C.B_vp, &C.B_pv})
-              bsr_make_fp32(*Q, s);
-            alloc_pw(C.pw32, C.n);
-          }
-        });
-    FSI_CUDA(cudaStreamSynchronize(s));   // before the near-nullspaces go
     C.built = true;
     if (demote) C.fp32_ready = true;
   }

@@ -92,7 +92,6 @@ struct Context {
   Bsr Mblk, Avv, Auu, Aff, Cpp;   // diagonal blocks, consumed by precond_build
   Hierarchy H[4];             // M, S_hat, A_ff, S_p
   ChebSolver mass;            // A_uu (solid mass)
-  bool blocks_used = false;   // a build (perhaps a failed one) has taken the diagonal blocks
   bool built = false;
   bool fp32_ready = false;    // FP32 copies of the current hierarchies and couplings exist
   Csr pattern;                // device CSR pattern of the operator (values not kept), for fsi_update_values

@@ -177,3 +177,48 @@ def test_training_step_after_a_failed_allocation(torch_cuda):
         T.close()
     assert failed >= 2
     S.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_build_after_a_failed_allocation(precision, torch_cuda):
+    """A build that runs out of memory, at whatever point, says so; the same call with memory builds what a
+    context that never failed has."""
+    torch = torch_cuda
+    import paper_1801_05648_gb300 as P
+    pb = fsigen.get_problem(fsigen.CONFIGS["2d_tiny"].with_(name="b", n=(128, 96)))
+    U = pb.seeded_state(0, 5e-3)
+    vals = torch.tensor(pb.jacobian(U, U), device="cuda")
+    r = torch.tensor(np.random.default_rng(2).standard_normal(pb.n), device="cuda")
+
+    def context():
+        S = P.FSISolver(pb.dim, pb.rowptr, pb.colind, None, pb.offsets, pb.solid_node_coords(), P.default_params(2))
+        S.update_values(vals)
+        return S
+
+    def applied(S):
+        z = torch.empty_like(r)
+        S.apply_block("precond", r, z)
+        return z
+    S = context()
+    S.precond_build(precision)
+    want = applied(S)
+    S.close()
+    failed = 0
+    for mb in (0, 40, 80, 120, 160, 200, 240, 280, 320, 400, 480):
+        S = context()
+        with _memory_left(torch, mb << 20):
+            try:
+                S.precond_build(precision)
+            except P.FSIError as e:
+                assert e.code == P.FSI_ENOMEM, e
+                failed += 1
+            else:
+                S.close()
+                break
+        S.precond_build(precision)
+        assert torch.equal(applied(S), want)
+        S.update_values(vals)
+        S.precond_build(precision)
+        assert torch.equal(applied(S), want)
+        S.close()
+    assert failed >= 3
