@@ -686,6 +686,10 @@ void extract_bsr(const CsrView& A, int64_t r0, int nbr, int br, int64_t c0, int 
     finalize_rowptr(cnt.p, out, s);
     alloc_values(out);
   }
+  // copies of the old values go: what is decided from a block's bytes must not depend on an earlier build
+  out.v32.release();
+  out.cd16.release();
+  out.stage_rows = out.stage_max = 0;
   if (nbr > 0) {
     k_extract<true><<<grid, 128, 0, s>>>(A.rowptr, A.colind, A.vals, r0, nbr, br, c0, c1, bc, nullptr, out.rowptr.p,
                                          out.colind.p, out.v64.p);

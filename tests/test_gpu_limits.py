@@ -222,3 +222,23 @@ def test_build_after_a_failed_allocation(precision, torch_cuda):
         assert torch.equal(applied(S), want)
         S.close()
     assert failed >= 3
+
+
+# meshes where the FP32 restriction's form changes with 2 bytes more or less per block of level 0
+@pytest.mark.parametrize("cells", [(32, 30), (30, 30), (48, 31)])
+def test_rebuild_equals_a_fresh_context(cells, torch_cuda):
+    """A second FP32 build of the same values has the bits of the first."""
+    torch = torch_cuda
+    import paper_1801_05648_gb300 as P
+    pb = fsigen.get_problem(fsigen.FSIConfig("c", 2, cells))
+    U = pb.seeded_state(0, 5e-3)
+    vals = torch.tensor(pb.jacobian(U, U), device="cuda")
+    r = torch.tensor(np.random.default_rng(2).standard_normal(pb.n), device="cuda")
+    S = P.FSISolver(pb.dim, pb.rowptr, pb.colind, None, pb.offsets, pb.solid_node_coords(), P.default_params(2))
+    z = [torch.empty_like(r) for _ in range(3)]
+    for k in range(3):
+        S.update_values(vals)
+        S.precond_build("fp32")
+        S.apply_block("precond", r, z[k])
+    assert torch.equal(z[0], z[1]) and torch.equal(z[0], z[2])
+    S.close()
