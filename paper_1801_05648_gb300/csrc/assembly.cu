@@ -1199,7 +1199,7 @@ void for_colours(const Assembler& A, F&& f) {
 template <int D, int PD>
 void run_residual(Assembler& A, const double* U, const double* Uold, double* out) {
   constexpr size_t sm = sizeof(ResSmem<D, PD>);
-  static std::atomic<unsigned long long> attr{0};
+  static OncePerDevice attr;
   once_per_device(attr, [](int) {
     FSI_CUDA(cudaFuncSetAttribute(k_residual<D, PD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   });
@@ -1213,7 +1213,7 @@ template <int D, int PD>
 void run_jacobian(Assembler& A, const double* U, const double* Uold, double* vals) {
   constexpr size_t sm = sizeof(JacSmem<D, PD>);
   static_assert(sm <= 227 * 1024, "Jacobian tables exceed the shared memory of a CTA");
-  static std::atomic<unsigned long long> attr{0};
+  static OncePerDevice attr;
   once_per_device(attr, [](int) {
     FSI_CUDA(cudaFuncSetAttribute(k_jacobian<D, PD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   });

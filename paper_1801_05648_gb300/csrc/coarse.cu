@@ -333,7 +333,7 @@ void launch(const CoarseRun<T>& run, const T* b0, T* x0, cudaStream_t s) {
 template <class T>
 int choose_grid() {
   static std::atomic<int> cached[64];
-  static std::atomic<unsigned long long> done{0};
+  static OncePerDevice done;
   once_per_device(done, [](int dev) {
     int nsm = 0, per_sm = 0, coop = 0;
     FSI_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -355,7 +355,7 @@ int find_cluster();
 template <class T>
 int choose_cluster() {
   static std::atomic<int> cached[64];
-  static std::atomic<unsigned long long> done{0};
+  static OncePerDevice done;
   once_per_device(done, [](int dev) { cached[dev].store(find_cluster<T>(), std::memory_order_relaxed); });
   int dev = 0;
   FSI_CUDA(cudaGetDevice(&dev));

@@ -4,6 +4,7 @@
 #include "error.cuh"
 #include "mempool.cuh"
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <atomic>
 #include <cstdint>
@@ -120,20 +121,50 @@ struct DeviceGuard {
   DeviceGuard& operator=(const DeviceGuard&) = delete;
 };
 
-// Runs setup(dev) once per device dev, on the current one: a kernel's function attributes
-// and a __device__ variable's address belong to the copy of the module that each
-// device loads, so what was set up on one device does not hold on another.  `done`
-// is the call site's set of devices already set up (bit d for device d).  Two
-// threads may both run it for the same device; it must be idempotent.
+// A number of the current CUDA context that no other one of this process has or had: a device that was reset
+// gets another.  (0 where the driver does not tell.)
+inline unsigned long long cuda_context_id() {
+  using GetCurrent = CUresult (*)(CUcontext*);
+  using GetId = CUresult (*)(CUcontext, unsigned long long*);
+  struct Entry {
+    void* current = nullptr;
+    void* id = nullptr;
+    Entry() {
+      cudaDriverEntryPointQueryResult r;
+      if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &current, 12000, cudaEnableDefault, &r) != cudaSuccess ||
+          cudaGetDriverEntryPointByVersion("cuCtxGetId", &id, 12000, cudaEnableDefault, &r) != cudaSuccess)
+        current = nullptr;
+      cudaGetLastError();
+    }
+  };
+  static const Entry e;
+  if (!e.current || !e.id) return 0;
+  CUcontext c = nullptr;
+  unsigned long long v = 0;
+  if (reinterpret_cast<GetCurrent>(e.current)(&c) != CUDA_SUCCESS || !c) {
+    FSI_CUDA(cudaFree(nullptr));   // makes the device's context, where this thread has none yet
+    if (reinterpret_cast<GetCurrent>(e.current)(&c) != CUDA_SUCCESS || !c) return 0;
+  }
+  return reinterpret_cast<GetId>(e.id)(c, &v) == CUDA_SUCCESS ? v : 0;
+}
+
+// Runs setup(dev) once per device dev, on the current one, and again after the device was reset: a
+// kernel's function attributes, a __device__ variable's address and a stream belong to one CUDA
+// context of one device, so what was set up in one does not hold in another.  `done` is the call
+// site's record: the context that each device was set up in.  Two threads may both run it for the
+// same device; it must be idempotent.
+struct OncePerDevice {
+  std::atomic<unsigned long long> context[64] = {};   // cuda_context_id() + 1, 0: not yet
+};
 template <class F>
-void once_per_device(std::atomic<unsigned long long>& done, F&& setup) {
+void once_per_device(OncePerDevice& done, F&& setup) {
   int dev = 0;
   FSI_CUDA(cudaGetDevice(&dev));
   require(dev >= 0 && dev < 64, "device ordinal above 63");
-  const unsigned long long bit = 1ull << dev;
-  if (done.load(std::memory_order_acquire) & bit) return;
+  const unsigned long long now = cuda_context_id() + 1;
+  if (done.context[dev].load(std::memory_order_acquire) == now) return;
   setup(dev);
-  done.fetch_or(bit, std::memory_order_release);
+  done.context[dev].store(now, std::memory_order_release);
 }
 
 // Block sparse row matrix on the device: nbr x nbc blocks of br x bc values,

@@ -286,7 +286,7 @@ cudaLaunchConfig_t panel_config(int n, int cs, cudaLaunchAttribute* attr, cudaSt
 // 8 is opt-in), else 8.  n <= 8192 needs 143 KB of shared memory in a 16-CTA cluster.
 int panel_cluster(int n) {
   constexpr int kMaxN16 = 8192;
-  static std::atomic<unsigned long long> done{0};
+  static OncePerDevice done;
   static std::atomic<int> big[64];
   once_per_device(done, [](int dev) {
     FSI_CUDA(cudaFuncSetAttribute(k_gj_panel, cudaFuncAttributeMaxDynamicSharedMemorySize,

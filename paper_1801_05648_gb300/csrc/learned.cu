@@ -353,7 +353,7 @@ template <int D, int MODE>
 void launch_mlp(const MlpGeom& g, const uint16_t* w16, const double* rp, double* c, float* F, float* rho,
                 float* G1, float* D1, float* G2, float* D2, int64_t ld, cudaStream_t s) {
   constexpr size_t smem = mlp_smem<D, MODE>();
-  static std::atomic<unsigned long long> attr{0};   // the opt-in above 48 KB, per instantiation and device
+  static OncePerDevice attr;   // the opt-in above 48 KB, per instantiation and device
   once_per_device(attr, [](int) {
     FSI_CUDA(cudaFuncSetAttribute(k_mlp<D, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   });

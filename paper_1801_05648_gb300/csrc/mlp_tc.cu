@@ -335,7 +335,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_mlp_tc(MlpGeom g, const uint1
 
 void mlp_apply_tc(const MlpGeom& g, const uint16_t* w16, const double* rp, double* c, int* err, cudaStream_t s) {
   require(g.dim == 2, "the tensor-core MLP takes the 2D layout (3x3 patch, 53 inputs)");
-  static std::atomic<unsigned long long> attr{0};   // the opt-in above 48 KB, per device
+  static OncePerDevice attr;   // the opt-in above 48 KB, per device
   once_per_device(attr, [](int) {
     FSI_CUDA(cudaFuncSetAttribute(k_mlp_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem));
   });

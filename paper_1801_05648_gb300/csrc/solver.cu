@@ -564,12 +564,13 @@ void context_update_values(Context& C, const double* vals_dev) {
   FSI_CUDA(cudaStreamSynchronize(C.s));
 }
 
-// The four streams of the hierarchies' set-ups on the current device, shared by its contexts
+// The four streams of the hierarchies' set-ups on the current device, shared by its contexts and made
+// again after a device reset
 // (work of several contexts on one of them only waits its turn).  Four more streams per
 // context slowed the launches of small captured solves by 6%: the device multiplexes
 // streams onto few connections.
 cudaStream_t branch_stream(int h) {
-  static std::atomic<unsigned long long> done{0};
+  static OncePerDevice done;
   static std::atomic<cudaStream_t> streams[64][4];
   static std::mutex making;
   std::lock_guard<std::mutex> g(making);

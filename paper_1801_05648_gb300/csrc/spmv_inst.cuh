@@ -26,7 +26,7 @@ __device__ int g_stage_err = 0;
 // The flag's device address on the current device (looked up once per device).
 int* stage_err_ptr() {
   static std::atomic<int*> addr[64];
-  static std::atomic<unsigned long long> done{0};
+  static OncePerDevice done;
   once_per_device(done, [](int dev) {
     int* a = nullptr;
     FSI_CUDA(cudaGetSymbolAddress((void**)&a, g_stage_err));
@@ -50,7 +50,7 @@ inline int staged_grid(int nchunks, int smax) {
 template <class Epi, class G1, int UREQ>
 void launch_staged(const Bsr& A1, const G1& g1, const Epi& epi, int tpr, int rows_per_cta, int nchunks, int grid,
                    int dep, cudaStream_t s) {
-  static std::atomic<unsigned long long> attr{0};   // the opt-in above 48 KB, per instantiation and device
+  static OncePerDevice attr;   // the opt-in above 48 KB, per instantiation and device
   once_per_device(attr, [](int) {
     FSI_CUDA(cudaFuncSetAttribute(k_bsr_cheb_staged<Epi, G1, UREQ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   kStageSmemMax));

@@ -1,6 +1,10 @@
 """Calls at the edges of what the solver takes: product rows around the length of the SpGEMM
-table, aggregates larger than shared memory, empty classes of unknowns, too little device memory."""
+table, aggregates larger than shared memory, empty classes of unknowns, too little device
+memory, a device that was reset."""
 import contextlib
+import os
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -242,3 +246,100 @@ def test_rebuild_equals_a_fresh_context(cells, torch_cuda):
         S.apply_block("precond", r, z[k])
     assert torch.equal(z[0], z[1]) and torch.equal(z[0], z[2])
     S.close()
+
+
+# Everything a Newton correction calls, on the library alone (a process's PyTorch does not outlive a reset).
+_RESET = r"""
+import ctypes
+import numpy as np
+import fsigen
+import paper_1801_05648_gb300.fsi as F
+
+lib = F.load_library()
+cudart = ctypes.CDLL("libcudart.so.13")
+cudart.cudaMalloc.argtypes = [ctypes.POINTER(ctypes.c_void_p), ctypes.c_size_t]
+cudart.cudaMemcpy.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_size_t, ctypes.c_int]
+pb = fsigen.get_problem(fsigen.FSIConfig("c", 2, (64, 48)))
+U = pb.seeded_state(0, 5e-3)
+rng = np.random.default_rng(0)
+b = rng.standard_normal(pb.n)
+bits = (rng.standard_normal(F.mlp_params(2)).astype(np.float32) * 0.1).view(np.uint32) >> 16
+bits = np.ascontiguousarray(bits, np.uint16)
+
+
+def ok(rc):
+    assert rc == 0, rc
+
+
+def dev(a):
+    p = ctypes.c_void_p()
+    ok(cudart.cudaMalloc(ctypes.byref(p), a.nbytes))
+    ok(cudart.cudaMemcpy(p, a.ctypes.data, a.nbytes, 1))
+    return p
+
+
+def host(p, n):
+    a = np.empty(n)
+    ok(cudart.cudaDeviceSynchronize())
+    ok(cudart.cudaMemcpy(a.ctypes.data, p, a.nbytes, 2))
+    return a
+
+
+def ptr(a, t):
+    return a.ctypes.data_as(ctypes.POINTER(t))
+
+
+def correction():
+    cd, cf = pb.cell_map()
+    cfg, m = pb.cfg, F.AsmMesh()
+    arrays = [np.ascontiguousarray(cd, np.int32), np.ascontiguousarray(cf, np.uint32),
+              np.ascontiguousarray(pb.rowptr, np.int64), np.ascontiguousarray(pb.colind, np.int32),
+              np.ascontiguousarray(pb.fixed, np.uint8), np.ascontiguousarray(pb.offsets, np.int64)]
+    m.dim, m.pressure, m.n = 2, 0, pb.n
+    for d in range(3):
+        m.cells[d], m.h[d] = (cfg.n[d], cfg.L[d] / cfg.n[d]) if d < 2 else (1, 1.0)
+    m.cell_dof, m.cell_flags = ptr(arrays[0], ctypes.c_int32), ptr(arrays[1], ctypes.c_uint32)
+    m.rowptr, m.colind, m.row_fixed = ptr(arrays[2], ctypes.c_int64), ptr(arrays[3], ctypes.c_int32), ptr(arrays[4], ctypes.c_uint8)
+    ph = F.AsmPhysics(**{k: float(getattr(cfg, k)) for k in ("rho_f", "nu_f", "mu_s", "lambda_s", "rho_s", "dt", "theta")})
+    asm, ctx = ctypes.c_void_p(), ctypes.c_void_p()
+    u, vals, r, z, x = dev(U), dev(np.zeros(pb.nnz)), dev(b), dev(np.zeros(pb.n)), dev(np.zeros(pb.n))
+    ok(lib.fsi_asm_create(ctypes.byref(asm), ctypes.byref(m), ctypes.byref(ph), None))
+    ok(lib.fsi_asm_residual(asm, u, u, z, None, None))
+    out = [host(z, pb.n)]
+    ok(lib.fsi_asm_jacobian(asm, u, u, vals, None))
+    prm = F.default_params(2)
+    prm.flags = F.FSI_USE_GRAPHS
+    ok(lib.fsi_setup(ctypes.byref(ctx), 2, pb.n, ptr(arrays[2], ctypes.c_int64), ptr(arrays[3], ctypes.c_int32), None,
+                     ptr(arrays[5], ctypes.c_int64), None, ctypes.byref(prm), None))
+    ok(lib.fsi_update_values(ctx, vals))
+    ok(lib.fsi_precond_build(ctx, 1, None))
+    ok(lib.fsi_apply_block(ctx, 7, r, z))
+    out.append(host(z, pb.n))
+    st = F.Stats()
+    ok(lib.fsi_solve(ctx, r, x, 1e-8, ctypes.byref(st)))
+    out.append(host(x, pb.n))
+    nd, pt = (np.ascontiguousarray(a, np.int32) for a in pb.node_map())
+    one = np.ones(5, np.float32)
+    ok(lib.fsi_learned_setup(ctx, len(nd), ptr(nd, ctypes.c_int32), ptr(pt, ctypes.c_int32)))
+    ok(lib.fsi_learned_set_weights(ctx, ptr(one, ctypes.c_float), ptr(one, ctypes.c_float), ptr(bits, ctypes.c_uint16)))
+    ok(lib.fsi_learned_apply(ctx, r, z))
+    out.append(host(z, pb.n))
+    lib.fsi_free(ctx)
+    lib.fsi_asm_free(asm)
+    return out
+
+
+first = correction()
+ok(cudart.cudaDeviceReset())
+second = correction()
+assert all(np.array_equal(a, c) and np.abs(a).max() > 0 for a, c in zip(first, second))
+print("same")
+"""
+
+
+def test_contexts_after_a_device_reset(torch_cuda):
+    """What is set up once per device (streams, kernels' attributes) is set up again for contexts made after a
+    reset of the device: same bits."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _RESET], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "same" in r.stdout, r.stdout[-2000:] + r.stderr[-4000:]
