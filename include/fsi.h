@@ -207,6 +207,13 @@ int fsi_setup(fsi_ctx** out, int dim, int64_t n, const int64_t* rowptr, const in
  *               built once).
  *   learned_weights  nullable: path of a weights file for the learned stage
  *               (as fsi_learned_load; needs fsi_learned_setup first).
+ * A call that fails (FSI_ENOMEM, say) may be repeated.
+ * Device memory: what fsi_setup, fsi_update_values and fsi_precond_build allocate
+ * for a while is kept with the context for the next such call: at most 1 GiB of
+ * released blocks, and at most 256 MiB of slabs that its arrays of up to 1 MiB are
+ * cut from.  fsi_free returns all of it; the blocks are also given up when an
+ * allocation of this library, for any context, finds too little memory (another
+ * allocator of the process cannot ask for them).
  */
 int fsi_precond_build(fsi_ctx* ctx, int precision, const char* learned_weights);
 

@@ -504,8 +504,21 @@ static void extract_blocks(Context& C, const CsrView& A, bool keep) {
   extract_bsr(A, o[4], nP, 1, o[4], nP, 1, C.Cpp, keep, s);
 }
 
+// The end of a set-up call: the pools go back to their bound.
+namespace {
+struct Settled {
+  Context& C;
+  ~Settled() {
+    C.pool->settle();
+    for (SetupBranch& b : C.branch)
+      if (b.pool) b.pool->settle();
+  }
+};
+}  // namespace
+
 void context_setup(Context& C, const int64_t* rowptr, const int32_t* colind, const double* vals,
                    const double* solid_coords) {
+  Settled settled{C};
   SetupPhase setup_phase(C.pool);
   auto t0 = clk::now();
   FSI_CUDA(cudaGetDevice(&C.device));
@@ -552,6 +565,7 @@ static void take_blocks_back(Context& C) {
 }
 
 void context_update_values(Context& C, const double* vals_dev) {
+  Settled settled{C};
   SetupPhase setup_phase(C.pool);
   CsrView v = C.pattern.view();
   v.vals = vals_dev;
@@ -710,6 +724,7 @@ static void build_parts(Context& C, bool first, bool demote, bool (&done)[5]) {
 }
 
 void precond_build(Context& C, int precision) {
+  Settled settled{C};
   SetupPhase setup_phase(C.pool);
   auto t0 = clk::now();
   auto& s = C.s;

@@ -84,9 +84,67 @@ void give_up() {
   EXPECT(thrown && !d.p && d.n == 0 && cudaGetLastError() == cudaSuccess);
 }
 
+void bounds() {
+  // a context's five pools together keep a limited amount, whichever of them it came from
+  capacity = 100000 * MB;
+  auto slabs = std::make_shared<Slabs>();
+  std::vector<std::shared_ptr<MemPool>> pools;
+  for (int i = 0; i < 5; ++i) pools.push_back(std::make_shared<MemPool>(slabs));
+  for (int round = 0; round < 2; ++round) {
+    std::vector<std::pair<void*, size_t>> b;
+    for (auto& p : pools)
+      for (int k = 0; k < 3; ++k) {
+        size_t got = 0;
+        void* x = p->take(200 * MB, got);
+        b.emplace_back(x, got);
+      }
+    EXPECT(used >= 3000 * MB);
+    for (size_t k = 0; k < b.size(); ++k) pools[k / 3]->give(b[k].first, b[k].second);
+    for (auto& p : pools) p->settle();
+    EXPECT(used > 0 && used <= 1024 * MB);
+  }
+  for (auto& p : pools) p->trim();
+  EXPECT(used == 0);
+  // small blocks: slabs up to a limit, then blocks of their own, all apart from each other and used again
+  constexpr size_t kBlocks = 600, kBytes = 900 * 1024;
+  for (int round = 0; round < 2; ++round) {
+    std::map<uintptr_t, size_t> at;
+    std::vector<std::pair<void*, size_t>> b;
+    for (size_t k = 0; k < kBlocks; ++k) {
+      size_t got = 0;
+      void* x = pools[k % 5]->take(kBytes, got);
+      EXPECT(got >= kBytes);
+      auto next = at.lower_bound((uintptr_t)x);
+      EXPECT(next == at.end() || (uintptr_t)x + kBytes <= next->first);
+      EXPECT(next == at.begin() || std::prev(next)->first + kBytes <= (uintptr_t)x);
+      at[(uintptr_t)x] = got;
+      b.emplace_back(x, got);
+    }
+    EXPECT(used <= 8 * 32 * MB + kBlocks * 2 * MB);
+    for (size_t k = 0; k < kBlocks; ++k) pools[k % 5]->give(b[k].first, b[k].second);
+  }
+  for (auto& p : pools) p->trim();
+  EXPECT(used <= 8 * 32 * MB);
+}
+
+void slab_under_pressure() {
+  // a slab that does not fit beside what its own context's pools hold
+  capacity = 100 * MB;
+  auto slabs = std::make_shared<Slabs>();
+  MemPool a(slabs);
+  size_t got = 0, small = 0;
+  void* big = a.take(90 * MB, got);
+  a.give(big, got);
+  void* x = a.take(1024, small);
+  EXPECT(x && small == 1024 && used == 32 * MB);
+  a.give(x, small);
+}
+
 int main(int argc, char** argv) {
   const std::string what = argc > 1 ? argv[1] : "";
   if (what == "give_up") give_up();
+  else if (what == "bounds") bounds();
+  else if (what == "slab_under_pressure") slab_under_pressure();
   else return 2;
   EXPECT(used == 0 && blocks.empty());           // everything came back
   return 0;
@@ -109,7 +167,7 @@ def program(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("what", ["give_up"])
+@pytest.mark.parametrize("what", ["give_up", "bounds", "slab_under_pressure"])
 def test_pool(what, program):
     r = subprocess.run([program, what], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr
