@@ -749,6 +749,10 @@ void precond_build(Context& C, int precision) {
     }
     C.built = true;
     if (demote) C.fp32_ready = true;
+    if (first) {   // S_hat and S_p hold what they went into; their patterns stay for the next values
+      C.Avv.v64.release();
+      C.Cpp.v64.release();
+    }
   }
   C.precision = precision;
   if (C.iter_graph) { cudaGraphExecDestroy(C.iter_graph); C.iter_graph = nullptr; }

@@ -89,7 +89,7 @@ struct Context {
   bool csf_u_zero = false;    // the s_u rows of C_sv_f and C_sv_p hold no entries
   Bsr C_fv_ms, C_p_ms;        // f_v rows x (m, s) cols, p rows x (m, s) cols
   Bsr B_vp, B_pv;             // fluid velocity-pressure couplings
-  Bsr Mblk, Avv, Auu, Aff, Cpp;   // diagonal blocks, consumed by precond_build
+  Bsr Mblk, Avv, Auu, Aff, Cpp;   // diagonal blocks, consumed by precond_build (Avv and Cpp keep their patterns)
   Hierarchy H[4];             // M, S_hat, A_ff, S_p
   ChebSolver mass;            // A_uu (solid mass)
   bool built = false;

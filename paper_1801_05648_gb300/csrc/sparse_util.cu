@@ -672,8 +672,7 @@ void extract_bsr(const CsrView& A, int64_t r0, int nbr, int br, int64_t c0, int 
   require(br <= 6, "extract_bsr: block rows > 6");
   const int64_t c1 = c0 + (int64_t)nbc * bc;
   const int grid = div_up((int64_t)nbr * 32, 128);
-  keep = keep && out.rowptr.p && out.colind.p && out.v64.p && out.nbr == nbr && out.nbc == nbc && out.br == br &&
-         out.bc == bc;
+  keep = keep && out.rowptr.p && out.colind.p && out.nbr == nbr && out.nbc == nbc && out.br == br && out.bc == bc;
   if (!keep) {
     out = Bsr();
     out.nbr = nbr; out.nbc = nbc; out.br = br; out.bc = bc;
@@ -684,8 +683,8 @@ void extract_bsr(const CsrView& A, int64_t r0, int nbr, int br, int64_t c0, int 
       FSI_CHECK_LAUNCH();
     }
     finalize_rowptr(cnt.p, out, s);
-    alloc_values(out);
   }
+  if (!out.v64.p) alloc_values(out);
   // copies of the old values go: what is decided from a block's bytes must not depend on an earlier build
   out.v32.release();
   out.cd16.release();

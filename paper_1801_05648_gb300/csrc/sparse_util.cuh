@@ -29,8 +29,8 @@ int64_t exclusive_scan(const int* in, int* out, int64_t n, cudaStream_t s);
 
 // BSR block of the monolithic CSR: scalar rows [r0, r0 + nbr*br), scalar columns
 // [c0, c0 + nbc*bc), blocks br x bc (column index (c - c0) / bc).  keep: out may hold this
-// block of a matrix with the same CSR pattern; its row pointers then stand (no counting, no
-// scan, no wait), and only the blocks are written.
+// block of a matrix with the same CSR pattern, with or without values; its row pointers then stand (no
+// counting, no scan, no wait), and only the blocks are written.
 void extract_bsr(const CsrView& A, int64_t r0, int nbr, int br, int64_t c0, int nbc, int bc, Bsr& out, bool keep,
                  cudaStream_t s);
 

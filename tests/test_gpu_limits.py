@@ -248,6 +248,34 @@ def test_rebuild_equals_a_fresh_context(cells, torch_cuda):
     S.close()
 
 
+def test_a_build_releases_the_blocks_it_used_up(torch_cuda):
+    """After a build the solid's velocity block lives on in S_hat alone: new values take its memory again
+    (memory is compared with the pools emptied, which a failed allocation does)."""
+    torch = torch_cuda
+    import paper_1801_05648_gb300 as P
+    pb = fsigen.get_problem(fsigen.CONFIGS["2d_tiny"].with_(name="b", n=(256, 128)))
+    U = pb.seeded_state(0, 5e-3)
+    vals = torch.tensor(pb.jacobian(U, U), device="cuda")
+    S = P.FSISolver(pb.dim, pb.rowptr, pb.colind, None, pb.offsets, pb.solid_node_coords(), P.default_params(2))
+
+    def free():
+        with _memory_left(torch, 1 << 20):
+            with contextlib.suppress(P.FSIError):
+                P.FSIAssembler.from_problem(pb).close()
+        return torch.cuda.mem_get_info()[0]
+    o = pb.offsets
+    rows = slice(int(pb.rowptr[o[1]]), int(pb.rowptr[o[2]]))
+    cols = pb.colind[rows]
+    avv = 8 * int(((cols >= o[1]) & (cols < o[2])).sum())
+    assert avv > 8 << 20
+    S.update_values(vals)
+    S.precond_build("fp64")
+    built = free()
+    S.update_values(vals)
+    assert built - free() >= avv - (4 << 20)                # whole driver pages of 2 MB
+    S.close()
+
+
 # Everything a Newton correction calls, on the library alone (a process's PyTorch does not outlive a reset).
 _RESET = r"""
 import ctypes
