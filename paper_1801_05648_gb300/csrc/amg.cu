@@ -497,6 +497,8 @@ double Hierarchy::vcycle_bytes(int vb) const {
 void amg_setup(Hierarchy& H, Bsr&& A0, const double* B0, int k0, const AmgParams& prm, cudaStream_t s) {
   require(A0.br == A0.bc && A0.nbr == A0.nbc, "amg_setup: square matrix with square blocks required");
   H.levels.clear();
+  H.crun64 = CoarseRun<double>();   // the plans point into the levels
+  H.crun32 = CoarseRun<float>();
   H.prm = prm;
   if (A0.nbr == 0) {   // empty block (e.g. no solid): a single empty level, nothing to solve
     H.levels.emplace_back();

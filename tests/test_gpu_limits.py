@@ -1,6 +1,6 @@
 """Calls at the edges of what the solver takes: product rows around the length of the SpGEMM
 table, aggregates larger than shared memory, empty classes of unknowns, too little device
-memory, a device that was reset."""
+memory, a hierarchy that changes its shape, a device that was reset."""
 import contextlib
 import os
 import subprocess
@@ -273,6 +273,43 @@ def test_a_build_releases_the_blocks_it_used_up(torch_cuda):
     built = free()
     S.update_values(vals)
     assert built - free() >= avv - (4 << 20)                # whole driver pages of 2 MB
+    S.close()
+
+
+def _anisotropic_grid(n, wy):
+    """Five-point operator on n x n nodes, coupling -1 in x and -wy in y, two components."""
+    T = sp.diags([-np.ones(n - 1), -np.ones(n - 1)], [-1, 1])
+    K = sp.kron(sp.identity(n), T) + wy * sp.kron(T, sp.identity(n))
+    K = K + sp.diags(np.asarray(-K.sum(1)).ravel() + 0.1)
+    return sp.kron(K, sp.identity(2)).tocsr()
+
+
+@pytest.mark.parametrize("flag", ["FSI_GRID_COARSE", "FSI_CLUSTER_COARSE"])
+def test_coarse_launch_follows_the_hierarchy(flag, torch_cuda):
+    """Values whose first coarse level is small enough for the single coarse launch, then values whose is not
+    (coarsened along x alone), then the first again: each build as the oracle's V-cycle."""
+    torch = torch_cuda
+    import paper_1801_05648_gb300 as P
+    from oracle import amg
+    values = [_anisotropic_grid(40, w) for w in (1.0, 1e-4)]
+    assert np.array_equal(values[0].indices, values[1].indices)
+    H = [amg.sa_setup(M, 2, amg.translations(1600, 2), amg.AMGParams(coarse_max=300)) for M in values]
+    limit = 1e5                                             # bytes of a level's FP64 values
+    size = [[sp.bsr_matrix(h.levels[k].A, blocksize=(2, 2)).indices.size * 32 for h in H] for k in (0, 1)]
+    assert [len(h.levels) for h in H] == [3, 3] and size[1][0] < limit < size[1][1] < size[0][0]
+    A, off = _system(m_m=values[0])
+    S = _context(A, off, coarse_max=300, cluster_max_bytes=limit, flags=getattr(P, flag))
+    b = np.random.default_rng(0).standard_normal(3200)
+    x = torch.empty(3200, dtype=torch.float64, device="cuda")
+    for k in (0, 1, 0):
+        data = A.copy()
+        data.data[: values[k].nnz] = values[k].data
+        S.update_values(torch.tensor(data.data, device="cuda"))
+        S.precond_build("fp64")
+        S.apply_block("mesh", torch.tensor(b, device="cuda"), x)
+        want = amg.vcycle(H[k], b)
+        assert np.linalg.norm(x.cpu().numpy() - want) <= 1e-10 * np.linalg.norm(want)
+    S.check_device_errors()
     S.close()
 
 
