@@ -19,7 +19,7 @@ void launch_operator(const Bsr& AVV, const Bsr& AVP, const Bsr& APV, const Bsr& 
   int cv = 0, cp = 0;
   const RowClass V = row_class(AVV, AVP, &cv), P = row_class(APV, APP, &cp);
   const bool built = tu.setup_depth == 0;
-  const bool early = built && cv + cp <= kEarlyCtas64 * device_sms();
+  const bool early = built && loads_early(cv + cp, V.rows_per_cta, V.tpr, kEarlyCtas64);
   launch_k(early ? k_operator_rows<D, Epi, true> : k_operator_rows<D, Epi, false>, cv + cp, 256, 0, s, V, P, cp,
            tu.prefetch > 0 ? kPrefetchCap : 0, built ? kDepBuilt : 0, x, x + AVV.rows(), ev, ep);
 }

@@ -71,11 +71,17 @@ inline int widened(const Bsr& A, int tpr) {
   return tpr;
 }
 
-// Loads before the wait for launches of up to this many CTAs per SM, which wait on latency.
+// Loads before the wait for launches of up to this many CTAs per SM, one pass each, which wait on latency.
 // FP32: 256x128 solve 8.85 / 8.71 / 8.61 / 8.62 ms with 4 / 8 / 16 / 32 (9.2 without), but
 // 1024x512 256 -> 282 ms when every launch does it; FP64: 64x32 outer operator 2.00 -> 1.96 ms of
 // solve with 1, nothing more with 4.
 constexpr int kEarlyCtas = 8, kEarlyCtas64 = 1;
+// Persistent CTAs (spmv_prefetch 2) walk several passes and are few however large the matrix: they neither load
+// early (512x256 level-0 step 29 us, 36.5 with the registers that it costs) nor trigger (256x128 9.0 us, 10.0).
+inline bool one_pass(int rows_per_cta, int tpr) { return rows_per_cta * tpr <= 256; }
+inline bool loads_early(int ctas, int rows_per_cta, int tpr, int per_sm) {
+  return ctas <= per_sm * device_sms() && one_pass(rows_per_cta, tpr);
+}
 
 // 256-thread CTAs over the block rows with tpr lanes each: {CTAs, block rows per CTA}.
 inline std::pair<int, int> cta_split(const Bsr& A, int tpr) {
@@ -111,9 +117,10 @@ void launch_g(const Bsr& A1, const G1& g1, const Bsr* A2, const T* x2, const Epi
   int64_t nnzb2 = 0;
   if (A2) { v2 = A2->vals<T>(); rp2 = A2->rowptr.p; ci2 = A2->colind.p; nnzb2 = A2->nnzb; }
   constexpr int per_sm = sizeof(T) == 4 ? kEarlyCtas : kEarlyCtas64;
-  const bool early = tu.setup_depth == 0 && blocks <= per_sm * device_sms();
+  const bool early = tu.setup_depth == 0 && loads_early(blocks, rows_per_cta, tpr, per_sm);
   // FP64 launches do not trigger, see common.cuh (21x11x10 FP64 solve 14.7 ms without, 16.4 with)
-  const int dep = (tu.setup_depth == 0 ? kDepBuilt : 0) | (sizeof(T) == 4 ? kDepTrigger : 0);
+  const int dep = (tu.setup_depth == 0 ? kDepBuilt : 0) |
+                  (sizeof(T) == 4 && one_pass(rows_per_cta, tpr) ? kDepTrigger : 0);
   const int pf = tu.prefetch > 0 ? kPrefetchCap : 0;
   const int4* ord2 = BC2 > 0 && A2 ? pair_order(A1, *A2) : nullptr;
   if constexpr (ALLOW16 && sizeof(T) == 4 && BC2 == 0) {

@@ -74,3 +74,25 @@ def test_overlapping_kernels_read_vectors_with_ordinary_loads():
             assert "ld.global.nc" not in _source(name), name
     for name in ("vec.cu", "solver.cu", "mlp_tc.cu", "amg.cu"):
         assert "__ldg" not in _source(name), name
+
+
+def _function(text, name):
+    """The body of the function whose definition names `name(`."""
+    start = text.index("{", text.index(name + "("))
+    depth, i = 1, start + 1
+    while depth:
+        depth += {"{": 1, "}": -1}.get(text[i], 0)
+        i += 1
+    return text[start:i]
+
+
+def test_persistent_launches_neither_load_early_nor_trigger():
+    """The registers of the early loads cost a launch that fills the GPU its occupancy; a persistent one
+    (more rows per CTA than threads allow in a pass) fills it although its CTAs are few."""
+    text = _source("spmv_inst.cuh")
+    assert "rows_per_cta * tpr <= 256" in _function(text, "bool one_pass")
+    assert "one_pass(rows_per_cta, tpr)" in _function(text, "bool loads_early")
+    assert re.search(r"one_pass\(rows_per_cta, tpr\) \? kDepTrigger : 0", text)
+    for name, source in (("spmv_inst.cuh", text), ("spmv64.cu", _source("spmv64.cu"))):
+        decided = re.findall(r"const bool early = ([^;]*);", source)
+        assert decided and all("loads_early(" in d for d in decided), name
