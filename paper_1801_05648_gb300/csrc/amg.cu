@@ -481,7 +481,8 @@ double Hierarchy::vcycle_bytes(int vb) const {
   const int nl = (int)levels.size();
   for (int l = 0; l + 1 < nl; ++l) {
     const AmgLevel& L = levels[l];
-    // smoother SpMVs (the first two steps from zero share one pass), the restricted
+    // smoother SpMVs (the first step from zero needs none, whether it shares the second's pass or is a
+    // launch of its own, see cheb_sweep), the restricted
     // residual R b + RAn x (one pass over both, one output) and the prolongation
     const int sweeps = prm.presmooth * prm.degree(l) - 1 + prm.postsmooth * prm.degree(l);
     tot += sweeps * L.A.spmv_bytes(vb) + L.P.spmv_bytes(vb);

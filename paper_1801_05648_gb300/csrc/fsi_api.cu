@@ -345,6 +345,7 @@ int fsi_smoother_step(fsi_ctx* ctx, int which, int level, int reps, double* byte
     fsi::Context& C = ctx->C;
     fsi::require(C.built, "fsi_smoother_step before fsi_precond_build");
     fsi::require(which >= 0 && which <= 3 && reps >= 0, "bad arguments");
+    fsi::WideRows64 wide(true);   // as the V-cycle's steps in FP64
     const double b = C.precision == 1 ? fsi::amg_smoother_steps<float>(C.H[which], level, reps, C.s)
                                       : fsi::amg_smoother_steps<double>(C.H[which], level, reps, C.s);
     if (bytes_per_step) *bytes_per_step = b;

@@ -96,3 +96,12 @@ def test_persistent_launches_neither_load_early_nor_trigger():
     for name, source in (("spmv_inst.cuh", text), ("spmv64.cu", _source("spmv64.cu"))):
         decided = re.findall(r"const bool early = ([^;]*);", source)
         assert decided and all("loads_early(" in d for d in decided), name
+
+
+def test_fp64_preconditioner_calls_share_their_launch_shapes():
+    """Every call that runs products of the FP64 preconditioner runs them as the solve does."""
+    solver = _source("solver.cu")
+    for text, name in ((solver, "void precond_apply"), (solver, "void apply_block"),
+                       (_source("noalloc.cu"), "int fsi_mass_solve_noalloc"),
+                       (_source("fsi_api.cu"), "int fsi_smoother_step")):
+        assert "WideRows64 wide(" in _function(text, name), name
