@@ -9,7 +9,8 @@
 // leaves the kNb multipliers of every row, and one launch over the whole GPU
 // (k_gj_update), which applies the panel's swaps and its kNb rank-1 updates to the other
 // columns.  Every entry sees the operations of the column-by-column elimination in the
-// same order with the same rounding (one fused multiply-add per step), so the inverse has the same bits as one launch per pivot gave.
+// same order with the same rounding (one fused multiply-add per step), so the inverse of a matrix whose
+// pivot rows stay finite is the one that a launch per pivot gave, up to the signs of zeros.
 //
 // Why panels: one launch per pivot took 11 us (n = 300) to 40 us (n = 1100) because each
 // read and wrote 2 n^2 entries and ended with one CTA's search for the next pivot.  The
@@ -55,7 +56,8 @@ struct Mail {
 // cyclically and stay in shared memory; one cluster barrier per step (the mailboxes
 // alternate: a CTA writes those of step s + 2 only after every CTA has arrived at step
 // s + 1, that is, has read those of step s).  A step is bound by that barrier and the
-// candidate search, about 1.5 us; the panel's own updates are n kNb FP64 FMAs per step,
+// candidate search: 3.4 us a pivot with the panel's loads and stores (11.2 ms for the 3,315 pivots of
+// a 32x16x16 build); the panel's own updates are n kNb FP64 FMAs per step,
 // which one SM alone could not hide (1.7 FMAs per clock), hence the cluster.
 __global__ void __launch_bounds__(kPanelThreads) k_gj_panel(int n, int P0, int nb, const double* __restrict__ Win,
                                                             double* __restrict__ Wout, double* __restrict__ Lg,

@@ -429,8 +429,8 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_spgemm_sym(int nbr, int
 // remaining entries goes (binary search in the chunk's columns, all lanes on different
 // entries), and then add the B rows one after the other, lanes side by side on (entry,
 // component), several loads ahead of the sums.  Bound by the FP64 pipe (BK FMAs per match
-// and component) as long as an SM holds about eight warps: the chunks are kept small for
-// that, and smaller when there are few rows.  All products of a 32x16x16 preconditioner build:
+// and component) as long as an SM holds enough warps to hide the loads: about 5 KB of sums a warp let 32 of them
+// fit, and chunks are cut smaller where rows x chunks would make fewer than 16.  All products of a 32x16x16 preconditioner build:
 // 24 ms; one lane per C entry searching every B row took 125 ms, whole rows per warp (two
 // CTAs' worth of sums per SM) 66 ms.
 constexpr int kSlots = 256;          // matches placed at a time

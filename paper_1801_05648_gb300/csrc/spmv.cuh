@@ -555,9 +555,10 @@ __global__ void __launch_bounds__(256) k_bsr_spmv(int nbr, int tpr, int rows_per
 // The outer operator's rows: D velocity components of a node (D x D blocks, and D x 1 to the
 // pressures) and pressures (1 x D and 1 x 1), in one launch.  The first ctas_p CTAs take the
 // pressure rows: few, long ones, which as a launch of their own wait on latency (10 us of the
-// 16x16 operator's 22, 14.6 of the 256x128 operator's 96) and here run beside the rest.  x is gathered with the default L2 policy: on the 1024x512 system
-// evict-last gathers cut the DRAM traffic from 7.5 to 6.4 GB but made the product 5% slower (it is
-// bound by the FP64 pipe).
+// 16x16 operator's 22, 14.6 of the 256x128 operator's 96) and here run beside the rest.  That pays on small
+// and mid-size systems; on 1024x512 one launch takes what the two took (1,258 us).  x is gathered with the
+// default L2 policy: on the 1024x512 system evict-last gathers cut the DRAM traffic from 7.5 to 6.4 GB but made
+// the product 5% slower (it is bound by the FP64 pipe).
 struct RowClass {
   int nbr, tpr, rows_per_cta;
   const int4* ord2;

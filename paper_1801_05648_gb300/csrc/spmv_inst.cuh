@@ -63,8 +63,9 @@ void launch_staged(const Bsr& A1, const G1& g1, const Epi& epi, int tpr, int row
 // FP64 launches of the preconditioner (WideRows64): lanes doubled until the launch holds
 // about 16 warps per SM or a lane has a single block of an average row.  The 8 blocks per lane of
 // the FP64 rule save shuffle additions, but leave the levels of small and mid-size systems a
-// few warps per SM walking rows of 64 blocks in dependent trips: the 21x11x10 FP64 solve went
-// from 25.3 to 16.0 ms with this and the epilogues per component.
+// few warps per SM walking rows of 64 blocks in dependent trips: with this, the epilogues per component and
+// the first Chebyshev iterate written first the 21x11x10 FP64 solve went from 25.3 to 16.0 ms (26.1 -> 16.4 and
+// 27.5 -> 17.1 ms on other GPUs).
 inline int widened(const Bsr& A, int tpr) {
   const double mean = (double)A.nnzb / A.nbr;
   while (tpr < 32 && (int64_t)A.nbr * tpr < (int64_t)device_sms() * 16 * 32 && mean >= 2 * tpr) tpr *= 2;
@@ -118,7 +119,7 @@ void launch_g(const Bsr& A1, const G1& g1, const Bsr* A2, const T* x2, const Epi
   if (A2) { v2 = A2->vals<T>(); rp2 = A2->rowptr.p; ci2 = A2->colind.p; nnzb2 = A2->nnzb; }
   constexpr int per_sm = sizeof(T) == 4 ? kEarlyCtas : kEarlyCtas64;
   const bool early = tu.setup_depth == 0 && loads_early(blocks, rows_per_cta, tpr, per_sm);
-  // FP64 launches do not trigger, see common.cuh (21x11x10 FP64 solve 14.7 ms without, 16.4 with)
+  // FP64 launches do not trigger, see common.cuh (21x11x10 FP64 solve 16.0 ms without, 21.1 with)
   const int dep = (tu.setup_depth == 0 ? kDepBuilt : 0) |
                   (sizeof(T) == 4 && one_pass(rows_per_cta, tpr) ? kDepTrigger : 0);
   const int pf = tu.prefetch > 0 ? kPrefetchCap : 0;

@@ -38,7 +38,6 @@ template <class T> void vfma(int64_t n, const T* w, const T* x, T* y, cudaStream
 template <class Ti, class To> void cast(int64_t n, const Ti* x, To* y, cudaStream_t s);
 // out[0] = sum_i x_i y_i (FP64 accumulation), device result; partials has kRedBlocks doubles
 template <class T> void dot_dev(int64_t n, const T* x, const T* y, double* partials, double* out, cudaStream_t s);
-// host convenience: synchronous dot
 
 // Gram-Schmidt pieces.  V holds basis vectors of length n with leading dimension
 // ldv (vector i at V + i*ldv); the number of active vectors is read on the
