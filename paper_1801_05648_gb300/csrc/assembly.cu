@@ -49,9 +49,9 @@ namespace {
 template <int D, int PD> struct Sh;
 template <int PD> struct Sh<2, PD> {
   static constexpr int NQ2 = 9, NQ1 = PD ? 3 : 4, NL = 36 + NQ1, NQP = 9, NFP = 3;
-  static constexpr int JCELLS = 8;    // cells per CTA of the Jacobian: 36 units of a kind per cell,
+  static constexpr int JCELLS = 8;    // most cells per CTA of the Jacobian: 36 units of a kind per cell,
   static constexpr int JTHREADS = 288;   // 288 in all, one per thread
-  static constexpr int RCELLS = 28;   // cells per CTA of the residual: 252 of 256 threads hold a point
+  static constexpr int RCELLS = 28;   // ... of the residual: 252 of 256 threads hold a point
 };
 template <int PD> struct Sh<3, PD> {
   static constexpr int NQ2 = 27, NQ1 = PD ? 4 : 8, NL = 162 + NQ1, NQP = 27, NFP = 9;
@@ -230,7 +230,7 @@ __device__ __forceinline__ void read_F(const double* gu, double (&F)[D][D]) {
 }
 
 // ====================================================================== residual
-// One CTA takes RCELLS cells of a colour.  All threads interpolate (one scalar of one
+// One CTA takes up to RCELLS cells of a colour (cells_per_cta).  All threads interpolate (one scalar of one
 // point per step), then one thread per point forms the point fluxes, then one thread per
 // element row sums its test function over the points.  2D 256x128: about 3,000 FP64
 // instructions per cell.  256x128 P1disc: 0.37 ms.  An earlier form gave each cell a CTA of
@@ -248,7 +248,7 @@ struct ResSmem {
 };
 
 template <int D, int PD>
-__global__ void __launch_bounds__(kAsmThreads) k_residual(CellGeom geom, int64_t ncol, Tables T, Phys P,
+__global__ void __launch_bounds__(kAsmThreads) k_residual(CellGeom geom, int64_t ncol, int per, Tables T, Phys P,
                                                           const int* __restrict__ cell_dof,
                                                           const unsigned* __restrict__ cell_flags,
                                                           const unsigned char* __restrict__ row_fixed,
@@ -262,8 +262,8 @@ __global__ void __launch_bounds__(kAsmThreads) k_residual(CellGeom geom, int64_t
   static_assert(G0 + 1 == kFlux<D> && kFlux<D> <= R::kAll, "fluxes fit the raw slots");
   extern __shared__ __align__(16) unsigned char asm_smem[];
   ResSmem<D, PD>& S = *reinterpret_cast<ResSmem<D, PD>*>(asm_smem);
-  const int64_t k0 = (int64_t)blockIdx.x * E::RCELLS;
-  const int nc = (int)(ncol - k0 < E::RCELLS ? ncol - k0 : E::RCELLS);
+  const int64_t k0 = (int64_t)blockIdx.x * per;
+  const int nc = (int)(ncol - k0 < per ? ncol - k0 : per);
   const bool prev = P.theta != 1.0;
   const double dtt = P.dt * P.theta, dto = P.dt * (1.0 - P.theta), mu = P.rho_f * P.nu_f;
   for (int t = threadIdx.x; t < nc * NL; t += blockDim.x) {
@@ -447,7 +447,7 @@ __global__ void __launch_bounds__(kAsmThreads) k_residual(CellGeom geom, int64_t
 }
 
 // ====================================================================== Jacobian
-// One CTA takes JCELLS cells of a colour.  What the variations above need is tabulated
+// One CTA takes up to JCELLS cells of a colour (cells_per_cta).  What the variations above need is tabulated
 // in shared memory once per point (PT slots) and once per (point, trial node) (TR slots,
 // quadrature weight folded in).  A unit of work is one trial component (b, k) against
 // one test component i: a thread forms the unit's f0 and reference flux f1 at a line of
@@ -556,7 +556,7 @@ __device__ __forceinline__ int find_col(const int* __restrict__ ci, int len, int
 }
 
 template <int D, int PD>
-__global__ void __launch_bounds__(Sh<D, PD>::JTHREADS, 2) k_jacobian(CellGeom geom, int64_t ncol, Tables T,
+__global__ void __launch_bounds__(Sh<D, PD>::JTHREADS, 2) k_jacobian(CellGeom geom, int64_t ncol, int per, Tables T,
                                                              const __grid_constant__ Basis1 B, Phys P,
                                                              const int* __restrict__ cell_dof,
                                                              const unsigned* __restrict__ cell_flags,
@@ -578,8 +578,8 @@ __global__ void __launch_bounds__(Sh<D, PD>::JTHREADS, 2) k_jacobian(CellGeom ge
   JacSmem<D, PD>& S = *reinterpret_cast<JacSmem<D, PD>*>(asm_smem);
   // the last cells first: the solid ones, a third of a fluid cell's work, lie at the low end of
   // the last direction in the meshes of Sec. 6 and fill the SMs' last slots better
-  const int64_t k0 = (int64_t)(gridDim.x - 1 - blockIdx.x) * E::JCELLS;
-  const int nc = (int)(ncol - k0 < E::JCELLS ? ncol - k0 : E::JCELLS);
+  const int64_t k0 = (int64_t)(gridDim.x - 1 - blockIdx.x) * per;
+  const int nc = (int)(ncol - k0 < per ? ncol - k0 : per);
   const bool prev = P.theta != 1.0;
   const double dtt = P.dt * P.theta, mu = P.rho_f * P.nu_f;
   for (int t = threadIdx.x; t < nc * NL; t += blockDim.x) {
@@ -1196,6 +1196,15 @@ void for_colours(const Assembler& A, F&& f) {
   }
 }
 
+// Cells per CTA for a colour of cnt cells: as many as the tables take, but no more than leave every SM two
+// CTAs.  What a CTA's cells cost is the FP64 pipe of its SM: with full groups on a mesh of a few
+// hundred cells, a handful of SMs did all the work (14x7: Jacobian 517 us, now 257, residual 262, now 94; one
+// CTA per cell and column chunk, before the groups, took 390 and 170).
+inline int cells_per_cta(int64_t cnt, int most) {
+  const int64_t spread = (cnt + 2 * device_sms() - 1) / (2 * device_sms());
+  return (int)(spread < most ? spread : most);
+}
+
 template <int D, int PD>
 void run_residual(Assembler& A, const double* U, const double* Uold, double* out) {
   constexpr size_t sm = sizeof(ResSmem<D, PD>);
@@ -1204,8 +1213,9 @@ void run_residual(Assembler& A, const double* U, const double* Uold, double* out
     FSI_CUDA(cudaFuncSetAttribute(k_residual<D, PD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   });
   for_colours<D>(A, [&](const CellGeom& g, int64_t cnt) {
-    k_residual<D, PD><<<div_up(cnt, Sh<D, PD>::RCELLS), kAsmThreads, sm, A.s>>>(
-        g, cnt, A.T, A.phys, A.cell_dof.p, A.cell_flags.p, A.fixed.p, U, Uold, out, A.res.p);
+    const int per = cells_per_cta(cnt, Sh<D, PD>::RCELLS);
+    k_residual<D, PD><<<div_up(cnt, per), kAsmThreads, sm, A.s>>>(
+        g, cnt, per, A.T, A.phys, A.cell_dof.p, A.cell_flags.p, A.fixed.p, U, Uold, out, A.res.p);
   });
 }
 
@@ -1218,8 +1228,9 @@ void run_jacobian(Assembler& A, const double* U, const double* Uold, double* val
     FSI_CUDA(cudaFuncSetAttribute(k_jacobian<D, PD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   });
   for_colours<D>(A, [&](const CellGeom& g, int64_t cnt) {
-    k_jacobian<D, PD><<<div_up(cnt, Sh<D, PD>::JCELLS), Sh<D, PD>::JTHREADS, sm, A.s>>>(
-        g, cnt, A.T, A.B1, A.phys, A.cell_dof.p, A.cell_flags.p, A.rowptr.p, A.colind.p, A.fixed.p, U, Uold, vals,
+    const int per = cells_per_cta(cnt, Sh<D, PD>::JCELLS);
+    k_jacobian<D, PD><<<div_up(cnt, per), Sh<D, PD>::JTHREADS, sm, A.s>>>(
+        g, cnt, per, A.T, A.B1, A.phys, A.cell_dof.p, A.cell_flags.p, A.rowptr.p, A.colind.p, A.fixed.p, U, Uold, vals,
         A.res.p, reinterpret_cast<int*>(A.res.p + 2));
   });
 }

@@ -1,10 +1,11 @@
 """Calls at the edges of what the solver takes: product rows around the length of the SpGEMM
 table, aggregates larger than shared memory, empty classes of unknowns, too little device
-memory, a hierarchy that changes its shape, a device that was reset."""
+memory, a hierarchy that changes its shape, meshes of few cells, a device that was reset."""
 import contextlib
 import os
 import subprocess
 import sys
+import time
 
 import numpy as np
 import pytest
@@ -311,6 +312,50 @@ def test_coarse_launch_follows_the_hierarchy(flag, torch_cuda):
         assert np.linalg.norm(x.cpu().numpy() - want) <= 1e-10 * np.linalg.norm(want)
     S.check_device_errors()
     S.close()
+
+
+# cells per colour that give a CTA 1, 2, 3, 8 (Jacobian) and 1, 2, 3, 9, 28 (residual) cells, the last CTA fewer
+@pytest.mark.parametrize("cells", [(34, 35), (38, 37), (50, 49), (101, 99), (190, 188), (14, 15, 13)])
+def test_assembly_of_groups_of_cells(cells, torch_cuda):
+    """Entries within 1e-12 of the row's largest magnitude of the host assembly's, however many cells a CTA takes."""
+    torch = torch_cuda
+    import paper_1801_05648_gb300 as P
+    pb = fsigen.get_problem(fsigen.FSIConfig("a", len(cells), cells, theta=0.5))
+    U = pb.seeded_state(4, 5e-3)
+    asm = P.FSIAssembler.from_problem(pb)
+    u, uo = torch.tensor(U, device="cuda"), torch.tensor(0.9 * U, device="cuda")
+    R, J = torch.empty_like(u), torch.empty(pb.nnz, dtype=torch.float64, device="cuda")
+    asm.residual(u, uo, R)
+    asm.jacobian(u, uo, J)
+    Rh, Jh = pb.residual(U, 0.9 * U), pb.jacobian(U, 0.9 * U)
+    assert np.abs(R.cpu().numpy() - Rh).max() <= 1e-12 * np.abs(Rh).max()
+    big = np.maximum.reduceat(np.abs(Jh), pb.rowptr[:-1])
+    assert np.max(np.abs(J.cpu().numpy() - Jh) / np.repeat(big, np.diff(pb.rowptr))) <= 1e-12
+    asm.close()
+
+
+def test_assembly_of_a_small_mesh_is_spread_over_the_gpu(torch_cuda):
+    """98 cells, a fortieth of the work of 90x45, take less than four fifths of its time (launches and host
+    work are in both; in groups of the size that suits large meshes they took as long)."""
+    torch = torch_cuda
+    import paper_1801_05648_gb300 as P
+
+    def median(cells, call):
+        pb = fsigen.get_problem(fsigen.FSIConfig("a", 2, cells))
+        u = torch.tensor(pb.seeded_state(4, 5e-3), device="cuda")
+        out = torch.empty(pb.nnz if call == "jacobian" else pb.n, dtype=torch.float64, device="cuda")
+        asm = P.FSIAssembler.from_problem(pb)
+        run = getattr(asm, call)
+        times = []
+        for _ in range(40):
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            run(u, u, out)
+            times.append(time.perf_counter() - t)
+        asm.close()
+        return sorted(times[10:])[15]
+    for call in ("jacobian", "residual"):
+        assert median((14, 7), call) < 0.8 * median((90, 45), call), call
 
 
 # Everything a Newton correction calls, on the library alone (a process's PyTorch does not outlive a reset).
