@@ -1291,6 +1291,7 @@ void asm_create(Assembler& A, const fsi_asm_mesh& m, const fsi_asm_physics& p, v
   require(m.n > 0 && m.n < ((int64_t)1 << 31), "fsi_asm: n out of range");
   require(m.cell_dof && m.cell_flags && m.rowptr && m.colind && m.row_fixed, "fsi_asm: null mesh array");
   require(m.pressure == 0 || m.pressure == 1, "fsi_asm: pressure must be 0 (continuous Q1) or 1 (P1disc)");
+  note_device_context();
   A.dim = m.dim;
   A.pdisc = m.pressure;
   A.n = m.n;

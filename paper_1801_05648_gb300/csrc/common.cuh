@@ -148,20 +148,36 @@ inline unsigned long long cuda_context_id() {
   return reinterpret_cast<GetId>(e.id)(c, &v) == CUDA_SUCCESS ? v : 0;
 }
 
-// Runs setup(dev) once per device dev, on the current one, and again after the device was reset: a
-// kernel's function attributes, a __device__ variable's address and a stream belong to one CUDA
-// context of one device, so what was set up in one does not hold in another.  `done` is the call
-// site's record: the context that each device was set up in.  Two threads may both run it for the
+// cuda_context_id() + 1 of each device, as of the last solver context or assembler made on it (0: none yet).
+// The driver is asked there and not in once_per_device, which short calls pass through.
+inline std::atomic<unsigned long long>& device_context(int dev) {
+  static std::atomic<unsigned long long> id[64];
+  return id[dev];
+}
+inline unsigned long long note_device_context() {
+  int dev = 0;
+  FSI_CUDA(cudaGetDevice(&dev));
+  require(dev >= 0 && dev < 64, "device ordinal above 63");
+  const unsigned long long id = cuda_context_id() + 1;
+  device_context(dev).store(id, std::memory_order_release);
+  return id;
+}
+
+// Runs setup(dev) once per device dev, on the current one, and again for solver contexts and assemblers made
+// after the device was reset: a kernel's function attributes, a __device__ variable's address and a stream
+// belong to one CUDA context of one device, so what was set up in one does not hold in another.  `done` is the
+// call site's record: the CUDA context that each device was set up in.  Two threads may both run it for the
 // same device; it must be idempotent.
 struct OncePerDevice {
-  std::atomic<unsigned long long> context[64] = {};   // cuda_context_id() + 1, 0: not yet
+  std::atomic<unsigned long long> context[64] = {};   // as device_context, 0: not yet
 };
 template <class F>
 void once_per_device(OncePerDevice& done, F&& setup) {
   int dev = 0;
   FSI_CUDA(cudaGetDevice(&dev));
   require(dev >= 0 && dev < 64, "device ordinal above 63");
-  const unsigned long long now = cuda_context_id() + 1;
+  unsigned long long now = device_context(dev).load(std::memory_order_acquire);
+  if (now == 0) now = note_device_context();
   if (done.context[dev].load(std::memory_order_acquire) == now) return;
   setup(dev);
   done.context[dev].store(now, std::memory_order_release);

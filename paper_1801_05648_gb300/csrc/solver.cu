@@ -522,6 +522,7 @@ void context_setup(Context& C, const int64_t* rowptr, const int32_t* colind, con
   SetupPhase setup_phase(C.pool);
   auto t0 = clk::now();
   FSI_CUDA(cudaGetDevice(&C.device));
+  note_device_context();
   FSI_CUDA(cudaStreamCreateWithFlags(&C.s2, cudaStreamNonBlocking));
   FSI_CUDA(cudaEventCreateWithFlags(&C.ev_fork, cudaEventDisableTiming));
   FSI_CUDA(cudaEventCreateWithFlags(&C.ev_join, cudaEventDisableTiming));
