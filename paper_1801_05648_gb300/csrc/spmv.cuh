@@ -553,10 +553,11 @@ __global__ void __launch_bounds__(256) k_bsr_spmv(int nbr, int tpr, int rows_per
 }
 
 // The outer operator's rows: D velocity components of a node (D x D blocks, and D x 1 to the
-// pressures) and pressures (1 x D and 1 x 1), in one launch.  The first ctas_p CTAs take the
+// pressures) and pressures (1 x D and 1 x 1), in one launch.  The last ctas_p CTAs take the
 // pressure rows: few, long ones, which as a launch of their own wait on latency (10 us of the
-// 16x16 operator's 22, 14.6 of the 256x128 operator's 96) and here run beside the rest.  That pays on small
-// and mid-size systems; on 1024x512 one launch takes what the two took (1,258 us).  x is gathered with the
+// 16x16 operator's 22) and here fill the last wave.  256x128 91.5 us as two launches, 87 with the
+// pressure rows first, 82 with them last; 32x16x16 264 and 256; 512x256 333, 332 and 324.  1024x512 1,262, 1,286 and
+// 1,279: there the gathers by ordinary loads (see dep_wait in common.cuh) cost 2%.  x is gathered with the
 // default L2 policy: on the 1024x512 system evict-last gathers cut the DRAM traffic from 7.5 to 6.4 GB but made
 // the product 5% slower (it is bound by the FP64 pipe).
 struct RowClass {
@@ -573,14 +574,15 @@ __global__ void __launch_bounds__(256) k_operator_rows(const __grid_constant__ R
                                                        const double* xp, Epi<double, D> epi_v,
                                                        Epi<double, 1> epi_p) {
   const GatherX<double, D> g{xv};
-  if ((int)blockIdx.x < ctas_p)
+  const int ctas_v = (int)gridDim.x - ctas_p;
+  if ((int)blockIdx.x >= ctas_v)
     bsr_rows<double, 1, D, 1, Epi<double, 1>, GatherX<double, D>, 4, int, false, EARLY>(
-        blockIdx.x, P.nbr, P.tpr, P.rows_per_cta, prefetch, dep, P.ord2, P.rp1, P.ci1, P.v1, P.nnzb1, g, P.rp2, P.ci2,
-        P.v2, P.nnzb2, xp, epi_p);
+        blockIdx.x - ctas_v, P.nbr, P.tpr, P.rows_per_cta, prefetch, dep, P.ord2, P.rp1, P.ci1, P.v1, P.nnzb1, g, P.rp2,
+        P.ci2, P.v2, P.nnzb2, xp, epi_p);
   else
     bsr_rows<double, D, D, 1, Epi<double, D>, GatherX<double, D>, 4, int, false, EARLY>(
-        blockIdx.x - ctas_p, V.nbr, V.tpr, V.rows_per_cta, prefetch, dep, V.ord2, V.rp1, V.ci1, V.v1, V.nnzb1, g, V.rp2,
-        V.ci2, V.v2, V.nnzb2, xp, epi_v);
+        blockIdx.x, V.nbr, V.tpr, V.rows_per_cta, prefetch, dep, V.ord2, V.rp1, V.ci1, V.v1, V.nnzb1, g, V.rp2, V.ci2,
+        V.v2, V.nnzb2, xp, epi_v);
 }
 
 // ------------------------------------------------------------------ staged 2 x 2 FP32 steps
